@@ -175,6 +175,11 @@ int psattn_exact_measure(psattn_plan_t *plan, const void *Q, const void *K, cons
 int psattn_project_qkv(psattn_plan_t *plan, const void *X, const void *Wt, int32_t d_x,
                        const int32_t *lengths, void *Q, void *K, void *V, float *vbar,
                        void *workspace, size_t workspace_bytes, void *stream);
+/* The same call, which also writes zeros to the rows of Q, K and V at positions >= lengths[b]: for callers that want
+ * fresh buffers defined everywhere without a pass over them before the call. */
+int psattn_project_qkv_zeroed(psattn_plan_t *plan, const void *X, const void *Wt, int32_t d_x,
+                              const int32_t *lengths, void *Q, void *K, void *V, float *vbar,
+                              void *workspace, size_t workspace_bytes, void *stream);
 
 /* The output matrix of the attention module, which merges the heads (Sec. 2.2, Eq. 5: the module inside the
  * Conformer block; Sec. 3.1: its heads):  Y[b][t][n] = sum_h sum_e O[b][h][t][e] W_o^h[e][n].  All pointers device.
@@ -192,6 +197,10 @@ int psattn_project_qkv(psattn_plan_t *plan, const void *X, const void *Wt, int32
 int psattn_project_out(psattn_plan_t *plan, const void *O, const int32_t *sel_idx, const int32_t *lengths,
                        const void *Wot, int32_t d_y, void *Y, void *workspace, size_t workspace_bytes,
                        void *stream);
+/* The same call, which also writes zeros to the rows of Y at positions >= lengths[b]. */
+int psattn_project_out_zeroed(psattn_plan_t *plan, const void *O, const int32_t *sel_idx, const int32_t *lengths,
+                              const void *Wot, int32_t d_y, void *Y, void *workspace, size_t workspace_bytes,
+                              void *stream);
 
 /* Step (c) only (Sec. 3.2): top-u positions of M (fp32 [B][H][T_max]) among i < lengths[b]. */
 int psattn_select(psattn_plan_t *plan, const float *M, const int32_t *lengths,

@@ -1,5 +1,5 @@
-"""Thin ctypes binding of libpsattn.so: same names as include/psattn.h, argument marshalling
-only.  torch supplies device memory and streams; every step of the computation runs in the
+"""Thin binding of libpsattn.so: same names as include/psattn.h, argument marshalling only (ctypes for plans
+and host-side calls, the native module psattn_torch for the calls that launch kernels).  torch supplies device memory and streams; every step of the computation runs in the
 library's CUDA kernels.  There is no fallback: if the library cannot be loaded or a call
 fails, an exception is raised.
 """
@@ -22,7 +22,8 @@ EXPORTS = [
     "psattn_forward", "psattn_forward_with_selection", "psattn_measure", "psattn_exact_measure", "psattn_select",
     "psattn_mean_v", "psattn_attend_rows", "psattn_dense_forward", "psattn_read_status",
     "psattn_plan_enable_host_io", "psattn_forward_host", "psattn_mean_v_noalloc", "psattn_project_qkv",
-    "psattn_probe_gather", "psattn_project_out", "psattn_plan_debug_waits",
+    "psattn_probe_gather", "psattn_project_out", "psattn_plan_debug_waits", "psattn_project_qkv_zeroed",
+    "psattn_project_out_zeroed",
 ]
 
 
@@ -44,6 +45,14 @@ class PsattnError(RuntimeError):
 
 
 _lib = None
+_native = None
+
+# order of the addresses that the native module is given
+_NATIVE_ENTRIES = [
+    "psattn_forward", "psattn_forward_with_selection", "psattn_measure", "psattn_exact_measure", "psattn_project_qkv",
+    "psattn_project_qkv_zeroed", "psattn_project_out", "psattn_project_out_zeroed", "psattn_select", "psattn_mean_v",
+    "psattn_attend_rows", "psattn_dense_forward",
+]
 
 
 def library_path() -> str:
@@ -83,6 +92,8 @@ def load(build_if_missing: bool = True):
     lib.psattn_project_qkv.argtypes = [vp, vp, vp, i32, vp, vp, vp, vp, vp, vp, sz, vp]
     lib.psattn_mean_v.argtypes = [vp] * 5 + [sz, vp]
     lib.psattn_project_out.argtypes = [vp, vp, vp, vp, vp, i32, vp, vp, sz, vp]
+    lib.psattn_project_qkv_zeroed.argtypes = lib.psattn_project_qkv.argtypes
+    lib.psattn_project_out_zeroed.argtypes = lib.psattn_project_out.argtypes
     lib.psattn_attend_rows.argtypes = [vp] * 6 + [i32, vp, vp, sz, vp]
     lib.psattn_dense_forward.argtypes = [vp] * 7 + [sz, vp]
     lib.psattn_read_status.argtypes = [vp, vp, vp, ctypes.POINTER(ctypes.c_uint32)]
@@ -95,12 +106,28 @@ def load(build_if_missing: bool = True):
     return lib
 
 
+def _load_native():
+    """The native module (built with the library), bound to the entry points of the loaded library."""
+    global _native
+    if _native is None:
+        import importlib.machinery
+        import importlib.util
+        lib = load()
+        path = _build.build_native() if _build.native_needs_build() else _build.NATIVE
+        loader = importlib.machinery.ExtensionFileLoader("psattn_torch", path)
+        mod = importlib.util.module_from_spec(importlib.util.spec_from_loader("psattn_torch", loader))
+        loader.exec_module(mod)
+        mod.bind(_check, tuple(ctypes.cast(getattr(lib, n), ctypes.c_void_p).value for n in _NATIVE_ENTRIES))
+        _native = mod
+    return _native
+
+
 def _check(rc: int, plan=None):
     if rc != 0:
         lib = load()
         msg = lib.psattn_status_string(rc).decode()
         if plan is not None and rc == 6:
-            msg += " (cudaError %d)" % lib.psattn_last_cuda_error(plan)
+            msg += " (cudaError %d)" % lib.psattn_last_cuda_error(plan if isinstance(plan, ctypes.c_void_p) else ctypes.c_void_p(plan))
         raise PsattnError("psattn status %d: %s" % (rc, msg))
 
 
@@ -181,14 +208,18 @@ class Plan:
         self.u_max, self.U_max = um.value, Um.value
         nbytes = ctypes.c_size_t()
         _check(lib.psattn_workspace_bytes(h, ctypes.byref(nbytes)))
-        self.workspace_bytes = nbytes.value
-        self.workspace = torch.zeros(nbytes.value, dtype=torch.uint8, device="cuda")
+        self._workspace = torch.zeros(nbytes.value, dtype=torch.uint8, device="cuda")
+        self._workspace_bytes = nbytes.value
         self.B, self.H, self.T_max, self.d_head, self.idx_cols = B, H, T_max, d_head, idx_cols
+        self._call = _load_native().Caller(h.value, self._workspace.data_ptr(), nbytes.value, B, H, T_max, d_head,
+                                           self.u_max, int(d.dtype == PSATTN_BF16))
 
     def close(self):
         if getattr(self, "handle", None):
             self.lib.psattn_plan_destroy(self.handle)
             self.handle = None
+            if hasattr(self, "_call"):
+                self._call.close()
 
     def __del__(self):
         try:
@@ -196,105 +227,63 @@ class Plan:
         except Exception:
             pass
 
+    # the workspace may be replaced by a caller's own
+    @property
+    def workspace(self):
+        return self._workspace
+
+    @workspace.setter
+    def workspace(self, tensor):
+        self._workspace = tensor
+        self._call.set_workspace(tensor.data_ptr(), self._workspace_bytes)
+
+    @property
+    def workspace_bytes(self):
+        return self._workspace_bytes
+
+    @workspace_bytes.setter
+    def workspace_bytes(self, n):
+        self._workspace_bytes = n
+        self._call.set_workspace(self._workspace.data_ptr(), n)
+
     def _ws(self):
         return _ptr(self.workspace), ctypes.c_size_t(self.workspace_bytes)
 
-    # -- same names as the C entry points --------------------------------------------------
+    # -- same names as the C entry points; outputs left out are allocated -----------------------
     def psattn_forward(self, Q, K, V, lengths, sample_idx, O=None, sel_idx=None, M_out=None):
-        if O is None:
-            O = torch.empty((self.B, self.H, self.T_max, self.d_head), dtype=self.dtype, device=Q.device)
-        if sel_idx is None:
-            sel_idx = torch.empty((self.B, self.H, self.u_max), dtype=torch.int32, device=Q.device)
-        ws, n = self._ws()
-        _check(self.lib.psattn_forward(self.handle, _ptr(Q), _ptr(K), _ptr(V), _ptr(lengths),
-                                       _ptr(sample_idx), _ptr(O), _ptr(sel_idx), _ptr(M_out),
-                                       ws, n, _stream()), self.handle)
-        return O, sel_idx
+        return self._call.forward(Q, K, V, lengths, sample_idx, O, sel_idx, M_out)
 
     def psattn_forward_with_selection(self, Q, K, V, lengths, sel_idx_in, O=None):
-        if O is None:
-            O = torch.empty((self.B, self.H, self.T_max, self.d_head), dtype=self.dtype, device=Q.device)
-        ws, n = self._ws()
-        _check(self.lib.psattn_forward_with_selection(self.handle, _ptr(Q), _ptr(K), _ptr(V),
-                                                      _ptr(lengths), _ptr(sel_idx_in), _ptr(O),
-                                                      ws, n, _stream()), self.handle)
-        return O
+        return self._call.forward_with_selection(Q, K, V, lengths, sel_idx_in, O)
 
     def psattn_measure(self, Q, K, lengths, sample_idx, M_out=None):
-        if M_out is None:
-            M_out = torch.empty((self.B, self.H, self.T_max), dtype=torch.float32, device=Q.device)
-        ws, n = self._ws()
-        _check(self.lib.psattn_measure(self.handle, _ptr(Q), _ptr(K), _ptr(lengths),
-                                       _ptr(sample_idx), _ptr(M_out), ws, n, _stream()), self.handle)
-        return M_out
+        return self._call.measure(Q, K, lengths, sample_idx, M_out)
 
     def psattn_exact_measure(self, Q, K, lengths, M_out=None):
-        if M_out is None:
-            M_out = torch.empty((self.B, self.H, self.T_max), dtype=torch.float32, device=Q.device)
-        ws, n = self._ws()
-        _check(self.lib.psattn_exact_measure(self.handle, _ptr(Q), _ptr(K), _ptr(lengths), _ptr(M_out),
-                                             ws, n, _stream()), self.handle)
-        return M_out
+        return self._call.exact_measure(Q, K, lengths, M_out)
 
     def psattn_project_qkv(self, X, Wt, lengths=None, Q=None, K=None, V=None, vbar=None):
         """Q, K, V = X W_q, X W_k, X W_v in the attention layout; X [B, T_max, d_x], Wt [3, H*64, d_x].
-        Rows at padded positions of freshly allocated outputs are zero (the kernel does not write them)."""
-        outs = []
-        for t in (Q, K, V):
-            if t is None:
-                t = torch.zeros((self.B, self.H, self.T_max, self.d_head), dtype=self.dtype, device=X.device)
-            outs.append(t)
-        ws, n = self._ws()
-        _check(self.lib.psattn_project_qkv(self.handle, _ptr(X), _ptr(Wt), int(X.shape[-1]), _ptr(lengths),
-                                           _ptr(outs[0]), _ptr(outs[1]), _ptr(outs[2]), _ptr(vbar), ws, n,
-                                           _stream()), self.handle)
-        return tuple(outs)
+        Rows at padded positions of freshly allocated outputs are zero, those of given ones are not written."""
+        return self._call.project_qkv(X, Wt, X.shape[-1], lengths, Q, K, V, vbar)
 
     def psattn_project_out(self, O, sel_idx, lengths, Wot, Y=None):
         """Y[b, t, :] = sum_h O[b, h, t, :] W_o^h; Wot [d_y, H*64] holds W_o transposed.  With sel_idx (the index
         sets psattn_forward wrote for this O) the broadcast-plus-corrections form runs, with None the dense product.
-        Rows at padded positions of a freshly allocated Y are zero (the kernels do not write them)."""
-        d_y = int(Wot.shape[0])
-        if Y is None:
-            Y = torch.zeros((self.B, self.T_max, d_y), dtype=self.dtype, device=O.device)
-        ws, n = self._ws()
-        _check(self.lib.psattn_project_out(self.handle, _ptr(O), _ptr(sel_idx), _ptr(lengths), _ptr(Wot), d_y,
-                                           _ptr(Y), ws, n, _stream()), self.handle)
-        return Y
+        Rows at padded positions of a freshly allocated Y are zero, those of a given one are not written."""
+        return self._call.project_out(O, sel_idx, lengths, Wot, Wot.shape[0], Y)
 
     def psattn_select(self, M, lengths, sel_idx=None):
-        if sel_idx is None:
-            sel_idx = torch.empty((self.B, self.H, self.u_max), dtype=torch.int32, device=M.device)
-        ws, n = self._ws()
-        _check(self.lib.psattn_select(self.handle, _ptr(M), _ptr(lengths), _ptr(sel_idx), ws, n,
-                                      _stream()), self.handle)
-        return sel_idx
+        return self._call.select(M, lengths, sel_idx)
 
     def psattn_mean_v(self, V, lengths, vbar=None):
-        if vbar is None:
-            vbar = torch.empty((self.B, self.H, self.d_head), dtype=torch.float32, device=V.device)
-        ws, n = self._ws()
-        _check(self.lib.psattn_mean_v(self.handle, _ptr(V), _ptr(lengths), _ptr(vbar), ws, n,
-                                      _stream()), self.handle)
-        return vbar
+        return self._call.mean_v(V, lengths, vbar)
 
     def psattn_attend_rows(self, Q, K, V, lengths, row_idx, out=None):
-        n_rows = int(row_idx.shape[-1])
-        if out is None:
-            out = torch.empty((self.B, self.H, n_rows, self.d_head), dtype=torch.float32, device=Q.device)
-        ws, n = self._ws()
-        _check(self.lib.psattn_attend_rows(self.handle, _ptr(Q), _ptr(K), _ptr(V), _ptr(lengths),
-                                           _ptr(row_idx), n_rows, _ptr(out), ws, n, _stream()),
-               self.handle)
-        return out
+        return self._call.attend_rows(Q, K, V, lengths, row_idx, row_idx.shape[-1], out)
 
     def psattn_dense_forward(self, Q, K, V, lengths, O=None):
-        if O is None:
-            O = torch.empty((self.B, self.H, self.T_max, self.d_head), dtype=self.dtype, device=Q.device)
-        ws, n = self._ws()
-        _check(self.lib.psattn_dense_forward(self.handle, _ptr(Q), _ptr(K), _ptr(V), _ptr(lengths),
-                                             _ptr(O), ws, n, _stream()), self.handle)
-        return O
+        return self._call.dense_forward(Q, K, V, lengths, O)
 
     def psattn_read_status(self) -> int:
         bits = ctypes.c_uint32()

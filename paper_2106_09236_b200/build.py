@@ -8,6 +8,8 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libpsattn.so")
+NATIVE = os.path.join(HERE, "psattn_torch.so")       # the native side of the Python binding (a CPython module)
+NATIVE_SOURCE = os.path.join(CSRC, "psattn_torch.cpp")
 SOURCES = ["psattn_api.cu", "psattn_staged.cu", "psattn_noalloc.cu", "psattn_attend_tc.cu", "psattn_measure_mma.cu", "psattn_measure_shared.cu", "psattn_exact_measure.cu", "psattn_project.cu", "psattn_attend64.cu", "psattn_fused.cu", "psattn_probe.cu", "psattn_project_out.cu"]
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -58,6 +60,31 @@ def build(force: bool = False, verbose: bool = False, phase_stamps: bool = False
     return LIB
 
 
+def native_needs_build() -> bool:
+    return not os.path.exists(NATIVE) or os.path.getmtime(NATIVE_SOURCE) > os.path.getmtime(NATIVE)
+
+
+def build_native(verbose: bool = False) -> str:
+    """Builds the module that marshals torch tensors into the C calls (g++ against torch's headers; no CUDA code)."""
+    import sysconfig
+
+    import torch
+    root = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(_nvcc())) if os.path.isabs(_nvcc()) else "/usr/local/cuda"
+    inc = [os.path.join(root, "include"), os.path.join(root, "include", "torch", "csrc", "api", "include"),
+           sysconfig.get_paths()["include"], os.path.join(cuda, "include")]
+    tmp = NATIVE + ".tmp.%d" % os.getpid()
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI), *["-I" + i for i in inc],
+           NATIVE_SOURCE, "-o", tmp, "-L" + os.path.join(root, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10",
+           "-lc10_cuda", "-Wl,-rpath," + os.path.join(root, "lib")]
+    if verbose:
+        print(" ".join(cmd), file=sys.stderr)
+    subprocess.check_call(cmd)
+    os.replace(tmp, NATIVE)
+    return NATIVE
+
+
 def _build_variant(name: str, extra: list, suffix: str, link: list = ()) -> str:
     out = os.path.join(HERE, name)
     objs = []
@@ -73,3 +100,5 @@ def _build_variant(name: str, extra: list, suffix: str, link: list = ()) -> str:
 
 if __name__ == "__main__":
     print(build(force="--force" in sys.argv, verbose="-v" in sys.argv, nvtx="--nvtx" in sys.argv))
+    if "--force" in sys.argv or native_needs_build():
+        print(build_native(verbose="-v" in sys.argv))

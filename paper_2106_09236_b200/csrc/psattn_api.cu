@@ -502,10 +502,9 @@ extern "C" int psattn_exact_measure(psattn_plan_t *plan, const void *Q, const vo
     return PSATTN_OK;
 }
 
-extern "C" int psattn_project_qkv(psattn_plan_t *plan, const void *X, const void *Wt, int32_t d_x,
-                                  const int32_t *lengths, void *Q, void *K, void *V, float *vbar,
-                                  void *workspace, size_t workspace_bytes, void *stream) {
-    PSATTN_RANGE();
+static int project_qkv(psattn_plan_t *plan, int zero_pad, const void *X, const void *Wt, int32_t d_x,
+                       const int32_t *lengths, void *Q, void *K, void *V, float *vbar, void *workspace,
+                       size_t workspace_bytes, void *stream) {
     if (!plan || !X || !Wt || !Q || !K || !V) return PSATTN_ERR_NULL;
     if (d_x < 1 || d_x > (1 << 20)) return PSATTN_ERR_BAD_DESC;
     if (!aligned16(X) || !aligned16(Wt) || !aligned16(Q) || !aligned16(K) || !aligned16(V)) return PSATTN_ERR_MISALIGNED;
@@ -513,15 +512,28 @@ extern "C" int psattn_project_qkv(psattn_plan_t *plan, const void *X, const void
     if (rc) return rc;
     const psattn_desc_t &d = plan->desc;
     Geom g = make_geom(plan, lengths, workspace);
-    PSATTN_CU(launch_project_qkv(d.dtype, d.path == PSATTN_PATH_STAGED, g, d_x, X, Wt, Q, K, V, vbar,
+    PSATTN_CU(launch_project_qkv(d.dtype, d.path == PSATTN_PATH_STAGED, zero_pad, g, d_x, X, Wt, Q, K, V, vbar,
                                  ws_at<float>(workspace, plan->off_pvsum), static_cast<cudaStream_t>(stream)));
     return PSATTN_OK;
 }
 
-extern "C" int psattn_project_out(psattn_plan_t *plan, const void *O, const int32_t *sel_idx, const int32_t *lengths,
-                                  const void *Wot, int32_t d_y, void *Y, void *workspace, size_t workspace_bytes,
-                                  void *stream) {
+extern "C" int psattn_project_qkv(psattn_plan_t *plan, const void *X, const void *Wt, int32_t d_x,
+                                  const int32_t *lengths, void *Q, void *K, void *V, float *vbar,
+                                  void *workspace, size_t workspace_bytes, void *stream) {
     PSATTN_RANGE();
+    return project_qkv(plan, 0, X, Wt, d_x, lengths, Q, K, V, vbar, workspace, workspace_bytes, stream);
+}
+
+extern "C" int psattn_project_qkv_zeroed(psattn_plan_t *plan, const void *X, const void *Wt, int32_t d_x,
+                                         const int32_t *lengths, void *Q, void *K, void *V, float *vbar,
+                                         void *workspace, size_t workspace_bytes, void *stream) {
+    PSATTN_RANGE();
+    return project_qkv(plan, 1, X, Wt, d_x, lengths, Q, K, V, vbar, workspace, workspace_bytes, stream);
+}
+
+static int project_out(psattn_plan_t *plan, int zero_pad, const void *O, const int32_t *sel_idx,
+                       const int32_t *lengths, const void *Wot, int32_t d_y, void *Y, void *workspace,
+                       size_t workspace_bytes, void *stream) {
     if (!plan || !O || !Wot || !Y) return PSATTN_ERR_NULL;
     if (d_y < 1 || d_y > (1 << 20)) return PSATTN_ERR_BAD_DESC;
     if (!aligned16(O) || !aligned16(Wot) || !aligned16(Y)) return PSATTN_ERR_MISALIGNED;
@@ -531,10 +543,24 @@ extern "C" int psattn_project_out(psattn_plan_t *plan, const void *O, const int3
     Geom g = make_geom(plan, lengths, workspace);
     // the shortcut needs Eq. 12's structure with the mean(V) fill; any other O goes through the dense product
     const int mode = d.path == PSATTN_PATH_STAGED ? 2 : (sel_idx != nullptr && d.fill_mode == PSATTN_FILL_MEAN_V ? 0 : 1);
-    cudaError_t e = launch_project_out(d.dtype, mode, g, d_y, O, sel_idx, Wot, Y, static_cast<cudaStream_t>(stream));
+    cudaError_t e = launch_project_out(d.dtype, mode, zero_pad, g, d_y, O, sel_idx, Wot, Y, static_cast<cudaStream_t>(stream));
     if (e == cudaErrorNotSupported) return PSATTN_ERR_UNSUPPORTED;
     PSATTN_CU(e);
     return PSATTN_OK;
+}
+
+extern "C" int psattn_project_out(psattn_plan_t *plan, const void *O, const int32_t *sel_idx, const int32_t *lengths,
+                                  const void *Wot, int32_t d_y, void *Y, void *workspace, size_t workspace_bytes,
+                                  void *stream) {
+    PSATTN_RANGE();
+    return project_out(plan, 0, O, sel_idx, lengths, Wot, d_y, Y, workspace, workspace_bytes, stream);
+}
+
+extern "C" int psattn_project_out_zeroed(psattn_plan_t *plan, const void *O, const int32_t *sel_idx,
+                                         const int32_t *lengths, const void *Wot, int32_t d_y, void *Y,
+                                         void *workspace, size_t workspace_bytes, void *stream) {
+    PSATTN_RANGE();
+    return project_out(plan, 1, O, sel_idx, lengths, Wot, d_y, Y, workspace, workspace_bytes, stream);
 }
 
 extern "C" int psattn_select(psattn_plan_t *plan, const float *M, const int32_t *lengths,

@@ -49,6 +49,7 @@ struct ProjArgs {
     const int *lengths;
     float *vpart;                                 // [B][tiles_per_seq][4][H][64] column sums of V per 32 rows, or null
     unsigned *status;
+    int zero_pad;                                 // rows at positions >= the length are written as zeros (else not written)
 };
 
 __device__ __forceinline__ int proj_len(const ProjArgs &a, int b) {
@@ -157,7 +158,20 @@ __global__ void __launch_bounds__(kPjThreads, 1) k_project_qkv(ProjArgs a, const
             const int n = tile % a.n_tiles_n, m = tile / a.n_tiles_n;
             const int b = m / a.tiles_per_seq, tt = m % a.tiles_per_seq;
             const int L = proj_len(a, b);
-            if (tt * kPjM >= L) continue;
+            if (tt * kPjM >= L) {
+                if (a.zero_pad) {                              // a tile of padding: no product, 64 columns = one row of 8 x 16 bytes
+                    for (int gc = n * (kPjN / 64); gc < min(a.n_blocks, (n + 1) * (kPjN / 64)); ++gc) {
+                        const int role = gc / a.H, h = gc - role * a.H;
+                        const long long *st = role == 0 ? a.qs : (role == 1 ? a.ks : a.vs);
+                        __nv_bfloat16 *base = (role == 0 ? a.Q : (role == 1 ? a.K : a.V)) + (long long)b * st[0] + (long long)h * st[1];
+                        for (int rr = lane >> 3; rr < 32; rr += 4) {
+                            const int tr = tt * kPjM + quarter * 32 + rr;
+                            if (tr < a.T) reinterpret_cast<uint4 *>(base + (long long)tr * st[2])[lane & 7] = make_uint4(0u, 0u, 0u, 0u);
+                        }
+                    }
+                }
+                continue;
+            }
             const uint32_t acc = tc & 1u, aph = (tc >> 1) & 1u;
             const bool mine = !*abort_flag && mbar_wait(&acc_full[acc], aph);
             uint32_t landed;                                   // the four drain warps decide together (they meet at
@@ -202,6 +216,7 @@ __global__ void __launch_bounds__(kPjThreads, 1) k_project_qkv(ProjArgs a, const
                     const int tr = tt * kPjM + quarter * 32 + rr;
                     const uint4 val = stage[rr * 8 + (c ^ (rr & 7))];
                     if (tr < L) reinterpret_cast<uint4 *>(base + (long long)tr * st[2])[c] = val;
+                    else if (a.zero_pad && tr < a.T) reinterpret_cast<uint4 *>(base + (long long)tr * st[2])[c] = make_uint4(0u, 0u, 0u, 0u);
                 }
                 if (role == 2 && a.vpart != nullptr) {
                     // column sums of this block over the warp's valid rows, from the values as stored (bf16):
@@ -280,12 +295,13 @@ __global__ void __launch_bounds__(64) k_project_simt(ProjArgs a, const DT *__res
                                                      DT *Q, DT *K, DT *V) {
     const int e = threadIdx.x, gc = blockIdx.y;
     const int b = blockIdx.x / a.T, t = blockIdx.x % a.T;
-    if (t >= proj_len(a, b)) return;
+    const bool valid = t < proj_len(a, b);
+    if (!valid && !a.zero_pad) return;
     const int role = gc / a.H, h = gc - role * a.H;
     const DT *x = X + ((long long)b * a.T + t) * a.dx;
     const DT *w = Wt + ((long long)gc * 64 + e) * a.dx;
     float acc = 0.f;
-    for (int k = 0; k < a.dx; ++k) acc = fmaf((float)x[k], (float)w[k], acc);
+    for (int k = 0; valid && k < a.dx; ++k) acc = fmaf((float)x[k], (float)w[k], acc);
     const long long *st = role == 0 ? a.qs : (role == 1 ? a.ks : a.vs);
     DT *base = role == 0 ? Q : (role == 1 ? K : V);
     base[(long long)b * st[0] + (long long)h * st[1] + (long long)t * st[2] + e] = (DT)acc;
@@ -328,8 +344,8 @@ size_t project_vpart_floats(int B, int H, int T) { return (size_t)B * ((T + kPjM
 // dtype 0 = bf16, 1 = fp32.  X [B][T][dx], Wt [3][H*64][dx], outputs with g.qs / g.ks / g.vs strides.
 // vbar (optional) fp32 [B][H][64]; vpart = scratch of project_vpart_floats() floats (needed with vbar on the
 // tensor-core path).  force_simt keeps bf16 inputs off the tensor cores.
-cudaError_t launch_project_qkv(int dtype, int force_simt, const Geom &g, int dx, const void *X, const void *Wt, void *Q,
-                               void *K, void *V, float *vbar, float *vpart, cudaStream_t st) {
+cudaError_t launch_project_qkv(int dtype, int force_simt, int zero_pad, const Geom &g, int dx, const void *X, const void *Wt,
+                               void *Q, void *K, void *V, float *vbar, float *vpart, cudaStream_t st) {
     if (g.B * g.H == 0) return cudaSuccess;
     ProjArgs a;
     a.B = g.B; a.H = g.H; a.T = g.T; a.dx = dx;
@@ -339,7 +355,7 @@ cudaError_t launch_project_qkv(int dtype, int force_simt, const Geom &g, int dx,
     a.n_tiles = g.B * a.tiles_per_seq * a.n_tiles_n;
     for (int k = 0; k < 3; ++k) { a.qs[k] = g.qs[k]; a.ks[k] = g.ks[k]; a.vs[k] = g.vs[k]; }
     a.Q = (__nv_bfloat16 *)Q; a.K = (__nv_bfloat16 *)K; a.V = (__nv_bfloat16 *)V;
-    a.lengths = g.lengths; a.status = g.status;
+    a.lengths = g.lengths; a.status = g.status; a.zero_pad = zero_pad;
     a.vpart = vbar ? vpart : nullptr;
     EncodeTiledFnP enc = proj_encode_fn();
     if (dtype == 0 && !force_simt && enc && dx % 8 == 0 && (vbar == nullptr || vpart != nullptr)) {
@@ -406,7 +422,7 @@ bool make_rows_map(CUtensorMap *map, const void *base, const Geom &g, const long
 // attention layout (slab kb = head kb, fetched through a 4-D tensor map of O), the 64-column blocks of Y
 // standing where the heads of one role stand for the projections.  bf16, dy a multiple of 64.
 // cudaErrorNotSupported: no tensor map for the layout.
-cudaError_t launch_project_out_dense(const Geom &g, int dy, const void *O, const void *Wot, void *Y, cudaStream_t st) {
+cudaError_t launch_project_out_dense(const Geom &g, int zero_pad, int dy, const void *O, const void *Wot, void *Y, cudaStream_t st) {
     if (g.B * g.H == 0) return cudaSuccess;
     EncodeTiledFnP enc = proj_encode_fn();
     if (!enc || dy % 64 != 0 || dy < 64) return cudaErrorNotSupported;
@@ -420,7 +436,7 @@ cudaError_t launch_project_out_dense(const Geom &g, int dy, const void *O, const
     const long long ys[3] = {(long long)g.T * dy, 64, dy};
     for (int k = 0; k < 3; ++k) { a.qs[k] = ys[k]; a.ks[k] = ys[k]; a.vs[k] = ys[k]; }
     a.Q = (__nv_bfloat16 *)Y; a.K = nullptr; a.V = nullptr;
-    a.lengths = g.lengths; a.status = g.status; a.vpart = nullptr;
+    a.lengths = g.lengths; a.status = g.status; a.vpart = nullptr; a.zero_pad = zero_pad;
     CUtensorMap tmX, tmW;
     int pos[3];
     if (!make_rows_map(&tmX, O, g, g.os, kPjM, 1, pos)) return cudaErrorNotSupported;

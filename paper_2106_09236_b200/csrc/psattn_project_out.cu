@@ -33,6 +33,7 @@ struct OutArgs {
     const int *sel, *lengths;
     __nv_bfloat16 *Y;
     unsigned *status;
+    int zero_pad;                // rows at positions >= the length are written as zeros (else not written)
 };
 
 __host__ __device__ inline uint32_t po_w_pitch(int H) { return (uint32_t)(H * 64 + 8) * 2u; }   // bytes per weight row
@@ -71,6 +72,9 @@ __global__ void __launch_bounds__(kPoThreads, 1) k_project_out_rows(OutArgs a) {
     int L = a.lengths ? a.lengths[b] : a.T;
     if (L < 0 || L > a.T) { if (tid == 0) atomicOr(a.status, kStatusLenClamped); L = L < 0 ? 0 : a.T; }
     const int t0 = chunk * a.t_chunk, t1 = min(t0 + a.t_chunk, L);
+    if (a.zero_pad && n0 + (tid & 7) * 8 < a.dy)
+        for (int i = max(t1, t0) + (tid >> 3); i < min(t0 + a.t_chunk, a.T); i += kPoThreads / 8)
+            reinterpret_cast<uint4 *>(a.Y + ((size_t)b * a.T + i) * a.dy + n0)[tid & 7] = make_uint4(0u, 0u, 0u, 0u);
     if (t0 >= L) return;
 
     // the weight slice: rows n0 .. n0 + 63 of Wot (zeros past dy), H * 64 bf16 each
@@ -304,9 +308,9 @@ __global__ void __launch_bounds__(128) k_project_out_simt(OutArgs a, const DT *_
     pdl_enter();
     int L = a.lengths ? a.lengths[b] : a.T;
     if (L < 0 || L > a.T) { if (threadIdx.x == 0) atomicOr(a.status, kStatusLenClamped); L = L < 0 ? 0 : a.T; }
-    if (t >= L || n >= a.dy) return;
+    if (n >= a.dy || (t >= L && !a.zero_pad)) return;
     float acc = 0.f;
-    for (int h = 0; h < a.H; ++h) {
+    for (int h = 0; t < L && h < a.H; ++h) {
         const DT *o = O + (long long)b * a.os[0] + (long long)h * a.os[1] + (long long)t * a.os[2];
         const DT *w = Wot + ((size_t)n * a.H + h) * 64;
         for (int e = 0; e < 64; ++e) acc = fmaf((float)o[e], (float)w[e], acc);
@@ -314,18 +318,18 @@ __global__ void __launch_bounds__(128) k_project_out_simt(OutArgs a, const DT *_
     Y[((size_t)b * a.T + t) * a.dy + n] = (DT)acc;
 }
 
-cudaError_t launch_project_out_dense(const Geom &g, int dy, const void *O, const void *Wot, void *Y, cudaStream_t st);
+cudaError_t launch_project_out_dense(const Geom &g, int zero_pad, int dy, const void *O, const void *Wot, void *Y, cudaStream_t st);
 
 // mode 0: pick (shortcut when an index set is given and the shape fits, else the dense GEMM, else one thread
 // per element); 1: never the shortcut; 2: one thread per element.
-cudaError_t launch_project_out(int dtype, int mode, const Geom &g, int dy, const void *O, const int *sel, const void *Wot,
-                               void *Y, cudaStream_t st) {
+cudaError_t launch_project_out(int dtype, int mode, int zero_pad, const Geom &g, int dy, const void *O, const int *sel,
+                               const void *Wot, void *Y, cudaStream_t st) {
     if (g.B * g.H == 0 || dy == 0) return cudaSuccess;
     OutArgs a;
     a.B = g.B; a.H = g.H; a.T = g.T; a.dy = dy; a.u_max = g.u_max;
     for (int k = 0; k < 3; ++k) a.os[k] = g.os[k];
     a.O = (const __nv_bfloat16 *)O; a.Wot = (const __nv_bfloat16 *)Wot; a.Y = (__nv_bfloat16 *)Y;
-    a.sel = sel; a.lengths = g.lengths; a.status = g.status;
+    a.sel = sel; a.lengths = g.lengths; a.status = g.status; a.zero_pad = zero_pad;
     a.t_chunk = 0; a.max_slots = 0; a.max_pairs = 0;
     if (dtype == 0 && mode == 0 && sel != nullptr && g.u_max <= kPoMaxRows && g.H <= 32 && dy % 8 == 0) {
         const int sms = device_sm_count();
@@ -357,7 +361,7 @@ cudaError_t launch_project_out(int dtype, int mode, const Geom &g, int dy, const
         }
     }
     if (dtype == 0 && mode != 2) {
-        cudaError_t e = launch_project_out_dense(g, dy, O, Wot, Y, st);
+        cudaError_t e = launch_project_out_dense(g, zero_pad, dy, O, Wot, Y, st);
         if (e != cudaErrorNotSupported) return e;
     }
     if (g.T > 65535 || g.B > 65535) return cudaErrorNotSupported;
