@@ -459,8 +459,8 @@ extern "C" int psattn_forward_with_selection(psattn_plan_t *plan, const void *Q,
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const psattn_desc_t &d = plan->desc;
     Geom g = make_geom(plan, lengths, workspace);
-    if (d.dtype == PSATTN_BF16 && d.path != PSATTN_PATH_STAGED && d.B * d.H >= device_sm_count() / 2) {
-        // one kernel for steps (d)+(e), one CTA per unit: where the units cover at least half of the SMs
+    if (d.dtype == PSATTN_BF16 && d.path != PSATTN_PATH_STAGED) {
+        // one kernel for steps (d)+(e): one CTA per unit, or a cluster of CTAs where the units are few
         cudaError_t e = launch_forward_fused(g, plan->U_max, d.fill_mode == PSATTN_FILL_OWN_V, Q, K, V, nullptr, O,
                                              nullptr, nullptr, sel_idx_in, st);
         if (e == cudaSuccess) return PSATTN_OK;

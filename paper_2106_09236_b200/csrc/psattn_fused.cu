@@ -13,6 +13,8 @@
 // 1 and 2 are skipped and the kernel is steps (d)+(e) in one launch.
 // HBM traffic is the algorithmic minimum: Q, K, V read once (K a second time out of L2), O
 // written once.  M~ never leaves the SM unless the caller asks for it.
+#include <atomic>
+
 #include "psattn_attend64.cuh"
 #include "psattn_launch.h"
 #include "psattn_measure_mma.cuh"
@@ -24,23 +26,82 @@ using namespace sm100;
 
 constexpr int kFusedThreads = 512;       // warp 0: control; warps 4-7, 8-11: attention warpgroups; all 16 warps measure
 
+#ifdef PSATTN_PHASE_STAMPS
+constexpr size_t kFusedMaxSmem = 226 * 1024;  // the stamps' static bytes push the dynamic memory to the next 1024-byte boundary
+#else
+constexpr size_t kFusedMaxSmem = 227 * 1024;
+#endif
+
 struct FusedArgs {
     uint32_t k_bytes, stage_bytes;       // measure phase: resident keys, one staging buffer
     uint32_t off_persist;                // M~, selection, flags: live through all phases
     int pos_t, pos_h, pos_b;             // TMA coordinate slots (same for the three maps)
     int own_v;                           // fill with the query's own value row instead of mean(V)
     int by_length;                       // CTAs take the sequences in descending order of length
+    int split;                           // CTAs per unit (one thread-block cluster): 1, 2, 4 or 8
+    int m_floats;                        // floats of the M~ array (0 with a given index set)
     const int *sel_in;                   // non-null: a given index set [unit][u_max] replaces steps (a)-(c)
 };
 
-struct FusedPersist {                    // at smem + off_persist + 4 * T (after the M~ array)
+struct FusedPersist {                    // at smem + off_persist, after the M~ array and the flags
     SelectScratch select;
     int sel[kA64MaxRows];
     float vbar[kD];
     uint64_t bar;
     uint32_t tmem_slot;
+    int b_ranked;
 };
 
+__host__ __device__ inline size_t fused_arrays_bytes(int m_floats, int T) { return ((size_t)4 * m_floats + T + 127) / 128 * 128; }
+
+// ---- the CTAs of a unit (a.split > 1): one thread-block cluster -----------------------------------------
+__device__ __forceinline__ void cluster_arrive() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t peer_addr(uint32_t addr, int rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void peer_store(uint32_t addr, float v) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
+}
+__device__ __forceinline__ float peer_load(uint32_t addr) {
+    float v;
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+    return v;
+}
+// Column c of row r over all CTAs of the unit: the states (m, l, acc) that every CTA left at `states` in its shared
+// memory (66 floats per row) merged in rank order; returns acc / l.
+template <int SPLIT>
+__device__ __forceinline__ float merge_states_n(uint32_t states, int r, int c) {
+    float m[SPLIT], l[SPLIT], a[SPLIT];
+#pragma unroll
+    for (int x = 0; x < SPLIT; ++x) {                          // all loads in flight together
+        const uint32_t p = peer_addr(states + (uint32_t)r * 264u, x);
+        m[x] = peer_load(p); l[x] = peer_load(p + 4u); a[x] = peer_load(p + 8u + 4u * (uint32_t)c);
+    }
+    float mw = -INFINITY, lw = 0.f, aw = 0.f;
+#pragma unroll
+    for (int x = 0; x < SPLIT; ++x) mw = fmaxf(mw, m[x]);
+#pragma unroll
+    for (int x = 0; x < SPLIT; ++x) {
+        const float f = l[x] > 0.f ? fast_exp2(m[x] - mw) : 0.f;
+        lw += l[x] * f; aw += a[x] * f;
+    }
+    return lw > 0.f ? aw / lw : 0.f;
+}
+__device__ __forceinline__ float merge_states(int split, uint32_t states, int r, int c) {
+    return split == 8 ? merge_states_n<8>(states, r, c) : split == 4 ? merge_states_n<4>(states, r, c) : merge_states_n<2>(states, r, c);
+}
+
+// SPLIT: the unit is shared by the a.split > 1 CTAs of a thread-block cluster.
+template <bool SPLIT>
 __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
     Geom g, FusedArgs a, const __nv_bfloat16 *__restrict__ Q, const __nv_bfloat16 *__restrict__ V,
     const int *__restrict__ sidx, __nv_bfloat16 *__restrict__ O, int *__restrict__ sel_out, float *__restrict__ M_out,
@@ -49,8 +110,9 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
     extern __shared__ __align__(1024) uint8_t smem[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     float *M_s = reinterpret_cast<float *>(smem + a.off_persist);
-    unsigned char *chosen = reinterpret_cast<unsigned char *>(M_s + g.T);
-    FusedPersist &P = *reinterpret_cast<FusedPersist *>(smem + a.off_persist + ((5 * (size_t)g.T + 127) / 128) * 128);
+    unsigned char *chosen = reinterpret_cast<unsigned char *>(M_s + a.m_floats);
+    FusedPersist &P = *reinterpret_cast<FusedPersist *>(smem + a.off_persist + fused_arrays_bytes(a.m_floats, g.T));
+    const int split = SPLIT ? a.split : 1, part = SPLIT ? (int)(blockIdx.x % split) : 0;   // clusters are consecutive blocks
 
     if ((smem_u32(smem) & 1023u) != 0u) {                      // swizzled tiles need a 1024-byte base
         if (tid == 0) atomicOr(g.status, kStatusWaitExpired);
@@ -63,15 +125,15 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
     // The trigger comes after this CTA's TMEM allocation (below, behind the barrier that publishes the slot):
     // a dependent CTA allocates TMEM and then waits for this grid, so it must never get columns that a CTA
     // of this grid still needs.
+    if (SPLIT) cluster_arrive();                            // this CTA runs: its shared memory may be written to
     if (warp == 0) tmem_alloc(&P.tmem_slot, kA64TmemCols);
     asm volatile("griddepcontrol.wait;" ::: "memory");
     // Which unit this CTA works on.  With ragged lengths the CTAs take the sequences longest first
     // (CTA x gets the sequence of rank x / H in descending length, ties by position): when there are
     // more units than SMs the long ones start in the first wave and the short ones fill the tail.
-    int b = blockIdx.x / g.H;
-    const int h = blockIdx.x % g.H;
-    if (a.by_length) {
-        __shared__ int b_ranked;
+    int b = (int)(blockIdx.x / split) / g.H;
+    const int h = (int)(blockIdx.x / split) % g.H;
+    if (!SPLIT && a.by_length) {
         const int rank = b;
         for (int c = tid; c < g.B; c += kFusedThreads) {
             const int lc = min(max(g.lengths[c], 0), g.T);
@@ -80,10 +142,10 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
                 const int lo = min(max(g.lengths[o], 0), g.T);
                 before += (lo > lc) || (lo == lc && o < c);
             }
-            if (before == rank) b_ranked = c;
+            if (before == rank) P.b_ranked = c;
         }
         __syncthreads();
-        b = b_ranked;
+        b = P.b_ranked;
     }
     const int unit = b * g.H + h;
     const int L = seq_len(g, b);
@@ -96,7 +158,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
         if (L > 0 && !given) measure_issue_keys(smem, &P.bar, &tmKrows, L, b, h, a.pos_t, a.pos_h, g.debug_extra_tx);
         tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV);
     }
-    for (int i = tid; i < g.T; i += kFusedThreads) { chosen[i] = 0; if (i >= L) M_s[i] = 0.f; }
+    for (int i = tid; i < g.T; i += kFusedThreads) { chosen[i] = 0; if (i >= L && !given) M_s[i] = 0.f; }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -105,19 +167,38 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
     phase_stamp(g, 0);
 
     // ---- steps (a)+(b) ------------------------------------------------------------------------
+    // (with several CTAs per unit each takes a range of the queries, a multiple of the eight of a warp, and sends
+    // its values to the others: every CTA then holds all of M~)
     bool ok = true;
-    if (L > 0 && !given)
-        ok = measure_resident<kFusedThreads>(smem, &P.bar, 0u, a.k_bytes, a.stage_bytes, g, unit, b, h, L, U, 0, L, Q,
-                                             sidx, M_s);
+    if (SPLIT) cluster_wait();                              // every CTA of the unit runs
+    if (L > 0 && !given) {
+        const int per = ((L + split - 1) / split + 7) & ~7;
+        const int q_lo = min(part * per, L), q_hi = min(q_lo + per, L);
+        ok = measure_resident<kFusedThreads>(smem, &P.bar, 0u, a.k_bytes, a.stage_bytes, g, unit, b, h, L, U, q_lo, q_hi,
+                                             Q, sidx, M_s);
+        __syncthreads();
+        if (SPLIT) {
+            for (int x = 1; x < split; ++x) {
+                const uint32_t dst = peer_addr(smem_u32(M_s), (part + x) & (split - 1));
+                for (int i = q_lo + tid; i < q_hi; i += kFusedThreads) peer_store(dst + 4u * (uint32_t)i, M_s[i]);
+            }
+            cluster_arrive();
+            cluster_wait();
+        }
+    }
     __syncthreads();
     phase_stamp(g, 2);                                         // steps (a)+(b) done (stamp 1: the keys had landed)
-    if (M_out != nullptr && !given)
+    if (M_out != nullptr && !given && part == 0)
         for (int i = tid; i < g.T; i += kFusedThreads) M_out[(long long)unit * g.T + i] = M_s[i];
 
     // The attention phase reuses the shared memory of the measure phase, which is free now; its first
     // K/V tiles depend only on the unit, so their copies start before the selection and land behind it.
     Attend64Job j;
     j.b = b; j.h = h; j.L = L; j.lo = 0; j.hi = L;
+    if (SPLIT) {                                            // a range of whole key tiles (possibly none) per CTA
+        const int per = (((L + 127) / 128 + split - 1) / split) * 128;
+        j.lo = min(part * per, L); j.hi = min(j.lo + per, L);
+    }
     const int n_rows = given ? g.u_max : u;                    // a given list is taken at its full width
     j.rows = P.sel; j.n_rows = n_rows;
     j.pos_t = a.pos_t; j.pos_h = a.pos_h; j.pos_b = a.pos_b;
@@ -131,7 +212,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
         block_select([&](int i) { return float_key(M_s[i]); }, L, u, kA64MaxRows, P.sel, P.select);
         for (int r = tid; r < g.u_max; r += kFusedThreads) {
             const int i = r < kA64MaxRows ? P.sel[r] : -1;
-            sel_out[(long long)unit * g.u_max + r] = i;
+            if (part == 0) sel_out[(long long)unit * g.u_max + r] = i;
             if (i >= 0) chosen[i] = 1;
         }
     } else {
@@ -145,10 +226,35 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
     phase_stamp(g, 3);                                         // step (c) done
 
     // ---- step (d), with the column sums of V riding along ------------------------------------------
-    if (ok && L > 0) {
-        float m_run, l_run, acc[kD];
-        ok = attend64_run(smem, tmem_base, g, j, Q, &tmK, &tmV, m_run, l_run, acc);
-        if (ok && warp >= 4 && warp < 8 && lane < 16) {
+    // (a CTA of a cluster whose wait for the keys ran out still takes part in the barriers below)
+    if (L > 0 && (ok || SPLIT)) {
+        float m_run = -INFINITY, l_run = 0.f, acc[kD];
+        if (ok) {
+            ok = attend64_run(smem, tmem_base, g, j, Q, &tmK, &tmV, m_run, l_run, acc);
+        } else {
+#pragma unroll
+            for (int c = 0; c < kD; ++c) acc[c] = 0.f;
+        }
+        if (SPLIT) {
+            // every CTA leaves the states of its key range in its shared memory; CTA p then finishes the rows
+            // r = p (mod split), and each CTA the fill row
+            float *mine = reinterpret_cast<float *>(smem + kA64OffWg + 4 * kA64Tile);
+            if (warp >= 4 && warp < 8 && lane < 16) {
+                float *dst = mine + (16 * (warp - 4) + lane) * 66;
+                dst[0] = m_run; dst[1] = ok ? l_run : 0.f;
+#pragma unroll
+                for (int c = 0; c < kD; c += 2) *reinterpret_cast<float2 *>(dst + 2 + c) = make_float2(acc[c], acc[c + 1]);
+            }
+            cluster_arrive();
+            cluster_wait();
+            const int c = tid & 63;
+            for (int r = part + (tid >> 6) * split; r < n_rows; r += (kFusedThreads / 64) * split) {
+                const int i = P.sel[r];
+                if (i >= 0) O[unit_off(g.os, b, h) + (long long)i * g.os[2] + c] = __float2bfloat16(merge_states(split, smem_u32(mine), r, c));
+            }
+            if (j.sum_row >= 0 && tid < kD) P.vbar[c] = merge_states(split, smem_u32(mine), j.sum_row, c);
+            cluster_arrive();                                   // done with the other CTAs' memory (awaited before the exit)
+        } else if (ok && warp >= 4 && warp < 8 && lane < 16) {
             const int r = 16 * (warp - 4) + lane;
             const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
             if (r < n_rows) {
@@ -178,7 +284,8 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
         for (int t = 0; t < 8; ++t) { fillv[t] = (L > 0 && !a.own_v && ok) ? P.vbar[sub * 8 + t] : 0.f; zero8[t] = 0.f; }
         __nv_bfloat16 *Ou = O + unit_off(g.os, b, h);
         const __nv_bfloat16 *Vu = V + unit_off(g.vs, b, h);
-        for (int i = r0; i < g.T; i += kFusedThreads / 8) {
+        const int per = (g.T + split - 1) / split;
+        for (int i = part * per + r0; i < min(g.T, (part + 1) * per); i += kFusedThreads / 8) {
             __nv_bfloat16 *dst = Ou + (long long)i * g.os[2];
             if (i >= L) store8(dst, sub, zero8);
             else if (chosen[i] && ok) continue;
@@ -188,11 +295,50 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
     }
     __syncthreads();
     phase_stamp(g, 5);                                         // step (e) done
+    if (SPLIT && L > 0) cluster_wait();                    // nobody reads this CTA's states any more
     if (warp == 0) tmem_dealloc(tmem_base, kA64TmemCols);
 }
 
 bool make_rows_map(CUtensorMap *map, const void *base, const Geom &g, const long long s[3], int box_rows,
                    int swizzle128, int pos[3]);
+
+// Clusters of `split` CTAs of this kernel (one CTA per SM, largest shared memory) that the current device holds at
+// once; asked once per device.
+static int fused_max_clusters(int split) {
+    static std::atomic<int> cached[kMaxDevices][4];
+    const int k = split == 8 ? 3 : split == 4 ? 2 : 1;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) { cudaGetLastError(); return 0; }
+    int n = cached[dev][k].load(std::memory_order_relaxed);
+    if (n == 0) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)split);
+        cfg.blockDim = dim3(kFusedThreads);
+        cfg.dynamicSmemBytes = kFusedMaxSmem;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)split; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(&n, k_forward_fused<true>, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+        if (n <= 0) n = -1;
+        cached[dev][k].store(n, std::memory_order_relaxed);
+    }
+    return n < 0 ? 0 : n;
+}
+
+// CTAs per unit: as many (up to 8) as leave every cluster resident at once, where the sequences are long enough that
+// the shared-out measure and key tiles outweigh the exchanges (three cluster barriers and the merge, about 2.5 us).
+// Measured, us per call with 1 / 2 / 4 / 8 CTAs per unit: B1 H4 T128 15.8 / 17.8 / 17.5 / 18.3, T203 18.8 / 18.9 /
+// 17.8 / 18.5, T512 30.0 / 23.3 / 20.9 / 19.9, T1000 47.3 / 33.4 / 25.7 / 22.1; with a given index set B1 H4 T512
+// 11.1 / 11.4 / 12.3 / 12.4, T1000 17.4 / 15.1 / 13.9 / 13.1, T3000 34.2 / 24.3 / 19.0 / 14.3.
+static int fused_split(const Geom &g, bool given) {
+    const int units = g.B * g.H;
+    if (g.T < (given ? 768 : 192)) return 1;
+    for (int split = 8; split > 1; split >>= 1)
+        if (units <= fused_max_clusters(split)) return split;
+    return 1;
+}
 
 // cudaErrorNotSupported when the shape does not fit this kernel (the caller runs the staged schedule):
 // keys + staging beyond shared memory, more than 63 selected rows or 64 samples, no tensor map.
@@ -202,13 +348,15 @@ cudaError_t launch_forward_fused(const Geom &g, int U_max, int own_v, const void
     if (g.u_max > kA64MaxRows - 1) return cudaErrorNotSupported;
     if (sel_in == nullptr && (U_max > kMeasureMaxU || U_max < 1)) return cudaErrorNotSupported;
     FusedArgs a;
-    a.k_bytes = (uint32_t)measure_k_bytes(g.T);
-    a.stage_bytes = (uint32_t)measure_stage_bytes(kFusedThreads, g.idx_cols);
+    const bool given = sel_in != nullptr;
+    a.k_bytes = given ? 0u : (uint32_t)measure_k_bytes(g.T);
+    a.stage_bytes = given ? 0u : (uint32_t)measure_stage_bytes(kFusedThreads, g.idx_cols);
+    a.m_floats = given ? 0 : g.T;
     size_t phase = (size_t)a.k_bytes + kMeasureStages * (size_t)a.stage_bytes;
     if (phase < kA64Bytes) phase = kA64Bytes;
     a.off_persist = (uint32_t)((phase + 1023) / 1024 * 1024);
-    const size_t smem = a.off_persist + ((5 * (size_t)g.T + 127) / 128) * 128 + sizeof(FusedPersist) + 128;
-    if (smem > 227 * 1024) return cudaErrorNotSupported;
+    const size_t smem = a.off_persist + fused_arrays_bytes(a.m_floats, g.T) + sizeof(FusedPersist) + 128;
+    if (smem > kFusedMaxSmem) return cudaErrorNotSupported;
     CUtensorMap tmKrows, tmK, tmV;
     int p0[3], p1[3], p2[3];
     if (!make_rows_map(&tmKrows, K, g, g.ks, kMeasureBoxRows, 0, p0) || !make_rows_map(&tmK, K, g, g.ks, 128, 1, p1) ||
@@ -222,20 +370,25 @@ cudaError_t launch_forward_fused(const Geom &g, int U_max, int own_v, const void
     // the ranking costs B comparisons per sequence in every CTA: only where a second wave exists and B is small
     a.by_length = g.lengths != nullptr && g.B * g.H > device_sm_count() && g.B <= 256;
     static SmemGrant grant;
-    if (cudaError_t e = grant_dynamic_smem(k_forward_fused, grant, smem)) return e;
+    static SmemGrant grant_split;
+    if (cudaError_t e = grant_dynamic_smem(k_forward_fused<false>, grant, kFusedMaxSmem)) return e;
+    if (cudaError_t e = grant_dynamic_smem(k_forward_fused<true>, grant_split, kFusedMaxSmem)) return e;
+    a.split = fused_split(g, given);
     // launched with programmatic stream serialization: the kernel may be scheduled while the previous
     // kernel of the stream drains; it orders itself with griddepcontrol.wait before its first read
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(g.B * g.H));
+    cfg.gridDim = dim3((unsigned)(g.B * g.H * a.split));
     cfg.blockDim = dim3(kFusedThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)a.split; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_forward_fused, g, a, (const __nv_bfloat16 *)Q, (const __nv_bfloat16 *)V,
+    cfg.numAttrs = a.split > 1 ? 2 : 1;
+    cudaError_t e = cudaLaunchKernelEx(&cfg, a.split > 1 ? k_forward_fused<true> : k_forward_fused<false>, g, a, (const __nv_bfloat16 *)Q, (const __nv_bfloat16 *)V,
                                        sidx, (__nv_bfloat16 *)O, sel, M_out, tmKrows, tmK, tmV);
     note_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
