@@ -61,7 +61,7 @@ def tensor_peak():
 
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum per launch) of the dominant kernel from the
 # ncu capture summarised under profiles/, valid only while the kernel's sources are unchanged.
-_FUSED_SOURCES = ["psattn_fused.cu", "psattn_measure_mma.cuh", "psattn_attend64.cuh", "psattn_select.cuh",
+_FUSED_SOURCES = ["psattn_fused.cu", "psattn_measure_mma.cuh", "psattn_attend_rows.cuh", "psattn_select.cuh",
                   "psattn_sm100.cuh", "psattn_common.cuh"]
 _STREAM_SOURCES = ["psattn_measure_mma.cu", "psattn_measure_stream.cuh", "psattn_measure_mma.cuh",
                    "psattn_sm100.cuh", "psattn_common.cuh"]

@@ -4,8 +4,8 @@
 //   1. TMA brings the unit's K rows in once; the measure routine (ldmatrix gather + mma.sync)
 //      leaves M~ of every query in shared memory                              (Eq. 11)
 //   2. block-wide radix select picks the u queries, in place                  (Sec. 3.2)
-//   3. the shared memory of step 1 is reused for the tcgen05 attention of the selected rows
-//      over all valid keys; an extra all-ones weight row accumulates the column sums of V on the
+//   3. the shared memory of step 1 is reused for the attention of the selected rows over all valid keys
+//      (psattn_attend_rows.cuh); an extra all-ones weight row accumulates the column sums of V on the
 //      tensor cores while V streams through, so V is read from HBM once        (Eq. 7-8; Sec. 3.1)
 //   4. mean(V) (or the query's own value row) is written to every other valid row of O, zeros
 //      to padded rows                                                         (Eq. 12)
@@ -15,7 +15,7 @@
 // written once.  M~ never leaves the SM unless the caller asks for it.
 #include <atomic>
 
-#include "psattn_attend64.cuh"
+#include "psattn_attend_rows.cuh"
 #include "psattn_launch.h"
 #include "psattn_measure_mma.cuh"
 #include "psattn_select.cuh"
@@ -24,7 +24,7 @@ namespace psattn {
 
 using namespace sm100;
 
-constexpr int kFusedThreads = 512;       // warp 0: control; warps 4-7, 8-11: attention warpgroups; all 16 warps measure
+constexpr int kFusedThreads = 512;       // every warp measures, selects and attends
 
 #ifdef PSATTN_PHASE_STAMPS
 constexpr size_t kFusedMaxSmem = 226 * 1024;  // the stamps' static bytes push the dynamic memory to the next 1024-byte boundary
@@ -45,10 +45,9 @@ struct FusedArgs {
 
 struct FusedPersist {                    // at smem + off_persist, after the M~ array and the flags
     SelectScratch select;
-    int sel[kA64MaxRows];
+    int sel[kArMaxRows];
     float vbar[kD];
     uint64_t bar;
-    uint32_t tmem_slot;
     int b_ranked;
 };
 
@@ -108,7 +107,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
     const __grid_constant__ CUtensorMap tmKrows, const __grid_constant__ CUtensorMap tmK,
     const __grid_constant__ CUtensorMap tmV) {
     extern __shared__ __align__(1024) uint8_t smem[];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x;
     float *M_s = reinterpret_cast<float *>(smem + a.off_persist);
     unsigned char *chosen = reinterpret_cast<unsigned char *>(M_s + a.m_floats);
     FusedPersist &P = *reinterpret_cast<FusedPersist *>(smem + a.off_persist + fused_arrays_bytes(a.m_floats, g.T));
@@ -118,15 +117,11 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
         if (tid == 0) atomicOr(g.status, kStatusWaitExpired);
         return;
     }
-    // Programmatic dependent launch: let the next kernel of the stream be scheduled already (its CTAs
-    // wait at their own griddepcontrol.wait until this grid has completed and its writes are visible),
-    // and do not touch global memory before the previous grid has completed.  Both are no-ops when the
-    // launch carries no programmatic dependency.
-    // The trigger comes after this CTA's TMEM allocation (below, behind the barrier that publishes the slot):
-    // a dependent CTA allocates TMEM and then waits for this grid, so it must never get columns that a CTA
-    // of this grid still needs.
+    // Programmatic dependent launch: let the next kernel of the stream be scheduled already (its CTAs wait at their own
+    // griddepcontrol.wait until this grid has completed and its writes are visible), and do not touch global memory
+    // before the previous grid has completed.  Both are no-ops when the launch carries no programmatic dependency.
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (SPLIT) cluster_arrive();                            // this CTA runs: its shared memory may be written to
-    if (warp == 0) tmem_alloc(&P.tmem_slot, kA64TmemCols);
     asm volatile("griddepcontrol.wait;" ::: "memory");
     // Which unit this CTA works on.  With ragged lengths the CTAs take the sequences longest first
     // (CTA x gets the sequence of rank x / H in descending length, ties by position): when there are
@@ -159,11 +154,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
         tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV);
     }
     for (int i = tid; i < g.T; i += kFusedThreads) { chosen[i] = 0; if (i >= L && !given) M_s[i] = 0.f; }
-    tc_fence_before();
     __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem_base = P.tmem_slot;
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     phase_stamp(g, 0);
 
     // ---- steps (a)+(b) ------------------------------------------------------------------------
@@ -193,7 +184,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
 
     // The attention phase reuses the shared memory of the measure phase, which is free now; its first
     // K/V tiles depend only on the unit, so their copies start before the selection and land behind it.
-    Attend64Job j;
+    AttendRowsJob j;
     j.b = b; j.h = h; j.L = L; j.lo = 0; j.hi = L;
     if (SPLIT) {                                            // a range of whole key tiles (possibly none) per CTA
         const int per = (((L + 127) / 128 + split - 1) / split) * 128;
@@ -202,21 +193,23 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
     const int n_rows = given ? g.u_max : u;                    // a given list is taken at its full width
     j.rows = P.sel; j.n_rows = n_rows;
     j.pos_t = a.pos_t; j.pos_h = a.pos_h; j.pos_b = a.pos_b;
-    j.ctrl_warp = 0; j.wg_warp0 = 4;
     j.sum_row = a.own_v ? -1 : n_rows;
-    j.started = 1;
-    if (ok && L > 0 && tid == 0) attend64_start(smem, j, &tmK, &tmV);
-
-    // ---- step (c) -----------------------------------------------------------------------------
-    if (!given) {
-        block_select([&](int i) { return float_key(M_s[i]); }, L, u, kA64MaxRows, P.sel, P.select);
-        for (int r = tid; r < g.u_max; r += kFusedThreads) {
-            const int i = r < kA64MaxRows ? P.sel[r] : -1;
+    // The last warp starts the copies (a dozen requests by one thread take about a microsecond), the others select.
+    constexpr int kSelectors = kFusedThreads - 32;
+    static_assert(kArLoader == kSelectors && kArThreads == kFusedThreads, "the last warp starts the copies");
+    const int ahead = given ? 1 : kArStages;                    // (nothing to hide the copies behind with a given set)
+    if (tid >= kSelectors) {
+        if (ok && L > 0 && tid == kArLoader) attend_rows_start(smem, j, &tmK, &tmV, ahead);
+    } else if (!given) {
+        // ---- step (c) ---------------------------------------------------------------------------
+        block_select_short<3>([&](int i) { return float_key(M_s[i]); }, L, u, kArMaxRows, P.sel, P.select, kSelectors, 1);
+        for (int r = tid; r < g.u_max; r += kSelectors) {
+            const int i = r < kArMaxRows ? P.sel[r] : -1;
             if (part == 0) sel_out[(long long)unit * g.u_max + r] = i;
             if (i >= 0) chosen[i] = 1;
         }
     } else {
-        for (int r = tid; r < kA64MaxRows; r += kFusedThreads) {
+        for (int r = tid; r < kArMaxRows; r += kSelectors) {
             const int i = r < g.u_max ? a.sel_in[(long long)unit * g.u_max + r] : -1;
             P.sel[r] = (i >= 0 && i < L) ? i : -1;              // entries outside the sequence are ignored
             if (i >= 0 && i < L) chosen[i] = 1;
@@ -228,51 +221,47 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
     // ---- step (d), with the column sums of V riding along ------------------------------------------
     // (a CTA of a cluster whose wait for the keys ran out still takes part in the barriers below)
     if (L > 0 && (ok || SPLIT)) {
-        float m_run = -INFINITY, l_run = 0.f, acc[kD];
+        float m_run = -INFINITY, l_run = 0.f, acc[8];
+        const int row = tid >> 3, c8 = tid & 7;
         if (ok) {
-            ok = attend64_run(smem, tmem_base, g, j, Q, &tmK, &tmV, m_run, l_run, acc);
+            ok = attend_rows_run(smem, g, j, Q, &tmK, &tmV, ahead, m_run, l_run, acc);
         } else {
 #pragma unroll
-            for (int c = 0; c < kD; ++c) acc[c] = 0.f;
+            for (int x = 0; x < 8; ++x) acc[x] = 0.f;
         }
         if (SPLIT) {
             // every CTA leaves the states of its key range in its shared memory; CTA p then finishes the rows
             // r = p (mod split), and each CTA the fill row
-            float *mine = reinterpret_cast<float *>(smem + kA64OffWg + 4 * kA64Tile);
-            if (warp >= 4 && warp < 8 && lane < 16) {
-                float *dst = mine + (16 * (warp - 4) + lane) * 66;
-                dst[0] = m_run; dst[1] = ok ? l_run : 0.f;
+            float *mine = reinterpret_cast<float *>(smem + kArOffStage + 5 * kArTile);        // behind the merge buffer
+            float *dst = mine + row * 66;
+            if (c8 == 0) { dst[0] = m_run; dst[1] = ok ? l_run : 0.f; }
 #pragma unroll
-                for (int c = 0; c < kD; c += 2) *reinterpret_cast<float2 *>(dst + 2 + c) = make_float2(acc[c], acc[c + 1]);
-            }
+            for (int x = 0; x < 8; x += 2) *reinterpret_cast<float2 *>(dst + 2 + 8 * c8 + x) = make_float2(acc[x], acc[x + 1]);
             cluster_arrive();
             cluster_wait();
             const int c = tid & 63;
-            for (int r = part + (tid >> 6) * split; r < n_rows; r += (kFusedThreads / 64) * split) {
-                const int i = P.sel[r];
-                if (i >= 0) O[unit_off(g.os, b, h) + (long long)i * g.os[2] + c] = __float2bfloat16(merge_states(split, smem_u32(mine), r, c));
+            for (int k = tid >> 6; k == 0 || part + (k - 1) * split < n_rows; k += kFusedThreads / 64) {   // 0: the fill row
+                const int r = k == 0 ? j.sum_row : part + (k - 1) * split;
+                const int i = k == 0 ? 0 : P.sel[r];
+                if (r < 0 || i < 0) continue;
+                const float v = merge_states(split, smem_u32(mine), r, c);
+                if (k == 0) P.vbar[c] = v;
+                else O[unit_off(g.os, b, h) + (long long)i * g.os[2] + c] = __float2bfloat16(v);
             }
-            if (j.sum_row >= 0 && tid < kD) P.vbar[c] = merge_states(split, smem_u32(mine), j.sum_row, c);
             cluster_arrive();                                   // done with the other CTAs' memory (awaited before the exit)
-        } else if (ok && warp >= 4 && warp < 8 && lane < 16) {
-            const int r = 16 * (warp - 4) + lane;
+        } else if (ok) {
             const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
-            if (r < n_rows) {
-                const int i = P.sel[r];
-                if (i >= 0) {
 #pragma unroll
-                    for (int c = 0; c < kD; ++c) acc[c] *= inv;
-                    __nv_bfloat16 *dst = O + unit_off(g.os, b, h) + (long long)i * g.os[2];
+            for (int x = 0; x < 8; ++x) acc[x] *= inv;
+            if (row < n_rows) {
+                const int i = P.sel[row];
+                if (i >= 0) store8(O + unit_off(g.os, b, h) + (long long)i * g.os[2], c8, acc);
+            } else if (row == j.sum_row) {
 #pragma unroll
-                    for (int c8 = 0; c8 < 8; ++c8) store8(dst, c8, acc + 8 * c8);
-                }
-            } else if (r == j.sum_row) {
-#pragma unroll
-                for (int c = 0; c < kD; ++c) P.vbar[c] = acc[c] * inv;     // l = number of valid keys
+                for (int x = 0; x < 8; ++x) P.vbar[8 * c8 + x] = acc[x];      // l = number of valid keys
             }
         }
     }
-    tc_fence_before();
     __syncthreads();
     phase_stamp(g, 4);                                         // step (d) done
 
@@ -296,7 +285,6 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
     __syncthreads();
     phase_stamp(g, 5);                                         // step (e) done
     if (SPLIT && L > 0) cluster_wait();                    // nobody reads this CTA's states any more
-    if (warp == 0) tmem_dealloc(tmem_base, kA64TmemCols);
 }
 
 bool make_rows_map(CUtensorMap *map, const void *base, const Geom &g, const long long s[3], int box_rows,
@@ -345,7 +333,7 @@ static int fused_split(const Geom &g, bool given) {
 cudaError_t launch_forward_fused(const Geom &g, int U_max, int own_v, const void *Q, const void *K, const void *V,
                                  const int *sidx, void *O, int *sel, float *M_out, const int *sel_in, cudaStream_t st) {
     if (g.B * g.H == 0) return cudaSuccess;
-    if (g.u_max > kA64MaxRows - 1) return cudaErrorNotSupported;
+    if (g.u_max > kArMaxRows - 1) return cudaErrorNotSupported;
     if (sel_in == nullptr && (U_max > kMeasureMaxU || U_max < 1)) return cudaErrorNotSupported;
     FusedArgs a;
     const bool given = sel_in != nullptr;
@@ -353,10 +341,10 @@ cudaError_t launch_forward_fused(const Geom &g, int U_max, int own_v, const void
     a.stage_bytes = given ? 0u : (uint32_t)measure_stage_bytes(kFusedThreads, g.idx_cols);
     a.m_floats = given ? 0 : g.T;
     size_t phase = (size_t)a.k_bytes + kMeasureStages * (size_t)a.stage_bytes;
-    if (phase < kA64Bytes) phase = kA64Bytes;
+    if (phase < kArBytes) phase = kArBytes;
     a.off_persist = (uint32_t)((phase + 1023) / 1024 * 1024);
     const size_t smem = a.off_persist + fused_arrays_bytes(a.m_floats, g.T) + sizeof(FusedPersist) + 128;
-    if (smem > kFusedMaxSmem) return cudaErrorNotSupported;
+    if (smem > kFusedMaxSmem || (!given && g.T > 3 * (kFusedThreads - 32))) return cudaErrorNotSupported;   // (block_select_short<3>)
     CUtensorMap tmKrows, tmK, tmV;
     int p0[3], p1[3], p2[3];
     if (!make_rows_map(&tmKrows, K, g, g.ks, kMeasureBoxRows, 0, p0) || !make_rows_map(&tmK, K, g, g.ks, 128, 1, p1) ||

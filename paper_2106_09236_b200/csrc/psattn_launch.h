@@ -7,7 +7,7 @@ namespace psattn {
 constexpr int kColsumRows = 256;      // rows of V per column-sum partial
 constexpr int kFillRows = 128;        // rows of O per fill block
 constexpr int kSelectThreads = 1024;
-constexpr int kSelectSmemKeys = 8192; // keys kept in shared memory by the select kernel (32 KB)
+constexpr int kSelectSliceKeys = 8192; // longest range of one block of the two-kernel selection
 constexpr int kSplitKeys = 1024;      // keys per split of the SIMT attention kernel
 constexpr int kMaxDevices = 64;       // device ordinals the per-device records below cover
 

@@ -146,15 +146,14 @@ __global__ void __launch_bounds__(kSelectThreads) k_select(Geom g, const float *
         vbar[(long long)unit * kD + threadIdx.x] = L > 0 ? s / (float)L : 0.f;
     }
     if (M == nullptr) return;                  // mean(V) only
-    // the routine reads every key several times: keep them in shared memory when they fit
-    __shared__ unsigned keys[kSelectSmemKeys];
-    if (L <= kSelectSmemKeys) {
-        for (int i = threadIdx.x; i < L; i += blockDim.x) keys[i] = float_key(Mu[i]);
-        __syncthreads();
-        block_select([&](int i) { return keys[i]; }, L, u, g.u_max, out, scratch);
-    } else {
+    if (L <= kSelectThreads)
+        block_select_short<1>([&](int i) { return float_key(Mu[i]); }, L, u, g.u_max, out, scratch, blockDim.x, 0);
+    else if (L <= 3 * kSelectThreads)
+        block_select_short<3>([&](int i) { return float_key(Mu[i]); }, L, u, g.u_max, out, scratch, blockDim.x, 0);
+    else if (L <= 8 * kSelectThreads)
+        block_select_short<8>([&](int i) { return float_key(Mu[i]); }, L, u, g.u_max, out, scratch, blockDim.x, 0);
+    else
         block_select([&](int i) { return float_key(Mu[i]); }, L, u, g.u_max, out, scratch);
-    }
 }
 
 // ---------------------------------------------------------------------------------------
@@ -162,14 +161,14 @@ __global__ void __launch_bounds__(kSelectThreads) k_select(Geom g, const float *
 // `width` positions; one block per (unit, range) finds the top-u of its range (an element of the unit's
 // top-u is also in the top-u of its own range); one small block per unit then picks the top-u among the
 // slices * u candidates, which sit in position order, so that the tie rule (equal values: lower position
-// first) carries over.  Four times as many SMs work on the long scan, and each block's scan is short.
+// first) carries over.  Only for sequences whose keys do
+// not fit the registers of one block (8192): below that one kernel is faster (4 units x 8 heads, T = 8192: 10.7 against 11.7 us).
 // ---------------------------------------------------------------------------------------
 constexpr int kSelectMaxSlices = 8;
 
 __global__ void __launch_bounds__(kSelectThreads) k_select_slice(Geom g, const float *__restrict__ M, int slices,
                                                                  int width, int *__restrict__ cand) {
     __shared__ SelectScratch scratch;
-    __shared__ unsigned keys[kSelectSmemKeys];
     const int unit = blockIdx.x / slices, sl = blockIdx.x % slices;
     const int b = unit / g.H;
     pdl_enter();
@@ -179,9 +178,10 @@ __global__ void __launch_bounds__(kSelectThreads) k_select_slice(Geom g, const f
     const int lo = sl * width, n = max(0, min(L - lo, width));
     const float *Mu = M + (long long)unit * g.T + lo;
     int *out = cand + ((long long)unit * slices + sl) * g.u_max;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) keys[i] = float_key(Mu[i]);
-    __syncthreads();
-    block_select([&](int i) { return keys[i]; }, n, min(u, n), g.u_max, out, scratch);
+    if (n <= 3 * kSelectThreads)
+        block_select_short<3>([&](int i) { return float_key(Mu[i]); }, n, min(u, n), g.u_max, out, scratch, blockDim.x, 0);
+    else
+        block_select_short<kSelectSliceKeys / kSelectThreads>([&](int i) { return float_key(Mu[i]); }, n, min(u, n), g.u_max, out, scratch, blockDim.x, 0);
     for (int r = threadIdx.x; r < g.u_max; r += blockDim.x) {       // positions within the range -> positions of the unit
         const int p = out[r];
         if (p >= 0) out[r] = p + lo;
@@ -208,7 +208,7 @@ __global__ void __launch_bounds__(256) k_select_merge(Geom g, const float *__res
     }
     __syncthreads();
     int *out = sel + (long long)unit * g.u_max;
-    block_select([&](int p) { return ckey[p]; }, n, u, g.u_max, out, scratch);
+    block_select_short<2>([&](int p) { return ckey[p]; }, n, u, g.u_max, out, scratch, blockDim.x, 0);
     for (int r = threadIdx.x; r < g.u_max; r += blockDim.x) {
         const int p = out[r];
         if (p >= 0) out[r] = cidx[p];
@@ -479,9 +479,9 @@ cudaError_t launch_select(const Geom &g, const float *M, int *sel, const float *
     const int units = g.B * g.H;
     int slices = device_sm_count() / units;
     if (slices > kSelectMaxSlices) slices = kSelectMaxSlices;
-    if (M != nullptr && vbar == nullptr && cand != nullptr && slices >= 2 && g.u_max <= 64 && g.T / slices >= 1024) {
+    if (M != nullptr && vbar == nullptr && cand != nullptr && slices >= 2 && g.u_max <= 64 && g.T > 8 * kSelectThreads) {
         const int width = (g.T + slices - 1) / slices;
-        if (width <= kSelectSmemKeys) {
+        if (width <= kSelectSliceKeys) {
             cudaError_t e = launch_pdl(k_select_slice, dim3((unsigned)(units * slices)), dim3(kSelectThreads), 0, st, g, M,
                                        slices, width, cand);
             note_launch();
