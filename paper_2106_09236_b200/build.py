@@ -10,7 +10,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libpsattn.so")
 NATIVE = os.path.join(HERE, "psattn_torch.so")       # the native side of the Python binding (a CPython module)
 NATIVE_SOURCE = os.path.join(CSRC, "psattn_torch.cpp")
-SOURCES = ["psattn_api.cu", "psattn_staged.cu", "psattn_noalloc.cu", "psattn_attend_tc.cu", "psattn_measure_mma.cu", "psattn_measure_shared.cu", "psattn_exact_measure.cu", "psattn_project.cu", "psattn_attend64.cu", "psattn_fused.cu", "psattn_probe.cu", "psattn_project_out.cu"]
+SOURCES = ["psattn_api.cu", "psattn_staged.cu", "psattn_noalloc.cu", "psattn_attend_tc.cu", "psattn_measure_mma.cu", "psattn_measure_shared.cu", "psattn_exact_measure.cu", "psattn_project.cu", "psattn_attend64.cu", "psattn_fused.cu", "psattn_fused_fp32.cu", "psattn_probe.cu", "psattn_project_out.cu"]
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
     "-Xcompiler", "-fPIC",

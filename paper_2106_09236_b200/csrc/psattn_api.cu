@@ -412,6 +412,11 @@ extern "C" int psattn_forward(psattn_plan_t *plan, const void *Q, const void *K,
         if (d.path == PSATTN_PATH_FUSED) return PSATTN_ERR_UNSUPPORTED;
     } else if (d.path == PSATTN_PATH_FUSED) {
         return PSATTN_ERR_UNSUPPORTED;
+    } else if (d.dtype == PSATTN_FP32 && d.path == PSATTN_PATH_AUTO) {
+        cudaError_t e = launch_forward_fused_fp32(g, plan->U_max, d.fill_mode == PSATTN_FILL_OWN_V, Q, K, V, sample_idx, O,
+                                                  sel_idx, M_out, nullptr, st);
+        if (e == cudaSuccess) return PSATTN_OK;
+        if (e != cudaErrorNotSupported) return cuda_fail(plan, e);
     }
     float *M = M_out ? M_out : ws_at<float>(workspace, plan->off_M);
     if (vbar_from_attention(plan, g, K, V)) {
@@ -463,6 +468,12 @@ extern "C" int psattn_forward_with_selection(psattn_plan_t *plan, const void *Q,
         // one kernel for steps (d)+(e): one CTA per unit, or a cluster of CTAs where the units are few
         cudaError_t e = launch_forward_fused(g, plan->U_max, d.fill_mode == PSATTN_FILL_OWN_V, Q, K, V, nullptr, O,
                                              nullptr, nullptr, sel_idx_in, st);
+        if (e == cudaSuccess) return PSATTN_OK;
+        if (e != cudaErrorNotSupported) return cuda_fail(plan, e);
+    }
+    if (d.dtype == PSATTN_FP32 && d.path == PSATTN_PATH_AUTO) {
+        cudaError_t e = launch_forward_fused_fp32(g, plan->U_max, d.fill_mode == PSATTN_FILL_OWN_V, Q, K, V, nullptr, O,
+                                                  nullptr, nullptr, sel_idx_in, st);
         if (e == cudaSuccess) return PSATTN_OK;
         if (e != cudaErrorNotSupported) return cuda_fail(plan, e);
     }

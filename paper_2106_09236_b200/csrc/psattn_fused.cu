@@ -13,9 +13,8 @@
 // 1 and 2 are skipped and the kernel is steps (d)+(e) in one launch.
 // HBM traffic is the algorithmic minimum: Q, K, V read once (K a second time out of L2), O
 // written once.  M~ never leaves the SM unless the caller asks for it.
-#include <atomic>
-
 #include "psattn_attend_rows.cuh"
+#include "psattn_cluster.cuh"
 #include "psattn_launch.h"
 #include "psattn_measure_mma.cuh"
 #include "psattn_select.cuh"
@@ -52,52 +51,6 @@ struct FusedPersist {                    // at smem + off_persist, after the M~ 
 };
 
 __host__ __device__ inline size_t fused_arrays_bytes(int m_floats, int T) { return ((size_t)4 * m_floats + T + 127) / 128 * 128; }
-
-// ---- the CTAs of a unit (a.split > 1): one thread-block cluster -----------------------------------------
-__device__ __forceinline__ void cluster_arrive() {
-    __syncwarp();
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void cluster_wait() {
-    __syncwarp();
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ uint32_t peer_addr(uint32_t addr, int rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-    return r;
-}
-__device__ __forceinline__ void peer_store(uint32_t addr, float v) {
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
-}
-__device__ __forceinline__ float peer_load(uint32_t addr) {
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
-    return v;
-}
-// Column c of row r over all CTAs of the unit: the states (m, l, acc) that every CTA left at `states` in its shared
-// memory (66 floats per row) merged in rank order; returns acc / l.
-template <int SPLIT>
-__device__ __forceinline__ float merge_states_n(uint32_t states, int r, int c) {
-    float m[SPLIT], l[SPLIT], a[SPLIT];
-#pragma unroll
-    for (int x = 0; x < SPLIT; ++x) {                          // all loads in flight together
-        const uint32_t p = peer_addr(states + (uint32_t)r * 264u, x);
-        m[x] = peer_load(p); l[x] = peer_load(p + 4u); a[x] = peer_load(p + 8u + 4u * (uint32_t)c);
-    }
-    float mw = -INFINITY, lw = 0.f, aw = 0.f;
-#pragma unroll
-    for (int x = 0; x < SPLIT; ++x) mw = fmaxf(mw, m[x]);
-#pragma unroll
-    for (int x = 0; x < SPLIT; ++x) {
-        const float f = l[x] > 0.f ? fast_exp2(m[x] - mw) : 0.f;
-        lw += l[x] * f; aw += a[x] * f;
-    }
-    return lw > 0.f ? aw / lw : 0.f;
-}
-__device__ __forceinline__ float merge_states(int split, uint32_t states, int r, int c) {
-    return split == 8 ? merge_states_n<8>(states, r, c) : split == 4 ? merge_states_n<4>(states, r, c) : merge_states_n<2>(states, r, c);
-}
 
 // SPLIT: the unit is shared by the a.split > 1 CTAs of a thread-block cluster.
 template <bool SPLIT>
@@ -290,41 +243,17 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
 bool make_rows_map(CUtensorMap *map, const void *base, const Geom &g, const long long s[3], int box_rows,
                    int swizzle128, int pos[3]);
 
-// Clusters of `split` CTAs of this kernel (one CTA per SM, largest shared memory) that the current device holds at
-// once; asked once per device.
-static int fused_max_clusters(int split) {
-    static std::atomic<int> cached[kMaxDevices][4];
-    const int k = split == 8 ? 3 : split == 4 ? 2 : 1;
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) { cudaGetLastError(); return 0; }
-    int n = cached[dev][k].load(std::memory_order_relaxed);
-    if (n == 0) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)split);
-        cfg.blockDim = dim3(kFusedThreads);
-        cfg.dynamicSmemBytes = kFusedMaxSmem;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = (unsigned)split; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        if (cudaOccupancyMaxActiveClusters(&n, k_forward_fused<true>, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
-        if (n <= 0) n = -1;
-        cached[dev][k].store(n, std::memory_order_relaxed);
-    }
-    return n < 0 ? 0 : n;
-}
-
 // CTAs per unit: as many (up to 8) as leave every cluster resident at once, where the sequences are long enough that
 // the shared-out measure and key tiles outweigh the exchanges (three cluster barriers and the merge, about 2.5 us).
 // Measured, us per call with 1 / 2 / 4 / 8 CTAs per unit: B1 H4 T128 15.8 / 17.8 / 17.5 / 18.3, T203 18.8 / 18.9 /
 // 17.8 / 18.5, T512 30.0 / 23.3 / 20.9 / 19.9, T1000 47.3 / 33.4 / 25.7 / 22.1; with a given index set B1 H4 T512
 // 11.1 / 11.4 / 12.3 / 12.4, T1000 17.4 / 15.1 / 13.9 / 13.1, T3000 34.2 / 24.3 / 19.0 / 14.3.
 static int fused_split(const Geom &g, bool given) {
+    static ClusterRecord clusters;
     const int units = g.B * g.H;
     if (g.T < (given ? 768 : 192)) return 1;
     for (int split = 8; split > 1; split >>= 1)
-        if (units <= fused_max_clusters(split)) return split;
+        if (units <= max_clusters(k_forward_fused<true>, clusters, split, kFusedThreads, kFusedMaxSmem)) return split;
     return 1;
 }
 
@@ -364,20 +293,9 @@ cudaError_t launch_forward_fused(const Geom &g, int U_max, int own_v, const void
     a.split = fused_split(g, given);
     // launched with programmatic stream serialization: the kernel may be scheduled while the previous
     // kernel of the stream drains; it orders itself with griddepcontrol.wait before its first read
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(g.B * g.H * a.split));
-    cfg.blockDim = dim3(kFusedThreads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = (unsigned)a.split; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = a.split > 1 ? 2 : 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, a.split > 1 ? k_forward_fused<true> : k_forward_fused<false>, g, a, (const __nv_bfloat16 *)Q, (const __nv_bfloat16 *)V,
-                                       sidx, (__nv_bfloat16 *)O, sel, M_out, tmKrows, tmK, tmV);
+    cudaError_t e = launch_split(a.split > 1 ? k_forward_fused<true> : k_forward_fused<false>, (unsigned)(g.B * g.H), a.split,
+                                 kFusedThreads, smem, st, g, a, (const __nv_bfloat16 *)Q, (const __nv_bfloat16 *)V, sidx,
+                                 (__nv_bfloat16 *)O, sel, M_out, tmKrows, tmK, tmV);
     note_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
 }

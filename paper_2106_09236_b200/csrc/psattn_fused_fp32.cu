@@ -1,0 +1,491 @@
+// The whole path (steps a-e) of one (batch, head) unit in one launch for fp32 inputs: psattn_fused.cu's plan in fp32
+// arithmetic on the FMA pipe (tf32 products would break the 1e-4 tolerance).
+//
+//   1. the unit's keys into shared memory where they fit (T up to about 870), then the measure, one warp per query, in the
+//      order of operations of the staged kernel, so that M~ has the same bits                       (Eq. 11)
+//   2. block-wide selection                                                                        (Sec. 3.2)
+//   3. attention of the selected rows: chunks of 128 keys, scores in 8 x 2 register tiles, softmax, values in 4 x 4 register
+//      tiles with the keys of the chunk spread over the threads that the rows leave free; a zero query row
+//      yields the column sums of V                                                                 (Eq. 7-8)
+//   4. fill                                                                                        (Eq. 12)
+// A unit is shared by the CTAs of a cluster as in psattn_fused.cu.
+// Bound: the measure's row reads (256 bytes per pair from shared memory at 128 B/clk), then latency.  The staged schedule ran
+// five kernels, of which the attention gave every (row, key split) to one warp that read all keys and values for itself: 99 us
+// of the 136 us at B8 H4 T777 (lengths 233..777), 14 of 29 us for B1 H4 T128.
+#include "psattn_cluster.cuh"
+#include "psattn_launch.h"
+#include "psattn_measure_mma.cuh"
+#include "psattn_select.cuh"
+
+namespace psattn {
+
+using namespace sm100;
+
+constexpr int kF32Threads = 512;
+constexpr int kF32MaxRows = 64;
+constexpr int kF32Chunk = 128;                                 // keys per step of the attention
+constexpr int kF32KPitch = 68, kF32PPitch = 72;                // floats: conflict-free 16-byte reads of eight rows; 16-byte rows
+constexpr uint32_t kF32OffQ = 0;                               // [64][64]
+constexpr uint32_t kF32OffK = kF32OffQ + 64 * 64 * 4;          // [128][68]
+constexpr uint32_t kF32OffV = kF32OffK + kF32Chunk * kF32KPitch * 4;       // [128][64]; afterwards the row states
+constexpr uint32_t kF32OffP = kF32OffV + kF32Chunk * 64 * 4;   // [128][72]: weights, key-major; afterwards partial sums
+constexpr uint32_t kF32AttendBytes = kF32OffP + kF32Chunk * kF32PPitch * 4;
+constexpr size_t kF32MaxSmem = 226 * 1024;
+
+struct Fused32Args {
+    uint32_t off_persist;                // M~, selection, flags: live through all phases
+    int resident;                        // the unit's keys fit in shared memory
+    int own_v, by_length, split, m_floats;
+    const int *sel_in;
+};
+
+struct Fused32Persist {
+    SelectScratch select;
+    int sel[kF32MaxRows];
+    float vbar[kD];
+    float m[kF32MaxRows], l[kF32MaxRows], alpha[kF32MaxRows];
+    float part[kF32MaxRows][2];          // row maxima, then row sums, of the two warps of a row group
+    int b_ranked;
+};
+
+__host__ __device__ inline size_t f32_arrays_bytes(int m_floats, int T) { return ((size_t)4 * m_floats + T + 127) / 128 * 128; }
+
+// One query's samples, kept one query ahead: its row (8 columns per lane) and up to 64 key positions.
+struct F32Query {
+    float q[8];
+    int key[2];
+};
+
+// M~ of the queries q_lo + warp, + 16, ... < q_hi of one unit, with the arithmetic of k_measure (psattn_staged.cu): four
+// groups of eight lanes, a group takes every fourth sampled key, 16 keys in flight.
+template <bool RESIDENT>
+__device__ __forceinline__ void f32_measure(const Geom &g, int unit, int b, int h, int L, int U, int q_lo, int q_hi,
+                                            const float *__restrict__ Qu, const float *Ku, long long k_pitch,
+                                            const int *__restrict__ sidx, float *M_s) {
+    const int lane = threadIdx.x & 31, sub = lane & 7, grp = lane >> 3, warp = threadIdx.x >> 5;
+    const int *idx0 = sidx + (g.idx_per_head ? (long long)unit : (long long)b) * g.T * g.idx_cols;
+    auto fetch = [&](int i, F32Query &x) {
+        if (i >= q_hi) return;
+        load8(Qu + (long long)i * g.qs[2], sub, x.q);
+        const int *row = idx0 + (long long)i * g.idx_cols;
+        x.key[0] = lane < U ? __ldg(row + lane) : 0;
+        x.key[1] = 32 + lane < U ? __ldg(row + 32 + lane) : 0;
+    };
+    F32Query cur, nxt;
+    fetch(q_lo + warp, cur);
+#pragma unroll 1
+    for (int i = q_lo + warp; i < q_hi; i += kF32Threads / 32) {
+        fetch(i + kF32Threads / 32, nxt);
+        MeasureState st = measure_init();
+#pragma unroll 1
+        for (int base = 0; base < U; base += 32) {
+            int my = base == 0 ? cur.key[0] : cur.key[1];
+            if (base + lane < U && (my < 0 || my >= L)) { atomicOr(g.status, kStatusIdxClamped); my = my < 0 ? 0 : L - 1; }
+            const int steps = (min(32, U - base) + 3) >> 2;
+#pragma unroll 1
+            for (int s0 = 0; s0 < steps; s0 += 4) {
+                float kk[4][8], part[4];
+                bool active[4];
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    const int src = (s0 + x) * 4 + grp;
+                    const int key = __shfl_sync(0xffffffffu, my, src & 31);
+                    active[x] = s0 + x < steps && base + src < U;
+                    const float *kr = Ku + (long long)(active[x] ? key : 0) * k_pitch;
+                    if (RESIDENT) {
+                        const float4 a = reinterpret_cast<const float4 *>(kr)[2 * sub], c = reinterpret_cast<const float4 *>(kr)[2 * sub + 1];
+                        kk[x][0] = a.x; kk[x][1] = a.y; kk[x][2] = a.z; kk[x][3] = a.w;
+                        kk[x][4] = c.x; kk[x][5] = c.y; kk[x][6] = c.z; kk[x][7] = c.w;
+                    } else {
+                        load8(kr, sub, kk[x]);
+                    }
+                }
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    part[x] = 0.f;
+#pragma unroll
+                    for (int t = 0; t < 8; ++t) part[x] = fmaf(cur.q[t], kk[x][t], part[x]);
+                }
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    part[x] += __shfl_xor_sync(0xffffffffu, part[x], 1);
+                    part[x] += __shfl_xor_sync(0xffffffffu, part[x], 2);
+                    part[x] += __shfl_xor_sync(0xffffffffu, part[x], 4);
+                }
+#pragma unroll
+                for (int x = 0; x < 4; ++x)
+                    if (active[x]) measure_push(st, part[x] * kScale);
+            }
+        }
+#pragma unroll
+        for (int o = 8; o <= 16; o <<= 1) {
+            MeasureState other;
+            other.m = __shfl_xor_sync(0xffffffffu, st.m, o);
+            other.D = __shfl_xor_sync(0xffffffffu, st.D, o);
+            other.n = __shfl_xor_sync(0xffffffffu, st.n, o);
+            st = (lane & o) ? measure_merge(other, st) : measure_merge(st, other);
+        }
+        if (lane == 0) M_s[i] = U > 0 ? st.D / (float)U : 0.f;
+        cur = nxt;
+    }
+}
+
+// Eight values per lane, reduced over the warp: lane l returns the result of value l >> 2 (the same in its four lanes).
+template <class Op>
+__device__ __forceinline__ float f32_reduce8(const float v[8], Op op) {
+    const int lane = threadIdx.x & 31;
+    float a[4], b[2];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+        const bool up = lane & 16;
+        const float keep = up ? v[4 + x] : v[x], send = up ? v[x] : v[4 + x];
+        a[x] = op(keep, __shfl_xor_sync(0xffffffffu, send, 16));
+    }
+#pragma unroll
+    for (int x = 0; x < 2; ++x) {
+        const bool up = lane & 8;
+        const float keep = up ? a[2 + x] : a[x], send = up ? a[x] : a[2 + x];
+        b[x] = op(keep, __shfl_xor_sync(0xffffffffu, send, 8));
+    }
+    const bool up = lane & 4;
+    float r = op(up ? b[1] : b[0], __shfl_xor_sync(0xffffffffu, up ? b[0] : b[1], 4));
+    r = op(r, __shfl_xor_sync(0xffffffffu, r, 2));
+    return op(r, __shfl_xor_sync(0xffffffffu, r, 1));
+}
+
+// Rows of 256 bytes from global memory into shared memory, `n` of them (zeros from `valid` on), pitch in floats.
+__device__ __forceinline__ void f32_stage_rows(uint32_t dst, uint32_t pitch, const float *src, long long stride, int n, int valid) {
+#pragma unroll 4
+    for (int e = threadIdx.x; e < n * 16; e += kF32Threads) {
+        const int r = e >> 4, c = e & 15;
+        const uint32_t d = dst + ((uint32_t)r * pitch + (uint32_t)c * 4u) * 4u;
+        if (r < valid) cp_async_16(d, src + (long long)r * stride + c * 4);
+        else asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(d), "r"(0) : "memory");
+    }
+}
+
+// The attention of the listed rows over the keys [lo, hi): on return P.m / P.l hold the row states and the partial sums of the
+// unnormalised rows lie at kF32OffP as [splits][rows][64]; returns splits.  Contains __syncthreads.
+__device__ __forceinline__ int f32_attend(uint8_t *smem, const Geom &g, Fused32Persist &P, int b, int h, int L, int lo, int hi,
+                                          int n_rows, int row_groups, const float *__restrict__ Qu,
+                                          const float *__restrict__ Ku, const float *__restrict__ Vu) {
+    const int tid = threadIdx.x, lane = tid & 31;
+    float *Qs = reinterpret_cast<float *>(smem + kF32OffQ), *Ks = reinterpret_cast<float *>(smem + kF32OffK);
+    float *Vs = reinterpret_cast<float *>(smem + kF32OffV), *Ps = reinterpret_cast<float *>(smem + kF32OffP);
+    const int n_chunks = (hi - lo + kF32Chunk - 1) / kF32Chunk;
+    auto stage_k = [&](int c) {
+        const int k0 = lo + c * kF32Chunk;
+        f32_stage_rows(smem_u32(Ks), kF32KPitch, Ku + (long long)k0 * g.ks[2], g.ks[2], kF32Chunk, hi - k0);
+        cp_async_commit();
+    };
+    auto stage_v = [&](int c) {
+        const int k0 = lo + c * kF32Chunk;
+        f32_stage_rows(smem_u32(Vs), 64, Vu + (long long)k0 * g.vs[2], g.vs[2], kF32Chunk, hi - k0);
+        cp_async_commit();
+    };
+#pragma unroll
+    for (int e = tid; e < kF32MaxRows * 16; e += kF32Threads) {        // the listed rows; unused rows are zero
+        const int r = e >> 4, c = e & 15, i = r < n_rows ? P.sel[r] : -1;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (i >= 0 && i < L) v = __ldg(reinterpret_cast<const float4 *>(Qu + (long long)i * g.qs[2]) + c);
+        reinterpret_cast<float4 *>(Qs)[e] = v;
+    }
+    if (tid < kF32MaxRows) { P.m[tid] = -INFINITY; P.l[tid] = 0.f; }
+    if (n_chunks > 0) { stage_k(0); stage_v(0); }
+
+    // scores: row group rg (8 rows), keys kg and kg + 64 of the chunk; values: row quad rq, columns 4 cq .., keys ks + splits * n
+    const int kg = tid & 63, rg = tid >> 6;
+    const int quads = 2 * row_groups, splits = kF32Threads / (16 * quads);
+    const int cq = tid & 15, rq = (tid >> 4) % quads, ks = (tid >> 4) / quads;
+    float o[4][4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x)
+#pragma unroll
+        for (int y = 0; y < 4; ++y) o[x][y] = 0.f;
+#pragma unroll 1
+    for (int c = 0; c < n_chunks; ++c) {
+        const int valid = min(kF32Chunk, hi - lo - c * kF32Chunk);
+        cp_async_wait<1>();                                    // K of this chunk (V may still be on its way)
+        __syncthreads();
+        float s[8][2];
+        if (rg < row_groups) {
+#pragma unroll
+            for (int x = 0; x < 8; ++x) s[x][0] = s[x][1] = 0.f;
+            const float4 *q = reinterpret_cast<const float4 *>(Qs + rg * 8 * 64);
+            const float4 *k0 = reinterpret_cast<const float4 *>(Ks + kg * kF32KPitch), *k1 = reinterpret_cast<const float4 *>(Ks + (kg + 64) * kF32KPitch);
+#pragma unroll 2
+            for (int d = 0; d < 16; ++d) {
+                const float4 a = k0[d], e = k1[d];
+#pragma unroll
+                for (int x = 0; x < 8; ++x) {
+                    const float4 v = q[x * 16 + d];
+                    s[x][0] = fmaf(v.x, a.x, s[x][0]); s[x][0] = fmaf(v.y, a.y, s[x][0]); s[x][0] = fmaf(v.z, a.z, s[x][0]); s[x][0] = fmaf(v.w, a.w, s[x][0]);
+                    s[x][1] = fmaf(v.x, e.x, s[x][1]); s[x][1] = fmaf(v.y, e.y, s[x][1]); s[x][1] = fmaf(v.z, e.z, s[x][1]); s[x][1] = fmaf(v.w, e.w, s[x][1]);
+                }
+            }
+            float mx[8];
+#pragma unroll
+            for (int x = 0; x < 8; ++x) {
+                s[x][0] = kg < valid ? s[x][0] * (kScale * kLog2e) : -INFINITY;
+                s[x][1] = kg + 64 < valid ? s[x][1] * (kScale * kLog2e) : -INFINITY;
+                mx[x] = fmaxf(s[x][0], s[x][1]);
+            }
+            const float r = f32_reduce8(mx, [](float a, float e) { return fmaxf(a, e); });
+            if ((lane & 3) == 0) P.part[rg * 8 + (lane >> 2)][(tid >> 5) & 1] = r;
+        }
+        __syncthreads();
+        if (c + 1 < n_chunks) stage_k(c + 1); else cp_async_commit();          // the K buffer is free
+        if (tid < row_groups * 8) {
+            const float m = P.m[tid], n = fmaxf(m, fmaxf(P.part[tid][0], P.part[tid][1]));
+            P.alpha[tid] = exp2f(m - n);                       // 0 on the first chunk (m = -inf)
+            P.m[tid] = n;
+        }
+        __syncthreads();
+        if (rg < row_groups) {
+            float sum[8];
+#pragma unroll
+            for (int x = 0; x < 8; ++x) {
+                const float m = P.m[rg * 8 + x];
+                s[x][0] = exp2f(s[x][0] - m); s[x][1] = exp2f(s[x][1] - m);
+                sum[x] = s[x][0] + s[x][1];
+            }
+#pragma unroll
+            for (int y = 0; y < 2; ++y) {
+                float4 *dst = reinterpret_cast<float4 *>(Ps + (kg + 64 * y) * kF32PPitch + rg * 8);
+                dst[0] = make_float4(s[0][y], s[1][y], s[2][y], s[3][y]);
+                dst[1] = make_float4(s[4][y], s[5][y], s[6][y], s[7][y]);
+            }
+            const float r = f32_reduce8(sum, [](float a, float e) { return a + e; });
+            if ((lane & 3) == 0) P.part[rg * 8 + (lane >> 2)][(tid >> 5) & 1] = r;
+        }
+        cp_async_wait<1>();                                    // V of this chunk
+        __syncthreads();
+        if (tid < row_groups * 8) P.l[tid] = P.l[tid] * P.alpha[tid] + (P.part[tid][0] + P.part[tid][1]);
+        if (ks < splits) {
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+                const float al = P.alpha[rq * 4 + x];
+#pragma unroll
+                for (int y = 0; y < 4; ++y) o[x][y] *= al;
+            }
+#pragma unroll 4
+            for (int k = ks; k < valid; k += splits) {
+                const float4 p = *reinterpret_cast<const float4 *>(Ps + k * kF32PPitch + rq * 4), v = *reinterpret_cast<const float4 *>(Vs + k * 64 + cq * 4);
+                o[0][0] = fmaf(p.x, v.x, o[0][0]); o[0][1] = fmaf(p.x, v.y, o[0][1]); o[0][2] = fmaf(p.x, v.z, o[0][2]); o[0][3] = fmaf(p.x, v.w, o[0][3]);
+                o[1][0] = fmaf(p.y, v.x, o[1][0]); o[1][1] = fmaf(p.y, v.y, o[1][1]); o[1][2] = fmaf(p.y, v.z, o[1][2]); o[1][3] = fmaf(p.y, v.w, o[1][3]);
+                o[2][0] = fmaf(p.z, v.x, o[2][0]); o[2][1] = fmaf(p.z, v.y, o[2][1]); o[2][2] = fmaf(p.z, v.z, o[2][2]); o[2][3] = fmaf(p.z, v.w, o[2][3]);
+                o[3][0] = fmaf(p.w, v.x, o[3][0]); o[3][1] = fmaf(p.w, v.y, o[3][1]); o[3][2] = fmaf(p.w, v.z, o[3][2]); o[3][3] = fmaf(p.w, v.w, o[3][3]);
+            }
+        }
+        __syncthreads();
+        if (c + 1 < n_chunks) stage_v(c + 1);                  // the V buffer is free
+    }
+    cp_async_wait<0>();
+    __syncthreads();
+    if (ks < splits) {
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+            *reinterpret_cast<float4 *>(Ps + ((ks * quads + rq) * 4 + x) * 64 + cq * 4) = make_float4(o[x][0], o[x][1], o[x][2], o[x][3]);
+    }
+    __syncthreads();
+    return splits;
+}
+
+template <bool SPLIT>
+__global__ void __launch_bounds__(kF32Threads, 1) k_forward_fused_fp32(
+    Geom g, Fused32Args a, const float *__restrict__ Q, const float *__restrict__ K, const float *__restrict__ V,
+    const int *__restrict__ sidx, float *__restrict__ O, int *__restrict__ sel_out, float *__restrict__ M_out) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    const int tid = threadIdx.x;
+    float *M_s = reinterpret_cast<float *>(smem + a.off_persist);
+    unsigned char *chosen = reinterpret_cast<unsigned char *>(M_s + a.m_floats);
+    Fused32Persist &P = *reinterpret_cast<Fused32Persist *>(smem + a.off_persist + f32_arrays_bytes(a.m_floats, g.T));
+    const int split = SPLIT ? a.split : 1, part = SPLIT ? (int)(blockIdx.x % split) : 0;
+    if (SPLIT) cluster_arrive();                                // this CTA runs: its shared memory may be written to
+    pdl_enter();
+    int b = (int)(blockIdx.x / split) / g.H;
+    const int h = (int)(blockIdx.x / split) % g.H;
+    if (!SPLIT && a.by_length) {                                // longest sequences first, as in k_forward_fused
+        const int rank = b;
+        for (int c = tid; c < g.B; c += kF32Threads) {
+            const int lc = min(max(g.lengths[c], 0), g.T);
+            int before = 0;
+            for (int o = 0; o < g.B; ++o) {
+                const int lo = min(max(g.lengths[o], 0), g.T);
+                before += (lo > lc) || (lo == lc && o < c);
+            }
+            if (before == rank) P.b_ranked = c;
+        }
+        __syncthreads();
+        b = P.b_ranked;
+    }
+    const int unit = b * g.H + h;
+    const int L = seq_len(g, b);
+    const int U = min(g.U_tab[L], g.idx_cols);
+    const int u = min(min(g.u_tab[L], g.u_max), L);
+    const bool given = a.sel_in != nullptr;                    // steps (d)+(e) only, for a given index set
+    const float *Qu = Q + unit_off(g.qs, b, h), *Ku = K + unit_off(g.ks, b, h), *Vu = V + unit_off(g.vs, b, h);
+    for (int i = tid; i < g.T; i += kF32Threads) { chosen[i] = 0; if (i >= L && !given) M_s[i] = 0.f; }
+
+    // ---- steps (a)+(b): every CTA of the unit a range of the queries; its values go to the others -----------------
+    if (SPLIT) cluster_wait();                                  // every CTA of the unit runs
+    if (L > 0 && !given) {
+        const int per = (L + split - 1) / split;
+        const int q_lo = min(part * per, L), q_hi = min(q_lo + per, L);
+        if (a.resident) {
+            f32_stage_rows(smem_u32(smem), 64, Ku, g.ks[2], L, L);
+            cp_async_commit();
+            cp_async_wait<0>();
+            __syncthreads();
+            f32_measure<true>(g, unit, b, h, L, U, q_lo, q_hi, Qu, reinterpret_cast<const float *>(smem), 64, sidx, M_s);
+        } else {
+            f32_measure<false>(g, unit, b, h, L, U, q_lo, q_hi, Qu, Ku, g.ks[2], sidx, M_s);
+        }
+        __syncthreads();
+        if (SPLIT) {
+            for (int x = 1; x < split; ++x) {
+                const uint32_t dst = peer_addr(smem_u32(M_s), (part + x) & (split - 1));
+                for (int i = q_lo + tid; i < q_hi; i += kF32Threads) peer_store(dst + 4u * (uint32_t)i, M_s[i]);
+            }
+            cluster_arrive();
+            cluster_wait();
+        }
+    }
+    __syncthreads();
+    if (M_out != nullptr && !given && part == 0)
+        for (int i = tid; i < g.T; i += kF32Threads) M_out[(long long)unit * g.T + i] = M_s[i];
+
+    // ---- step (c) -----------------------------------------------------------------------------
+    const int n_rows = given ? g.u_max : u;                    // a given list is taken at its full width
+    if (!given) {
+        block_select_short<3>([&](int i) { return float_key(M_s[i]); }, L, u, kF32MaxRows, P.sel, P.select, kF32Threads, 0);
+        for (int r = tid; r < g.u_max; r += kF32Threads) {
+            const int i = r < kF32MaxRows ? P.sel[r] : -1;
+            if (part == 0) sel_out[(long long)unit * g.u_max + r] = i;
+            if (i >= 0) chosen[i] = 1;
+        }
+    } else {
+        for (int r = tid; r < kF32MaxRows; r += kF32Threads) {
+            const int i = r < g.u_max ? a.sel_in[(long long)unit * g.u_max + r] : -1;
+            P.sel[r] = (i >= 0 && i < L) ? i : -1;              // entries outside the sequence are ignored
+            if (i >= 0 && i < L) chosen[i] = 1;
+        }
+    }
+    __syncthreads();
+
+    // ---- step (d), with the column sums of V as one more row ------------------------------------------------
+    if (L > 0) {
+        const int sum_row = a.own_v ? -1 : n_rows;
+        const int row_groups = (max(n_rows, sum_row + 1) + 7) / 8;
+        const int per = SPLIT ? (L + split - 1) / split : L;
+        const int lo = min(part * per, L), hi = min(lo + per, L);
+        const int splits = f32_attend(smem, g, P, b, h, L, lo, hi, n_rows, row_groups, Qu, Ku, Vu);
+        const float *Ps = reinterpret_cast<const float *>(smem + kF32OffP);
+        const int row = tid >> 3, c8 = tid & 7;
+        float acc[8];
+#pragma unroll
+        for (int x = 0; x < 8; ++x) acc[x] = 0.f;
+        if (row < row_groups * 8)
+            for (int s = 0; s < splits; ++s) {
+                const float4 *src = reinterpret_cast<const float4 *>(Ps + (s * row_groups * 8 + row) * 64 + c8 * 8);
+                const float4 x = src[0], y = src[1];
+                acc[0] += x.x; acc[1] += x.y; acc[2] += x.z; acc[3] += x.w;
+                acc[4] += y.x; acc[5] += y.y; acc[6] += y.z; acc[7] += y.w;
+            }
+        if (SPLIT) {
+            // as in k_forward_fused: the states of every CTA's key range stay in its shared memory, CTA p finishes the rows
+            // r = p (mod split), and each CTA the fill row
+            float *mine = reinterpret_cast<float *>(smem + kF32OffV);
+            if (row < row_groups * 8) {
+                float *dst = mine + row * 66;
+                if (c8 == 0) { dst[0] = P.m[row]; dst[1] = P.l[row]; }
+#pragma unroll
+                for (int x = 0; x < 8; x += 2) *reinterpret_cast<float2 *>(dst + 2 + 8 * c8 + x) = make_float2(acc[x], acc[x + 1]);
+            }
+            cluster_arrive();
+            cluster_wait();
+            const int c = tid & 63;
+            for (int k = tid >> 6; k == 0 || part + (k - 1) * split < n_rows; k += kF32Threads / 64) {   // 0: the fill row
+                const int r = k == 0 ? sum_row : part + (k - 1) * split;
+                const int i = k == 0 ? 0 : P.sel[r];
+                if (r < 0 || i < 0) continue;
+                const float v = merge_states(split, smem_u32(mine), r, c);
+                if (k == 0) P.vbar[c] = v;
+                else O[unit_off(g.os, b, h) + (long long)i * g.os[2] + c] = v;
+            }
+            cluster_arrive();                                   // done with the other CTAs' memory (awaited before the exit)
+        } else {
+            const float l = row < row_groups * 8 ? P.l[row] : 0.f, inv = l > 0.f ? 1.f / l : 0.f;
+#pragma unroll
+            for (int x = 0; x < 8; ++x) acc[x] *= inv;
+            if (row < n_rows) {
+                const int i = P.sel[row];
+                if (i >= 0) store8(O + unit_off(g.os, b, h) + (long long)i * g.os[2], c8, acc);
+            } else if (row == sum_row) {
+#pragma unroll
+                for (int x = 0; x < 8; ++x) P.vbar[8 * c8 + x] = acc[x];
+            }
+        }
+    }
+    __syncthreads();
+
+    // ---- step (e) -----------------------------------------------------------------------------
+    {
+        const int sub = tid & 7, per = (g.T + split - 1) / split;
+        float fillv[8], zero8[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) { fillv[t] = (L > 0 && !a.own_v) ? P.vbar[sub * 8 + t] : 0.f; zero8[t] = 0.f; }
+        float *Ou = O + unit_off(g.os, b, h);
+        for (int i = part * per + (tid >> 3); i < min(g.T, (part + 1) * per); i += kF32Threads / 8) {
+            float *dst = Ou + (long long)i * g.os[2];
+            if (i >= L) store8(dst, sub, zero8);
+            else if (chosen[i]) continue;
+            else if (a.own_v) { float v[8]; load8(Vu + (long long)i * g.vs[2], sub, v); store8(dst, sub, v); }
+            else store8(dst, sub, fillv);
+        }
+    }
+    if (SPLIT && L > 0) cluster_wait();                        // nobody reads this CTA's states any more
+}
+
+// CTAs per unit: as many (up to 8) as leave every cluster resident at once; see fused_split in psattn_fused.cu.
+static int f32_split(const Geom &g) {
+    static ClusterRecord clusters;
+    const int units = g.B * g.H;
+    if (g.T < 96) return 1;
+    for (int split = 8; split > 1; split >>= 1)
+        if (units <= max_clusters(k_forward_fused_fp32<true>, clusters, split, kF32Threads, kF32MaxSmem)) return split;
+    return 1;
+}
+
+// cudaErrorNotSupported: more than 63 selected rows or 64 samples, sequences too long for the selection's registers, or
+// sample lists shared by the queries (the caller runs the staged schedule).
+cudaError_t launch_forward_fused_fp32(const Geom &g, int U_max, int own_v, const void *Q, const void *K, const void *V,
+                                      const int *sidx, void *O, int *sel, float *M_out, const int *sel_in, cudaStream_t st) {
+    if (g.B * g.H == 0) return cudaSuccess;
+    const bool given = sel_in != nullptr;
+    if (g.u_max > kF32MaxRows - 1) return cudaErrorNotSupported;
+    if (!given && (U_max > 64 || U_max < 1 || g.idx_shared || g.T > 3 * kF32Threads)) return cudaErrorNotSupported;
+    Fused32Args a;
+    a.m_floats = given ? 0 : g.T;
+    const size_t tail = f32_arrays_bytes(a.m_floats, g.T) + sizeof(Fused32Persist) + 128;
+    const size_t keys = (size_t)g.T * 256;
+    a.resident = !given && keys + tail <= kF32MaxSmem;
+    const size_t phase = a.resident && keys > kF32AttendBytes ? keys : kF32AttendBytes;
+    a.off_persist = (uint32_t)((phase + 127) / 128 * 128);
+    const size_t smem = a.off_persist + tail;
+    if (smem > kF32MaxSmem) return cudaErrorNotSupported;
+    a.own_v = own_v;
+    a.sel_in = sel_in;
+    static SmemGrant grant, grant_split;
+    if (cudaError_t e = grant_dynamic_smem(k_forward_fused_fp32<false>, grant, kF32MaxSmem)) return e;
+    if (cudaError_t e = grant_dynamic_smem(k_forward_fused_fp32<true>, grant_split, kF32MaxSmem)) return e;
+    a.split = f32_split(g);
+    a.by_length = g.lengths != nullptr && g.B * g.H > device_sm_count() && g.B <= 256;
+    cudaError_t e = launch_split(a.split > 1 ? k_forward_fused_fp32<true> : k_forward_fused_fp32<false>, (unsigned)(g.B * g.H),
+                                 a.split, kF32Threads, smem, st, g, a, (const float *)Q, (const float *)K, (const float *)V,
+                                 sidx, (float *)O, sel, M_out);
+    note_launch();
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+}  // namespace psattn
