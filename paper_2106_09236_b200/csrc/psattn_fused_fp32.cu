@@ -1,8 +1,7 @@
 // The whole path (steps a-e) of one (batch, head) unit in one launch for fp32 inputs: psattn_fused.cu's plan in fp32
 // arithmetic on the FMA pipe (tf32 products would break the 1e-4 tolerance).
 //
-//   1. the unit's keys into shared memory where they fit (T up to about 870), then the measure, one warp per query, in the
-//      order of operations of the staged kernel, so that M~ has the same bits                       (Eq. 11)
+//   1. the unit's keys into shared memory where they fit (T up to about 870), then the measure, one warp per query (Eq. 11)
 //   2. block-wide selection                                                                        (Sec. 3.2)
 //   3. attention of the selected rows: chunks of 128 keys, scores in 8 x 2 register tiles, softmax, values in 4 x 4 register
 //      tiles with the keys of the chunk spread over the threads that the rows leave free; a zero query row
@@ -43,8 +42,8 @@ struct Fused32Persist {
     SelectScratch select;
     int sel[kF32MaxRows];
     float vbar[kD];
-    float m[kF32MaxRows], l[kF32MaxRows], alpha[kF32MaxRows];
-    float part[kF32MaxRows][2];          // row maxima, then row sums, of the two warps of a row group
+    float m[2][kF32MaxRows], l[kF32MaxRows];       // references before and after a chunk, in turn
+    float part[kF32MaxRows][2], sum[kF32MaxRows][2];         // row maxima and row sums of the two warps of a row group
     int b_ranked;
 };
 
@@ -56,14 +55,24 @@ struct F32Query {
     int key[2];
 };
 
-// M~ of the queries q_lo + warp, + 16, ... < q_hi of one unit, with the arithmetic of k_measure (psattn_staged.cu): four
-// groups of eight lanes, a group takes every fourth sampled key, 16 keys in flight.
-template <bool RESIDENT>
-__device__ __forceinline__ void f32_measure(const Geom &g, int unit, int b, int h, int L, int U, int q_lo, int q_hi,
+// M~ of the queries q_lo + warp, + 16, ... < q_hi of one unit.  Four groups of eight lanes, a group takes every fourth sampled
+// key (lane `sub` its columns 8 sub .. 8 sub + 7); 16 keys are in flight, and their 16 dot products are summed over the
+// eight lanes by exchanging halves (four shuffles instead of twelve), after which lane (grp, sub) holds the score of
+// sample 16 n + 4 x + grp, x = 2 (sub & 1) + (sub >> 1 & 1).  At most 64 samples, so all scores of a query stay in
+// registers: M~ = (1/U) sum_j (max - s_j) exactly as written, never negative and 0 for equal scores.
+// Resident rows hold their 16-byte piece c at c ^ (c >> 3): the even pieces of a row lie in eight different bank groups, and
+// so do the odd ones.
+// NB = ceil(U / 16) batches, straight-line, so that the loads of one run under the sums of another.
+template <bool RESIDENT, int NB>
+__device__ __forceinline__ void f32_measure_n(const Geom &g, int unit, int b, int h, int L, int U, int q_lo, int q_hi,
                                             const float *__restrict__ Qu, const float *Ku, long long k_pitch,
                                             const int *__restrict__ sidx, float *M_s) {
     const int lane = threadIdx.x & 31, sub = lane & 7, grp = lane >> 3, warp = threadIdx.x >> 5;
     const int *idx0 = sidx + (g.idx_per_head ? (long long)unit : (long long)b) * g.T * g.idx_cols;
+    const float4 *Kl = reinterpret_cast<const float4 *>(Ku) + (RESIDENT ? 0 : 2 * sub);    // (dense shared rows: 32-bit indices)
+    const int at_lo = 2 * sub ^ (sub >> 2), at_hi = (2 * sub + 1) ^ (sub >> 2);
+    const int mine = 4 * (2 * (sub & 1) + ((sub >> 1) & 1)) + grp;         // this lane's sample in a batch of 16
+    const bool b0 = sub & 1, b1 = sub & 2;
     auto fetch = [&](int i, F32Query &x) {
         if (i >= q_hi) return;
         load8(Qu + (long long)i * g.qs[2], sub, x.q);
@@ -76,58 +85,60 @@ __device__ __forceinline__ void f32_measure(const Geom &g, int unit, int b, int 
 #pragma unroll 1
     for (int i = q_lo + warp; i < q_hi; i += kF32Threads / 32) {
         fetch(i + kF32Threads / 32, nxt);
-        MeasureState st = measure_init();
-#pragma unroll 1
-        for (int base = 0; base < U; base += 32) {
-            int my = base == 0 ? cur.key[0] : cur.key[1];
-            if (base + lane < U && (my < 0 || my >= L)) { atomicOr(g.status, kStatusIdxClamped); my = my < 0 ? 0 : L - 1; }
-            const int steps = (min(32, U - base) + 3) >> 2;
-#pragma unroll 1
-            for (int s0 = 0; s0 < steps; s0 += 4) {
-                float kk[4][8], part[4];
-                bool active[4];
 #pragma unroll
-                for (int x = 0; x < 4; ++x) {
-                    const int src = (s0 + x) * 4 + grp;
-                    const int key = __shfl_sync(0xffffffffu, my, src & 31);
-                    active[x] = s0 + x < steps && base + src < U;
-                    const float *kr = Ku + (long long)(active[x] ? key : 0) * k_pitch;
-                    if (RESIDENT) {
-                        const float4 a = reinterpret_cast<const float4 *>(kr)[2 * sub], c = reinterpret_cast<const float4 *>(kr)[2 * sub + 1];
-                        kk[x][0] = a.x; kk[x][1] = a.y; kk[x][2] = a.z; kk[x][3] = a.w;
-                        kk[x][4] = c.x; kk[x][5] = c.y; kk[x][6] = c.z; kk[x][7] = c.w;
-                    } else {
-                        load8(kr, sub, kk[x]);
-                    }
+        for (int x = 0; x < 2; ++x)
+            if ((unsigned)cur.key[x] >= (unsigned)L) { atomicOr(g.status, kStatusIdxClamped); cur.key[x] = cur.key[x] < 0 ? 0 : L - 1; }
+        float s[NB];
+        float mx = -INFINITY;
+#pragma unroll
+        for (int n = 0; n < NB; ++n) {
+            float part[4];
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {                      // (a sample behind the last reads row 0; its score is dropped)
+                const int key = __shfl_sync(0xffffffffu, cur.key[n >> 1], (n & 1) * 16 + x * 4 + grp);
+                float4 lo, hi;
+                if (RESIDENT) { lo = Kl[key * 16 + at_lo]; hi = Kl[key * 16 + at_hi]; }
+                else {
+                    const float4 *kr = Kl + (long long)key * (k_pitch >> 2);
+                    lo = __ldg(kr); hi = __ldg(kr + 1);
                 }
-#pragma unroll
-                for (int x = 0; x < 4; ++x) {
-                    part[x] = 0.f;
-#pragma unroll
-                    for (int t = 0; t < 8; ++t) part[x] = fmaf(cur.q[t], kk[x][t], part[x]);
-                }
-#pragma unroll
-                for (int x = 0; x < 4; ++x) {
-                    part[x] += __shfl_xor_sync(0xffffffffu, part[x], 1);
-                    part[x] += __shfl_xor_sync(0xffffffffu, part[x], 2);
-                    part[x] += __shfl_xor_sync(0xffffffffu, part[x], 4);
-                }
-#pragma unroll
-                for (int x = 0; x < 4; ++x)
-                    if (active[x]) measure_push(st, part[x] * kScale);
+                float p = cur.q[0] * lo.x;
+                p = fmaf(cur.q[1], lo.y, p); p = fmaf(cur.q[2], lo.z, p); p = fmaf(cur.q[3], lo.w, p);
+                p = fmaf(cur.q[4], hi.x, p); p = fmaf(cur.q[5], hi.y, p); p = fmaf(cur.q[6], hi.z, p); p = fmaf(cur.q[7], hi.w, p);
+                part[x] = p;
             }
+            const float r0 = (b0 ? part[2] : part[0]) + __shfl_xor_sync(0xffffffffu, b0 ? part[0] : part[2], 1);
+            const float r1 = (b0 ? part[3] : part[1]) + __shfl_xor_sync(0xffffffffu, b0 ? part[1] : part[3], 1);
+            float v = (b1 ? r1 : r0) + __shfl_xor_sync(0xffffffffu, b1 ? r0 : r1, 2);
+            v += __shfl_xor_sync(0xffffffffu, v, 4);
+            s[n] = n * 16 + mine < U ? v * kScale : -INFINITY;
+            mx = fmaxf(mx, s[n]);
         }
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
+        float D = 0.f;
 #pragma unroll
-        for (int o = 8; o <= 16; o <<= 1) {
-            MeasureState other;
-            other.m = __shfl_xor_sync(0xffffffffu, st.m, o);
-            other.D = __shfl_xor_sync(0xffffffffu, st.D, o);
-            other.n = __shfl_xor_sync(0xffffffffu, st.n, o);
-            st = (lane & o) ? measure_merge(other, st) : measure_merge(st, other);
-        }
-        if (lane == 0) M_s[i] = U > 0 ? st.D / (float)U : 0.f;
+        for (int n = 0; n < NB; ++n)
+            if (n * 16 + mine < U) D += mx - s[n];
+        D += __shfl_xor_sync(0xffffffffu, D, 1);
+        D += __shfl_xor_sync(0xffffffffu, D, 2);
+        D += __shfl_xor_sync(0xffffffffu, D, 8);
+        D += __shfl_xor_sync(0xffffffffu, D, 16);
+        if (lane == 0) M_s[i] = U > 0 ? D / (float)U : 0.f;
         cur = nxt;
     }
+}
+
+template <bool RESIDENT>
+__device__ __forceinline__ void f32_measure(const Geom &g, int unit, int b, int h, int L, int U, int q_lo, int q_hi,
+                                            const float *__restrict__ Qu, const float *Ku, long long k_pitch,
+                                            const int *__restrict__ sidx, float *M_s) {
+    if (U <= 16) f32_measure_n<RESIDENT, 1>(g, unit, b, h, L, U, q_lo, q_hi, Qu, Ku, k_pitch, sidx, M_s);
+    else if (U <= 32) f32_measure_n<RESIDENT, 2>(g, unit, b, h, L, U, q_lo, q_hi, Qu, Ku, k_pitch, sidx, M_s);
+    else if (U <= 48) f32_measure_n<RESIDENT, 3>(g, unit, b, h, L, U, q_lo, q_hi, Qu, Ku, k_pitch, sidx, M_s);
+    else f32_measure_n<RESIDENT, 4>(g, unit, b, h, L, U, q_lo, q_hi, Qu, Ku, k_pitch, sidx, M_s);
 }
 
 // Eight values per lane, reduced over the warp: lane l returns the result of value l >> 2 (the same in its four lanes).
@@ -154,17 +165,27 @@ __device__ __forceinline__ float f32_reduce8(const float v[8], Op op) {
 }
 
 // Rows of 256 bytes from global memory into shared memory, `n` of them (zeros from `valid` on), pitch in floats.
-__device__ __forceinline__ void f32_stage_rows(uint32_t dst, uint32_t pitch, const float *src, long long stride, int n, int valid) {
+// `spread`: 16-byte piece c at c ^ (c >> 3) (see f32_measure).
+__device__ __forceinline__ void f32_stage_rows(uint32_t dst, uint32_t pitch, const float *src, long long stride, int n, int valid,
+                                               bool spread = false) {
 #pragma unroll 4
     for (int e = threadIdx.x; e < n * 16; e += kF32Threads) {
         const int r = e >> 4, c = e & 15;
-        const uint32_t d = dst + ((uint32_t)r * pitch + (uint32_t)c * 4u) * 4u;
+        const int at = spread ? c ^ (c >> 3) : c;
+        const uint32_t d = dst + ((uint32_t)r * pitch + (uint32_t)at * 4u) * 4u;
         if (r < valid) cp_async_16(d, src + (long long)r * stride + c * 4);
         else asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(d), "r"(0) : "memory");
     }
 }
 
-// The attention of the listed rows over the keys [lo, hi): on return P.m / P.l hold the row states and the partial sums of the
+// acc += (a0 b0, a1 b1) in one instruction
+__device__ __forceinline__ void f32_fma2(float2 &acc, float a0, float a1, float b0, float b1) {
+    asm("{\n\t.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tmov.b64 z, {%0, %1};\n\t"
+        "fma.rn.f32x2 z, x, y, z;\n\tmov.b64 {%0, %1}, z;\n\t}"
+        : "+f"(acc.x), "+f"(acc.y) : "f"(a0), "f"(a1), "f"(b0), "f"(b1));
+}
+
+// The attention of the listed rows over the keys [lo, hi): on return P.m[0] / P.l hold the row states and the partial sums of the
 // unnormalised rows lie at kF32OffP as [splits][rows][64]; returns splits.  Contains __syncthreads.
 __device__ __forceinline__ int f32_attend(uint8_t *smem, const Geom &g, Fused32Persist &P, int b, int h, int L, int lo, int hi,
                                           int n_rows, int row_groups, const float *__restrict__ Qu,
@@ -190,39 +211,55 @@ __device__ __forceinline__ int f32_attend(uint8_t *smem, const Geom &g, Fused32P
         if (i >= 0 && i < L) v = __ldg(reinterpret_cast<const float4 *>(Qu + (long long)i * g.qs[2]) + c);
         reinterpret_cast<float4 *>(Qs)[e] = v;
     }
-    if (tid < kF32MaxRows) { P.m[tid] = -INFINITY; P.l[tid] = 0.f; }
+    if (tid < kF32MaxRows) { P.m[0][tid] = -INFINITY; P.l[tid] = 0.f; }
     if (n_chunks > 0) { stage_k(0); stage_v(0); }
 
     // scores: row group rg (8 rows), keys kg and kg + 64 of the chunk; values: row quad rq, columns 4 cq .., keys ks + splits * n
     const int kg = tid & 63, rg = tid >> 6;
     const int quads = 2 * row_groups, splits = kF32Threads / (16 * quads);
     const int cq = tid & 15, rq = (tid >> 4) % quads, ks = (tid >> 4) / quads;
-    float o[4][4];
+    float2 o[4][2];
 #pragma unroll
     for (int x = 0; x < 4; ++x)
 #pragma unroll
-        for (int y = 0; y < 4; ++y) o[x][y] = 0.f;
+        for (int y = 0; y < 2; ++y) o[x][y] = make_float2(0.f, 0.f);
 #pragma unroll 1
     for (int c = 0; c < n_chunks; ++c) {
         const int valid = min(kF32Chunk, hi - lo - c * kF32Chunk);
         cp_async_wait<1>();                                    // K of this chunk (V may still be on its way)
         __syncthreads();
         float s[8][2];
+        const bool lower = kg - lane < valid, upper = kg - lane + 64 < valid;  // of this warp's keys any exist (uniform)
         if (rg < row_groups) {
-#pragma unroll
-            for (int x = 0; x < 8; ++x) s[x][0] = s[x][1] = 0.f;
             const float4 *q = reinterpret_cast<const float4 *>(Qs + rg * 8 * 64);
-            const float4 *k0 = reinterpret_cast<const float4 *>(Ks + kg * kF32KPitch), *k1 = reinterpret_cast<const float4 *>(Ks + (kg + 64) * kF32KPitch);
-#pragma unroll 2
-            for (int d = 0; d < 16; ++d) {
-                const float4 a = k0[d], e = k1[d];
+            const float4 *k = reinterpret_cast<const float4 *>(Ks + kg * kF32KPitch);
+            float2 e[8][2];                                    // sums over the even and the odd columns
 #pragma unroll
-                for (int x = 0; x < 8; ++x) {
-                    const float4 v = q[x * 16 + d];
-                    s[x][0] = fmaf(v.x, a.x, s[x][0]); s[x][0] = fmaf(v.y, a.y, s[x][0]); s[x][0] = fmaf(v.z, a.z, s[x][0]); s[x][0] = fmaf(v.w, a.w, s[x][0]);
-                    s[x][1] = fmaf(v.x, e.x, s[x][1]); s[x][1] = fmaf(v.y, e.y, s[x][1]); s[x][1] = fmaf(v.z, e.z, s[x][1]); s[x][1] = fmaf(v.w, e.w, s[x][1]);
+            for (int x = 0; x < 8; ++x) e[x][0] = e[x][1] = make_float2(0.f, 0.f);
+            if (upper) {                                       // both keys share the loads of the query rows
+#pragma unroll 1
+                for (int d = 0; d < 16; ++d) {
+                    const float4 a0 = k[d], a1 = k[64 * kF32KPitch / 4 + d];
+#pragma unroll
+                    for (int x = 0; x < 8; ++x) {
+                        const float4 v = q[x * 16 + d];
+                        f32_fma2(e[x][0], v.x, v.y, a0.x, a0.y); f32_fma2(e[x][0], v.z, v.w, a0.z, a0.w);
+                        f32_fma2(e[x][1], v.x, v.y, a1.x, a1.y); f32_fma2(e[x][1], v.z, v.w, a1.z, a1.w);
+                    }
+                }
+            } else if (lower) {
+#pragma unroll 2
+                for (int d = 0; d < 16; ++d) {
+                    const float4 a0 = k[d];
+#pragma unroll
+                    for (int x = 0; x < 8; ++x) {
+                        const float4 v = q[x * 16 + d];
+                        f32_fma2(e[x][0], v.x, v.y, a0.x, a0.y); f32_fma2(e[x][0], v.z, v.w, a0.z, a0.w);
+                    }
                 }
             }
+#pragma unroll
+            for (int x = 0; x < 8; ++x) { s[x][0] = e[x][0].x + e[x][0].y; s[x][1] = e[x][1].x + e[x][1].y; }
             float mx[8];
 #pragma unroll
             for (int x = 0; x < 8; ++x) {
@@ -235,17 +272,15 @@ __device__ __forceinline__ int f32_attend(uint8_t *smem, const Geom &g, Fused32P
         }
         __syncthreads();
         if (c + 1 < n_chunks) stage_k(c + 1); else cp_async_commit();          // the K buffer is free
-        if (tid < row_groups * 8) {
-            const float m = P.m[tid], n = fmaxf(m, fmaxf(P.part[tid][0], P.part[tid][1]));
-            P.alpha[tid] = exp2f(m - n);                       // 0 on the first chunk (m = -inf)
-            P.m[tid] = n;
-        }
-        __syncthreads();
+        // the new reference of a row, from what everyone can read; P.m of the next chunk is written beside it
+        const float *m_old = P.m[c & 1];
+        auto m_new = [&](int r) { return fmaxf(m_old[r], fmaxf(P.part[r][0], P.part[r][1])); };
+        if (tid < row_groups * 8) P.m[(c + 1) & 1][tid] = m_new(tid);
         if (rg < row_groups) {
             float sum[8];
 #pragma unroll
             for (int x = 0; x < 8; ++x) {
-                const float m = P.m[rg * 8 + x];
+                const float m = m_new(rg * 8 + x);
                 s[x][0] = exp2f(s[x][0] - m); s[x][1] = exp2f(s[x][1] - m);
                 sum[x] = s[x][0] + s[x][1];
             }
@@ -256,25 +291,25 @@ __device__ __forceinline__ int f32_attend(uint8_t *smem, const Geom &g, Fused32P
                 dst[1] = make_float4(s[4][y], s[5][y], s[6][y], s[7][y]);
             }
             const float r = f32_reduce8(sum, [](float a, float e) { return a + e; });
-            if ((lane & 3) == 0) P.part[rg * 8 + (lane >> 2)][(tid >> 5) & 1] = r;
+            if ((lane & 3) == 0) P.sum[rg * 8 + (lane >> 2)][(tid >> 5) & 1] = r;
         }
         cp_async_wait<1>();                                    // V of this chunk
         __syncthreads();
-        if (tid < row_groups * 8) P.l[tid] = P.l[tid] * P.alpha[tid] + (P.part[tid][0] + P.part[tid][1]);
+        const float *m_cur = P.m[(c + 1) & 1];                 // alpha = exp2(old - new): 0 on the first chunk (m = -inf)
+        if (tid < row_groups * 8) P.l[tid] = P.l[tid] * exp2f(m_old[tid] - m_cur[tid]) + (P.sum[tid][0] + P.sum[tid][1]);
         if (ks < splits) {
 #pragma unroll
             for (int x = 0; x < 4; ++x) {
-                const float al = P.alpha[rq * 4 + x];
+                const float al = exp2f(m_old[rq * 4 + x] - m_cur[rq * 4 + x]);
 #pragma unroll
-                for (int y = 0; y < 4; ++y) o[x][y] *= al;
+                for (int y = 0; y < 2; ++y) { o[x][y].x *= al; o[x][y].y *= al; }
             }
 #pragma unroll 4
             for (int k = ks; k < valid; k += splits) {
                 const float4 p = *reinterpret_cast<const float4 *>(Ps + k * kF32PPitch + rq * 4), v = *reinterpret_cast<const float4 *>(Vs + k * 64 + cq * 4);
-                o[0][0] = fmaf(p.x, v.x, o[0][0]); o[0][1] = fmaf(p.x, v.y, o[0][1]); o[0][2] = fmaf(p.x, v.z, o[0][2]); o[0][3] = fmaf(p.x, v.w, o[0][3]);
-                o[1][0] = fmaf(p.y, v.x, o[1][0]); o[1][1] = fmaf(p.y, v.y, o[1][1]); o[1][2] = fmaf(p.y, v.z, o[1][2]); o[1][3] = fmaf(p.y, v.w, o[1][3]);
-                o[2][0] = fmaf(p.z, v.x, o[2][0]); o[2][1] = fmaf(p.z, v.y, o[2][1]); o[2][2] = fmaf(p.z, v.z, o[2][2]); o[2][3] = fmaf(p.z, v.w, o[2][3]);
-                o[3][0] = fmaf(p.w, v.x, o[3][0]); o[3][1] = fmaf(p.w, v.y, o[3][1]); o[3][2] = fmaf(p.w, v.z, o[3][2]); o[3][3] = fmaf(p.w, v.w, o[3][3]);
+                const float pr[4] = {p.x, p.y, p.z, p.w};
+#pragma unroll
+                for (int x = 0; x < 4; ++x) { f32_fma2(o[x][0], pr[x], pr[x], v.x, v.y); f32_fma2(o[x][1], pr[x], pr[x], v.z, v.w); }
             }
         }
         __syncthreads();
@@ -282,10 +317,11 @@ __device__ __forceinline__ int f32_attend(uint8_t *smem, const Geom &g, Fused32P
     }
     cp_async_wait<0>();
     __syncthreads();
+    if ((n_chunks & 1) && tid < row_groups * 8) P.m[0][tid] = P.m[1][tid];
     if (ks < splits) {
 #pragma unroll
         for (int x = 0; x < 4; ++x)
-            *reinterpret_cast<float4 *>(Ps + ((ks * quads + rq) * 4 + x) * 64 + cq * 4) = make_float4(o[x][0], o[x][1], o[x][2], o[x][3]);
+            *reinterpret_cast<float4 *>(Ps + ((ks * quads + rq) * 4 + x) * 64 + cq * 4) = make_float4(o[x][0].x, o[x][0].y, o[x][1].x, o[x][1].y);
     }
     __syncthreads();
     return splits;
@@ -327,16 +363,18 @@ __global__ void __launch_bounds__(kF32Threads, 1) k_forward_fused_fp32(
     const float *Qu = Q + unit_off(g.qs, b, h), *Ku = K + unit_off(g.ks, b, h), *Vu = V + unit_off(g.vs, b, h);
     for (int i = tid; i < g.T; i += kF32Threads) { chosen[i] = 0; if (i >= L && !given) M_s[i] = 0.f; }
 
+    phase_stamp(g, 0);
     // ---- steps (a)+(b): every CTA of the unit a range of the queries; its values go to the others -----------------
     if (SPLIT) cluster_wait();                                  // every CTA of the unit runs
     if (L > 0 && !given) {
         const int per = (L + split - 1) / split;
         const int q_lo = min(part * per, L), q_hi = min(q_lo + per, L);
         if (a.resident) {
-            f32_stage_rows(smem_u32(smem), 64, Ku, g.ks[2], L, L);
+            f32_stage_rows(smem_u32(smem), 64, Ku, g.ks[2], L, L, true);
             cp_async_commit();
             cp_async_wait<0>();
             __syncthreads();
+            phase_stamp(g, 1);                                 // the keys have landed
             f32_measure<true>(g, unit, b, h, L, U, q_lo, q_hi, Qu, reinterpret_cast<const float *>(smem), 64, sidx, M_s);
         } else {
             f32_measure<false>(g, unit, b, h, L, U, q_lo, q_hi, Qu, Ku, g.ks[2], sidx, M_s);
@@ -352,6 +390,7 @@ __global__ void __launch_bounds__(kF32Threads, 1) k_forward_fused_fp32(
         }
     }
     __syncthreads();
+    phase_stamp(g, 2);                                         // steps (a)+(b) done
     if (M_out != nullptr && !given && part == 0)
         for (int i = tid; i < g.T; i += kF32Threads) M_out[(long long)unit * g.T + i] = M_s[i];
 
@@ -372,6 +411,7 @@ __global__ void __launch_bounds__(kF32Threads, 1) k_forward_fused_fp32(
         }
     }
     __syncthreads();
+    phase_stamp(g, 3);                                         // step (c) done
 
     // ---- step (d), with the column sums of V as one more row ------------------------------------------------
     if (L > 0) {
@@ -380,6 +420,7 @@ __global__ void __launch_bounds__(kF32Threads, 1) k_forward_fused_fp32(
         const int per = SPLIT ? (L + split - 1) / split : L;
         const int lo = min(part * per, L), hi = min(lo + per, L);
         const int splits = f32_attend(smem, g, P, b, h, L, lo, hi, n_rows, row_groups, Qu, Ku, Vu);
+        phase_stamp(g, 6);                                     // step (d): the merge is left
         const float *Ps = reinterpret_cast<const float *>(smem + kF32OffP);
         const int row = tid >> 3, c8 = tid & 7;
         float acc[8];
@@ -398,7 +439,7 @@ __global__ void __launch_bounds__(kF32Threads, 1) k_forward_fused_fp32(
             float *mine = reinterpret_cast<float *>(smem + kF32OffV);
             if (row < row_groups * 8) {
                 float *dst = mine + row * 66;
-                if (c8 == 0) { dst[0] = P.m[row]; dst[1] = P.l[row]; }
+                if (c8 == 0) { dst[0] = P.m[0][row]; dst[1] = P.l[row]; }
 #pragma unroll
                 for (int x = 0; x < 8; x += 2) *reinterpret_cast<float2 *>(dst + 2 + 8 * c8 + x) = make_float2(acc[x], acc[x + 1]);
             }
@@ -428,6 +469,7 @@ __global__ void __launch_bounds__(kF32Threads, 1) k_forward_fused_fp32(
         }
     }
     __syncthreads();
+    phase_stamp(g, 4);                                         // step (d) done
 
     // ---- step (e) -----------------------------------------------------------------------------
     {
@@ -444,6 +486,8 @@ __global__ void __launch_bounds__(kF32Threads, 1) k_forward_fused_fp32(
             else store8(dst, sub, fillv);
         }
     }
+    __syncthreads();
+    phase_stamp(g, 5);                                         // step (e) done
     if (SPLIT && L > 0) cluster_wait();                        // nobody reads this CTA's states any more
 }
 
