@@ -406,7 +406,7 @@ extern "C" int psattn_forward(psattn_plan_t *plan, const void *Q, const void *K,
     Geom g = make_geom(plan, lengths, workspace);
     if (d.dtype == PSATTN_BF16 && d.path != PSATTN_PATH_STAGED && !d.idx_shared) {
         cudaError_t e = launch_forward_fused(g, plan->U_max, d.fill_mode == PSATTN_FILL_OWN_V, Q, K, V, sample_idx, O,
-                                             sel_idx, M_out, nullptr, st);
+                                             sel_idx, M_out, nullptr, nullptr, st);
         if (e == cudaSuccess) return PSATTN_OK;
         if (e != cudaErrorNotSupported) return cuda_fail(plan, e);
         if (d.path == PSATTN_PATH_FUSED) return PSATTN_ERR_UNSUPPORTED;
@@ -419,6 +419,13 @@ extern "C" int psattn_forward(psattn_plan_t *plan, const void *Q, const void *K,
         if (e != cudaErrorNotSupported) return cuda_fail(plan, e);
     }
     float *M = M_out ? M_out : ws_at<float>(workspace, plan->off_M);
+    if (d.dtype == PSATTN_BF16 && d.path == PSATTN_PATH_AUTO && fused_from_measure_supported(g, K, V)) {
+        // keys too long for shared memory: the measure by itself, the rest in one kernel
+        if ((rc = run_measure(plan, g, Q, K, sample_idx, M, st)) != PSATTN_OK) return rc;
+        PSATTN_CU(launch_forward_fused(g, plan->U_max, d.fill_mode == PSATTN_FILL_OWN_V, Q, K, V, nullptr, O, sel_idx, nullptr,
+                                       nullptr, M, st));
+        return PSATTN_OK;
+    }
     if (vbar_from_attention(plan, g, K, V)) {
         // Steps (a)-(c) do not touch V or O, and they are bound by on-chip gathers, not by HBM: the fill of
         // step (e) - column sums of V, mean(V), every valid row of O - runs beside them on the plan's side
@@ -467,7 +474,7 @@ extern "C" int psattn_forward_with_selection(psattn_plan_t *plan, const void *Q,
     if (d.dtype == PSATTN_BF16 && d.path != PSATTN_PATH_STAGED) {
         // one kernel for steps (d)+(e): one CTA per unit, or a cluster of CTAs where the units are few
         cudaError_t e = launch_forward_fused(g, plan->U_max, d.fill_mode == PSATTN_FILL_OWN_V, Q, K, V, nullptr, O,
-                                             nullptr, nullptr, sel_idx_in, st);
+                                             nullptr, nullptr, sel_idx_in, nullptr, st);
         if (e == cudaSuccess) return PSATTN_OK;
         if (e != cudaErrorNotSupported) return cuda_fail(plan, e);
     }

@@ -10,7 +10,8 @@
 //   4. mean(V) (or the query's own value row) is written to every other valid row of O, zeros
 //      to padded rows                                                         (Eq. 12)
 // With a given index set (the reuse of one layer's selection by the following layers, Sec. 4.4) steps
-// 1 and 2 are skipped and the kernel is steps (d)+(e) in one launch.
+// 1 and 2 are skipped and the kernel is steps (d)+(e) in one launch; where the keys do not fit, a measure kernel runs before and the
+// kernel starts at step 2.
 // HBM traffic is the algorithmic minimum: Q, K, V read once (K a second time out of L2), O
 // written once.  M~ never leaves the SM unless the caller asks for it.
 #include "psattn_attend_rows.cuh"
@@ -39,7 +40,8 @@ struct FusedArgs {
     int by_length;                       // CTAs take the sequences in descending order of length
     int split;                           // CTAs per unit (one thread-block cluster): 1, 2, 4 or 8
     int m_floats;                        // floats of the M~ array (0 with a given index set)
-    const int *sel_in;                   // non-null: a given index set [unit][u_max] replaces steps (a)-(c)
+    const int *sel_in;                   // kGivenSet: the index set [unit][u_max]
+    const float *M_in;                   // kGivenMeasure: M~ [unit][T]
 };
 
 struct FusedPersist {                    // at smem + off_persist, after the M~ array and the flags
@@ -53,7 +55,11 @@ struct FusedPersist {                    // at smem + off_persist, after the M~ 
 __host__ __device__ inline size_t fused_arrays_bytes(int m_floats, int T) { return ((size_t)4 * m_floats + T + 127) / 128 * 128; }
 
 // SPLIT: the unit is shared by the a.split > 1 CTAs of a thread-block cluster.
-template <bool SPLIT>
+// MODE: all steps, or from step (c) on with M~ in global memory (sequences too long for resident keys), or steps (d)+(e).
+enum FusedMode { kAllSteps = 0, kGivenMeasure = 1, kGivenSet = 2 };
+constexpr int kFusedSelectKeys = kSelectMaxSlots * (kFusedThreads - 32);       // longest sequence of the block-wide selection
+
+template <bool SPLIT, int MODE>
 __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
     Geom g, FusedArgs a, const __nv_bfloat16 *__restrict__ Q, const __nv_bfloat16 *__restrict__ V,
     const int *__restrict__ sidx, __nv_bfloat16 *__restrict__ O, int *__restrict__ sel_out, float *__restrict__ M_out,
@@ -99,14 +105,14 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
     const int L = seq_len(g, b);
     const int U = min(g.U_tab[L], g.idx_cols);
     const int u = min(min(g.u_tab[L], g.u_max), L);
-    const bool given = a.sel_in != nullptr;                    // steps (d)+(e) only, for a given index set
+    constexpr bool all_steps = MODE == kAllSteps, given = MODE == kGivenSet;
     if (tid == 32) {
         mbar_init(&P.bar, 1);
         fence_barrier_init();
-        if (L > 0 && !given) measure_issue_keys(smem, &P.bar, &tmKrows, L, b, h, a.pos_t, a.pos_h, g.debug_extra_tx);
+        if (all_steps && L > 0) measure_issue_keys(smem, &P.bar, &tmKrows, L, b, h, a.pos_t, a.pos_h, g.debug_extra_tx);
         tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV);
     }
-    for (int i = tid; i < g.T; i += kFusedThreads) { chosen[i] = 0; if (i >= L && !given) M_s[i] = 0.f; }
+    for (int i = tid; i < g.T; i += kFusedThreads) { chosen[i] = 0; if (all_steps && i >= L) M_s[i] = 0.f; }
     __syncthreads();
     phase_stamp(g, 0);
 
@@ -115,7 +121,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
     // its values to the others: every CTA then holds all of M~)
     bool ok = true;
     if (SPLIT) cluster_wait();                              // every CTA of the unit runs
-    if (L > 0 && !given) {
+    if (all_steps && L > 0) {
         const int per = ((L + split - 1) / split + 7) & ~7;
         const int q_lo = min(part * per, L), q_hi = min(q_lo + per, L);
         ok = measure_resident<kFusedThreads>(smem, &P.bar, 0u, a.k_bytes, a.stage_bytes, g, unit, b, h, L, U, q_lo, q_hi,
@@ -132,7 +138,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
     }
     __syncthreads();
     phase_stamp(g, 2);                                         // steps (a)+(b) done (stamp 1: the keys had landed)
-    if (M_out != nullptr && !given && part == 0)
+    if (all_steps && M_out != nullptr && part == 0)
         for (int i = tid; i < g.T; i += kFusedThreads) M_out[(long long)unit * g.T + i] = M_s[i];
 
     // The attention phase reuses the shared memory of the measure phase, which is free now; its first
@@ -155,7 +161,14 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
         if (ok && L > 0 && tid == kArLoader) attend_rows_start(smem, j, &tmK, &tmV, ahead);
     } else if (!given) {
         // ---- step (c) ---------------------------------------------------------------------------
-        block_select_short<3>([&](int i) { return float_key(M_s[i]); }, L, u, kArMaxRows, P.sel, P.select, kSelectors, 1);
+        if (all_steps) {
+            block_select_short<3>([&](int i) { return float_key(M_s[i]); }, L, u, kArMaxRows, P.sel, P.select, kSelectors, 1);
+        } else {
+            const float *Mu = a.M_in + (long long)unit * g.T;
+            auto key_of = [&](int i) { return float_key(__ldg(Mu + i)); };
+            if (L <= 6 * kSelectors) block_select_short<6>(key_of, L, u, kArMaxRows, P.sel, P.select, kSelectors, 1);
+            else block_select_short<kSelectMaxSlots>(key_of, L, u, kArMaxRows, P.sel, P.select, kSelectors, 1);
+        }
         for (int r = tid; r < g.u_max; r += kSelectors) {
             const int i = r < kArMaxRows ? P.sel[r] : -1;
             if (part == 0) sel_out[(long long)unit * g.u_max + r] = i;
@@ -248,24 +261,36 @@ bool make_rows_map(CUtensorMap *map, const void *base, const Geom &g, const long
 // Measured, us per call with 1 / 2 / 4 / 8 CTAs per unit: B1 H4 T128 15.8 / 17.8 / 17.5 / 18.3, T203 18.8 / 18.9 /
 // 17.8 / 18.5, T512 30.0 / 23.3 / 20.9 / 19.9, T1000 47.3 / 33.4 / 25.7 / 22.1; with a given index set B1 H4 T512
 // 11.1 / 11.4 / 12.3 / 12.4, T1000 17.4 / 15.1 / 13.9 / 13.1, T3000 34.2 / 24.3 / 19.0 / 14.3.
-static int fused_split(const Geom &g, bool given) {
+static int fused_split(const Geom &g, int mode) {
     static ClusterRecord clusters;
     const int units = g.B * g.H;
-    if (g.T < (given ? 768 : 192)) return 1;
+    if (g.T < (mode == kAllSteps ? 192 : 768)) return 1;
     for (int split = 8; split > 1; split >>= 1)
-        if (units <= max_clusters(k_forward_fused<true>, clusters, split, kFusedThreads, kFusedMaxSmem)) return split;
+        if (units <= max_clusters(k_forward_fused<true, kAllSteps>, clusters, split, kFusedThreads, kFusedMaxSmem)) return split;
     return 1;
+}
+
+static size_t fused_given_smem(int T) {
+    return (kArBytes + 1023) / 1024 * 1024 + fused_arrays_bytes(0, T) + sizeof(FusedPersist) + 128;
+}
+
+// Host-side check with no side effect: would launch_forward_fused take this call with M~ given?
+bool fused_from_measure_supported(const Geom &g, const void *K, const void *V) {
+    return g.u_max <= kArMaxRows - 1 && g.T <= kFusedSelectKeys && fused_given_smem(g.T) <= kFusedMaxSmem &&
+           attend64_supported(g, K, V, g.u_max, 1);
 }
 
 // cudaErrorNotSupported when the shape does not fit this kernel (the caller runs the staged schedule):
 // keys + staging beyond shared memory, more than 63 selected rows or 64 samples, no tensor map.
 cudaError_t launch_forward_fused(const Geom &g, int U_max, int own_v, const void *Q, const void *K, const void *V,
-                                 const int *sidx, void *O, int *sel, float *M_out, const int *sel_in, cudaStream_t st) {
+                                 const int *sidx, void *O, int *sel, float *M_out, const int *sel_in, const float *M_in,
+                                 cudaStream_t st) {
     if (g.B * g.H == 0) return cudaSuccess;
     if (g.u_max > kArMaxRows - 1) return cudaErrorNotSupported;
-    if (sel_in == nullptr && (U_max > kMeasureMaxU || U_max < 1)) return cudaErrorNotSupported;
+    if (sel_in == nullptr && M_in == nullptr && (U_max > kMeasureMaxU || U_max < 1)) return cudaErrorNotSupported;
     FusedArgs a;
-    const bool given = sel_in != nullptr;
+    const int mode = sel_in != nullptr ? kGivenSet : (M_in != nullptr ? kGivenMeasure : kAllSteps);
+    const bool given = mode != kAllSteps;
     a.k_bytes = given ? 0u : (uint32_t)measure_k_bytes(g.T);
     a.stage_bytes = given ? 0u : (uint32_t)measure_stage_bytes(kFusedThreads, g.idx_cols);
     a.m_floats = given ? 0 : g.T;
@@ -273,7 +298,9 @@ cudaError_t launch_forward_fused(const Geom &g, int U_max, int own_v, const void
     if (phase < kArBytes) phase = kArBytes;
     a.off_persist = (uint32_t)((phase + 1023) / 1024 * 1024);
     const size_t smem = a.off_persist + fused_arrays_bytes(a.m_floats, g.T) + sizeof(FusedPersist) + 128;
-    if (smem > kFusedMaxSmem || (!given && g.T > 3 * (kFusedThreads - 32))) return cudaErrorNotSupported;   // (block_select_short<3>)
+    if (smem > kFusedMaxSmem) return cudaErrorNotSupported;
+    if (mode == kAllSteps && g.T > 3 * (kFusedThreads - 32)) return cudaErrorNotSupported;     // (block_select_short<3>)
+    if (mode == kGivenMeasure && g.T > kFusedSelectKeys) return cudaErrorNotSupported;
     CUtensorMap tmKrows, tmK, tmV;
     int p0[3], p1[3], p2[3];
     if (!make_rows_map(&tmKrows, K, g, g.ks, kMeasureBoxRows, 0, p0) || !make_rows_map(&tmK, K, g, g.ks, 128, 1, p1) ||
@@ -284,18 +311,23 @@ cudaError_t launch_forward_fused(const Geom &g, int U_max, int own_v, const void
     a.pos_t = p0[0]; a.pos_h = p0[1]; a.pos_b = p0[2];
     a.own_v = own_v;
     a.sel_in = sel_in;
+    a.M_in = M_in;
     // the ranking costs B comparisons per sequence in every CTA: only where a second wave exists and B is small
     a.by_length = g.lengths != nullptr && g.B * g.H > device_sm_count() && g.B <= 256;
-    static SmemGrant grant;
-    static SmemGrant grant_split;
-    if (cudaError_t e = grant_dynamic_smem(k_forward_fused<false>, grant, kFusedMaxSmem)) return e;
-    if (cudaError_t e = grant_dynamic_smem(k_forward_fused<true>, grant_split, kFusedMaxSmem)) return e;
-    a.split = fused_split(g, given);
+    using Kernel = decltype(&k_forward_fused<false, kAllSteps>);
+    static const Kernel kernels[3][2] = {{k_forward_fused<false, kAllSteps>, k_forward_fused<true, kAllSteps>},
+                                         {k_forward_fused<false, kGivenMeasure>, k_forward_fused<true, kGivenMeasure>},
+                                         {k_forward_fused<false, kGivenSet>, k_forward_fused<true, kGivenSet>}};
+    static SmemGrant grants[3][2];
+    for (int x = 0; x < 2; ++x)
+        if (cudaError_t e = grant_dynamic_smem(kernels[mode][x], grants[mode][x], kFusedMaxSmem)) return e;
+    if (cudaError_t e = grant_dynamic_smem(kernels[0][1], grants[0][1], kFusedMaxSmem)) return e;        // (asked by fused_split)
+    a.split = fused_split(g, mode);
     // launched with programmatic stream serialization: the kernel may be scheduled while the previous
     // kernel of the stream drains; it orders itself with griddepcontrol.wait before its first read
-    cudaError_t e = launch_split(a.split > 1 ? k_forward_fused<true> : k_forward_fused<false>, (unsigned)(g.B * g.H), a.split,
-                                 kFusedThreads, smem, st, g, a, (const __nv_bfloat16 *)Q, (const __nv_bfloat16 *)V, sidx,
-                                 (__nv_bfloat16 *)O, sel, M_out, tmKrows, tmK, tmV);
+    cudaError_t e = launch_split(kernels[mode][a.split > 1], (unsigned)(g.B * g.H), a.split, kFusedThreads, smem, st, g, a,
+                                 (const __nv_bfloat16 *)Q, (const __nv_bfloat16 *)V, sidx, (__nv_bfloat16 *)O, sel, M_out,
+                                 tmKrows, tmK, tmV);
     note_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
 }

@@ -58,8 +58,11 @@ cudaError_t launch_measure_mma(const Geom &g, int U_max, const void *Q, const vo
 // Steps (a)-(e) of every unit in one kernel (bf16, keys resident in shared memory).
 // cudaErrorNotSupported: shape outside the kernel's limits; run the staged schedule instead.
 // sel_in != nullptr: steps (d)+(e) only, for the given index set [unit][u_max] (sidx, sel, M_out unused).
+// M_in != nullptr: steps (c)-(e), M~ [unit][T] given (sidx, M_out unused).
 cudaError_t launch_forward_fused(const Geom &g, int U_max, int own_v, const void *Q, const void *K, const void *V,
-                                 const int *sidx, void *O, int *sel, float *M_out, const int *sel_in, cudaStream_t st);
+                                 const int *sidx, void *O, int *sel, float *M_out, const int *sel_in, const float *M_in,
+                                 cudaStream_t st);
+bool fused_from_measure_supported(const Geom &g, const void *K, const void *V);
 // The same for fp32 inputs (psattn_fused_fp32.cu).
 cudaError_t launch_forward_fused_fp32(const Geom &g, int U_max, int own_v, const void *Q, const void *K, const void *V,
                                       const int *sidx, void *O, int *sel, float *M_out, const int *sel_in, cudaStream_t st);

@@ -48,31 +48,117 @@ __global__ void __launch_bounds__(kMeasureThreads, 1) k_measure_mma(Geom g, Meas
 }
 
 // Streaming form (keys gathered from L2 through per-warp rings): any T_max.
-constexpr int kStreamThreads = 768;
+constexpr int kStreamThreads = 768;      // at most: fewer warps where long sample rows leave no room for their buffers
 
-__global__ void __launch_bounds__(kStreamThreads, 1) k_measure_stream(Geom g, int q_slices, uint32_t stage_bytes,
+__global__ void __launch_bounds__(kStreamThreads, 1) k_measure_stream(Geom g, uint32_t warp_stage_bytes,
                                                                       const __nv_bfloat16 *__restrict__ Q,
                                                                       const __nv_bfloat16 *__restrict__ K,
-                                                                      const int *__restrict__ sidx,
-                                                                      float *__restrict__ M) {
-    extern __shared__ __align__(1024) uint8_t smem[];
-    const int tid = threadIdx.x;
-    const int unit = blockIdx.x / q_slices, slice = blockIdx.x % q_slices;
-    const int b = unit / g.H, h = unit % g.H;
+                                                                      const int *__restrict__ sidx, float *__restrict__ M) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    __shared__ unsigned long long warp_sum[kStreamThreads / 32];
+    const int n_threads = blockDim.x, n_warps = n_threads >> 5;
+    // shared memory: rings, staging buffers, weight of all groups of the sequences before b (b = 0 .. B)
+    unsigned long long *before = reinterpret_cast<unsigned long long *>(smem + n_warps * (kStreamRing * kStreamRoundBytes + 2 * warp_stage_bytes));
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     pdl_enter();
     KernelSpan span(g, kKernelMeasure);
-    const int L = seq_len(g, b);
-    const int U = min(g.U_tab[L], g.idx_cols);
-    // slices in whole staged blocks so that every CTA but the last works on full blocks
-    constexpr int kBlock = measure_block_queries(kStreamThreads);
-    const int blocks_total = (g.T + kBlock - 1) / kBlock;
-    const int per = (blocks_total + q_slices - 1) / q_slices * kBlock;
-    const int q_lo = min(g.T, slice * per), q_hi = min(g.T, q_lo + per);
-    const int q_end = min(q_hi, L);
-    float *Mu = M + (long long)unit * g.T;
-    for (int i = max(q_lo, L) + tid; i < q_hi; i += kStreamThreads) Mu[i] = 0.f;   // padded queries
-    if (L == 0 || q_lo >= L) return;
-    measure_stream<kStreamThreads>(smem, stage_bytes, g, unit, b, h, L, U, q_lo, q_end, Q, K, sidx, Mu);
+    // weights of the sequences, added up in order (thread t takes sequences t * per ..)
+    {
+        const int per = (g.B + n_threads - 1) / n_threads;
+        auto weight_of = [&](int b) {
+            const int L = seq_len(g, b);
+            return L > 0 ? (unsigned long long)stream_groups(L) * g.H * stream_weight(min(g.U_tab[L], g.idx_cols)) : 0ull;
+        };
+        unsigned long long mine = 0;
+        for (int b = tid * per; b < min(g.B, (tid + 1) * per); ++b) mine += weight_of(b);
+        unsigned long long incl = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        if (lane == 31) warp_sum[warp] = incl;
+        __syncthreads();
+        unsigned long long at = incl - mine;
+        for (int w = 0; w < warp; ++w) at += warp_sum[w];
+        for (int b = tid * per; b < min(g.B, (tid + 1) * per); ++b) { before[b] = at; at += weight_of(b); }
+        if (tid == 0) {
+            unsigned long long all = 0;
+            for (int w = 0; w < n_warps; ++w) all += warp_sum[w];
+            before[g.B] = all;
+        }
+        __syncthreads();
+    }
+    const unsigned long long all = before[g.B];
+    const unsigned long long w_lo = all * blockIdx.x / gridDim.x, w_hi = all * (blockIdx.x + 1) / gridDim.x;
+    // zeros at padded positions, unit by unit
+    for (int unit = blockIdx.x; unit < g.B * g.H; unit += gridDim.x)
+        for (int i = seq_len(g, unit / g.H) + tid; i < g.T; i += n_threads) M[(long long)unit * g.T + i] = 0.f;
+
+    // this warp's groups: every n_warps-th of the CTA's range
+    int b = 0;
+    for (int step = kStreamMaxB / 2; step > 0; step >>= 1)                 // last sequence that starts at or before w_lo
+        if (b + step < g.B && before[b + step] <= w_lo) b += step;
+    struct Group { int b, h, i0, rows, L, U; };
+    int k = 0, k_hi = 0, skip = warp;                          // within sequence b: next group number, end; groups to skip first
+    bool open = false;
+    auto next = [&](Group &x) {                                // false: no more groups
+        for (; b < g.B && before[b] < w_hi; ++b, open = false) {
+            const int L = seq_len(g, b);
+            if (L == 0) continue;
+            const int ng = stream_groups(L), U = min(g.U_tab[L], g.idx_cols);
+            if (!open) {
+                stream_range(before[b], ng * g.H, stream_weight(U), w_lo, w_hi, k, k_hi);
+                open = true;
+            }
+            if (k + skip >= k_hi) { skip -= max(0, k_hi - k); continue; }
+            k += skip; skip = 0;
+            x.b = b; x.h = k / ng; x.i0 = (k - x.h * ng) * 8; x.rows = min(8, L - x.i0); x.L = L; x.U = U;
+            ++k; skip = n_warps - 1;
+            return true;
+        }
+        return false;
+    };
+    StreamCtx cx;
+    cx.ring = smem_u32(smem) + (uint32_t)warp * kStreamRing * kStreamRoundBytes;
+    cx.idx_cols = g.idx_cols; cx.status = g.status; cx.k_row_bytes = (uint32_t)(g.ks[2] * 2);
+    const uint32_t stage0 = smem_u32(smem) + n_warps * kStreamRing * kStreamRoundBytes + (uint32_t)warp * 2u * warp_stage_bytes;
+    // Q rows, then sample rows, of a group into one of the warp's two buffers; nobody else reads them, so the warps never meet at
+    // a barrier and drift apart: the pipeline bubble at the start of a group does not hit all of them at once
+    auto stage = [&](const Group &x, int buf) {
+        const uint32_t dst = stage0 + (uint32_t)buf * warp_stage_bytes;
+        const __nv_bfloat16 *Qu = Q + unit_off(g.qs, x.b, x.h);
+        for (int e = lane; e < x.rows * 8; e += 32)
+            cp_async_16(dst + (uint32_t)e * 16u, Qu + (long long)(x.i0 + (e >> 3)) * g.qs[2] + (e & 7) * 8);
+        const int words = x.rows * g.idx_cols;
+        const int *src = sidx + ((g.idx_per_head ? (long long)(x.b * g.H + x.h) : (long long)x.b) * g.T + x.i0) * g.idx_cols;
+        const uint32_t idst = dst + 1024u;
+        if (((reinterpret_cast<uintptr_t>(src) | (uintptr_t)(words * 4)) & 15u) == 0u) {
+            for (int w = lane; w < words / 4; w += 32) cp_async_16(idst + (uint32_t)w * 16u, src + 4 * w);
+        } else {
+            for (int w = lane; w < words; w += 32) cp_async_4(idst + (uint32_t)w * 4u, src + w);
+        }
+        cp_async_commit();
+    };
+    Group cur, nxt;
+    bool have = next(cur);
+    if (have) stage(cur, 0);
+    for (int n = 0; have; ++n) {
+        cp_async_wait<0>();                                    // this lane's part of the group (nothing else is pending)
+        __syncwarp();
+        asm volatile("mov.u32 %0, %1;" : "=r"(cx.epoch0) : "r"(n << 8) : "memory");
+        have = next(nxt);
+        if (have) stage(nxt, (n + 1) & 1);                     // lands while this group is worked on
+        cx.q_tile = stage0 + (uint32_t)(n & 1) * warp_stage_bytes;
+        cx.idx_tile = cx.q_tile + 1024u;
+        cx.rows = cur.rows; cx.L = cur.L; cx.U = min(cur.U, kMeasureMaxU);
+        cx.Ku = K + unit_off(g.ks, cur.b, cur.h);
+        cx.out = M + (long long)(cur.b * g.H + cur.h) * g.T + cur.i0;
+        measure_stream_group(cx);
+        __syncwarp();                                          // the group's buffer may be staged again from now on
+        cur = nxt;
+    }
+    cp_async_wait<0>();
 }
 
 // ---- host side ----------------------------------------------------------------------------------
@@ -149,27 +235,34 @@ cudaError_t launch_measure_mma(const Geom &g, int U_max, const void *Q, const vo
 
 namespace psattn {
 
-// cudaErrorNotSupported: more than 64 samples per query, or key rows of a unit spread over 4 GB or more.
+// cudaErrorNotSupported: more than 64 samples per query, sample rows too wide for shared memory, or key rows of a unit
+// spread over 4 GB or more.
 cudaError_t launch_measure_stream(const Geom &g, int U_max, const void *Q, const void *K, const int *sidx, float *M,
                                   cudaStream_t st) {
     if (g.B * g.H == 0) return cudaSuccess;
     if (U_max > kMeasureMaxU || U_max < 1) return cudaErrorNotSupported;
     if (g.ks[2] <= 0 || (long long)g.T * g.ks[2] * 2 >= (1ll << 32)) return cudaErrorNotSupported;
-    const size_t stage_bytes = measure_stage_bytes(kStreamThreads, g.idx_cols);
-    const size_t smem = (size_t)(kStreamThreads / 32) * kStreamRing * kStreamRoundBytes + 2 * stage_bytes;
-    if (smem > 225 * 1024) return cudaErrorNotSupported;
-    const int units = g.B * g.H;
-    constexpr int kBlock = measure_block_queries(kStreamThreads);
-    const int blocks_total = (g.T + kBlock - 1) / kBlock;
-    int slices = (2 * device_sm_count() + units - 1) / units;             // about two CTAs' worth of work per SM
-    if (slices > blocks_total) slices = blocks_total;
-    if (slices < 1) slices = 1;
+    const size_t warp_stage = (1024 + (size_t)8 * g.idx_cols * 4 + 15) / 16 * 16;
+    const size_t table = ((size_t)(g.B < kStreamMaxB ? g.B : kStreamMaxB) + 1) * 8;
+    const size_t per_warp = kStreamRing * kStreamRoundBytes + 2 * warp_stage, room = 226 * 1024 - table;
+    int warps = (int)(room / per_warp);
+    if (warps > kStreamThreads / 32) warps = kStreamThreads / 32;
+    if (warps < 8) return cudaErrorNotSupported;               // sample rows of hundreds of columns: the plain kernel
+    const size_t smem = (size_t)warps * per_warp + table;
     static SmemGrant grant;
     if (cudaError_t e = grant_dynamic_smem(k_measure_stream, grant, smem)) return e;
-    cudaError_t e = launch_pdl(k_measure_stream, dim3((unsigned)(units * slices)), dim3(kStreamThreads), smem, st, g, slices,
-                               (uint32_t)stage_bytes, (const __nv_bfloat16 *)Q, (const __nv_bfloat16 *)K, sidx, M);
-    note_launch();
-    return e != cudaSuccess ? e : cudaGetLastError();
+    for (int b0 = 0; b0 < g.B; b0 += kStreamMaxB) {
+        Geom part = g;
+        part.B = g.B - b0 < kStreamMaxB ? g.B - b0 : kStreamMaxB;
+        if (g.lengths) part.lengths = g.lengths + b0;
+        const long long idx_b = (long long)(g.idx_per_head ? g.H : 1) * g.T * g.idx_cols;
+        cudaError_t e = launch_pdl(k_measure_stream, dim3((unsigned)device_sm_count()), dim3((unsigned)warps * 32), smem, st, part,
+                                   (uint32_t)warp_stage, (const __nv_bfloat16 *)Q + b0 * g.qs[0], (const __nv_bfloat16 *)K + b0 * g.ks[0],
+                                   sidx + b0 * idx_b, M + (long long)b0 * g.H * g.T);
+        note_launch();
+        if (e != cudaSuccess) return e;
+    }
+    return cudaGetLastError();
 }
 
 }  // namespace psattn

@@ -94,14 +94,12 @@ __device__ __forceinline__ void stream_round(const StreamLane &ln, const uint32_
     asm volatile("" ::"f"(c[0]), "f"(c[1]), "f"(c[2]), "f"(c[3]) : "memory");
 }
 
-template <int THREADS>
-__device__ __forceinline__ void measure_stream_block(const StreamCtx &cx) {
+// The eight (or fewer) queries of the warp's group.
+__device__ __forceinline__ void measure_stream_group(const StreamCtx &cx) {
     static_assert(kStreamRing == 2, "two ring stages");
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
     const int l7 = lane & 7;
-    const int q0 = warp * 8;
-    if (q0 >= cx.rows) return;
-    const int qn = min(q0 + l7, cx.rows - 1);
+    const int qn = min(l7, cx.rows - 1);                       // a short group recomputes its last query
     uint32_t bq[8];
     {
         const uint32_t qa = cx.q_tile + (uint32_t)qn * 128u;
@@ -163,70 +161,31 @@ __device__ __forceinline__ void measure_stream_block(const StreamCtx &cx) {
             take(!odd);
         }
     }
-    if ((lane & 3) == (g >> 1) && q0 + g < cx.rows)
-        cx.out[q0 + g] = fmaxf((mx - ds / (float)cx.U) * kScale, 0.f);
+    if ((lane & 3) == (g >> 1) && g < cx.rows)
+        cx.out[g] = fmaxf((mx - ds / (float)cx.U) * kScale, 0.f);
 }
 
-// All THREADS threads of the CTA: M~ of the queries [q_lo, q_end) (q_end <= L, L >= 1) of unit (b, h)
-// into out[i].  Shared memory: THREADS / 32 rings, then two staging buffers of stage_bytes.
-// No block-wide barrier inside: the caller orders the result with one of its own where it needs to.
-template <int THREADS>
-__device__ __forceinline__ void measure_stream(uint8_t *smem, uint32_t stage_bytes, const Geom &g, int unit, int b, int h,
-                                               int L, int U, int q_lo, int q_end, const __nv_bfloat16 *__restrict__ Q,
-                                               const __nv_bfloat16 *__restrict__ K, const int *__restrict__ sidx,
-                                               float *out) {
-    using namespace sm100;
-    constexpr int kBlock = measure_block_queries(THREADS);
-    constexpr uint32_t kRingBytes = (THREADS / 32) * kStreamRing * kStreamRoundBytes;
-    const int tid = threadIdx.x;
-    const int *idx_base = sidx + ((g.idx_per_head ? (long long)unit : (long long)b) * g.T) * g.idx_cols;
-    const __nv_bfloat16 *Qu = Q + unit_off(g.qs, b, h);
-    const uint32_t stage0 = smem_u32(smem) + kRingBytes;
-    const int n_blocks = (q_end - q_lo + kBlock - 1) / kBlock;
-    // every warp stages the rows of its own eight queries (see measure_resident): no barrier between blocks,
-    // so the warps drift apart and the pipeline bubble at the start of a group of queries does not hit all
-    // of them at once
-    const int warp = tid >> 5, lane = tid & 31;
-    auto stage_block = [&](int blk) {
-        if (blk < n_blocks) {
-            const int i0 = q_lo + blk * kBlock + warp * 8;
-            const int rows = min(8, q_end - i0);
-            if (rows > 0) {
-                const uint32_t base = stage0 + (uint32_t)(blk & 1) * stage_bytes;
-                const uint32_t qdst = base + (uint32_t)warp * 1024u;
-                for (int e = lane; e < rows * 8; e += 32)
-                    cp_async_16(qdst + (uint32_t)e * 16u, Qu + (long long)(i0 + (e >> 3)) * g.qs[2] + (e & 7) * 8);
-                const int words = rows * g.idx_cols;
-                const int *src = idx_base + (long long)i0 * g.idx_cols;
-                const uint32_t idst = base + kBlock * 128u + (uint32_t)(warp * 8 * g.idx_cols) * 4u;
-                if (((reinterpret_cast<uintptr_t>(src) | (uintptr_t)(words * 4)) & 15u) == 0u) {
-                    for (int w = lane; w < words / 4; w += 32) cp_async_16(idst + (uint32_t)w * 16u, src + 4 * w);
-                } else {
-                    for (int w = lane; w < words; w += 32) cp_async_4(idst + (uint32_t)w * 4u, src + w);
-                }
-            }
-        }
-        cp_async_commit();
+// ---------------------------------------------------------------------------------------------
+// How the work is split: the groups of eight queries of all sequences and heads, in order, each weighing its rounds (plus a
+// few for its start), are cut into one range of equal weight per CTA (one CTA per SM), and the warps of a CTA take
+// the groups of its range in turn.  With a fixed number of query ranges per unit the ragged batch (B6 H8, lengths
+// 1050..3001) left most SMs idle behind the longest units: 64 us, where the gathers alone need 28.
+// ---------------------------------------------------------------------------------------------
+constexpr int kStreamMaxB = 2048;                               // sequences per launch (their weights sit in shared memory)
+
+__device__ __forceinline__ int stream_groups(int L) { return (L + 7) >> 3; }
+__device__ __forceinline__ int stream_weight(int U) { return ((U + 1) >> 1) + 3; }
+
+// The range of group numbers (head * groups + group) of sequence b that start within [w_lo, w_hi).
+__device__ __forceinline__ void stream_range(unsigned long long before, int n, int weight, unsigned long long w_lo,
+                                             unsigned long long w_hi, int &k_lo, int &k_hi) {
+    auto first_at = [&](unsigned long long w) {
+        if (w <= before) return 0;
+        const unsigned long long k = (w - before + weight - 1) / weight;
+        return k < (unsigned long long)n ? (int)k : n;
     };
-    StreamCtx cx;
-    cx.ring = smem_u32(smem) + (uint32_t)(tid >> 5) * kStreamRing * kStreamRoundBytes;
-    cx.U = min(U, kMeasureMaxU); cx.L = L; cx.idx_cols = g.idx_cols; cx.status = g.status;
-    cx.Ku = K + unit_off(g.ks, b, h); cx.k_row_bytes = (uint32_t)(g.ks[2] * 2);
-    stage_block(0);
-    for (int blk = 0; blk < n_blocks; ++blk) {
-        cp_async_wait<0>();                                    // this lane's part of block blk (nothing else is pending)
-        __syncwarp();
-        asm volatile("mov.u32 %0, %1;" : "=r"(cx.epoch0) : "r"(blk << 8) : "memory");
-        stage_block(blk + 1);                                  // lands while this block is worked on
-        cx.q_tile = stage0 + (uint32_t)(blk & 1) * stage_bytes;
-        cx.idx_tile = cx.q_tile + kBlock * 128u;
-        const int i0 = q_lo + blk * kBlock;
-        cx.rows = min(kBlock, q_end - i0);
-        cx.out = out + i0;
-        measure_stream_block<THREADS>(cx);
-        __syncwarp();                                          // the warp's part of buffer blk & 1 may be restaged next time
-    }
-    cp_async_wait<0>();
+    k_lo = first_at(w_lo);
+    k_hi = first_at(w_hi);
 }
 
 }  // namespace psattn

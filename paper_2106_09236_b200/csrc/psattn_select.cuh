@@ -6,6 +6,8 @@
 
 namespace psattn {
 
+constexpr int kSelectMaxSlots = 18;       // keys per thread of block_select_short at most
+
 struct SelectScratch {
     int hist[256];
     int wtot_gt[32], wtot_eq[32];
@@ -16,7 +18,7 @@ struct SelectScratch {
     // block_select_short
     uint2 count[2][32];                                    // warp totals of a round (two rounds in turn)
     unsigned lo[32], hi[32];
-    unsigned taken[8][32];                                 // per key slot and warp: keys above tau, keys equal to it << 16
+    unsigned taken[kSelectMaxSlots][32];                                 // per key slot and warp: keys above tau, keys equal to it << 16
 };
 
 // The same selection for lists that fit the block's registers (L <= KPT * nthr): every thread keeps its keys
