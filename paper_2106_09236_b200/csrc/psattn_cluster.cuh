@@ -9,6 +9,8 @@
 
 namespace psattn {
 
+constexpr int kMaxSplit = 8;           // CTAs per cluster at most (the portable limit)
+
 __device__ __forceinline__ void cluster_arrive() {
     __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
@@ -32,36 +34,38 @@ __device__ __forceinline__ float peer_load(uint32_t addr) {
 }
 // Column c of row r over all CTAs of the unit: the states (m, l, acc) that every CTA left at `states` in its shared
 // memory (66 floats per row) merged in rank order; returns acc / l.
-template <int SPLIT>
-__device__ __forceinline__ float merge_states_n(uint32_t states, int r, int c) {
-    float m[SPLIT], l[SPLIT], a[SPLIT];
+template <int MOST>
+__device__ __forceinline__ float merge_states_n(int split, uint32_t states, int r, int c) {
+    float m[MOST], l[MOST], a[MOST];
 #pragma unroll
-    for (int x = 0; x < SPLIT; ++x) {                          // all loads in flight together
+    for (int x = 0; x < MOST; ++x) {                          // all loads in flight together
+        m[x] = -INFINITY; l[x] = 0.f; a[x] = 0.f;
+        if (x >= split) continue;
         const uint32_t p = peer_addr(states + (uint32_t)r * 264u, x);
         m[x] = peer_load(p); l[x] = peer_load(p + 4u); a[x] = peer_load(p + 8u + 4u * (uint32_t)c);
     }
     float mw = -INFINITY, lw = 0.f, aw = 0.f;
 #pragma unroll
-    for (int x = 0; x < SPLIT; ++x) mw = fmaxf(mw, m[x]);
+    for (int x = 0; x < MOST; ++x) mw = fmaxf(mw, m[x]);
 #pragma unroll
-    for (int x = 0; x < SPLIT; ++x) {
+    for (int x = 0; x < MOST; ++x) {
         const float f = l[x] > 0.f ? sm100::fast_exp2(m[x] - mw) : 0.f;
         lw += l[x] * f; aw += a[x] * f;
     }
     return lw > 0.f ? aw / lw : 0.f;
 }
 __device__ __forceinline__ float merge_states(int split, uint32_t states, int r, int c) {
-    return split == 8 ? merge_states_n<8>(states, r, c) : split == 4 ? merge_states_n<4>(states, r, c) : merge_states_n<2>(states, r, c);
+    return split > 4 ? merge_states_n<kMaxSplit>(split, states, r, c) : split > 2 ? merge_states_n<4>(split, states, r, c) : merge_states_n<2>(split, states, r, c);
 }
 
 // Clusters of `split` CTAs of `kernel` (at the given shared memory) that the current device holds at once; asked once per
 // device and kernel (`cached`: one record per kernel).
 struct ClusterRecord {
-    std::atomic<int> n[kMaxDevices][4];
+    std::atomic<int> n[kMaxDevices][kMaxSplit + 1];
 };
 template <typename... KArgs>
 inline int max_clusters(void (*kernel)(KArgs...), ClusterRecord &cached, int split, int threads, size_t smem) {
-    const int k = split == 8 ? 3 : split == 4 ? 2 : 1;
+    const int k = split;
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) { cudaGetLastError(); return 0; }
     int n = cached.n[dev][k].load(std::memory_order_relaxed);

@@ -38,7 +38,7 @@ struct FusedArgs {
     int pos_t, pos_h, pos_b;             // TMA coordinate slots (same for the three maps)
     int own_v;                           // fill with the query's own value row instead of mean(V)
     int by_length;                       // CTAs take the sequences in descending order of length
-    int split;                           // CTAs per unit (one thread-block cluster): 1, 2, 4 or 8
+    int split;                           // CTAs per unit (one thread-block cluster): 1 to 8
     int m_floats;                        // floats of the M~ array (0 with a given index set)
     const int *sel_in;                   // kGivenSet: the index set [unit][u_max]
     const float *M_in;                   // kGivenMeasure: M~ [unit][T]
@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
         __syncthreads();
         if (SPLIT) {
             for (int x = 1; x < split; ++x) {
-                const uint32_t dst = peer_addr(smem_u32(M_s), (part + x) & (split - 1));
+                const uint32_t dst = peer_addr(smem_u32(M_s), part + x < split ? part + x : part + x - split);
                 for (int i = q_lo + tid; i < q_hi; i += kFusedThreads) peer_store(dst + 4u * (uint32_t)i, M_s[i]);
             }
             cluster_arrive();
@@ -166,8 +166,8 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
         } else {
             const float *Mu = a.M_in + (long long)unit * g.T;
             auto key_of = [&](int i) { return float_key(__ldg(Mu + i)); };
-            if (L <= 6 * kSelectors) block_select_short<6>(key_of, L, u, kArMaxRows, P.sel, P.select, kSelectors, 1);
-            else block_select_short<kSelectMaxSlots>(key_of, L, u, kArMaxRows, P.sel, P.select, kSelectors, 1);
+            if (L <= 6 * kSelectors) block_select_few<6>(key_of, L, u, kArMaxRows, P.sel, P.select, kSelectors, 1);
+            else block_select_few<kSelectMaxSlots>(key_of, L, u, kArMaxRows, P.sel, P.select, kSelectors, 1);
         }
         for (int r = tid; r < g.u_max; r += kSelectors) {
             const int i = r < kArMaxRows ? P.sel[r] : -1;
@@ -265,7 +265,7 @@ static int fused_split(const Geom &g, int mode) {
     static ClusterRecord clusters;
     const int units = g.B * g.H;
     if (g.T < (mode == kAllSteps ? 192 : 768)) return 1;
-    for (int split = 8; split > 1; split >>= 1)
+    for (int split = kMaxSplit; split > 1; --split)
         if (units <= max_clusters(k_forward_fused<true, kAllSteps>, clusters, split, kFusedThreads, kFusedMaxSmem)) return split;
     return 1;
 }

@@ -382,7 +382,7 @@ __global__ void __launch_bounds__(kF32Threads, 1) k_forward_fused_fp32(
         __syncthreads();
         if (SPLIT) {
             for (int x = 1; x < split; ++x) {
-                const uint32_t dst = peer_addr(smem_u32(M_s), (part + x) & (split - 1));
+                const uint32_t dst = peer_addr(smem_u32(M_s), part + x < split ? part + x : part + x - split);
                 for (int i = q_lo + tid; i < q_hi; i += kF32Threads) peer_store(dst + 4u * (uint32_t)i, M_s[i]);
             }
             cluster_arrive();
@@ -496,7 +496,7 @@ static int f32_split(const Geom &g) {
     static ClusterRecord clusters;
     const int units = g.B * g.H;
     if (g.T < 96) return 1;
-    for (int split = 8; split > 1; split >>= 1)
+    for (int split = kMaxSplit; split > 1; --split)
         if (units <= max_clusters(k_forward_fused_fp32<true>, clusters, split, kF32Threads, kF32MaxSmem)) return split;
     return 1;
 }

@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(kSelectThreads) k_select(Geom g, const float *
     else if (L <= 8 * kSelectThreads)
         block_select_short<8>([&](int i) { return float_key(Mu[i]); }, L, u, g.u_max, out, scratch, blockDim.x, 0);
     else
-        block_select([&](int i) { return float_key(Mu[i]); }, L, u, g.u_max, out, scratch);
+        block_select([&](int i) { return float_key(Mu[i]); }, L, u, g.u_max, out, scratch, blockDim.x, 0);
 }
 
 // ---------------------------------------------------------------------------------------
