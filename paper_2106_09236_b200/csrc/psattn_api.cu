@@ -426,7 +426,7 @@ extern "C" int psattn_forward(psattn_plan_t *plan, const void *Q, const void *K,
                                        nullptr, M, st));
         return PSATTN_OK;
     }
-    if (vbar_from_attention(plan, g, K, V)) {
+    if (d.path != PSATTN_PATH_STAGED) {
         // Steps (a)-(c) do not touch V or O, and they are bound by on-chip gathers, not by HBM: the fill of
         // step (e) - column sums of V, mean(V), every valid row of O - runs beside them on the plan's side
         // stream (forked and joined with events, so the call stays ordered on the caller's stream and can be
@@ -487,9 +487,11 @@ extern "C" int psattn_forward_with_selection(psattn_plan_t *plan, const void *Q,
     if (vbar_from_attention(plan, g, K, V))
         return run_attend_and_fill(plan, g, Q, K, V, sel_idx_in, O, workspace, st, false);
     // mean(V) by a column-sum pass (the select kernel, run without keys, only finishes the mean)
-    PSATTN_CU(launch_colsum(d.dtype, g, V, ws_at<float>(workspace, plan->off_vpart), plan->n_chunks, st));
-    PSATTN_CU(launch_select(g, nullptr, nullptr, ws_at<float>(workspace, plan->off_vpart),
-                            plan->n_chunks, ws_at<float>(workspace, plan->off_vbar), nullptr, st));
+    if (d.fill_mode == PSATTN_FILL_MEAN_V) {
+        PSATTN_CU(launch_colsum(d.dtype, g, V, ws_at<float>(workspace, plan->off_vpart), plan->n_chunks, st));
+        PSATTN_CU(launch_select(g, nullptr, nullptr, ws_at<float>(workspace, plan->off_vpart),
+                                plan->n_chunks, ws_at<float>(workspace, plan->off_vbar), nullptr, st));
+    }
     return run_attend_and_fill(plan, g, Q, K, V, sel_idx_in, O, workspace, st, true);
 }
 

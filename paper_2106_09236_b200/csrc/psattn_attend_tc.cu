@@ -9,8 +9,8 @@
 //                    both query tiles use the same key tile, so K and V cross L2 -> shared memory once per 256 rows
 // Per key tile t and warpgroup w:
 //   tcgen05   S_w = Q_w K_t^T            -> TMEM (128 lanes x 128 fp32 columns)
-//   threads   one pass over the row's 128 scores (32 at a time in registers, the next 32 in flight): exponentials
-//             relative to the row's reference, P (bf16) -> shared memory (A-operand layout), the maximum on the side
+//   threads   two passes over the row's 128 scores (32 at a time in registers, the next 32 in flight): the maximum; the
+//             exponentials relative to the row's reference, P (bf16) -> shared memory (A-operand layout)
 //   tcgen05   O_w += P_w V_t             -> TMEM (64 columns), accumulated across key tiles; V is the MN-major B
 //                                           operand exactly as TMA wrote it
 // The issuing thread runs "P V of tile t, then S of tile t + 1" for A and for B in turn, so the tensor pipe
@@ -72,8 +72,8 @@ __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.
 
 // One pass over a row's 128 scores in TMEM, 32 columns at a time, the next block of 32 in flight while the
 // current one is worked on.  EXP: the exponentials relative to `ref` (scaled log2 units) go to the row's place in
-// P as bf16 (two panels of 64 keys in the A-operand layout, 128-byte swizzle) and their sum to `lsum`; the largest
-// raw score of the valid columns goes to `mx` in any case.  FULL: all 128 keys exist.
+// P as bf16 (two panels of 64 keys in the A-operand layout, 128-byte swizzle) and their sum to `lsum`.  Otherwise the largest
+// raw score of the valid columns goes to `mx`.  FULL: all 128 keys exist.
 template <bool EXP, bool FULL>
 __device__ __forceinline__ void tc_row_pass(uint32_t t_s, float ref, int valid, uint8_t *prow, int row, float &mx, float &lsum) {
     const float kScaleLog2 = kScale * kLog2e;
@@ -93,9 +93,10 @@ __device__ __forceinline__ void tc_row_pass(uint32_t t_s, float ref, int valid, 
             for (int x = 0; x < 8; x += 2) {
                 const int c = ch * 8 + x, col = q * 32 + c;
                 const float s0 = __uint_as_float(cur[c]), s1 = __uint_as_float(cur[c + 1]);
-                if (FULL || col < valid) m0 = fmaxf(m0, s0);
-                if (FULL || col + 1 < valid) m1 = fmaxf(m1, s1);
-                if (EXP) {
+                if (!EXP) {
+                    if (FULL || col < valid) m0 = fmaxf(m0, s0);
+                    if (FULL || col + 1 < valid) m1 = fmaxf(m1, s1);
+                } else {
                     const float p0 = (FULL || col < valid) ? fast_exp2(fmaf(s0, kScaleLog2, -ref)) : 0.f;
                     const float p1 = (FULL || col + 1 < valid) ? fast_exp2(fmaf(s1, kScaleLog2, -ref)) : 0.f;
                     l0 += p0; l1 += p1;
@@ -131,8 +132,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_attend_tc(Geom g, AttendTcArg
     const int b = unit / g.H, h = unit % g.H;
     const int L = seq_len(g, b);
     const int lo = min(L, split * a.split_keys), hi = min(L, lo + a.split_keys);
-    const int n_tiles = (hi - lo + kTileKeys - 1) / kTileKeys;
-    const bool has_b = pair * kCtaRows + kTileRows < a.n_rows;  // the second query tile lists rows
+    int n_tiles = (hi - lo + kTileKeys - 1) / kTileKeys;
 
     if ((smem_u32(smem) & 1023u) != 0u) {                      // swizzled tiles need a 1024-byte base
         if (tid == 0) atomicOr(g.status, kStatusWaitExpired);
@@ -165,7 +165,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_attend_tc(Geom g, AttendTcArg
     }
     fence_proxy_async_smem();
     tc_fence_before();
-    __syncthreads();
+    // Lists are padded to the longest one of the batch: a query tile that lists no position of this sequence is left out (with
+    // u = L / 2 and lengths 384..960 a third of the tiles), and a CTA with none has only its zero rows to write.
+    const bool has_a = __syncthreads_or(wg == 0 && row_ok);
+    const bool has_b = __syncthreads_or(wg == 1 && row_ok);
+    if (!has_a && !has_b) n_tiles = 0;
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
     auto give_up = [&]() { *abort_flag = 1u; atomicOr(g.status, kStatusWaitExpired); };
@@ -240,19 +244,43 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_attend_tc(Geom g, AttendTcArg
                 if (*abort_flag) break;
             }
         }
-    } else if (wg == 0 || has_b) {
+    } else {
         // ---------------- softmax warpgroups: thread = row = TMEM lane ------------------------------------------
         const uint32_t lane_base = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
         const uint32_t t_s = lane_base + wg * 128, t_o = lane_base + 256 + wg * 64;
         uint8_t *prow = smem + kOffP + wg * 2 * kTileBytes + wrow * 128;
         const float kScaleLog2 = kScale * kLog2e;
-        for (int t = 0; t < n_tiles; ++t) {
+        const int my_tiles = wg == 0 || has_b ? n_tiles : 0;
+        for (int t = 0; t < my_tiles; ++t) {
             if (*abort_flag) break;
             if (!mbar_wait(&s_full[wg], (uint32_t)(t & 1), g.wait_ns)) { give_up(); break; }
             tc_fence_after();
             const int valid = min(kTileKeys, hi - (lo + t * kTileKeys));     // keys of this tile that exist (>= 1)
             const bool full = valid == kTileKeys;
-            float mx, lsum;
+            // The maximum first: a pass without exponentials, which lies under the other warpgroup's exponentials.  Where it has
+            // run away from the reference (by more than 2^8; always in the first tile) the reference follows, and the row
+            // sum and the row of O are scaled (P V of tile t - 1 has finished, see the head of the file).  Exponentials
+            // first and the pass taken again where the reference moved cost more: with rows that attend to few keys most
+            // tiles move some row of a warp.
+            float mx, lsum, alpha = 1.f;
+            if (full) tc_row_pass<false, true>(t_s, 0.f, valid, prow, wrow, mx, lsum);
+            else tc_row_pass<false, false>(t_s, 0.f, valid, prow, wrow, mx, lsum);
+            const float mxs = mx * kScaleLog2;
+            if (t == 0) {
+                m_ref = mxs;
+            } else if (__any_sync(0xffffffffu, mxs > m_ref + kRefSlack)) {
+                if (mxs > m_ref + kRefSlack) { alpha = fast_exp2(m_ref - mxs); m_ref = mxs; }
+                uint32_t ov[2][32];
+                tmem_ld32_issue(t_o, ov[0]);
+                tmem_ld32_issue(t_o + 32, ov[1]);
+                tmem_ld_wait();
+                tmem_ld_fence32(ov[0]); tmem_ld_fence32(ov[1]);
+#pragma unroll
+                for (int x = 0; x < 64; ++x) ov[x >> 5][x & 31] = __float_as_uint(__uint_as_float(ov[x >> 5][x & 31]) * alpha);
+                tmem_st32(t_o, ov[0]);
+                tmem_st32(t_o + 32, ov[1]);
+                tmem_st_wait();
+            }
             // The exponentials are bound by the special-function unit (16 per clock and SM).  Left alone, the two
             // warpgroups fall into step: both take it at half speed, then both wait for their products while it idles.
             // So they take turns: B starts the exponentials of tile t when A has issued its own, A those of tile t + 1
@@ -260,44 +288,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_attend_tc(Geom g, AttendTcArg
             if (kTakeTurns && has_b && (wg == 1 || t > 0)) {
                 if (!mbar_wait(&turn[wg], (uint32_t)((wg == 1 ? t : t - 1) & 1), g.wait_ns)) { give_up(); break; }
             }
-            if (t == 0) {
-                // the first tile fixes the reference: a pass for the maximum, then the exponentials
-                if (full) tc_row_pass<false, true>(t_s, 0.f, valid, prow, wrow, mx, lsum);
-                else tc_row_pass<false, false>(t_s, 0.f, valid, prow, wrow, mx, lsum);
-                m_ref = mx * kScaleLog2;
-                if (full) tc_row_pass<true, true>(t_s, m_ref, valid, prow, wrow, mx, lsum);
-                else tc_row_pass<true, false>(t_s, m_ref, valid, prow, wrow, mx, lsum);
-                l_run = lsum;
-            } else {
-                // Later tiles take ONE pass: the exponentials relative to the standing reference, the maximum on the
-                // side.  P V of tile t - 1 has finished (see the head of the file), so P may be overwritten.
-                if (full) tc_row_pass<true, true>(t_s, m_ref, valid, prow, wrow, mx, lsum);
-                else tc_row_pass<true, false>(t_s, m_ref, valid, prow, wrow, mx, lsum);
-                const float mxs = mx * kScaleLog2;
-                const bool moved = mxs > m_ref + kRefSlack;
-                if (__any_sync(0xffffffffu, moved)) {
-                    // rare: the maximum has run away from the reference (the weights just written may even have
-                    // overflowed).  The reference follows, the row of O (stable: no product is in flight) and the
-                    // row sum are scaled, and the row's weights are written again.
-                    const float alpha = moved ? fast_exp2(m_ref - mxs) : 1.f;
-                    uint32_t ov[2][32];
-                    tmem_ld32_issue(t_o, ov[0]);
-                    tmem_ld32_issue(t_o + 32, ov[1]);
-                    tmem_ld_wait();
-                    tmem_ld_fence32(ov[0]); tmem_ld_fence32(ov[1]);
-#pragma unroll
-                    for (int x = 0; x < 64; ++x) ov[x >> 5][x & 31] = __float_as_uint(__uint_as_float(ov[x >> 5][x & 31]) * alpha);
-                    tmem_st32(t_o, ov[0]);
-                    tmem_st32(t_o + 32, ov[1]);
-                    tmem_st_wait();
-                    if (moved) m_ref = mxs;
-                    if (full) tc_row_pass<true, true>(t_s, m_ref, valid, prow, wrow, mx, lsum);
-                    else tc_row_pass<true, false>(t_s, m_ref, valid, prow, wrow, mx, lsum);
-                    l_run = l_run * alpha + lsum;
-                } else {
-                    l_run += lsum;
-                }
-            }
+            if (full) tc_row_pass<true, true>(t_s, m_ref, valid, prow, wrow, mx, lsum);
+            else tc_row_pass<true, false>(t_s, m_ref, valid, prow, wrow, mx, lsum);
+            l_run = l_run * alpha + lsum;
             if (kTakeTurns && has_b && (wg == 0 || t + 1 < n_tiles)) mbar_arrive(&turn[wg ^ 1]);
             // rows of V past the valid length may hold anything (even NaN): zero them so that 0 * x stays 0
             if (valid < kTileKeys) {                                // uniform over the CTA (both warpgroups write zeros)
@@ -314,7 +307,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_attend_tc(Geom g, AttendTcArg
         float acc[kD];
 #pragma unroll
         for (int c = 0; c < kD; ++c) acc[c] = 0.f;
-        if (n_tiles > 0 && !*abort_flag) {
+        if (my_tiles > 0 && !*abort_flag) {
             if (!mbar_wait(&o_final[wg], 0u, g.wait_ns)) give_up();
             else {
                 tc_fence_after();
@@ -351,8 +344,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_attend_tc(Geom g, AttendTcArg
                 }
             } else {
                 const long long slot = ((long long)unit * a.n_rows + r) * a.n_splits + split;
-                a.part_ml[2 * slot] = (row_ok && n_tiles > 0) ? m_ref : -INFINITY;
-                a.part_ml[2 * slot + 1] = (row_ok && n_tiles > 0) ? l_run : 0.f;
+                a.part_ml[2 * slot] = (row_ok && my_tiles > 0) ? m_ref : -INFINITY;
+                a.part_ml[2 * slot + 1] = (row_ok && my_tiles > 0) ? l_run : 0.f;
                 float *dst = a.part_acc + slot * kD;
 #pragma unroll
                 for (int c8 = 0; c8 < 8; ++c8) store8(dst, c8, acc + 8 * c8);
