@@ -54,6 +54,7 @@ struct AttendTcArgs {
     long long out_unit_stride, out_row_stride;
     int out_by_position, out_fp32;
     int pos_t, pos_h, pos_b;    // which TMA coordinate (1..3) carries t, h, b
+    int by_length;              // CTAs take the sequences in descending order of length
 };
 
 // 32 consecutive fp32 columns of this thread's TMEM lane, written from registers.
@@ -128,8 +129,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_attend_tc(Geom g, AttendTcArg
     volatile uint32_t *abort_flag = tmem_slot + 1;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int split = blockIdx.x, pair = blockIdx.y, unit = blockIdx.z;
-    const int b = unit / g.H, h = unit % g.H;
+    const int split = blockIdx.x, pair = blockIdx.y;
+    int b = blockIdx.z / g.H;
+    const int h = blockIdx.z % g.H;
+    // longest sequences first: the short ones (and the tiles that list nothing) fill the tail of the last wave
+    if (a.by_length) b = sequence_of_rank(g, b, kTcThreads, reinterpret_cast<int *>(smem + kOffBar + 240));
+    const int unit = b * g.H + h;
     const int L = seq_len(g, b);
     const int lo = min(L, split * a.split_keys), hi = min(L, lo + a.split_keys);
     int n_tiles = (hi - lo + kTileKeys - 1) / kTileKeys;
@@ -435,6 +440,7 @@ cudaError_t launch_attend_tc(const Geom &g, const void *Q, const void *K, const 
     if (posK[0] != posV[0] || posK[1] != posV[1] || posK[2] != posV[2]) return cudaErrorNotSupported;
     a.pos_t = posK[0]; a.pos_h = posK[1]; a.pos_b = posK[2];
     // one CTA per SM: 192 KB of shared memory, all 512 TMEM columns
+    a.by_length = g.lengths != nullptr && g.B > 1 && g.B <= 256;
     static SmemGrant grant;
     if (cudaError_t e = grant_dynamic_smem(k_attend_tc, grant, kAttendSmem, true)) return e;
     dim3 grid((unsigned)n_splits, (unsigned)((n_rows + kCtaRows - 1) / kCtaRows), (unsigned)(g.B * g.H));

@@ -159,4 +159,20 @@ __device__ __forceinline__ unsigned float_key(float f) {
     return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
 }
 
+// The sequence of rank `rank` in descending order of length (ties by position), for kernels whose CTAs take the long
+// sequences first.  All n_threads threads call it (one block barrier inside); `slot` is in shared memory.
+__device__ __forceinline__ int sequence_of_rank(const Geom &g, int rank, int n_threads, int *slot) {
+    for (int c = threadIdx.x; c < g.B; c += n_threads) {
+        const int lc = min(max(g.lengths[c], 0), g.T);
+        int before = 0;
+        for (int o = 0; o < g.B; ++o) {
+            const int lo = min(max(g.lengths[o], 0), g.T);
+            before += (lo > lc) || (lo == lc && o < c);
+        }
+        if (before == rank) *slot = c;
+    }
+    __syncthreads();
+    return *slot;
+}
+
 }  // namespace psattn

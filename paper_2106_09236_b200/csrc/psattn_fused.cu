@@ -88,18 +88,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
     int b = (int)(blockIdx.x / split) / g.H;
     const int h = (int)(blockIdx.x / split) % g.H;
     if (!SPLIT && a.by_length) {
-        const int rank = b;
-        for (int c = tid; c < g.B; c += kFusedThreads) {
-            const int lc = min(max(g.lengths[c], 0), g.T);
-            int before = 0;
-            for (int o = 0; o < g.B; ++o) {
-                const int lo = min(max(g.lengths[o], 0), g.T);
-                before += (lo > lc) || (lo == lc && o < c);
-            }
-            if (before == rank) P.b_ranked = c;
-        }
-        __syncthreads();
-        b = P.b_ranked;
+        b = sequence_of_rank(g, b, kFusedThreads, &P.b_ranked);
     }
     const int unit = b * g.H + h;
     const int L = seq_len(g, b);
