@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) k_measure_stream(Geom g, ui
     };
     StreamCtx cx;
     cx.ring = smem_u32(smem) + (uint32_t)warp * kStreamRing * kStreamRoundBytes;
-    cx.idx_cols = g.idx_cols; cx.status = g.status; cx.k_row_bytes = (uint32_t)(g.ks[2] * 2);
+    cx.idx_pitch = measure_idx_pitch(g.idx_cols); cx.status = g.status; cx.k_row_bytes = (uint32_t)(g.ks[2] * 2);
     const uint32_t stage0 = smem_u32(smem) + n_warps * kStreamRing * kStreamRoundBytes + (uint32_t)warp * 2u * warp_stage_bytes;
     // Q rows, then sample rows, of a group into one of the warp's two buffers; nobody else reads them, so the warps never meet at
     // a barrier and drift apart: the pipeline bubble at the start of a group does not hit all of them at once
@@ -130,14 +130,8 @@ __global__ void __launch_bounds__(kStreamThreads, 1) k_measure_stream(Geom g, ui
         const __nv_bfloat16 *Qu = Q + unit_off(g.qs, x.b, x.h);
         for (int e = lane; e < x.rows * 8; e += 32)
             cp_async_16(dst + (uint32_t)e * 16u, Qu + (long long)(x.i0 + (e >> 3)) * g.qs[2] + (e & 7) * 8);
-        const int words = x.rows * g.idx_cols;
-        const int *src = sidx + ((g.idx_per_head ? (long long)(x.b * g.H + x.h) : (long long)x.b) * g.T + x.i0) * g.idx_cols;
-        const uint32_t idst = dst + 1024u;
-        if (((reinterpret_cast<uintptr_t>(src) | (uintptr_t)(words * 4)) & 15u) == 0u) {
-            for (int w = lane; w < words / 4; w += 32) cp_async_16(idst + (uint32_t)w * 16u, src + 4 * w);
-        } else {
-            for (int w = lane; w < words; w += 32) cp_async_4(idst + (uint32_t)w * 4u, src + w);
-        }
+        measure_stage_samples(dst + 1024u, sidx + ((g.idx_per_head ? (long long)(x.b * g.H + x.h) : (long long)x.b) * g.T + x.i0) * g.idx_cols,
+                              x.rows, g.idx_cols);
         cp_async_commit();
     };
     Group cur, nxt;
@@ -242,7 +236,7 @@ cudaError_t launch_measure_stream(const Geom &g, int U_max, const void *Q, const
     if (g.B * g.H == 0) return cudaSuccess;
     if (U_max > kMeasureMaxU || U_max < 1) return cudaErrorNotSupported;
     if (g.ks[2] <= 0 || (long long)g.T * g.ks[2] * 2 >= (1ll << 32)) return cudaErrorNotSupported;
-    const size_t warp_stage = (1024 + (size_t)8 * g.idx_cols * 4 + 15) / 16 * 16;
+    const size_t warp_stage = (1024 + (size_t)8 * measure_idx_pitch(g.idx_cols) * 4 + 15) / 16 * 16;
     const size_t table = ((size_t)(g.B < kStreamMaxB ? g.B : kStreamMaxB) + 1) * 8;
     const size_t per_warp = kStreamRing * kStreamRoundBytes + 2 * warp_stage, room = 226 * 1024 - table;
     int warps = (int)(room / per_warp);

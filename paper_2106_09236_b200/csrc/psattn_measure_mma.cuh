@@ -72,14 +72,35 @@ __host__ __device__ constexpr int measure_block_queries(int threads) { return th
 __host__ __device__ inline size_t measure_k_bytes(int T) {
     return (size_t)((T + kMeasureBoxRows - 1) / kMeasureBoxRows * kMeasureBoxRows) * 128;
 }
+// Words per staged sample row.  A round reads two neighbouring words of eight rows at once: with a multiple of eight words
+// per row these fall into one to four banks (32 words, T = 493 .. 601 at c = 5: all eight rows in one; B32 H4 T512
+// 28.8 us against 25.6 with the rows 36 words apart).
+__host__ __device__ inline int measure_idx_pitch(int idx_cols) { return idx_cols % 8 == 0 ? idx_cols + 4 : idx_cols; }
+// Sample rows of a warp's queries into its staging buffer (all lanes; cp.async, not committed).
+__device__ __forceinline__ void measure_stage_samples(uint32_t dst, const int *src, int rows, int idx_cols) {
+    const int lane = threadIdx.x & 31, pitch = measure_idx_pitch(idx_cols);
+    if (pitch != idx_cols && (reinterpret_cast<uintptr_t>(src) & 15u) == 0u) {             // rows of whole 16-byte pieces
+        const int per_row = idx_cols / 4;
+        for (int w = lane; w < rows * per_row; w += 32) {
+            const int r = w / per_row;
+            cp_async_16(dst + (uint32_t)(w * 4 + r * 4) * 4u, src + 4 * w);
+        }
+    } else if (pitch != idx_cols) {
+        for (int w = lane; w < rows * idx_cols; w += 32) cp_async_4(dst + (uint32_t)(w + w / idx_cols * 4) * 4u, src + w);
+    } else if (((reinterpret_cast<uintptr_t>(src) | (uintptr_t)(rows * idx_cols * 4)) & 15u) == 0u) {
+        for (int w = lane; w < rows * idx_cols / 4; w += 32) cp_async_16(dst + (uint32_t)w * 16u, src + 4 * w);
+    } else {
+        for (int w = lane; w < rows * idx_cols; w += 32) cp_async_4(dst + (uint32_t)w * 4u, src + w);
+    }
+}
 __host__ __device__ inline size_t measure_stage_bytes(int threads, int idx_cols) {
     const size_t q = measure_block_queries(threads);
-    return (q * 128 + q * idx_cols * 4 + 127) / 128 * 128;
+    return (q * 128 + q * measure_idx_pitch(idx_cols) * 4 + 127) / 128 * 128;
 }
 
 struct MeasureCtx {
     uint32_t k_base, q_tile, idx_tile;      // shared-memory addresses
-    int rows, U, L, idx_cols;
+    int rows, U, L, idx_pitch;
     uint32_t epoch;                         // see ldmatrix_x4
     float *out;                             // M~ of the first query of the block (global or shared)
     unsigned *status;
@@ -119,7 +140,7 @@ __device__ __forceinline__ void measure_block(const MeasureCtx &cx) {
     uint32_t off[4];
 #pragma unroll
     for (int t = 0; t < 4; ++t) off[t] = (uint32_t)((2 * t + (lane >> 4) + l7) & 7) << 4;
-    const uint32_t krow = cx.idx_tile + (uint32_t)(qn * cx.idx_cols + ((lane >> 3) & 1)) * 4u;
+    const uint32_t krow = cx.idx_tile + (uint32_t)(qn * cx.idx_pitch + ((lane >> 3) & 1)) * 4u;
     // D: lane 4g + g / 2 holds D[g][g] (register g & 1) and D[g + 8][g] (register 2 + (g & 1)):
     // the two scores of query g in this round
     const int g = lane >> 2;
@@ -227,14 +248,8 @@ __device__ __forceinline__ bool measure_resident(uint8_t *smem, uint64_t *bar, u
                 const uint32_t qdst = base + (uint32_t)warp * 1024u;
                 for (int e = lane; e < rows * 8; e += 32)
                     cp_async_16(qdst + (uint32_t)e * 16u, Qu + (long long)(i0 + (e >> 3)) * g.qs[2] + (e & 7) * 8);
-                const int words = rows * g.idx_cols;
-                const int *src = idx_base + (long long)i0 * g.idx_cols;
-                const uint32_t idst = base + kBlock * 128u + (uint32_t)(warp * 8 * g.idx_cols) * 4u;
-                if (((reinterpret_cast<uintptr_t>(src) | (uintptr_t)(words * 4)) & 15u) == 0u) {
-                    for (int w = lane; w < words / 4; w += 32) cp_async_16(idst + (uint32_t)w * 16u, src + 4 * w);
-                } else {
-                    for (int w = lane; w < words; w += 32) cp_async_4(idst + (uint32_t)w * 4u, src + w);
-                }
+                measure_stage_samples(base + kBlock * 128u + (uint32_t)(warp * 8 * measure_idx_pitch(g.idx_cols)) * 4u,
+                                      idx_base + (long long)i0 * g.idx_cols, rows, g.idx_cols);
             }
         }
         cp_async_commit();
@@ -254,7 +269,7 @@ __device__ __forceinline__ bool measure_resident(uint8_t *smem, uint64_t *bar, u
     phase_stamp(g, 1);                                    // the unit's keys are in shared memory
     U = min(U, kMeasureMaxU);
     MeasureCtx cx;
-    cx.k_base = smem_u32(smem); cx.U = U; cx.L = L; cx.idx_cols = g.idx_cols; cx.status = g.status;
+    cx.k_base = smem_u32(smem); cx.U = U; cx.L = L; cx.idx_pitch = measure_idx_pitch(g.idx_cols); cx.status = g.status;
 
     for (int blk = 0; blk < n_blocks; ++blk) {
         stage_block(blk + kMeasureStages - 1);            // into the buffer this warp left at the end of the trip before

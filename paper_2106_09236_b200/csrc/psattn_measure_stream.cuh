@@ -20,7 +20,7 @@ constexpr uint32_t kStreamRoundBytes = 16 * 128;
 struct StreamCtx {
     uint32_t ring;                        // shared-memory address of this warp's ring
     uint32_t q_tile, idx_tile;            // staged Q rows and sample rows of the block
-    int rows, U, L, idx_cols;
+    int rows, U, L, idx_pitch;
     uint32_t epoch0;                      // see ldmatrix_x4: produced after the barrier that published the block
     const __nv_bfloat16 *Ku;              // key rows of the unit
     uint32_t k_row_bytes;                 // row pitch of K in bytes (T_max * pitch < 2^32, checked by the launcher)
@@ -112,8 +112,8 @@ __device__ __forceinline__ void measure_stream_group(const StreamCtx &cx) {
     for (int t = 0; t < 4; ++t)
         ln.la[t] = cx.ring + (uint32_t)(l7 + 8 * slot) * 128u + ((uint32_t)((2 * t + (lane >> 4) + l7) & 7) << 4);
     ln.dst = cx.ring + (uint32_t)lane * 16u;
-    ln.kp = cx.idx_tile + (uint32_t)(qn * cx.idx_cols + slot) * 4u;
-    ln.kp_last = cx.idx_tile + (uint32_t)(qn * cx.idx_cols + cx.U - 1) * 4u;
+    ln.kp = cx.idx_tile + (uint32_t)(qn * cx.idx_pitch + slot) * 4u;
+    ln.kp_last = cx.idx_tile + (uint32_t)(qn * cx.idx_pitch + cx.U - 1) * 4u;
     ln.kb = reinterpret_cast<const char *>(cx.Ku) + l7 * 16;
     ln.k_row_bytes = cx.k_row_bytes;
     ln.src0 = lane >> 3;
