@@ -21,7 +21,8 @@
 
 namespace psattn {
 
-constexpr int kPoThreads = 256;
+constexpr int kPoThreads = 512;              // the CTA is alone on its SM and a chain of latencies: 512 against 256 threads 14.8 / 16.8 us
+                                             // (B16 H8 T1024), 10.2 / 14.3 us (B32 H4 T700)
 constexpr int kPoCols = 64;                  // output columns per CTA
 constexpr int kPoMaxRows = 64;               // selected rows of one head (u_max <= 64)
 constexpr int kPoMaxChunk = 1024;            // positions per CTA at most
@@ -331,8 +332,14 @@ cudaError_t launch_project_out(int dtype, int mode, int zero_pad, const Geom &g,
     a.O = (const __nv_bfloat16 *)O; a.Wot = (const __nv_bfloat16 *)Wot; a.Y = (__nv_bfloat16 *)Y;
     a.sel = sel; a.lengths = g.lengths; a.status = g.status; a.zero_pad = zero_pad;
     a.t_chunk = 0; a.max_slots = 0; a.max_pairs = 0;
-    if (dtype == 0 && mode == 0 && sel != nullptr && g.u_max <= kPoMaxRows && g.H <= 32 && dy % 8 == 0) {
-        const int sms = device_sm_count();
+    // The dense product runs at the tensor cores' rate; the shortcut reads less but is a chain of dependent steps.  Where the
+    // dense product is at most one tile per SM (or three, with 512 columns and more to sum over, whose tiles hide their starts), it
+    // is the faster one.  us, shortcut / dense: B1 H4 T300 8.1 / 6.2, B2 H8 T3000 9.1 / 7.7, B16 H8 T1024 14.8 / 13.8, but
+    // B32 H4 T700 10.2 / 12.3.
+    const int sms = device_sm_count();
+    const long long dense_tiles = (long long)g.B * ((g.T + 127) / 128) * ((dy + 191) / 192);
+    const bool dense = mode == 0 && dtype == 0 && dy % 64 == 0 && dense_tiles <= (g.H >= 8 ? 3ll : 1ll) * sms;
+    if (dtype == 0 && mode == 0 && !dense && sel != nullptr && g.u_max <= kPoMaxRows && g.H <= 32 && dy % 8 == 0) {
         const int slices = (dy + kPoCols - 1) / kPoCols;
         // ranges of positions: about one CTA per SM (every CTA loads its weight slice once), 256 .. 1024 positions each
         int chunks = sms / (slices * g.B);

@@ -1,0 +1,36 @@
+"""The output matrix on either side of the line between its two forms: many short ragged sequences (broadcast plus corrections) and
+batches that a dense tile per SM or a few cover."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import psattn_oracle as orc
+from paper_2106_09236_b200 import binding as ps
+from paper_2106_09236_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,H,T,dy,longest", [(80, 4, 130, 256, 130), (160, 3, 70, 64, 69), (40, 4, 129, 128, 129),
+                                              (3, 5, 1030, 72, 1030), (2, 8, 257, 512, 255)])
+def test_output_matrix_forms(B, H, T, dy, longest):
+    rng = np.random.default_rng(B)
+    lengths = rng.integers(0, longest + 1, size=B).astype(np.int32)
+    lengths[0] = longest
+    w = wl.Workload("out", 0, B, H, T, 64, "bf16", 5.0, 0.1, 3.0)
+    n = max(orc.count(5.0, L) for L in range(1, T + 1))
+    inp = wl.make_inputs(w, n, seed=7, lengths=lengths)
+    plan = ps.Plan(B, H, T, c=5.0, idx_cols=n)
+    q, k, v = (torch.from_numpy(inp[x]).to("cuda", torch.bfloat16) for x in ("Q", "K", "V"))
+    ln, idx = (torch.from_numpy(inp[x]).cuda() for x in ("lengths", "sample_idx"))
+    O, sel = plan.psattn_forward(q, k, v, ln, idx)
+    Wot = wl.round_to_bf16((rng.standard_normal((dy, H * 64)) / 16).astype(np.float32))
+    Y = torch.full((B, T, dy), float("nan"), dtype=torch.bfloat16, device="cuda")
+    plan.psattn_project_out(O, sel, ln, torch.from_numpy(Wot).to("cuda", torch.bfloat16), Y=Y)
+    got = Y.float().cpu().numpy()
+    want = orc.project_out(O.float().cpu().numpy(), Wot, inp["lengths"], nthreads=4)
+    for b, L in enumerate(lengths):
+        assert np.isnan(got[b, L:]).all()
+        err = np.abs(got[b, :L] - want[b, :L])
+        assert (err <= 2.0 ** -8 * np.abs(want[b, :L]) + 1e-3).all()
+    plan.close()
