@@ -61,17 +61,17 @@ def tensor_peak():
 
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum per launch) of the dominant kernel from the
 # ncu capture summarised under profiles/, valid only while the kernel's sources are unchanged.
-_FUSED_SOURCES = ["psattn_fused.cu", "psattn_measure_mma.cuh", "psattn_attend_rows.cuh", "psattn_select.cuh",
+_FUSED_SOURCES = ["psattn_fused.cu", "psattn_measure_mma.cuh", "psattn_attend_rows.cuh", "psattn_select.cuh", "psattn_cluster.cuh",
                   "psattn_sm100.cuh", "psattn_common.cuh"]
 _STREAM_SOURCES = ["psattn_measure_mma.cu", "psattn_measure_stream.cuh", "psattn_measure_mma.cuh",
                    "psattn_sm100.cuh", "psattn_common.cuh"]
 TRAFFIC = {
-    "large_bf16": {"kernel": "k_forward_fused", "bytes": 54344192, "sources": _FUSED_SOURCES,
+    "large_bf16": {"kernel": "k_forward_fused", "bytes": 53223936, "sources": _FUSED_SOURCES,
                    "profile": "profiles/ncu_full_k_forward_fused_large_bf16.txt",
-                   "sources_sha1": "605a5cec63dc810331d622f1397e716836f31c53"},
-    "long_bf16": {"kernel": "k_measure_stream", "bytes": 75986944, "sources": _STREAM_SOURCES,
+                   "sources_sha1": "1187c13b8a60e9ee288234d3619fb7046442a2ea"},
+    "long_bf16": {"kernel": "k_measure_stream", "bytes": 75015424, "sources": _STREAM_SOURCES,
                   "profile": "profiles/ncu_full_k_measure_stream_long_bf16.txt",
-                  "sources_sha1": "3d85716f75af55982a00d06ed97d69c0403d17ba"},
+                  "sources_sha1": "a13c10c3f47b3db47a5c576634599e33ed45e89d"},
 }
 
 
