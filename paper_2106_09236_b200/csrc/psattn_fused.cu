@@ -247,17 +247,19 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
 bool make_rows_map(CUtensorMap *map, const void *base, const Geom &g, const long long s[3], int box_rows,
                    int swizzle128, int pos[3]);
 
-// CTAs per unit: as many (up to 8) as leave every cluster resident at once, where the sequences are long enough that
-// the shared-out measure and key tiles outweigh the exchanges (three cluster barriers and the merge, about 2.5 us).
-// Measured, us per call with 1 / 2 / 4 / 8 CTAs per unit: B1 H4 T128 15.8 / 17.8 / 17.5 / 18.3, T203 18.8 / 18.9 /
-// 17.8 / 18.5, T512 30.0 / 23.3 / 20.9 / 19.9, T1000 47.3 / 33.4 / 25.7 / 22.1; with a given index set B1 H4 T512
-// 11.1 / 11.4 / 12.3 / 12.4, T1000 17.4 / 15.1 / 13.9 / 13.1, T3000 34.2 / 24.3 / 19.0 / 14.3.
+// CTAs per unit: as many (up to 8) as leave every cluster resident at once, where the sequences are long enough that the
+// shared-out measure and key tiles outweigh the exchanges (three cluster barriers and the merge, about 2.5 us).
+// Measured, us per call with 1 / 2 / 4 / 8 CTAs per unit: B1 H4 T128 11.4 / 13.3 / 13.1 / 13.6, T203 14.0 / 14.1 / 13.2 /
+// 13.6, T512 24.8 / 20.2 / 15.6 / 14.5, T800 35.4 / 27.5 / 19.4 / 15.8; with a given index set T300 7.1 / 8.2 / 8.0 / 7.6,
+// T512 8.8 / 9.0 / 8.0 / 7.7, T768 11.2 / 10.4 / 9.0 / 8.0 (two CTAs pay from about 700 on, four from 450).
 static int fused_split(const Geom &g, int mode) {
     static ClusterRecord clusters;
     const int units = g.B * g.H;
-    if (g.T < (mode == kAllSteps ? 192 : 768)) return 1;
-    for (int split = kMaxSplit; split > 1; --split)
+    if (g.T < (mode == kAllSteps ? 192 : 448)) return 1;
+    for (int split = kMaxSplit; split > 1; --split) {
+        if (mode != kAllSteps && split < 4 && g.T < 704) return 1;
         if (units <= max_clusters(k_forward_fused<true, kAllSteps>, clusters, split, kFusedThreads, kFusedMaxSmem)) return split;
+    }
     return 1;
 }
 

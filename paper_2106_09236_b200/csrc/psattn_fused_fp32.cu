@@ -480,11 +480,12 @@ __global__ void __launch_bounds__(kF32Threads, 1) k_forward_fused_fp32(
     if (SPLIT && L > 0) cluster_wait();                        // nobody reads this CTA's states any more
 }
 
-// CTAs per unit: as many (up to 8) as leave every cluster resident at once; see fused_split in psattn_fused.cu.
+// CTAs per unit: as many (up to 8) as leave every cluster resident at once; see fused_split in psattn_fused.cu.  us per call with
+// 1 / 2 / 4 / 8 CTAs per unit: B1 H4 T64 14.4 / 14.1 / 12.8 / 13.0, T128 21.4 / 17.7 / 14.6 / 13.9, T200 32.0 / 21.9 / 17.1 / 15.1.
 static int f32_split(const Geom &g) {
     static ClusterRecord clusters;
     const int units = g.B * g.H;
-    if (g.T < 96) return 1;
+    if (g.T < 48) return 1;
     for (int split = kMaxSplit; split > 1; --split)
         if (units <= max_clusters(k_forward_fused_fp32<true>, clusters, split, kF32Threads, kF32MaxSmem)) return split;
     return 1;
