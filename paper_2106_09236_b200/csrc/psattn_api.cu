@@ -26,8 +26,9 @@ struct psattn_plan {
     bool host_io;
     void *h_Q, *h_K, *h_V, *h_O, *h_ws;
     int *h_len, *h_idx, *h_sel;
+    cudaStream_t h_in_stream;     // host-to-device copies of the chunks run here, one behind the other
     cudaStream_t h_copy_stream;   // device-to-host copies of finished chunks run here
-    cudaEvent_t h_ev[2];          // [0]: a chunk is finished; [1]: its results have been copied out
+    cudaEvent_t h_ev[2];          // [0]: a chunk is finished; [1]: a chunk has been copied in (or: the caller's earlier work)
     int b_override;               // > 0: number of sequences of the current (chunked) call
     // side stream of the staged schedule: the fill of step (e) runs there while steps (a)-(c) run on the caller's
     cudaStream_t side_stream;
@@ -209,7 +210,7 @@ extern "C" int psattn_plan_destroy(psattn_plan_t *p) {
     if (p->host_io) {
         cudaFree(p->h_Q); cudaFree(p->h_K); cudaFree(p->h_V); cudaFree(p->h_O); cudaFree(p->h_ws);
         cudaFree(p->h_len); cudaFree(p->h_idx); cudaFree(p->h_sel);
-        cudaStreamDestroy(p->h_copy_stream); cudaEventDestroy(p->h_ev[0]); cudaEventDestroy(p->h_ev[1]);
+        cudaStreamDestroy(p->h_in_stream); cudaStreamDestroy(p->h_copy_stream); cudaEventDestroy(p->h_ev[0]); cudaEventDestroy(p->h_ev[1]);
     }
     delete p;
     return PSATTN_OK;
@@ -675,6 +676,7 @@ extern "C" int psattn_plan_enable_host_io(psattn_plan_t *plan) {
         }
     }
     PSATTN_CU(cudaMemset(plan->h_ws, 0, 256));
+    PSATTN_CU(cudaStreamCreateWithFlags(&plan->h_in_stream, cudaStreamNonBlocking));
     PSATTN_CU(cudaStreamCreateWithFlags(&plan->h_copy_stream, cudaStreamNonBlocking));
     PSATTN_CU(cudaEventCreateWithFlags(&plan->h_ev[0], cudaEventDisableTiming));
     PSATTN_CU(cudaEventCreateWithFlags(&plan->h_ev[1], cudaEventDisableTiming));
@@ -692,35 +694,47 @@ extern "C" int psattn_forward_host(psattn_plan_t *plan, const void *Q, const voi
     psattn_desc_t &d = plan->desc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const size_t es = d.dtype == PSATTN_BF16 ? 2 : 4;
-    // Sequences are independent, so the batch goes through in chunks: while chunk k is copied in and
-    // computed on `stream`, the results of chunk k - 1 travel back on a second stream (PCIe is full
-    // duplex).  All chunks share the one workspace; they are ordered by `stream`.
+    // Sequences are independent, so the batch goes through in chunks: the copies in run one behind the other on a stream of
+    // their own, chunk k is computed on `stream` while chunk k + 1 is copied in, and the results of chunk k - 1 travel
+    // back on a third stream (PCIe is full duplex).  All chunks share the one workspace; they are ordered by `stream`.
+    // The link is the bound: copies in run at 52 GB/s with 2 us between copies, a copy out slows them by a third to a half of its
+    // time, and behind the last copy in stand one chunk's kernel and copy out.  So two chunks, the second a quarter of the
+    // batch (a short tail, few copies), and one chunk below 8 MB.  us per call with 1 chunk / 1/2 + 1/2 / 3/4 + 1/4 / four
+    // halving ones: B32 H4 T512 722 / 700 / 683 / 704, B64 H4 T256 721 / 689 / 672 / 699, B8 H4 T300 159 / 171 / 173 / 203.
     const size_t per_b = (size_t)d.H * d.T_max * kD * es;
     const size_t idx_b = (size_t)(d.idx_per_head ? d.H : 1) * (d.idx_shared ? 1 : d.T_max) * d.idx_cols * sizeof(int);
     const size_t sel_b = (size_t)d.H * plan->u_max * sizeof(int);
-    if (lengths) PSATTN_CU(cudaMemcpyAsync(plan->h_len, lengths, (size_t)d.B * sizeof(int), cudaMemcpyHostToDevice, st));
+    const cudaStream_t in = plan->h_in_stream;
+    PSATTN_CU(cudaEventRecord(plan->h_ev[1], st));              // the copies in stay behind the caller's earlier work
+    PSATTN_CU(cudaStreamWaitEvent(in, plan->h_ev[1], 0));
+    if (lengths) PSATTN_CU(cudaMemcpyAsync(plan->h_len, lengths, (size_t)d.B * sizeof(int), cudaMemcpyHostToDevice, in));
     // the staging buffers are dense: run with dense strides whatever the descriptor says
     psattn_desc_t saved = d;
     std::memset(d.q_stride, 0, sizeof(d.q_stride)); std::memset(d.k_stride, 0, sizeof(d.k_stride));
     std::memset(d.v_stride, 0, sizeof(d.v_stride)); std::memset(d.o_stride, 0, sizeof(d.o_stride));
     check_strides(d.q_stride, d); check_strides(d.k_stride, d);
     check_strides(d.v_stride, d); check_strides(d.o_stride, d);
-    int n_chunks = 2;       // measured: every extra chunk costs ~50 us of copy set-up, more than it hides
+    constexpr size_t kOneChunkBytes = 8u << 20;
+    int n_chunks = 0;       // 0: as above
     if (const char *env = std::getenv("PSATTN_HOST_CHUNKS")) { const int v = std::atoi(env); if (v >= 1 && v <= 64) n_chunks = v; }
     if (n_chunks > d.B) n_chunks = d.B > 0 ? d.B : 1;
     int rc = PSATTN_OK;
     cudaError_t ce = cudaSuccess;
-    for (int k = 0; k < n_chunks && rc == PSATTN_OK && ce == cudaSuccess; ++k) {
-        const int b0 = (int)((long long)d.B * k / n_chunks), b1 = (int)((long long)d.B * (k + 1) / n_chunks);
-        const int nb = b1 - b0;
-        if (nb == 0) continue;
+    int nb = 0;
+    for (int b0 = 0, k = 0; b0 < d.B; b0 += nb, ++k) {
+        const int rest = d.B - b0;
+        if (n_chunks > 0) nb = (int)((long long)d.B * (k + 1) / n_chunks) - b0;
+        else nb = k == 0 && d.B > 1 && d.B * (3 * per_b + idx_b) >= kOneChunkBytes ? (d.B == 2 ? 1 : (3 * d.B + 2) / 4) : rest;
+        if (nb <= 0) continue;
         char *dq = (char *)plan->h_Q + b0 * per_b, *dk = (char *)plan->h_K + b0 * per_b;
         char *dv = (char *)plan->h_V + b0 * per_b, *dout = (char *)plan->h_O + b0 * per_b;
         char *di = (char *)plan->h_idx + b0 * idx_b, *ds = (char *)plan->h_sel + b0 * sel_b;
-        if ((ce = cudaMemcpyAsync(dq, (const char *)Q + b0 * per_b, nb * per_b, cudaMemcpyHostToDevice, st)) != cudaSuccess) break;
-        if ((ce = cudaMemcpyAsync(dk, (const char *)K + b0 * per_b, nb * per_b, cudaMemcpyHostToDevice, st)) != cudaSuccess) break;
-        if ((ce = cudaMemcpyAsync(dv, (const char *)V + b0 * per_b, nb * per_b, cudaMemcpyHostToDevice, st)) != cudaSuccess) break;
-        if ((ce = cudaMemcpyAsync(di, (const char *)sample_idx + b0 * idx_b, nb * idx_b, cudaMemcpyHostToDevice, st)) != cudaSuccess) break;
+        if ((ce = cudaMemcpyAsync(dq, (const char *)Q + b0 * per_b, nb * per_b, cudaMemcpyHostToDevice, in)) != cudaSuccess) break;
+        if ((ce = cudaMemcpyAsync(dk, (const char *)K + b0 * per_b, nb * per_b, cudaMemcpyHostToDevice, in)) != cudaSuccess) break;
+        if ((ce = cudaMemcpyAsync(dv, (const char *)V + b0 * per_b, nb * per_b, cudaMemcpyHostToDevice, in)) != cudaSuccess) break;
+        if ((ce = cudaMemcpyAsync(di, (const char *)sample_idx + b0 * idx_b, nb * idx_b, cudaMemcpyHostToDevice, in)) != cudaSuccess) break;
+        if ((ce = cudaEventRecord(plan->h_ev[1], in)) != cudaSuccess) break;
+        if ((ce = cudaStreamWaitEvent(st, plan->h_ev[1], 0)) != cudaSuccess) break;
         plan->b_override = nb;
         rc = psattn_forward(plan, dq, dk, dv, lengths ? plan->h_len + b0 : nullptr, (const int32_t *)di, dout,
                             (int32_t *)ds, nullptr, plan->h_ws, plan->ws_bytes, stream);
@@ -734,6 +748,7 @@ extern "C" int psattn_forward_host(psattn_plan_t *plan, const void *Q, const voi
     d = saved;
     plan->b_override = 0;
     // never return with copies in flight, whatever happened above
+    cudaStreamSynchronize(in);
     cudaStreamSynchronize(plan->h_copy_stream);
     if (rc != PSATTN_OK) { cudaStreamSynchronize(st); return rc; }
     if (ce != cudaSuccess) { cudaStreamSynchronize(st); return cuda_fail(plan, ce); }
