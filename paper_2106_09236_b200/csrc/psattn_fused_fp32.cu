@@ -49,6 +49,13 @@ struct Fused32Persist {
 
 __host__ __device__ inline size_t f32_arrays_bytes(int m_floats, int T) { return ((size_t)4 * m_floats + T + 127) / 128 * 128; }
 
+// acc += (a0 b0, a1 b1) in one instruction
+__device__ __forceinline__ void f32_fma2(float2 &acc, float a0, float a1, float b0, float b1) {
+    asm("{\n\t.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tmov.b64 z, {%0, %1};\n\t"
+        "fma.rn.f32x2 z, x, y, z;\n\tmov.b64 {%0, %1}, z;\n\t}"
+        : "+f"(acc.x), "+f"(acc.y) : "f"(a0), "f"(a1), "f"(b0), "f"(b1));
+}
+
 // One query's samples, kept one query ahead: its row (8 columns per lane) and up to 64 key positions.
 struct F32Query {
     float q[8];
@@ -89,7 +96,6 @@ __device__ __forceinline__ void f32_measure_n(const Geom &g, int unit, int b, in
         for (int x = 0; x < 2; ++x)
             if ((unsigned)cur.key[x] >= (unsigned)L) { atomicOr(g.status, kStatusIdxClamped); cur.key[x] = cur.key[x] < 0 ? 0 : L - 1; }
         float s[NB];
-        float mx = -INFINITY;
 #pragma unroll
         for (int n = 0; n < NB; ++n) {
             float part[4];
@@ -102,31 +108,32 @@ __device__ __forceinline__ void f32_measure_n(const Geom &g, int unit, int b, in
                     const float4 *kr = Kl + (long long)key * (k_pitch >> 2);
                     lo = __ldg(kr); hi = __ldg(kr + 1);
                 }
-                float p = cur.q[0] * lo.x;
-                p = fmaf(cur.q[1], lo.y, p); p = fmaf(cur.q[2], lo.z, p); p = fmaf(cur.q[3], lo.w, p);
-                p = fmaf(cur.q[4], hi.x, p); p = fmaf(cur.q[5], hi.y, p); p = fmaf(cur.q[6], hi.z, p); p = fmaf(cur.q[7], hi.w, p);
-                part[x] = p;
+                float2 p = make_float2(cur.q[0] * lo.x, cur.q[1] * lo.y);
+                f32_fma2(p, cur.q[2], cur.q[3], lo.z, lo.w);
+                f32_fma2(p, cur.q[4], cur.q[5], hi.x, hi.y);
+                f32_fma2(p, cur.q[6], cur.q[7], hi.z, hi.w);
+                part[x] = p.x + p.y;
             }
             const float r0 = (b0 ? part[2] : part[0]) + __shfl_xor_sync(0xffffffffu, b0 ? part[0] : part[2], 1);
             const float r1 = (b0 ? part[3] : part[1]) + __shfl_xor_sync(0xffffffffu, b0 ? part[1] : part[3], 1);
             float v = (b1 ? r1 : r0) + __shfl_xor_sync(0xffffffffu, b1 ? r0 : r1, 2);
             v += __shfl_xor_sync(0xffffffffu, v, 4);
-            s[n] = n * 16 + mine < U ? v * kScale : -INFINITY;
-            mx = fmaxf(mx, s[n]);
+            s[n] = v;
         }
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
-        float D = 0.f;
+        float mx = -INFINITY, D = 0.f;
+#pragma unroll
+        for (int n = 0; n < NB; ++n)
+            if (n * 16 + mine < U) mx = fmaxf(mx, s[n]);
+#pragma unroll
+        for (int o = 1; o <= 16; o <<= 1)
+            if (o != 4) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));           // (lanes l and l ^ 4 hold the same scores)
 #pragma unroll
         for (int n = 0; n < NB; ++n)
             if (n * 16 + mine < U) D += mx - s[n];
-        D += __shfl_xor_sync(0xffffffffu, D, 1);
-        D += __shfl_xor_sync(0xffffffffu, D, 2);
-        D += __shfl_xor_sync(0xffffffffu, D, 8);
-        D += __shfl_xor_sync(0xffffffffu, D, 16);
-        if (lane == 0) M_s[i] = U > 0 ? D / (float)U : 0.f;
+#pragma unroll
+        for (int o = 1; o <= 16; o <<= 1)
+            if (o != 4) D += __shfl_xor_sync(0xffffffffu, D, o);
+        if (lane == 0) M_s[i] = U > 0 ? D * kScale / (float)U : 0.f;
         cur = nxt;
     }
 }
@@ -176,13 +183,6 @@ __device__ __forceinline__ void f32_stage_rows(uint32_t dst, uint32_t pitch, con
         if (r < valid) cp_async_16(d, src + (long long)r * stride + c * 4);
         else asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(d), "r"(0) : "memory");
     }
-}
-
-// acc += (a0 b0, a1 b1) in one instruction
-__device__ __forceinline__ void f32_fma2(float2 &acc, float a0, float a1, float b0, float b1) {
-    asm("{\n\t.reg .b64 x, y, z;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tmov.b64 z, {%0, %1};\n\t"
-        "fma.rn.f32x2 z, x, y, z;\n\tmov.b64 {%0, %1}, z;\n\t}"
-        : "+f"(acc.x), "+f"(acc.y) : "f"(a0), "f"(a1), "f"(b0), "f"(b1));
 }
 
 // The attention of the listed rows over the keys [lo, hi): on return P.m[0] / P.l hold the row states and the partial sums of the
