@@ -19,7 +19,7 @@ struct Attend64Args {
     float *vbar;                // if non-null: mean(V) [unit][64], from an extra all-weights-1 row (slot n_rows)
 };
 
-__global__ void __launch_bounds__(kArThreads, 1) k_attend64(Geom g, Attend64Args a, const __nv_bfloat16 *__restrict__ Q,
+__global__ void __launch_bounds__(ArWide::kThreads, 1) k_attend64(Geom g, Attend64Args a, const __nv_bfloat16 *__restrict__ Q,
                                                             const __grid_constant__ CUtensorMap tmK,
                                                             const __grid_constant__ CUtensorMap tmV) {
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -39,9 +39,11 @@ __global__ void __launch_bounds__(kArThreads, 1) k_attend64(Geom g, Attend64Args
     j.rows = a.rows + (long long)unit * a.rows_stride; j.n_rows = a.n_rows;
     j.pos_t = a.pos_t; j.pos_h = a.pos_h; j.pos_b = a.pos_b;
     j.sum_row = a.vbar ? a.n_rows : -1;
-    if (tid == kArLoader) attend_rows_start(smem, j, &tmK, &tmV, 1);
-    float m_run, l_run, acc[8];
-    if (!attend_rows_run(smem, g, j, Q, &tmK, &tmV, 1, m_run, l_run, acc)) return;
+    if (tid == ArWide::kLoader) attend_rows_start<ArWide>(smem, j, &tmK, &tmV, 1);
+    float m_rows[1], l_rows[1], acc_rows[1][8];
+    if (!attend_rows_run<ArWide>(smem, g, j, Q, &tmK, &tmV, 1, m_rows, l_rows, acc_rows)) return;
+    const float m_run = m_rows[0], l_run = l_rows[0];
+    float (&acc)[8] = acc_rows[0];
 
     const int r = tid >> 3, c8 = tid & 7;
     const int n_slots = a.n_rows + (a.vbar ? 1 : 0);               // row slots per unit in the split partials
@@ -105,9 +107,9 @@ cudaError_t launch_attend64(const Geom &g, const void *Q, const void *K, const v
     if (posK[0] != posV[0] || posK[1] != posV[1] || posK[2] != posV[2]) return cudaErrorNotSupported;
     a.pos_t = posK[0]; a.pos_h = posK[1]; a.pos_b = posK[2];
     static SmemGrant grant;
-    if (cudaError_t e = grant_dynamic_smem(k_attend64, grant, kArBytes)) return e;
+    if (cudaError_t e = grant_dynamic_smem(k_attend64, grant, ArWide::kBytes)) return e;
     dim3 grid((unsigned)n_splits, (unsigned)(g.B * g.H));
-    cudaError_t le = launch_pdl(k_attend64, grid, dim3(kArThreads), kArBytes, st, g, a, (const __nv_bfloat16 *)Q, tmK, tmV);
+    cudaError_t le = launch_pdl(k_attend64, grid, dim3(ArWide::kThreads), ArWide::kBytes, st, g, a, (const __nv_bfloat16 *)Q, tmK, tmV);
     if (le != cudaSuccess) { note_launch(); return le; }
     note_launch();
     return cudaGetLastError();

@@ -1,4 +1,4 @@
-// Step (d) (Eq. 7-8) for up to 64 listed rows of one unit, as a routine of a 512-thread CTA on mma.sync.
+// Step (d) (Eq. 7-8) for up to 64 listed rows of one unit, as a routine of a CTA of 512 (or 256) threads on mma.sync.
 //
 // The step is short and its operands are thin (u <= 64 rows), so what it costs is the chain of dependent steps, not
 // the tensor pipe: on tcgen05 every key tile went TMA -> product -> TMEM -> registers -> shared memory -> product ->
@@ -6,7 +6,7 @@
 // products kept the pipe a few per cent busy.  Here scores and weights stay in the registers of one warp from the first
 // product to the second, and no warp waits for another before the merge at the end.
 //
-//   K and V stream in chunks of 256 keys by TMA (128-byte swizzle) through a ring of three stages; a chunk's stage is
+//   K and V stream in chunks of 256 (128) keys by TMA (128-byte swizzle) through a ring of three (two) stages; a chunk's stage is
 //   refilled by whichever warp is the last to leave it.
 //   A warp owns one tile of 16 rows and one key group: the blocks of 32 keys whose number is the group's modulo the
 //   number of groups, so that short sequences spread over all warps as well.  Groups: 16, 8, 5 or 4 for one to four
@@ -27,18 +27,25 @@
 
 namespace psattn {
 
-constexpr int kArThreads = 512;
-constexpr int kArLoader = kArThreads - 32;                   // the thread that starts the copies of the first stages
 constexpr int kArMaxRows = 64;
-constexpr int kArChunk = 256;                                // keys per stage
-constexpr int kArStages = 3;
 constexpr int kArBlock = 32;                                 // keys per trip of a warp
-constexpr int kArPerChunk = kArChunk / kArBlock;
 constexpr uint32_t kArTile = 16384;                          // one 128-key K or V tile
 constexpr uint32_t kArOffQ = 0;                              // 64 rows x 128 B
-constexpr uint32_t kArOffStage = 8192;                       // per stage: two K tiles, two V tiles
-constexpr uint32_t kArOffBar = kArOffStage + kArStages * 4 * kArTile;
-constexpr uint32_t kArBytes = kArOffBar + 128;
+constexpr uint32_t kArOffStage = 8192;                       // per stage: K tiles, then V tiles
+// Shape of the CTA: threads, keys per stage, stages of the ring.
+template <int THREADS, int CHUNK, int STAGES>
+struct AttendRowsShape {
+    static constexpr int kThreads = THREADS, kChunk = CHUNK, kStages = STAGES;
+    static constexpr int kLoader = THREADS - 32;             // the thread that starts the copies of the first stages
+    static constexpr int kPerChunk = CHUNK / kArBlock;
+    static constexpr int kRows = kArMaxRows * 8 / THREADS;   // rows per thread of the result
+    static constexpr uint32_t kOffV = CHUNK * 128, kStageBytes = 2 * kOffV;
+    static constexpr uint32_t kOffBar = kArOffStage + STAGES * kStageBytes;
+    static constexpr uint32_t kBytes = kOffBar + 128;
+};
+typedef AttendRowsShape<512, 256, 3> ArWide;                 // alone on its SM
+typedef AttendRowsShape<256, 128, 2> ArHalf;                 // two CTAs per SM
+constexpr int kArMostStages = 3;
 constexpr int kArPitch = 72;                                 // floats per row of the merge buffer: O[64], m, l
 
 struct AttendRowsJob {
@@ -51,48 +58,50 @@ struct AttendRowsJob {
 };
 
 struct AttendRowsBars {
-    uint64_t full[kArStages];
-    int left[kArStages];         // warps that have left the stage
-    int issued[kArStages];       // copies started into the stage
+    uint64_t full[kArMostStages];
+    int left[kArMostStages];         // warps that have left the stage
+    int issued[kArMostStages];       // copies started into the stage
     int abort_flag;
 };
 
 // One thread: the TMA copies of chunk c.
+template <class S>
 __device__ __forceinline__ void attend_rows_load(uint8_t *smem, const AttendRowsJob &j, const CUtensorMap *tmK,
                                                  const CUtensorMap *tmV, int c) {
     using namespace sm100;
-    AttendRowsBars &B = *reinterpret_cast<AttendRowsBars *>(smem + kArOffBar);
-    const int s = c % kArStages;
-    B.issued[s] = c / kArStages + 1;
-    const int tiles = min(2, (j.hi - j.lo - c * kArChunk + 127) / 128);
+    AttendRowsBars &B = *reinterpret_cast<AttendRowsBars *>(smem + S::kOffBar);
+    const int s = c % S::kStages;
+    B.issued[s] = c / S::kStages + 1;
+    const int tiles = min(S::kChunk / 128, (j.hi - j.lo - c * S::kChunk + 127) / 128);
     mbar_expect_tx(&B.full[s], 2 * kArTile * (uint32_t)tiles);
 #pragma unroll 1
     for (int t = 0; t < tiles; ++t) {
-        const int key0 = j.lo + c * kArChunk + t * 128;
+        const int key0 = j.lo + c * S::kChunk + t * 128;
         const int c1 = j.pos_t == 1 ? key0 : (j.pos_h == 1 ? j.h : j.b);
         const int c2 = j.pos_t == 2 ? key0 : (j.pos_h == 2 ? j.h : j.b);
         const int c3 = j.pos_t == 3 ? key0 : (j.pos_h == 3 ? j.h : j.b);
-        uint8_t *dst = smem + kArOffStage + s * 4 * kArTile + t * kArTile;
+        uint8_t *dst = smem + kArOffStage + s * S::kStageBytes + t * kArTile;
         tma_load_4d(dst, tmK, &B.full[s], 0, c1, c2, c3);
-        tma_load_4d(dst + 2 * kArTile, tmV, &B.full[s], 0, c1, c2, c3);
+        tma_load_4d(dst + S::kOffV, tmV, &B.full[s], 0, c1, c2, c3);
     }
 }
 
-// Thread kArLoader: initialise the barriers and start the copies of the first `ahead` chunks.  They depend only on the
+// Thread kLoader: initialise the barriers and start the copies of the first `ahead` chunks.  They depend only on the
 // unit and its length, not on the listed rows, so that a caller may run this early; the shared memory of the routine must
 // be free.  In attend_rows_run the same thread (so that no block barrier is needed in between) starts the rest of the ring
 // behind the loads of the query rows, which otherwise queue behind the copies of all CTAs (128 of them, K and V cold:
 // 3.3 us instead of 2.1 us for the rows with three chunks ahead).
+template <class S>
 __device__ __forceinline__ void attend_rows_start(uint8_t *smem, const AttendRowsJob &j, const CUtensorMap *tmK,
                                                   const CUtensorMap *tmV, int ahead) {
     using namespace sm100;
-    AttendRowsBars &B = *reinterpret_cast<AttendRowsBars *>(smem + kArOffBar);
-    for (int s = 0; s < kArStages; ++s) { mbar_init(&B.full[s], 1); B.left[s] = 0; B.issued[s] = 0; }
+    AttendRowsBars &B = *reinterpret_cast<AttendRowsBars *>(smem + S::kOffBar);
+    for (int s = 0; s < S::kStages; ++s) { mbar_init(&B.full[s], 1); B.left[s] = 0; B.issued[s] = 0; }
     B.abort_flag = 0;
     fence_barrier_init();
-    const int n_chunks = (j.hi - j.lo + kArChunk - 1) / kArChunk;
+    const int n_chunks = (j.hi - j.lo + S::kChunk - 1) / S::kChunk;
 #pragma unroll 1
-    for (int c = 0; c < ahead && c < n_chunks; ++c) attend_rows_load(smem, j, tmK, tmV, c);
+    for (int c = 0; c < ahead && c < n_chunks; ++c) attend_rows_load<S>(smem, j, tmK, tmV, c);
 }
 
 // Not volatile, so that the compiler may place them; `epoch` (see ldmatrix_x4) ties them to the wait before them.
@@ -128,13 +137,14 @@ __device__ __forceinline__ uint32_t ar_pack(float a, float b) {
 // The loop is kept short on purpose: unrolled over a chunk, or software pipelined (the scores of the next block ahead of the
 // softmax of this one), the warps of a scheduler thrash its instruction cache: a third of the issue slots went to missing
 // instructions, 7.5 and 10 us at T = 1024.  With 16 keys per trip instead of 32 the overhead of a trip weighs twice: 8.3 us.
+template <class S>
 __device__ __forceinline__ void attend_rows_warp(uint8_t *smem, const AttendRowsJob &j, const CUtensorMap *tmK,
                                                  const CUtensorMap *tmV, const Geom &g, int mt, int grp, int groups,
                                                  int n_warps, bool ones, float m[2], float l[2], float o[8][4]) {
     using namespace sm100;
-    AttendRowsBars &B = *reinterpret_cast<AttendRowsBars *>(smem + kArOffBar);
+    AttendRowsBars &B = *reinterpret_cast<AttendRowsBars *>(smem + S::kOffBar);
     const int lane = threadIdx.x & 31, l7 = lane & 7;
-    const int n_keys = j.hi - j.lo, n_chunks = (n_keys + kArChunk - 1) / kArChunk, n_blocks = (n_keys + kArBlock - 1) / kArBlock;
+    const int n_keys = j.hi - j.lo, n_chunks = (n_keys + S::kChunk - 1) / S::kChunk, n_blocks = (n_keys + kArBlock - 1) / kArBlock;
     constexpr float kScaleLog2 = kScale * kLog2e;
     constexpr float kSlack = 8.f;                              // weights may grow to 2^8 before the reference moves
     uint32_t q[4][4], epoch;
@@ -147,7 +157,7 @@ __device__ __forceinline__ void attend_rows_warp(uint8_t *smem, const AttendRows
     }
     auto arrived = [&](int c) {                                // bounded wait, agreed on by the warp
         bool ok = *reinterpret_cast<volatile int *>(&B.abort_flag) == 0;
-        if (ok) ok = mbar_wait(&B.full[c % kArStages], (uint32_t)(c / kArStages) & 1u, g.wait_ns);
+        if (ok) ok = mbar_wait(&B.full[c % S::kStages], (uint32_t)(c / S::kStages) & 1u, g.wait_ns);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok && lane == 0) { *reinterpret_cast<volatile int *>(&B.abort_flag) = 1; atomicOr(g.status, kStatusWaitExpired); }
         return ok;
@@ -157,17 +167,17 @@ __device__ __forceinline__ void attend_rows_warp(uint8_t *smem, const AttendRows
     // multiple of eight rows, so the swizzle depends on the lane alone
     const uint32_t base = smem_u32(smem + kArOffStage);
     const uint32_t k_lane = (uint32_t)l7 * 128u + ((uint32_t)((lane >> 3) ^ l7) << 4);
-    const uint32_t v_lane = 2 * kArTile + (uint32_t)(l7 + 8 * ((lane >> 3) & 1)) * 128u + ((uint32_t)((lane >> 4) ^ l7) << 4);
+    const uint32_t v_lane = S::kOffV + (uint32_t)(l7 + 8 * ((lane >> 3) & 1)) * 128u + ((uint32_t)((lane >> 4) ^ l7) << 4);
     float2 l0 = make_float2(0.f, 0.f), l1 = l0;
-    int c = -1, stage = -1, in_chunk = grp + kArPerChunk;      // chunk, its stage, block inside it (normalised at the top)
+    int c = -1, stage = -1, in_chunk = grp + S::kPerChunk;      // chunk, its stage, block inside it (normalised at the top)
 #pragma unroll 1
     for (int i = grp; i < n_blocks; i += groups, in_chunk += groups) {
-        if (in_chunk >= kArPerChunk) {                         // on to another chunk
-            do { in_chunk -= kArPerChunk; ++c; stage = stage == kArStages - 1 ? 0 : stage + 1; } while (in_chunk >= kArPerChunk);
+        if (in_chunk >= S::kPerChunk) {                         // on to another chunk
+            do { in_chunk -= S::kPerChunk; ++c; stage = stage == S::kStages - 1 ? 0 : stage + 1; } while (in_chunk >= S::kPerChunk);
             if (!arrived(c)) return;
         }
         asm volatile("mov.u32 %0, %1;" : "=r"(epoch) : "r"(i) : "memory");
-        const uint32_t at = base + (uint32_t)stage * (4 * kArTile) + (uint32_t)in_chunk * (kArBlock * 128u);
+        const uint32_t at = base + (uint32_t)stage * S::kStageBytes + (uint32_t)in_chunk * (kArBlock * 128u);
         const int left = n_keys - i * kArBlock;                // keys from the block's first on
         float s[4][4];
 #pragma unroll
@@ -199,7 +209,7 @@ __device__ __forceinline__ void attend_rows_warp(uint8_t *smem, const AttendRows
             }
 #pragma unroll 1
             for (int e = left * 8 + lane; e < kArBlock * 8; e += 32)
-                asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(at + 2 * kArTile + (uint32_t)e * 16u), "r"(0) : "memory");
+                asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(at + S::kOffV + (uint32_t)e * 16u), "r"(0) : "memory");
             __syncwarp();
             asm volatile("mov.u32 %0, %1;" : "=r"(epoch) : "r"(i) : "memory");
         }
@@ -236,14 +246,14 @@ __device__ __forceinline__ void attend_rows_warp(uint8_t *smem, const AttendRows
             mma_bf16_16816(o[2 * d], p[2][0], p[2][1], p[3][0], p[3][1], w[0], w[1]);
             mma_bf16_16816(o[2 * d + 1], p[2][0], p[2][1], p[3][0], p[3][1], w[2], w[3]);
         }
-        if (in_chunk + groups >= kArPerChunk && c + kArStages < n_chunks) {
+        if (in_chunk + groups >= S::kPerChunk && c + S::kStages < n_chunks) {
             __syncwarp();                                      // every lane has read its fragments
             if (lane == 0) {
                 __threadfence_block();
                 if (atomicAdd(&B.left[stage], 1) == n_warps - 1) { // the last warp to leave the stage refills it
                     B.left[stage] = 0;
                     __threadfence_block();
-                    attend_rows_load(smem, j, tmK, tmV, c + kArStages);
+                    attend_rows_load<S>(smem, j, tmK, tmV, c + S::kStages);
                 }
             }
             __syncwarp();
@@ -252,35 +262,44 @@ __device__ __forceinline__ void attend_rows_warp(uint8_t *smem, const AttendRows
     l[0] = l0.x + l0.y; l[1] = l1.x + l1.y;
 }
 
-// All 512 threads of the CTA (contains __syncthreads); attend_rows_start must have been run with the same
+// All threads of the CTA (contains __syncthreads); attend_rows_start must have been run with the same
 // `ahead`.  On return thread t holds, of
-// row t / 8, the softmax state over [lo, hi): m (scaled log2 units), l, and the unnormalised columns 8 (t % 8) .. + 7.
+// rows t / 8 + x kThreads / 8, the softmax state over [lo, hi): m (scaled log2 units), l, and the unnormalised columns 8 (t % 8) .. + 7.
 // Returns false if a wait ran out (status bit set).
+template <class S>
 __device__ __forceinline__ bool attend_rows_run(uint8_t *smem, const Geom &g, const AttendRowsJob &j,
                                                 const __nv_bfloat16 *__restrict__ Q, const CUtensorMap *tmK,
-                                                const CUtensorMap *tmV, int ahead, float &m_out, float &l_out,
-                                                float acc[8]) {
+                                                const CUtensorMap *tmV, int ahead, float (&m_out)[S::kRows],
+                                                float (&l_out)[S::kRows], float (&acc)[S::kRows][8]) {
     using namespace sm100;
-    AttendRowsBars &B = *reinterpret_cast<AttendRowsBars *>(smem + kArOffBar);
+    AttendRowsBars &B = *reinterpret_cast<AttendRowsBars *>(smem + S::kOffBar);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    {   // the listed rows of Q, one 16-byte piece per thread; unused rows are zero
-        const int r = tid >> 3, c = tid & 7;
-        int i = -1;
-        if (r < j.n_rows) i = j.rows ? j.rows[r] : r;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (i >= 0 && i < j.L)
-            v = __ldg(reinterpret_cast<const uint4 *>(Q + unit_off(g.qs, j.b, j.h) + (long long)i * g.qs[2]) + c);
-        if (tid == kArLoader) {
-            const int n_chunks = (j.hi - j.lo + kArChunk - 1) / kArChunk;
-#pragma unroll 1
-            for (int x = ahead; x < kArStages && x < n_chunks; ++x) attend_rows_load(smem, j, tmK, tmV, x);
+    {   // the listed rows of Q, 16-byte pieces; unused rows are zero
+        uint4 v[S::kRows];
+#pragma unroll
+        for (int x = 0; x < S::kRows; ++x) {
+            const int r = (tid + x * S::kThreads) >> 3, c = tid & 7;
+            int i = -1;
+            if (r < j.n_rows) i = j.rows ? j.rows[r] : r;
+            v[x] = make_uint4(0u, 0u, 0u, 0u);
+            if (i >= 0 && i < j.L)
+                v[x] = __ldg(reinterpret_cast<const uint4 *>(Q + unit_off(g.qs, j.b, j.h) + (long long)i * g.qs[2]) + c);
         }
-        *reinterpret_cast<uint4 *>(smem + kArOffQ + r * 128 + ((c ^ (r & 7)) << 4)) = v;
+        if (tid == S::kLoader) {
+            const int n_chunks = (j.hi - j.lo + S::kChunk - 1) / S::kChunk;
+#pragma unroll 1
+            for (int x = ahead; x < S::kStages && x < n_chunks; ++x) attend_rows_load<S>(smem, j, tmK, tmV, x);
+        }
+#pragma unroll
+        for (int x = 0; x < S::kRows; ++x) {
+            const int r = (tid + x * S::kThreads) >> 3, c = tid & 7;
+            *reinterpret_cast<uint4 *>(smem + kArOffQ + r * 128 + ((c ^ (r & 7)) << 4)) = v[x];
+        }
     }
     __syncthreads();
     phase_stamp(g, 6);
     const int used = max(j.n_rows, j.sum_row + 1), tiles = (used + 15) / 16;
-    const int groups = tiles <= 1 ? 16 : 16 / tiles;           // 16, 8, 5, 4
+    const int groups = (S::kThreads / 32) / max(tiles, 1);     // of 16 warps: 16, 8, 5, 4
     const int mt = warp / groups, grp = warp % groups;
     const bool ones = j.sum_row >= 0 && mt * 16 >= j.n_rows;   // a tile with no query but the all-ones row
     float m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f}, o[8][4];
@@ -289,7 +308,7 @@ __device__ __forceinline__ bool attend_rows_run(uint8_t *smem, const Geom &g, co
 #pragma unroll
         for (int e = 0; e < 4; ++e) o[x][e] = 0.f;
     if (mt < tiles) {
-        attend_rows_warp(smem, j, tmK, tmV, g, mt, grp, groups, min(groups, kArPerChunk) * tiles, ones, m, l, o);
+        attend_rows_warp<S>(smem, j, tmK, tmV, g, mt, grp, groups, min(groups, S::kPerChunk) * tiles, ones, m, l, o);
     }
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
@@ -302,14 +321,17 @@ __device__ __forceinline__ bool attend_rows_run(uint8_t *smem, const Geom &g, co
     if (!ok) {
         // copies that were issued but never consumed: give them a bounded chance to land
         if (tid == 0)
-            for (int s = 0; s < kArStages; ++s)
+            for (int s = 0; s < S::kStages; ++s)
                 if (B.issued[s] > 0) {
                     mbar_wait(&B.full[s], (uint32_t)(B.issued[s] - 1) & 1u, g.wait_ns);
                 }
         __syncthreads();
-        m_out = -INFINITY; l_out = 0.f;
 #pragma unroll
-        for (int x = 0; x < 8; ++x) acc[x] = 0.f;
+        for (int y = 0; y < S::kRows; ++y) {
+            m_out[y] = -INFINITY; l_out[y] = 0.f;
+#pragma unroll
+            for (int x = 0; x < 8; ++x) acc[y][x] = 0.f;
+        }
         return false;
     }
     // merge: state of (group, row) at [group][row][kArPitch] in the stages' memory, which nobody reads any more
@@ -325,23 +347,27 @@ __device__ __forceinline__ bool attend_rows_run(uint8_t *smem, const Geom &g, co
         if ((lane & 3) == 0) { lo[64] = m[0]; lo[65] = l[0]; hi[64] = m[1]; hi[65] = l[1]; }
     }
     __syncthreads();
-    const int r = tid >> 3, c8 = tid & 7;
-    float mw = -INFINITY, lw = 0.f;
+    const int c8 = tid & 7;
 #pragma unroll
-    for (int x = 0; x < 8; ++x) acc[x] = 0.f;
-    if (r < rows) {
-        for (int x = 0; x < groups; ++x) mw = fmaxf(mw, buf[(x * rows + r) * kArPitch + 64]);
+    for (int y = 0; y < S::kRows; ++y) {
+        const int r = (tid + y * S::kThreads) >> 3;
+        float mw = -INFINITY, lw = 0.f;
+#pragma unroll
+        for (int x = 0; x < 8; ++x) acc[y][x] = 0.f;
+        if (r < rows) {
+            for (int x = 0; x < groups; ++x) mw = fmaxf(mw, buf[(x * rows + r) * kArPitch + 64]);
 #pragma unroll 4
-        for (int x = 0; x < groups; ++x) {
-            const float *src = buf + (x * rows + r) * kArPitch;
-            const float f = src[65] > 0.f ? fast_exp2(src[64] - mw) : 0.f;
-            const float4 u = *reinterpret_cast<const float4 *>(src + 8 * c8), v = *reinterpret_cast<const float4 *>(src + 8 * c8 + 4);
-            lw += src[65] * f;
-            acc[0] = fmaf(u.x, f, acc[0]); acc[1] = fmaf(u.y, f, acc[1]); acc[2] = fmaf(u.z, f, acc[2]); acc[3] = fmaf(u.w, f, acc[3]);
-            acc[4] = fmaf(v.x, f, acc[4]); acc[5] = fmaf(v.y, f, acc[5]); acc[6] = fmaf(v.z, f, acc[6]); acc[7] = fmaf(v.w, f, acc[7]);
+            for (int x = 0; x < groups; ++x) {
+                const float *src = buf + (x * rows + r) * kArPitch;
+                const float f = src[65] > 0.f ? fast_exp2(src[64] - mw) : 0.f;
+                const float4 u = *reinterpret_cast<const float4 *>(src + 8 * c8), v = *reinterpret_cast<const float4 *>(src + 8 * c8 + 4);
+                lw += src[65] * f;
+                acc[y][0] = fmaf(u.x, f, acc[y][0]); acc[y][1] = fmaf(u.y, f, acc[y][1]); acc[y][2] = fmaf(u.z, f, acc[y][2]); acc[y][3] = fmaf(u.w, f, acc[y][3]);
+                acc[y][4] = fmaf(v.x, f, acc[y][4]); acc[y][5] = fmaf(v.y, f, acc[y][5]); acc[y][6] = fmaf(v.z, f, acc[y][6]); acc[y][7] = fmaf(v.w, f, acc[y][7]);
+            }
         }
+        m_out[y] = mw; l_out[y] = lw;
     }
-    m_out = mw; l_out = lw;
     return true;
 }
 

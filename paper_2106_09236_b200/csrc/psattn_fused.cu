@@ -26,7 +26,8 @@ namespace psattn {
 
 using namespace sm100;
 
-constexpr int kFusedThreads = 512;       // every warp measures, selects and attends
+constexpr int kFusedThreads = ArWide::kThreads;   // every warp measures, selects and attends
+constexpr size_t kFusedHalfSmem = 113 * 1024;      // two CTAs per SM (228 KB, of which 1 KB per CTA is the system's)
 
 #ifdef PSATTN_PHASE_STAMPS
 constexpr size_t kFusedMaxSmem = 226 * 1024;  // the stamps' static bytes push the dynamic memory to the next 1024-byte boundary
@@ -61,8 +62,11 @@ __host__ __device__ inline size_t fused_arrays_bytes(int m_floats, int T) { retu
 enum FusedMode { kAllSteps = 0, kGivenMeasure = 1, kGivenSet = 2 };
 constexpr int kFusedSelectKeys = kSelectMaxSlots * (kFusedThreads - 32);       // longest sequence of the block-wide selection
 
-template <bool SPLIT, int MODE>
-__global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
+// S: the shape of the CTA.  ArWide has the SM to itself.  ArHalf (256 threads, half of the shared memory) leaves room for a
+// second CTA, for more units than SMs: the chains of dependent steps of one unit (selection, query rows, merge, fill) then
+// lie under the measure or the attention of another one.
+template <bool SPLIT, int MODE, class S>
+__global__ void __launch_bounds__(S::kThreads, S::kThreads <= 256 ? 2 : 1) k_forward_fused(
     Geom g, FusedArgs a, const __nv_bfloat16 *__restrict__ Q, const __nv_bfloat16 *__restrict__ V,
     const int *__restrict__ sidx, __nv_bfloat16 *__restrict__ O, int *__restrict__ sel_out, float *__restrict__ M_out,
     const __grid_constant__ CUtensorMap tmKrows, const __grid_constant__ CUtensorMap tmK,
@@ -90,7 +94,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
     int b = (int)(blockIdx.x / split) / g.H;
     const int h = (int)(blockIdx.x / split) % g.H;
     if (!SPLIT && a.by_length) {
-        b = sequence_of_rank(g, b, kFusedThreads, &P.b_ranked);
+        b = sequence_of_rank(g, b, S::kThreads, &P.b_ranked);
     }
     const int unit = b * g.H + h;
     const int L = seq_len(g, b);
@@ -103,7 +107,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
         if (all_steps && L > 0) measure_issue_keys(smem, &P.bar, &tmKrows, L, b, h, a.pos_t, a.pos_h, g.debug_extra_tx);
         tma_prefetch_desc(&tmK); tma_prefetch_desc(&tmV);
     }
-    for (int i = tid; i < g.T; i += kFusedThreads) { chosen[i] = 0; if (all_steps && i >= L) M_s[i] = 0.f; }
+    for (int i = tid; i < g.T; i += S::kThreads) { chosen[i] = 0; if (all_steps && i >= L) M_s[i] = 0.f; }
     __syncthreads();
     phase_stamp(g, 0);
 
@@ -115,13 +119,13 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
     if (all_steps && L > 0) {
         const int per = ((L + split - 1) / split + 7) & ~7;
         const int q_lo = min(part * per, L), q_hi = min(q_lo + per, L);
-        ok = measure_resident<kFusedThreads>(smem, &P.bar, 0u, a.k_bytes, a.stage_bytes, g, unit, b, h, L, U, q_lo, q_hi,
+        ok = measure_resident<S::kThreads>(smem, &P.bar, 0u, a.k_bytes, a.stage_bytes, g, unit, b, h, L, U, q_lo, q_hi,
                                              Q, sidx, M_s);
         __syncthreads();
         if (SPLIT) {
             for (int x = 1; x < split; ++x) {
                 const uint32_t dst = peer_addr(smem_u32(M_s), part + x < split ? part + x : part + x - split);
-                for (int i = q_lo + tid; i < q_hi; i += kFusedThreads) peer_store(dst + 4u * (uint32_t)i, M_s[i]);
+                for (int i = q_lo + tid; i < q_hi; i += S::kThreads) peer_store(dst + 4u * (uint32_t)i, M_s[i]);
             }
             cluster_arrive();
             cluster_wait();
@@ -130,7 +134,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
     __syncthreads();
     phase_stamp(g, 2);                                         // steps (a)+(b) done (stamp 1: the keys had landed)
     if (all_steps && M_out != nullptr && part == 0)
-        for (int i = tid; i < g.T; i += kFusedThreads) M_out[(long long)unit * g.T + i] = M_s[i];
+        for (int i = tid; i < g.T; i += S::kThreads) M_out[(long long)unit * g.T + i] = M_s[i];
 
     // The attention phase reuses the shared memory of the measure phase, which is free now; its first
     // K/V tiles depend only on the unit, so their copies start before the selection and land behind it.
@@ -145,11 +149,11 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
     j.pos_t = a.pos_t; j.pos_h = a.pos_h; j.pos_b = a.pos_b;
     j.sum_row = a.own_v ? -1 : n_rows;
     // The last warp starts the copies (a dozen requests by one thread take about a microsecond), the others select.
-    constexpr int kSelectors = kFusedThreads - 32;
-    static_assert(kArLoader == kSelectors && kArThreads == kFusedThreads, "the last warp starts the copies");
-    const int ahead = given ? 1 : kArStages;                    // (nothing to hide the copies behind with a given set)
+    constexpr int kSelectors = S::kThreads - 32;
+    static_assert(S::kLoader == kSelectors, "the last warp starts the copies");
+    const int ahead = given ? 1 : S::kStages;                    // (nothing to hide the copies behind with a given set)
     if (tid >= kSelectors) {
-        if (ok && L > 0 && tid == kArLoader) attend_rows_start(smem, j, &tmK, &tmV, ahead);
+        if (ok && L > 0 && tid == S::kLoader) attend_rows_start<S>(smem, j, &tmK, &tmV, ahead);
     } else if (!given) {
         // ---- step (c) ---------------------------------------------------------------------------
         if (all_steps) {
@@ -178,26 +182,33 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
     // ---- step (d), with the column sums of V riding along ------------------------------------------
     // (a CTA of a cluster whose wait for the keys ran out still takes part in the barriers below)
     if (L > 0 && (ok || SPLIT)) {
-        float m_run = -INFINITY, l_run = 0.f, acc[8];
-        const int row = tid >> 3, c8 = tid & 7;
+        float m_run[S::kRows], l_run[S::kRows], acc[S::kRows][8];
+        const int c8 = tid & 7;
         if (ok) {
-            ok = attend_rows_run(smem, g, j, Q, &tmK, &tmV, ahead, m_run, l_run, acc);
+            ok = attend_rows_run<S>(smem, g, j, Q, &tmK, &tmV, ahead, m_run, l_run, acc);
         } else {
 #pragma unroll
-            for (int x = 0; x < 8; ++x) acc[x] = 0.f;
+            for (int y = 0; y < S::kRows; ++y) {
+                m_run[y] = -INFINITY; l_run[y] = 0.f;
+#pragma unroll
+                for (int x = 0; x < 8; ++x) acc[y][x] = 0.f;
+            }
         }
         if (SPLIT) {
             // every CTA leaves the states of its key range in its shared memory; CTA p then finishes the rows
             // r = p (mod split), and each CTA the fill row
             float *mine = reinterpret_cast<float *>(smem + kArOffStage + 5 * kArTile);        // behind the merge buffer
-            float *dst = mine + row * 66;
-            if (c8 == 0) { dst[0] = m_run; dst[1] = ok ? l_run : 0.f; }
 #pragma unroll
-            for (int x = 0; x < 8; x += 2) *reinterpret_cast<float2 *>(dst + 2 + 8 * c8 + x) = make_float2(acc[x], acc[x + 1]);
+            for (int y = 0; y < S::kRows; ++y) {
+                float *dst = mine + ((tid + y * S::kThreads) >> 3) * 66;
+                if (c8 == 0) { dst[0] = m_run[y]; dst[1] = ok ? l_run[y] : 0.f; }
+#pragma unroll
+                for (int x = 0; x < 8; x += 2) *reinterpret_cast<float2 *>(dst + 2 + 8 * c8 + x) = make_float2(acc[y][x], acc[y][x + 1]);
+            }
             cluster_arrive();
             cluster_wait();
             const int c = tid & 63;
-            for (int k = tid >> 6; k == 0 || part + (k - 1) * split < n_rows; k += kFusedThreads / 64) {   // 0: the fill row
+            for (int k = tid >> 6; k == 0 || part + (k - 1) * split < n_rows; k += S::kThreads / 64) {   // 0: the fill row
                 const int r = k == 0 ? j.sum_row : part + (k - 1) * split;
                 const int i = k == 0 ? 0 : P.sel[r];
                 if (r < 0 || i < 0) continue;
@@ -207,15 +218,19 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
             }
             cluster_arrive();                                   // done with the other CTAs' memory (awaited before the exit)
         } else if (ok) {
-            const float inv = l_run > 0.f ? 1.f / l_run : 0.f;
 #pragma unroll
-            for (int x = 0; x < 8; ++x) acc[x] *= inv;
-            if (row < n_rows) {
-                const int i = P.sel[row];
-                if (i >= 0) store8(O + unit_off(g.os, b, h) + (long long)i * g.os[2], c8, acc);
-            } else if (row == j.sum_row) {
+            for (int y = 0; y < S::kRows; ++y) {
+                const int row = (tid + y * S::kThreads) >> 3;
+                const float inv = l_run[y] > 0.f ? 1.f / l_run[y] : 0.f;
 #pragma unroll
-                for (int x = 0; x < 8; ++x) P.vbar[8 * c8 + x] = acc[x];      // l = number of valid keys
+                for (int x = 0; x < 8; ++x) acc[y][x] *= inv;
+                if (row < n_rows) {
+                    const int i = P.sel[row];
+                    if (i >= 0) store8(O + unit_off(g.os, b, h) + (long long)i * g.os[2], c8, acc[y]);
+                } else if (row == j.sum_row) {
+#pragma unroll
+                    for (int x = 0; x < 8; ++x) P.vbar[8 * c8 + x] = acc[y][x];       // l = number of valid keys
+                }
             }
         }
     }
@@ -231,7 +246,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) k_forward_fused(
         __nv_bfloat16 *Ou = O + unit_off(g.os, b, h);
         const __nv_bfloat16 *Vu = V + unit_off(g.vs, b, h);
         const int per = (g.T + split - 1) / split;
-        for (int i = part * per + r0; i < min(g.T, (part + 1) * per); i += kFusedThreads / 8) {
+        for (int i = part * per + r0; i < min(g.T, (part + 1) * per); i += S::kThreads / 8) {
             __nv_bfloat16 *dst = Ou + (long long)i * g.os[2];
             if (i >= L) store8(dst, sub, zero8);
             else if (chosen[i] && ok) continue;
@@ -258,13 +273,30 @@ static int fused_split(const Geom &g, int mode) {
     if (g.T < (mode == kAllSteps ? 192 : 448)) return 1;
     for (int split = kMaxSplit; split > 1; --split) {
         if (mode != kAllSteps && split < 4 && g.T < 704) return 1;
-        if (units <= max_clusters(k_forward_fused<true, kAllSteps>, clusters, split, kFusedThreads, kFusedMaxSmem)) return split;
+        if (units <= max_clusters(k_forward_fused<true, kAllSteps, ArWide>, clusters, split, kFusedThreads, kFusedMaxSmem)) return split;
     }
     return 1;
 }
 
+// Two CTAs of 256 threads per SM instead of one of 512?  More units than SMs, and selections that fit 224 threads.  us per call,
+// half / wide, lengths all T and uniform in [T / 10, T]:
+//   all steps    512 units T128 30 / 46, 25 / 42; T500 87 / 103, 53 / 71;  320 units T200 37 / 42, 21 / 34; T500 73 / 76, 42 / 47
+//                256 units T200 22 / 30, 22 / 25; T360 32 / 40, 30 / 31; T500 45 / 53, 42 / 36;  152 units T200 22 / 28, 21 / 20; T360 31 / 38, 29 / 21
+//   given set    512 units T500 33 / 44, 25 / 37;  152 units T128 7.5 / 11.7, 7.4 / 11.8
+// Up to two units per SM and ragged lengths, the wide CTAs pack long and short units and run the long ones faster: there the line
+// lies where no mix of lengths loses.
+static bool fused_half(const Geom &g, int mode) {
+    const long long units = (long long)g.B * g.H, sms = device_sm_count();
+    constexpr int kSelectors = ArHalf::kThreads - 32;
+    if (units <= sms) return false;
+    if (mode == kGivenSet) return true;
+    if (mode == kGivenMeasure) return g.T <= kSelectMaxSlots * kSelectors;
+    if (g.T > 3 * kSelectors) return false;
+    return units > 2 * sms || g.T <= 208 || (g.T <= 400 && 5 * units >= 8 * sms);
+}
+
 static size_t fused_given_smem(int T) {
-    return (kArBytes + 1023) / 1024 * 1024 + fused_arrays_bytes(0, T) + sizeof(FusedPersist) + 128;
+    return (ArWide::kBytes + 1023) / 1024 * 1024 + fused_arrays_bytes(0, T) + sizeof(FusedPersist) + 128;
 }
 
 // Host-side check with no side effect: would launch_forward_fused take this call with M~ given?
@@ -284,13 +316,24 @@ cudaError_t launch_forward_fused(const Geom &g, int U_max, int own_v, const void
     FusedArgs a;
     const int mode = sel_in != nullptr ? kGivenSet : (M_in != nullptr ? kGivenMeasure : kAllSteps);
     const bool given = mode != kAllSteps;
-    a.k_bytes = given ? 0u : (uint32_t)measure_k_bytes(g.T);
-    a.stage_bytes = given ? 0u : (uint32_t)measure_stage_bytes(kFusedThreads, g.idx_cols);
-    a.m_floats = given ? 0 : g.T;
-    size_t phase = (size_t)a.k_bytes + kMeasureStages * (size_t)a.stage_bytes;
-    if (phase < kArBytes) phase = kArBytes;
-    a.off_persist = (uint32_t)((phase + 1023) / 1024 * 1024);
-    const size_t smem = a.off_persist + fused_arrays_bytes(a.m_floats, g.T) + sizeof(FusedPersist) + 128;
+    // The shared memory of a CTA of the given shape
+    auto layout = [&](int threads, uint32_t attend_bytes) {
+        a.k_bytes = given ? 0u : (uint32_t)measure_k_bytes(g.T);
+        a.stage_bytes = given ? 0u : (uint32_t)measure_stage_bytes(threads, g.idx_cols);
+        a.m_floats = given ? 0 : g.T;
+        size_t phase = (size_t)a.k_bytes + kMeasureStages * (size_t)a.stage_bytes;
+        if (phase < attend_bytes) phase = attend_bytes;
+        a.off_persist = (uint32_t)((phase + 1023) / 1024 * 1024);
+        return a.off_persist + fused_arrays_bytes(a.m_floats, g.T) + sizeof(FusedPersist) + 128;
+    };
+    // Two CTAs per SM where there are more units than SMs and their shared memory fits twice (the keys of T up to about 510).
+    bool half = fused_half(g, mode);
+    size_t smem = 0;
+    if (half) {
+        smem = layout(ArHalf::kThreads, ArHalf::kBytes);
+        half = smem <= kFusedHalfSmem;
+    }
+    if (!half) smem = layout(ArWide::kThreads, ArWide::kBytes);
     if (smem > kFusedMaxSmem) return cudaErrorNotSupported;
     if (mode == kAllSteps && g.T > 3 * (kFusedThreads - 32)) return cudaErrorNotSupported;     // (block_select_short<3>)
     if (mode == kGivenMeasure && g.T > kFusedSelectKeys) return cudaErrorNotSupported;
@@ -307,18 +350,20 @@ cudaError_t launch_forward_fused(const Geom &g, int U_max, int own_v, const void
     a.M_in = M_in;
     // the ranking costs B comparisons per sequence in every CTA: only where a second wave exists and B is small
     a.by_length = g.lengths != nullptr && g.B * g.H > device_sm_count() && g.B <= 256;
-    using Kernel = decltype(&k_forward_fused<false, kAllSteps>);
-    static const Kernel kernels[3][2] = {{k_forward_fused<false, kAllSteps>, k_forward_fused<true, kAllSteps>},
-                                         {k_forward_fused<false, kGivenMeasure>, k_forward_fused<true, kGivenMeasure>},
-                                         {k_forward_fused<false, kGivenSet>, k_forward_fused<true, kGivenSet>}};
-    static SmemGrant grants[3][2];
-    for (int x = 0; x < 2; ++x)
-        if (cudaError_t e = grant_dynamic_smem(kernels[mode][x], grants[mode][x], kFusedMaxSmem)) return e;
+    using Kernel = decltype(&k_forward_fused<false, kAllSteps, ArWide>);
+    static const Kernel kernels[3][3] = {
+        {k_forward_fused<false, kAllSteps, ArWide>, k_forward_fused<true, kAllSteps, ArWide>, k_forward_fused<false, kAllSteps, ArHalf>},
+        {k_forward_fused<false, kGivenMeasure, ArWide>, k_forward_fused<true, kGivenMeasure, ArWide>, k_forward_fused<false, kGivenMeasure, ArHalf>},
+        {k_forward_fused<false, kGivenSet, ArWide>, k_forward_fused<true, kGivenSet, ArWide>, k_forward_fused<false, kGivenSet, ArHalf>}};
+    static SmemGrant grants[3][3];
+    for (int x = 0; x < 3; ++x)
+        if (cudaError_t e = grant_dynamic_smem(kernels[mode][x], grants[mode][x], x == 2 ? kFusedHalfSmem : kFusedMaxSmem, x == 2)) return e;
     if (cudaError_t e = grant_dynamic_smem(kernels[0][1], grants[0][1], kFusedMaxSmem)) return e;        // (asked by fused_split)
-    a.split = fused_split(g, mode);
+    a.split = half ? 1 : fused_split(g, mode);
     // launched with programmatic stream serialization: the kernel may be scheduled while the previous
     // kernel of the stream drains; it orders itself with griddepcontrol.wait before its first read
-    cudaError_t e = launch_split(kernels[mode][a.split > 1], (unsigned)(g.B * g.H), a.split, kFusedThreads, smem, st, g, a,
+    cudaError_t e = launch_split(kernels[mode][half ? 2 : a.split > 1], (unsigned)(g.B * g.H), a.split,
+                                 half ? ArHalf::kThreads : ArWide::kThreads, smem, st, g, a,
                                  (const __nv_bfloat16 *)Q, (const __nv_bfloat16 *)V, sidx, (__nv_bfloat16 *)O, sel, M_out,
                                  tmKrows, tmK, tmV);
     note_launch();
