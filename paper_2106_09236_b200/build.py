@@ -60,8 +60,21 @@ def build(force: bool = False, verbose: bool = False, phase_stamps: bool = False
     return LIB
 
 
+def native_built_for() -> bytes:
+    """What the native module is compiled against: the layout of torch's and Python's objects belongs to these versions."""
+    import sysconfig
+
+    import torch
+    return ("built for torch %s, C++11 ABI %d, %s" % (torch.__version__, int(torch._C._GLIBCXX_USE_CXX11_ABI),
+                                                      sysconfig.get_config_var("SOABI"))).encode()
+
+
 def native_needs_build() -> bool:
-    return not os.path.exists(NATIVE) or os.path.getmtime(NATIVE_SOURCE) > os.path.getmtime(NATIVE)
+    """Missing, older than its source, or compiled against another torch or Python (the module holds the text as a string)."""
+    if not os.path.exists(NATIVE) or os.path.getmtime(NATIVE_SOURCE) > os.path.getmtime(NATIVE):
+        return True
+    with open(NATIVE, "rb") as f:
+        return native_built_for() + b"\0" not in f.read()
 
 
 def build_native(verbose: bool = False) -> str:
@@ -75,7 +88,8 @@ def build_native(verbose: bool = False) -> str:
            sysconfig.get_paths()["include"], os.path.join(cuda, "include")]
     tmp = NATIVE + ".tmp.%d" % os.getpid()
     cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden",
-           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI), *["-I" + i for i in inc],
+           "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
+           '-DPSATTN_BUILT_FOR="%s"' % native_built_for().decode(), *["-I" + i for i in inc],
            NATIVE_SOURCE, "-o", tmp, "-L" + os.path.join(root, "lib"), "-ltorch_python", "-ltorch_cpu", "-lc10",
            "-lc10_cuda", "-Wl,-rpath," + os.path.join(root, "lib")]
     if verbose:

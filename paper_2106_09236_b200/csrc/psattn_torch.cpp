@@ -16,6 +16,11 @@
 
 #include <cstdint>
 
+#ifdef PSATTN_BUILT_FOR
+// read back from the file by build.py: a module compiled against another torch or Python is built again, not loaded
+extern "C" __attribute__((used)) const char psattn_built_for[] = PSATTN_BUILT_FOR;
+#endif
+
 namespace {
 
 typedef int (*fn_forward)(void *, const void *, const void *, const void *, const void *, const void *, void *, void *,
