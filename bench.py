@@ -66,12 +66,12 @@ _FUSED_SOURCES = ["psattn_fused.cu", "psattn_measure_mma.cuh", "psattn_attend_ro
 _STREAM_SOURCES = ["psattn_measure_mma.cu", "psattn_measure_stream.cuh", "psattn_measure_mma.cuh",
                    "psattn_sm100.cuh", "psattn_common.cuh"]
 TRAFFIC = {
-    "large_bf16": {"kernel": "k_forward_fused", "bytes": 53233664, "sources": _FUSED_SOURCES,
+    "large_bf16": {"kernel": "k_forward_fused", "bytes": 52913920, "sources": _FUSED_SOURCES,
                    "profile": "profiles/ncu_full_k_forward_fused_large_bf16.txt",
-                   "sources_sha1": "e1b007495ba3efae26ae30725e146e1da3accf82"},
-    "long_bf16": {"kernel": "k_measure_stream", "bytes": 74967808, "sources": _STREAM_SOURCES,
+                   "sources_sha1": "4551b1dfb39a3f91d15a10b0d3101a22ad69c050"},
+    "long_bf16": {"kernel": "k_measure_stream", "bytes": 74937344, "sources": _STREAM_SOURCES,
                   "profile": "profiles/ncu_full_k_measure_stream_long_bf16.txt",
-                  "sources_sha1": "a13c10c3f47b3db47a5c576634599e33ed45e89d"},
+                  "sources_sha1": "e5eafeb3613a091b4d268c321177f6906e7d21af"},
 }
 
 

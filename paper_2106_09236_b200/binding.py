@@ -292,7 +292,7 @@ class Plan:
         return bits.value
 
     def psattn_plan_debug_waits(self, wait_limit_ns=0, extra_expected_bytes=0):
-        """Test hook: shorten the bounded device-side waits and/or make the first TMA barrier never complete."""
+        """Test hook: shorten the bounded device-side waits and/or make a TMA barrier of the kernels never complete."""
         _check(self.lib.psattn_plan_debug_waits(self.handle, int(wait_limit_ns), int(extra_expected_bytes)), self.handle)
 
     def psattn_plan_enable_host_io(self):

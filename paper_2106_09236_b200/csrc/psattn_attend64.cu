@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(ArWide::kThreads, 1) k_attend64(Geom g, Attend
     j.rows = a.rows + (long long)unit * a.rows_stride; j.n_rows = a.n_rows;
     j.pos_t = a.pos_t; j.pos_h = a.pos_h; j.pos_b = a.pos_b;
     j.sum_row = a.vbar ? a.n_rows : -1;
-    if (tid == ArWide::kLoader) attend_rows_start<ArWide>(smem, j, &tmK, &tmV, 1);
+    if (tid == ArWide::kLoader) attend_rows_start<ArWide>(smem, g, j, &tmK, &tmV, 1);
     float m_rows[1], l_rows[1], acc_rows[1][8];
     if (!attend_rows_run<ArWide>(smem, g, j, Q, &tmK, &tmV, 1, m_rows, l_rows, acc_rows)) return;
     const float m_run = m_rows[0], l_run = l_rows[0];

@@ -64,16 +64,18 @@ struct AttendRowsBars {
     int abort_flag;
 };
 
-// One thread: the TMA copies of chunk c.
+// One thread: the TMA copies of chunk c.  (The test hook makes the last chunk wait for more bytes than are sent: with more
+// chunks than stages that is a refilled stage, and the copies of other stages are in flight when the wait runs out.)
 template <class S>
-__device__ __forceinline__ void attend_rows_load(uint8_t *smem, const AttendRowsJob &j, const CUtensorMap *tmK,
+__device__ __forceinline__ void attend_rows_load(uint8_t *smem, const Geom &g, const AttendRowsJob &j, const CUtensorMap *tmK,
                                                  const CUtensorMap *tmV, int c) {
     using namespace sm100;
     AttendRowsBars &B = *reinterpret_cast<AttendRowsBars *>(smem + S::kOffBar);
     const int s = c % S::kStages;
     B.issued[s] = c / S::kStages + 1;
     const int tiles = min(S::kChunk / 128, (j.hi - j.lo - c * S::kChunk + 127) / 128);
-    mbar_expect_tx(&B.full[s], 2 * kArTile * (uint32_t)tiles);
+    const bool last = j.hi - j.lo <= (c + 1) * S::kChunk;
+    mbar_expect_tx(&B.full[s], 2 * kArTile * (uint32_t)tiles + (last ? g.debug_extra_tx : 0u));
 #pragma unroll 1
     for (int t = 0; t < tiles; ++t) {
         const int key0 = j.lo + c * S::kChunk + t * 128;
@@ -92,8 +94,8 @@ __device__ __forceinline__ void attend_rows_load(uint8_t *smem, const AttendRows
 // behind the loads of the query rows, which otherwise queue behind the copies of all CTAs (128 of them, K and V cold:
 // 3.3 us instead of 2.1 us for the rows with three chunks ahead).
 template <class S>
-__device__ __forceinline__ void attend_rows_start(uint8_t *smem, const AttendRowsJob &j, const CUtensorMap *tmK,
-                                                  const CUtensorMap *tmV, int ahead) {
+__device__ __forceinline__ void attend_rows_start(uint8_t *smem, const Geom &g, const AttendRowsJob &j,
+                                                  const CUtensorMap *tmK, const CUtensorMap *tmV, int ahead) {
     using namespace sm100;
     AttendRowsBars &B = *reinterpret_cast<AttendRowsBars *>(smem + S::kOffBar);
     for (int s = 0; s < S::kStages; ++s) { mbar_init(&B.full[s], 1); B.left[s] = 0; B.issued[s] = 0; }
@@ -101,7 +103,7 @@ __device__ __forceinline__ void attend_rows_start(uint8_t *smem, const AttendRow
     fence_barrier_init();
     const int n_chunks = (j.hi - j.lo + S::kChunk - 1) / S::kChunk;
 #pragma unroll 1
-    for (int c = 0; c < ahead && c < n_chunks; ++c) attend_rows_load<S>(smem, j, tmK, tmV, c);
+    for (int c = 0; c < ahead && c < n_chunks; ++c) attend_rows_load<S>(smem, g, j, tmK, tmV, c);
 }
 
 // Not volatile, so that the compiler may place them; `epoch` (see ldmatrix_x4) ties them to the wait before them.
@@ -253,7 +255,7 @@ __device__ __forceinline__ void attend_rows_warp(uint8_t *smem, const AttendRows
                 if (atomicAdd(&B.left[stage], 1) == n_warps - 1) { // the last warp to leave the stage refills it
                     B.left[stage] = 0;
                     __threadfence_block();
-                    attend_rows_load<S>(smem, j, tmK, tmV, c + S::kStages);
+                    attend_rows_load<S>(smem, g, j, tmK, tmV, c + S::kStages);
                 }
             }
             __syncwarp();
@@ -288,7 +290,7 @@ __device__ __forceinline__ bool attend_rows_run(uint8_t *smem, const Geom &g, co
         if (tid == S::kLoader) {
             const int n_chunks = (j.hi - j.lo + S::kChunk - 1) / S::kChunk;
 #pragma unroll 1
-            for (int x = ahead; x < S::kStages && x < n_chunks; ++x) attend_rows_load<S>(smem, j, tmK, tmV, x);
+            for (int x = ahead; x < S::kStages && x < n_chunks; ++x) attend_rows_load<S>(smem, g, j, tmK, tmV, x);
         }
 #pragma unroll
         for (int x = 0; x < S::kRows; ++x) {

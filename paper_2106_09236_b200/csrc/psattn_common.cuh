@@ -27,8 +27,8 @@ struct Geom {
     unsigned *status;                     // device status word
     unsigned long long wait_ns;           // limit of the bounded device-side waits that take it from here (1 s unless a
                                           // test shortens it, see psattn_plan_debug_waits)
-    unsigned debug_extra_tx;              // test hook: bytes added to the first expected-bytes count of a kernel's
-                                          // first TMA barrier, so that the barrier never completes and the wait runs out
+    unsigned debug_extra_tx;              // test hook: bytes added to what a TMA barrier expects, so that it never completes
+                                          // and the wait on it runs out
 };
 
 // Programmatic dependent launch, for kernels that are launched with launch_pdl (psattn_launch.h): lets the

@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(S::kThreads, S::kThreads <= 256 ? 2 : 1) k_for
     static_assert(S::kLoader == kSelectors, "the last warp starts the copies");
     const int ahead = given ? 1 : S::kStages;                    // (nothing to hide the copies behind with a given set)
     if (tid >= kSelectors) {
-        if (ok && L > 0 && tid == S::kLoader) attend_rows_start<S>(smem, j, &tmK, &tmV, ahead);
+        if (ok && L > 0 && tid == S::kLoader) attend_rows_start<S>(smem, g, j, &tmK, &tmV, ahead);
     } else if (!given) {
         // ---- step (c) ---------------------------------------------------------------------------
         if (all_steps) {

@@ -1,9 +1,10 @@
 """A bounded device-side wait that really runs out: the kernel must set the status bit, unwind (drain its
 copies, free its TMEM) and return, and the next call on the same plan must be correct again.
 
-No invalid access is involved: through the test hook psattn_plan_debug_waits the first TMA barrier of the
+No invalid access is involved: through the test hook psattn_plan_debug_waits a TMA barrier of the
 kernel expects 16 bytes more than are ever sent, so it never completes, and the wait limit is cut from 1 s
-to 20 microseconds.  Covered: the long-row-list / dense attention kernel and the fused forward kernel."""
+to 20 microseconds.  Covered: the long-row-list / dense attention kernel, the fused forward kernel (its key barrier), and the ring of
+the attention of listed rows in every kernel that has one."""
 import time
 
 import numpy as np
@@ -71,4 +72,40 @@ def test_fused_forward_kernel_gives_up_and_recovers():
     torch.cuda.synchronize()
     assert plan.psattn_read_status() == 0
     parity.check_forward(O2.float().cpu().numpy(), sel2.cpu().numpy(), M.cpu().numpy(), inp, inp["lengths"], "bf16", c)
+    plan.close()
+
+
+# units on their own CTA, sharing a cluster of eight, two per SM; one chunk of keys, and more chunks than the ring has stages
+@pytest.mark.parametrize("mode,B,H,T", [("given set", 2, 2, 200), ("given set", 1, 2, 1700), ("given set", 37, 4, 1100),
+                                        ("given set", 38, 4, 300), ("given measure", 1, 2, 2500), ("given measure", 19, 8, 1300),
+                                        ("row list", 2, 2, 200), ("row list", 1, 2, 3000), ("row list", 37, 4, 1100)])
+def test_attention_of_listed_rows_gives_up_and_recovers(mode, B, H, T):
+    inp, dev, c = _inputs(B, H, T, 73)
+    plan = ps.Plan(B, H, T, dtype=torch.bfloat16, c=c, idx_cols=inp["sample_idx"].shape[-1])
+    q, k, v, ln, idx = (dev[x] for x in ("Q", "K", "V", "lengths", "sample_idx"))
+    rows = torch.arange(0, plan.u_max, dtype=torch.int32, device="cuda").expand(B, H, plan.u_max).contiguous()
+
+    def call():
+        if mode == "given set":
+            return plan.psattn_forward_with_selection(q, k, v, ln, rows)
+        if mode == "row list":
+            return plan.psattn_attend_rows(q, k, v, ln, rows)
+        return plan.psattn_forward(q, k, v, ln, idx)[0]
+
+    want = call()
+    torch.cuda.synchronize()
+    assert plan.psattn_read_status() == 0
+    plan.psattn_plan_debug_waits(20_000, 16)
+    t0 = time.perf_counter()
+    got = call()
+    torch.cuda.synchronize()
+    assert time.perf_counter() - t0 < 5.0
+    assert plan.psattn_read_status() & WAIT_EXPIRED
+    if mode != "row list":                                    # no row could be finished: zeros everywhere
+        assert float(got.float().abs().max()) == 0.0
+    plan.psattn_plan_debug_waits(0, 0)
+    again = call()
+    torch.cuda.synchronize()
+    assert plan.psattn_read_status() == 0
+    assert torch.equal(again, want)
     plan.close()
