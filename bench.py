@@ -69,9 +69,9 @@ TRAFFIC = {
     "large_bf16": {"kernel": "k_forward_fused", "bytes": 52913920, "sources": _FUSED_SOURCES,
                    "profile": "profiles/ncu_full_k_forward_fused_large_bf16.txt",
                    "sources_sha1": "4551b1dfb39a3f91d15a10b0d3101a22ad69c050"},
-    "long_bf16": {"kernel": "k_measure_stream", "bytes": 74937344, "sources": _STREAM_SOURCES,
+    "long_bf16": {"kernel": "k_measure_stream", "bytes": 76630528, "sources": _STREAM_SOURCES,
                   "profile": "profiles/ncu_full_k_measure_stream_long_bf16.txt",
-                  "sources_sha1": "e5eafeb3613a091b4d268c321177f6906e7d21af"},
+                  "sources_sha1": "1d064db1ba6464687590a19f6429439836b866f8"},
 }
 
 

@@ -14,6 +14,10 @@ constexpr int kMaxDevices = 64;       // device ordinals the per-device records 
 // Multiprocessors of the current device (read once per device from its attributes).
 int device_sm_count();
 
+// The driver's cuTensorMapEncodeTiled, or null.  Callers keep it in a function-local `static const`, whose initialisation
+// is safe with several threads making their first calls at once.
+void *tensor_map_encoder();
+
 // cudaFuncAttributeMaxDynamicSharedMemorySize belongs to the current device's context: one record per
 // kernel holds, per device, the size already granted there.  grant_dynamic_smem raises it when needed
 // (thread safe; `carveout`: also ask for the largest shared-memory carve-out).

@@ -163,18 +163,7 @@ typedef CUresult (*EncodeTiledFn2)(CUtensorMap *, CUtensorMapDataType, cuuint32_
 
 bool make_rows_map(CUtensorMap *map, const void *base, const Geom &g, const long long s[3], int box_rows,
                    int swizzle128, int pos[3]) {
-    static EncodeTiledFn2 enc = nullptr;
-    static bool tried = false;
-    if (!tried) {
-        tried = true;
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult qres;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &qres) == cudaSuccess &&
-            qres == cudaDriverEntryPointSuccess)
-            enc = reinterpret_cast<EncodeTiledFn2>(p);
-        else
-            cudaGetLastError();
-    }
+    static const EncodeTiledFn2 enc = reinterpret_cast<EncodeTiledFn2>(tensor_map_encoder());
     if (!enc) return false;
     struct Dim { long long size, stride; int which; } dims[3] = {{g.T, s[2], 0}, {g.H, s[1], 1}, {g.B, s[0], 2}};
     for (int x = 0; x < 3; ++x)

@@ -324,18 +324,7 @@ typedef CUresult (*EncodeTiledFnP)(CUtensorMap *, CUtensorMapDataType, cuuint32_
                                    CUtensorMapFloatOOBfill);
 
 static EncodeTiledFnP proj_encode_fn() {
-    static EncodeTiledFnP fn = nullptr;
-    static bool tried = false;
-    if (!tried) {
-        tried = true;
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult qres;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &qres) == cudaSuccess &&
-            qres == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeTiledFnP>(p);
-        else
-            cudaGetLastError();
-    }
+    static const EncodeTiledFnP fn = reinterpret_cast<EncodeTiledFnP>(tensor_map_encoder());
     return fn;
 }
 

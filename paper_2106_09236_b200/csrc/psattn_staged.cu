@@ -425,6 +425,13 @@ int device_sm_count() {
     return n;
 }
 
+void *tensor_map_encoder() {
+    void *p = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &found) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    return found == cudaDriverEntryPointSuccess ? p : nullptr;
+}
+
 cudaError_t grant_dynamic_smem_impl(const void *kernel, SmemGrant &rec, size_t smem, bool carveout) {
     static std::mutex mu;
     int dev = 0;
