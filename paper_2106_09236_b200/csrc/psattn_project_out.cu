@@ -339,7 +339,11 @@ cudaError_t launch_project_out(int dtype, int mode, int zero_pad, const Geom &g,
     const int sms = device_sm_count();
     const long long dense_tiles = (long long)g.B * ((g.T + 127) / 128) * ((dy + 191) / 192);
     const bool dense = mode == 0 && dtype == 0 && dy % 64 == 0 && dense_tiles <= (g.H >= 8 ? 3ll : 1ll) * sms;
-    if (dtype == 0 && mode == 0 && !dense && sel != nullptr && g.u_max <= kPoMaxRows && g.H <= 32 && dy % 8 == 0) {
+    if (dense) {                          // it has no tensor map for some layouts (a stride of 0), which the shortcut takes
+        cudaError_t e = launch_project_out_dense(g, zero_pad, dy, O, Wot, Y, st);
+        if (e != cudaErrorNotSupported) return e;
+    }
+    if (dtype == 0 && mode == 0 && sel != nullptr && g.u_max <= kPoMaxRows && g.H <= 32 && dy % 8 == 0) {
         const int slices = (dy + kPoCols - 1) / kPoCols;
         // ranges of positions: about one CTA per SM (every CTA loads its weight slice once), 256 .. 1024 positions each
         int chunks = sms / (slices * g.B);
@@ -367,7 +371,7 @@ cudaError_t launch_project_out(int dtype, int mode, int zero_pad, const Geom &g,
             return e != cudaSuccess ? e : cudaGetLastError();
         }
     }
-    if (dtype == 0 && mode != 2) {
+    if (dtype == 0 && mode != 2 && !dense) {
         cudaError_t e = launch_project_out_dense(g, zero_pad, dy, O, Wot, Y, st);
         if (e != cudaErrorNotSupported) return e;
     }

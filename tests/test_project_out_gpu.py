@@ -9,6 +9,7 @@ import numpy as np
 import pytest
 import torch
 
+from kernels import launched
 from oracle import psattn_oracle as orc
 from paper_2106_09236_b200 import binding as ps
 from paper_2106_09236_b200 import workloads as wl
@@ -147,6 +148,30 @@ def test_own_value_fill_takes_the_dense_product():
     inp = wl.make_inputs(wk, n_cols, seed=66, lengths=[256, 100])
     plan, O, sel, lengths, tdt = _forward(inp, "bf16", c, fill_mode=ps.PSATTN_FILL_OWN_V)
     _run_all_forms(plan, O, sel, lengths, _weights(H, 256, 10, "bf16"), tdt, "bf16", inp["lengths"], forms=("shortcut",))
+    plan.close()
+
+
+@pytest.mark.parametrize("B", [1, 2])
+def test_output_matrix_of_an_o_with_a_stride_of_zero(B):
+    """No tensor map describes such a layout (one O for all sequences, or an unused batch stride left at 0), so the dense product
+    refuses it: the corrections form takes the call, not the kernel with one thread per element."""
+    H, T, c, dy = 8, 300, 5.0, 512
+    n_cols = orc.count(c, T)
+    wk = wl.Workload("adhoc", 0, 1, H, T, 64, "bf16", c, 0.1, 3.0)
+    inp = wl.make_inputs(wk, n_cols, seed=67, lengths=[T - 5])
+    first, O, sel, _, tdt = _forward(inp, "bf16", c)
+    first.close()
+    plan = ps.Plan(B, H, T, dtype=tdt, c=c, idx_cols=n_cols, strides={"o": (0, T * 64, 64)})
+    Wot_np = _weights(H, dy, 11, "bf16")
+    Wot = torch.from_numpy(Wot_np).to("cuda", tdt)
+    lengths = torch.full((B,), T - 5, dtype=torch.int32, device="cuda")
+    Y = torch.full((B, T, dy), 7.0, dtype=tdt, device="cuda")
+    sels = sel.expand(B, H, plan.u_max).contiguous()
+    _, ran = launched(lambda: plan.psattn_project_out(O, sels, lengths, Wot, Y))
+    assert ran == {"k_project_out_rows"}
+    ref = orc.project_out(O.float().cpu().numpy(), Wot_np, inp["lengths"], nthreads=8)
+    _check(Y, np.repeat(ref, B, axis=0), [T - 5] * B, "bf16", 7.0)
+    assert plan.psattn_read_status() == 0
     plan.close()
 
 
