@@ -172,12 +172,33 @@ __device__ __forceinline__ void attend_rows_warp(uint8_t *smem, const AttendRows
     const uint32_t v_lane = S::kOffV + (uint32_t)(l7 + 8 * ((lane >> 3) & 1)) * 128u + ((uint32_t)((lane >> 4) ^ l7) << 4);
     float2 l0 = make_float2(0.f, 0.f), l1 = l0;
     int c = -1, stage = -1, in_chunk = grp + S::kPerChunk;      // chunk, its stage, block inside it (normalised at the top)
+    // Every warp passes every chunk in order, also one that holds no block of its group (one row tile: more groups than blocks per
+    // chunk): a wait tells the two phases of a stage's barrier apart by parity only, so no warp may be two phases ahead of it, and a
+    // stage is refilled when all warps have left it.
 #pragma unroll 1
-    for (int i = grp; i < n_blocks; i += groups, in_chunk += groups) {
-        if (in_chunk >= S::kPerChunk) {                         // on to another chunk
-            do { in_chunk -= S::kPerChunk; ++c; stage = stage == S::kStages - 1 ? 0 : stage + 1; } while (in_chunk >= S::kPerChunk);
+    for (int i = grp;; i += groups, in_chunk += groups) {
+        while (in_chunk >= S::kPerChunk) {                      // on to the next chunk
+            if (c >= 0 && c + S::kStages < n_chunks) {
+#pragma unroll
+                for (int x = 0; x < 8; ++x)                    // the fragments of the chunk have been read
+                    asm volatile("" : "+f"(o[x][0]), "+f"(o[x][1]), "+f"(o[x][2]), "+f"(o[x][3]) :: "memory");
+                __syncwarp();
+                if (lane == 0) {
+                    __threadfence_block();
+                    if (atomicAdd(&B.left[stage], 1) == n_warps - 1) { // the last warp to leave the stage refills it
+                        B.left[stage] = 0;
+                        __threadfence_block();
+                        attend_rows_load<S>(smem, g, j, tmK, tmV, c + S::kStages);
+                    }
+                }
+                __syncwarp();
+            }
+            in_chunk -= S::kPerChunk;
+            if (++c >= n_chunks) break;
+            stage = stage == S::kStages - 1 ? 0 : stage + 1;
             if (!arrived(c)) return;
         }
+        if (i >= n_blocks) break;
         asm volatile("mov.u32 %0, %1;" : "=r"(epoch) : "r"(i) : "memory");
         const uint32_t at = base + (uint32_t)stage * S::kStageBytes + (uint32_t)in_chunk * (kArBlock * 128u);
         const int left = n_keys - i * kArBlock;                // keys from the block's first on
@@ -248,18 +269,6 @@ __device__ __forceinline__ void attend_rows_warp(uint8_t *smem, const AttendRows
             mma_bf16_16816(o[2 * d], p[2][0], p[2][1], p[3][0], p[3][1], w[0], w[1]);
             mma_bf16_16816(o[2 * d + 1], p[2][0], p[2][1], p[3][0], p[3][1], w[2], w[3]);
         }
-        if (in_chunk + groups >= S::kPerChunk && c + S::kStages < n_chunks) {
-            __syncwarp();                                      // every lane has read its fragments
-            if (lane == 0) {
-                __threadfence_block();
-                if (atomicAdd(&B.left[stage], 1) == n_warps - 1) { // the last warp to leave the stage refills it
-                    B.left[stage] = 0;
-                    __threadfence_block();
-                    attend_rows_load<S>(smem, g, j, tmK, tmV, c + S::kStages);
-                }
-            }
-            __syncwarp();
-        }
     }
     l[0] = l0.x + l0.y; l[1] = l1.x + l1.y;
 }
@@ -310,7 +319,7 @@ __device__ __forceinline__ bool attend_rows_run(uint8_t *smem, const Geom &g, co
 #pragma unroll
         for (int e = 0; e < 4; ++e) o[x][e] = 0.f;
     if (mt < tiles) {
-        attend_rows_warp<S>(smem, j, tmK, tmV, g, mt, grp, groups, min(groups, S::kPerChunk) * tiles, ones, m, l, o);
+        attend_rows_warp<S>(smem, j, tmK, tmV, g, mt, grp, groups, groups * tiles, ones, m, l, o);
     }
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
