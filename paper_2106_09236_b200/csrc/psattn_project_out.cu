@@ -321,7 +321,25 @@ __global__ void __launch_bounds__(128) k_project_out_simt(OutArgs a, const DT *_
 
 cudaError_t launch_project_out_dense(const Geom &g, int zero_pad, int dy, const void *O, const void *Wot, void *Y, cudaStream_t st);
 
-// mode 0: pick (shortcut when an index set is given and the shape fits, else the dense GEMM, else one thread
+// Is the shortcut faster than the dense product?  The shortcut reads less, but its CTAs are alone on their SMs and chains of
+// dependent steps, so a second wave of them costs as much as the first; the dense tiles hide their starts behind one another.  Both
+// are estimated in us (constants fitted to 366 measured shapes: H 1 .. 8, d_y 64 .. 512, T 64 .. 8192, c 2 .. 6, lengths all T and
+// uniform from T / 10 on; 0.3 % above the better form on average, 16 % at worst):
+//   shortcut  waves of its CTAs, each a start, its positions' rows of Y, and the products of the selected rows among them
+//   dense     a start, and the tiles of the SM with most of them
+// us, shortcut / dense, d_y = 64 H: few picks per position, one wave: B2 H8 T8192 11.4 / 14.8, B4 H4 T8192 10.2 / 15.8, B32 H4 T1024
+// 12.9 / 15.8; more picks: B16 H8 T1024 16.2 / 14.9; several waves of short sequences: B148 H8 T128 89 / 15, B64 H4 T300 17.7 / 12.6,
+// B64 H8 T1024 61 / 43; about equal: B8 H8 T8192 42.0 / 42.7, B64 H4 T1024 24.2 / 24.7.
+static bool rows_pay(const Geom &g, long long ctas, int t_chunk, int dy, int sms) {
+    const long long tiles = (long long)g.B * ((g.T + 127) / 128) * ((dy + 191) / 192);
+    const int positions = g.T < t_chunk ? g.T : t_chunk;
+    const double picks = (double)g.H * g.u_max * positions / g.T;
+    const double rows_us = (double)((ctas + sms - 1) / sms) * (5.0 + 0.3 * g.H + 0.003 * positions + 0.02 * picks);
+    const double dense_us = 3.3 + 0.15 * g.H + (double)((tiles + sms - 1) / sms) * (2.0 + 0.2 * g.H);
+    return rows_us < dense_us;
+}
+
+// mode 0: pick (shortcut when an index set is given, the shape fits and it pays, else the dense GEMM, else one thread
 // per element); 1: never the shortcut; 2: one thread per element.
 cudaError_t launch_project_out(int dtype, int mode, int zero_pad, const Geom &g, int dy, const void *O, const int *sel,
                                const void *Wot, void *Y, cudaStream_t st) {
@@ -332,21 +350,16 @@ cudaError_t launch_project_out(int dtype, int mode, int zero_pad, const Geom &g,
     a.O = (const __nv_bfloat16 *)O; a.Wot = (const __nv_bfloat16 *)Wot; a.Y = (__nv_bfloat16 *)Y;
     a.sel = sel; a.lengths = g.lengths; a.status = g.status; a.zero_pad = zero_pad;
     a.t_chunk = 0; a.max_slots = 0; a.max_pairs = 0;
-    // The dense product runs at the tensor cores' rate; the shortcut reads less but is a chain of dependent steps.  Where the
-    // dense product is at most one tile per SM (or three, with 512 columns and more to sum over, whose tiles hide their starts), it
-    // is the faster one.  us, shortcut / dense: B1 H4 T300 8.1 / 6.2, B2 H8 T3000 9.1 / 7.7, B16 H8 T1024 14.8 / 13.8, but
-    // B32 H4 T700 10.2 / 12.3.
     const int sms = device_sm_count();
-    const long long dense_tiles = (long long)g.B * ((g.T + 127) / 128) * ((dy + 191) / 192);
-    const bool dense = mode == 0 && dtype == 0 && dy % 64 == 0 && dense_tiles <= (g.H >= 8 ? 3ll : 1ll) * sms;
-    if (dense) {                          // it has no tensor map for some layouts (a stride of 0), which the shortcut takes
-        cudaError_t e = launch_project_out_dense(g, zero_pad, dy, O, Wot, Y, st);
-        if (e != cudaErrorNotSupported) return e;
-    }
-    if (dtype == 0 && mode == 0 && sel != nullptr && g.u_max <= kPoMaxRows && g.H <= 32 && dy % 8 == 0) {
-        const int slices = (dy + kPoCols - 1) / kPoCols;
+    // the shortcut's launch
+    bool rows_fit = dtype == 0 && mode == 0 && sel != nullptr && g.u_max <= kPoMaxRows && g.H <= 32 && dy % 8 == 0 && g.B <= 65535;
+    bool rows = false;
+    const int slices = (dy + kPoCols - 1) / kPoCols;
+    int chunks = 1;
+    size_t smem = 0;
+    if (rows_fit) {
         // ranges of positions: about one CTA per SM (every CTA loads its weight slice once), 256 .. 1024 positions each
-        int chunks = sms / (slices * g.B);
+        chunks = (int)(sms / ((long long)slices * g.B));
         if (chunks < 1) chunks = 1;
         int t_chunk = (g.T + chunks - 1) / chunks;
         t_chunk = ((t_chunk + 63) / 64) * 64;
@@ -357,23 +370,25 @@ cudaError_t launch_project_out(int dtype, int mode, int zero_pad, const Geom &g,
         a.max_slots = g.H * g.u_max < t_chunk ? g.H * g.u_max : t_chunk;
         a.max_pairs = g.H * ((g.u_max + 15) / 16 * 16);         // every head's rows padded to whole 16-row tiles
         // the kernel's layout: weights, fill rows, c, base, pair positions, slot positions, pair_of | slot_of | P
-        size_t smem = (size_t)kPoCols * po_w_pitch(g.H) + (size_t)g.H * 64 * 2 + (size_t)g.H * 64 * 4 + 64 * 4 +
-                      (size_t)a.max_pairs * 4 + (size_t)a.max_slots * 4;
+        smem = (size_t)kPoCols * po_w_pitch(g.H) + (size_t)g.H * 64 * 2 + (size_t)g.H * 64 * 4 + 64 * 4 +
+               (size_t)a.max_pairs * 4 + (size_t)a.max_slots * 4;
         smem = po_align16(smem + (size_t)g.H * a.max_slots * 2);
         smem = po_align16(smem + (size_t)t_chunk * 2);
         smem += (size_t)a.max_pairs * 64 * 4 + 128;
-        if (smem <= 200 * 1024 && chunks <= 65535 && g.B <= 65535) {
-            static SmemGrant grant;
-            if (cudaError_t e = grant_dynamic_smem(k_project_out_rows, grant, smem)) return e;
-            cudaError_t e = launch_pdl(k_project_out_rows, dim3((unsigned)slices, (unsigned)chunks, (unsigned)g.B),
-                                       dim3(kPoThreads), smem, st, a);
-            note_launch();
-            return e != cudaSuccess ? e : cudaGetLastError();
-        }
+        rows_fit = smem <= 200 * 1024 && chunks <= 65535;
+        rows = rows_fit && (dy % 64 != 0 || rows_pay(g, (long long)slices * chunks * g.B, t_chunk, dy, sms));
     }
-    if (dtype == 0 && mode != 2 && !dense) {
+    if (dtype == 0 && mode != 2 && !rows) {
         cudaError_t e = launch_project_out_dense(g, zero_pad, dy, O, Wot, Y, st);
-        if (e != cudaErrorNotSupported) return e;
+        if (e != cudaErrorNotSupported) return e;               // no tensor map for some layouts (a stride of 0)
+    }
+    if (rows_fit) {
+        static SmemGrant grant;
+        if (cudaError_t e = grant_dynamic_smem(k_project_out_rows, grant, smem)) return e;
+        cudaError_t e = launch_pdl(k_project_out_rows, dim3((unsigned)slices, (unsigned)chunks, (unsigned)g.B),
+                                   dim3(kPoThreads), smem, st, a);
+        note_launch();
+        return e != cudaSuccess ? e : cudaGetLastError();
     }
     if (g.T > 65535 || g.B > 65535) return cudaErrorNotSupported;
     const dim3 grid((unsigned)((dy + 127) / 128), (unsigned)g.T, (unsigned)g.B);

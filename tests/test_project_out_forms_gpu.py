@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 import torch
 
+from kernels import launched
 from oracle import psattn_oracle as orc
 from paper_2106_09236_b200 import binding as ps
 from paper_2106_09236_b200 import workloads as wl
@@ -33,4 +34,29 @@ def test_output_matrix_forms(B, H, T, dy, longest):
         assert np.isnan(got[b, L:]).all()
         err = np.abs(got[b, :L] - want[b, :L])
         assert (err <= 2.0 ** -8 * np.abs(want[b, :L]) + 1e-3).all()
+    plan.close()
+
+
+# one wave of long ranges with few picks; many picks; several waves of short sequences; a second wave; widths beside 64
+@pytest.mark.parametrize("B,H,T,dy,corrections", [
+    (2, 8, 8192, 512, True), (1, 8, 8191, 512, True), (32, 4, 1024, 256, True), (32, 8, 1024, 256, True), (16, 8, 1024, 512, False),
+    (148, 8, 128, 512, False), (64, 4, 300, 256, False), (24, 8, 1024, 512, False), (1, 1, 64, 64, False), (3, 8, 700, 520, True),
+])
+def test_output_matrix_form_by_size(B, H, T, dy, corrections):
+    """Which form a call with an index set takes, and that it agrees with the dense product of the same call without one."""
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(B * T)
+    plan = ps.Plan(B, H, T, c=5.0)
+    q, k, v = (torch.randn((B, H, T, 64), generator=gen, device="cuda").bfloat16() for _ in range(3))
+    ln = torch.randint(1, T + 1, (B,), generator=gen, device="cuda", dtype=torch.int32)
+    ln[0] = T
+    idx = (torch.rand((B, T, plan.idx_cols), generator=gen, device="cuda") * ln.view(B, 1, 1)).int()
+    O, sel = plan.psattn_forward(q, k, v, ln, idx)
+    Wot = (torch.randn((dy, H * 64), generator=gen, device="cuda") / 16).bfloat16()
+    Y, ran = launched(lambda: plan.psattn_project_out(O, sel, ln, Wot))
+    assert ran == {"k_project_out_rows" if corrections else "k_project_qkv"}
+    want = O.permute(0, 2, 1, 3).reshape(B, T, H * 64).double() @ Wot.double().T       # O is zero at padded positions
+    err = (Y.double() - want).abs()
+    assert bool((err <= 2.0 ** -8 * want.abs() + 1e-3).all())
+    assert plan.psattn_read_status() == 0
     plan.close()
