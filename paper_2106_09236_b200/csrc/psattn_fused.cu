@@ -278,21 +278,28 @@ static int fused_split(const Geom &g, int mode) {
     return 1;
 }
 
-// Two CTAs of 256 threads per SM instead of one of 512?  More units than SMs, and selections that fit 224 threads.  us per call,
-// half / wide, lengths all T and uniform in [T / 10, T]:
-//   all steps    512 units T128 30 / 46, 25 / 42; T500 87 / 103, 53 / 71;  320 units T200 37 / 42, 21 / 34; T500 73 / 76, 42 / 47
-//                256 units T200 22 / 30, 22 / 25; T360 32 / 40, 30 / 31; T500 45 / 53, 42 / 36;  152 units T200 22 / 28, 21 / 20; T360 31 / 38, 29 / 21
-//   given set    512 units T500 33 / 44, 25 / 37;  152 units T128 7.5 / 11.7, 7.4 / 11.8
-// Up to two units per SM and ragged lengths, the wide CTAs pack long and short units and run the long ones faster: there the line
-// lies where no mix of lengths loses.
+// Two CTAs of 256 threads per SM instead of one of 512?  More units than SMs, and selections that fit 224 threads.  Two per SM hide
+// one unit's chains under the other's work, but take a unit longer, which shows where the long units of a ragged batch end last,
+// and they run in waves of 2 sms units where the wide ones run in waves of sms: between two and three units per SM that is four
+// unit times against three.  The lengths are not known here, so the line lies where the worse of the losses, over lengths all T and
+// uniform from T / 2 and from T / 10 on, is the smaller one (with all steps and up to two units per SM: where none loses).
+// us per call, half / wide, lengths all T and from T / 10:
+//   all steps    152 units T128 22 / 28, 21 / 20; T360 31 / 38, 29 / 21    256 units T200 22 / 30, 22 / 25; T360 32 / 40, 30 / 31; T500 45 / 53, 42 / 36
+//                304 units T500 73 / 75, 42 / 47    440 units T128 30 / 36, 24 / 32; T500 84 / 79, 47 / 56    512 units T128 31 / 46, 25 / 42; T500 86 / 103, 53 / 70
+//   given set    152 units T128 6.9 / 10.9, 6.8 / 10.9; T1024 25.7 / 29.1, 21.6 / 20.0; T1536 35.5 / 38.0, 28.6 / 23.9; T4096 82 / 85, 64 / 48
+//                240 units T1024 28 / 33, 25 / 26; T1536 38 / 42, 33 / 33; T2048 48 / 51, 42 / 40
+//                440 units T1024 53 / 52, 38 / 41; T1536 71 / 65, 48 / 51; T4096 161 / 139, 100 / 98    512 units T4096 169 / 176, 115 / 123
+//   given measure (with the measure kernel before it)
+//                152 units T1152 96 / 100, 68 / 60; T4000 297 / 299, 219 / 181    240 units T1152 123 / 128, 88 / 86; T1536 161 / 167, 109 / 106; T2048 216 / 220, 148 / 141
+//                440 units T1152 215 / 216, 128 / 136; T3000 594 / 589, 349 / 349    512 units T1152 239 / 256, 144 / 160; T2048 436 / 446, 259 / 273
 static bool fused_half(const Geom &g, int mode) {
     const long long units = (long long)g.B * g.H, sms = device_sm_count();
     constexpr int kSelectors = ArHalf::kThreads - 32;
     if (units <= sms) return false;
-    if (mode == kGivenSet) return true;
-    if (mode == kGivenMeasure) return g.T <= kSelectMaxSlots * kSelectors;
-    if (g.T > 3 * kSelectors) return false;
-    return units > 2 * sms || g.T <= 208 || (g.T <= 400 && 5 * units >= 8 * sms);
+    if (mode == kAllSteps) return g.T <= 3 * kSelectors && (units > 2 * sms || g.T <= 208 || (g.T <= 400 && 5 * units >= 8 * sms));
+    if (mode == kGivenMeasure && g.T > kSelectMaxSlots * kSelectors) return false;
+    const bool many = mode == kGivenSet ? 3 * units >= 4 * sms : 5 * units >= 8 * sms;
+    return units > 3 * sms || g.T <= (many ? 1536 : 1024);
 }
 
 static size_t fused_given_smem(int T) {
