@@ -41,7 +41,6 @@ constexpr uint32_t kOffQ = 0, kOffK = 2 * kTileBytes, kOffV = kOffK + kTcStages 
                    kOffBar = kOffP + 4 * kTileBytes;
 constexpr uint32_t kAttendSmem = kOffBar + 256;
 static_assert(kAttendSmem <= 227 * 1024, "the CTA's tiles must fit the shared memory of one SM");
-static_assert(kAttendSmem <= 227 * 1024, "the CTA's tiles must fit the shared memory of one SM");
 constexpr bool kTakeTurns = true;                            // the softmax warpgroups alternate on the exponential unit
 constexpr float kRefSlack = 8.f;                             // the reference follows the row maximum in steps of 2^8
 

@@ -74,7 +74,7 @@ __host__ __device__ inline size_t measure_k_bytes(int T) {
 }
 // Words per staged sample row.  A round reads two neighbouring words of eight rows at once: with a multiple of eight words
 // per row these fall into one to four banks (32 words, T = 493 .. 601 at c = 5: all eight rows in one; B32 H4 T512
-// 28.8 us against 25.6 with the rows 36 words apart).
+// 29.0 us against 26.4 with the rows 36 words apart).
 __host__ __device__ inline int measure_idx_pitch(int idx_cols) { return idx_cols % 8 == 0 ? idx_cols + 4 : idx_cols; }
 // Sample rows of a warp's queries into its staging buffer (all lanes; cp.async, not committed).
 __device__ __forceinline__ void measure_stage_samples(uint32_t dst, const int *src, int rows, int idx_cols) {

@@ -168,8 +168,10 @@ __device__ __forceinline__ void measure_stream_group(const StreamCtx &cx) {
 // ---------------------------------------------------------------------------------------------
 // How the work is split: the groups of eight queries of all sequences and heads, in order, each weighing its rounds (plus a
 // few for its start), are cut into one range of equal weight per CTA (one CTA per SM), and the warps of a CTA take
-// the groups of its range in turn.  With a fixed number of query ranges per unit the ragged batch (B6 H8, lengths
-// 1050..3001) left most SMs idle behind the longest units: 64 us, where the gathers alone need 28.
+// the groups of its range in turn.  us, a fixed number of query ranges per unit / this split (the gathers alone, at 17.6 TB/s):
+// B6 H8, lengths 1050..3001 55 / 47 (about 30), B16 H8 T2048 102 / 91 (74), B8 H8 T4096 104 / 94 (80), B3 H8 T8192 79 / 75.5 (66).
+// Where fixed ranges happened to fit, it costs: B4 H8 T8192 97.7 / 101.1 (88), B1 H8 T32768 109.0 / 111.6 (99).  A range of
+// 221 groups for 24 warps ends in a pass with 5 of them, at the latency of a whole group, on all SMs at once.
 // ---------------------------------------------------------------------------------------------
 constexpr int kStreamMaxB = 2048;                               // sequences per launch (their weights sit in shared memory)
 
