@@ -12,7 +12,7 @@ from test_parity_gpu import _dev, _synth
 
 pytestmark = pytest.mark.gpu
 
-CASES = {"fused": (4, 8, 1024, 1), "staged": (2, 8, 3000, 2), "short": (16, 4, 300, 3)}
+CASES = {"fused": (4, 8, 1024, 1), "staged": (1, 4, 9000, 2), "short": (16, 4, 300, 3)}
 
 
 def _work(name, out, repeats):

@@ -7,6 +7,7 @@ import pytest
 import torch
 
 import parity
+from kernels import launched
 from oracle import psattn_oracle as orc
 from paper_2106_09236_b200 import binding as ps
 from paper_2106_09236_b200 import workloads as wl
@@ -249,10 +250,12 @@ def test_workspace_contents_do_not_matter_and_its_bounds_are_kept(dtype, T, path
     plan.close()
 
 
-@pytest.mark.parametrize("dtype,T", [("bf16", 300), ("bf16", 1500), ("fp32", 200)])
-def test_forward_inside_a_cuda_graph_matches_the_direct_call(dtype, T):
-    """The call may fork work onto the plan's side stream and uses programmatic dependent launches: a stream
-    capture has to follow all of it, and a replay on new input values has to give what a direct call gives."""
+@pytest.mark.parametrize("dtype,T,forks", [("bf16", 300, False), ("bf16", 1500, False), ("fp32", 200, False), ("bf16", 9000, True),
+                                           ("fp32", 2500, True)])
+def test_forward_inside_a_cuda_graph_matches_the_direct_call(dtype, T, forks):
+    """The call may fork work onto the plan's side stream (the fill, where the steps are kernels of their own) and uses
+    programmatic dependent launches: a stream capture has to follow all of it, and a replay on new input values has to
+    give what a direct call gives."""
     B, H, c = 3, 2, 5.0
     n = max(orc.count(c, L) for L in range(1, T + 1))
     lengths = [T, T // 2, T - 3]
@@ -287,6 +290,7 @@ def test_forward_inside_a_cuda_graph_matches_the_direct_call(dtype, T):
     np.testing.assert_array_equal(O.float().cpu().numpy(), want[0])
     np.testing.assert_array_equal(sel.cpu().numpy(), want[1])
     np.testing.assert_array_equal(M.cpu().numpy(), want[2])
+    assert ("k_fill" in launched(call)[1]) == forks
     plan.close()
 
 
@@ -624,19 +628,23 @@ def test_dense_comparator(dtype):
     plan.close()
 
 
-def test_host_buffer_front_end():
-    w = wl.WORKLOADS["ragged_bf16"]
+# one chunk (less than 8 MB to copy in), three quarters and one quarter, one and one of two kernels each
+@pytest.mark.parametrize("name,B", [("ragged_bf16", 4), ("ragged_bf16", 13), ("long_bf16", 2)])
+def test_host_buffer_front_end(name, B):
+    w = wl.WORKLOADS[name]
     n = max(orc.count(w.c, L) for L in range(1, w.T + 1))
-    inp = wl.make_inputs(w, n, B=4)
+    inp = wl.make_inputs(w, n, B=B)
     tdt = torch.bfloat16
-    plan = ps.Plan(4, w.H, w.T, dtype=tdt, c=w.c, idx_cols=n)
+    plan = ps.Plan(B, w.H, w.T, dtype=tdt, c=w.c, idx_cols=n)
     plan.psattn_plan_enable_host_io()
     hQ, hK, hV = (torch.from_numpy(inp[k]).to(tdt).pin_memory() for k in ("Q", "K", "V"))
     hl = torch.from_numpy(inp["lengths"]).pin_memory()
     hi = torch.from_numpy(inp["sample_idx"]).pin_memory()
-    hO = torch.empty((4, w.H, w.T, 64), dtype=tdt).pin_memory()
-    hs = torch.empty((4, w.H, plan.u_max), dtype=torch.int32).pin_memory()
+    hO = torch.empty((B, w.H, w.T, 64), dtype=tdt).pin_memory()
+    hs = torch.empty((B, w.H, plan.u_max), dtype=torch.int32).pin_memory()
+    launches = ps.psattn_launch_count()
     plan.psattn_forward_host(hQ, hK, hV, hl, hi, hO, hs)
+    assert ps.psattn_launch_count() - launches == {4: 1, 13: 2, 2: 4}[B]
     parity.check_forward(hO.float().numpy(), hs.numpy(), None, inp, inp["lengths"], "bf16", w.c)
     plan.close()
 

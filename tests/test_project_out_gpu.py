@@ -49,6 +49,7 @@ def _run_all_forms(plan, O, sel, lengths, Wot_np, tdt, dtype, inp_lengths, forms
     Wot = torch.from_numpy(Wot_np).to("cuda", tdt)
     ref = orc.project_out(O.float().cpu().numpy(), Wot_np, inp_lengths, nthreads=8)
     sentinel = 7.0
+    ran = {}
     for form in forms:
         Y = torch.full((B, T, dy), sentinel, dtype=tdt, device="cuda")
         before = ps.psattn_launch_count()
@@ -57,6 +58,8 @@ def _run_all_forms(plan, O, sel, lengths, Wot_np, tdt, dtype, inp_lengths, forms
         assert ps.psattn_launch_count() == before + 1
         assert plan.psattn_read_status() == 0
         _check(Y, ref, inp_lengths, dtype, sentinel)
+        ran[form], = launched(lambda: plan.psattn_project_out(O, sel if form == "shortcut" else None, lengths, Wot, Y))[1]
+    return ran                                               # kernel by form: with an index set the call takes the faster one
 
 
 @pytest.mark.parametrize("name,nb", [("ragged_bf16", None), ("large_bf16", None), ("long_bf16", 1)])
@@ -65,7 +68,11 @@ def test_output_matrix_on_workloads(name, nb):
     n_cols = max(orc.count(w.c, L) for L in range(1, w.T + 1))
     inp = wl.make_inputs(w, n_cols, B=nb)
     plan, O, sel, lengths, tdt = _forward(inp, w.dtype, w.c)
-    _run_all_forms(plan, O, sel, lengths, _weights(w.H, w.H * 64, 5, w.dtype), tdt, w.dtype, inp["lengths"])
+    ran = _run_all_forms(plan, O, sel, lengths, _weights(w.H, w.H * 64, 5, w.dtype), tdt, w.dtype, inp["lengths"])
+    assert ran["dense"] == "k_project_qkv"
+    # a width that the dense tiles do not take: the corrections
+    ran = _run_all_forms(plan, O, sel, lengths, _weights(w.H, w.H * 64 + 8, 5, w.dtype), tdt, w.dtype, inp["lengths"], forms=("shortcut",))
+    assert ran["shortcut"] == "k_project_out_rows"
     plan.close()
 
 
@@ -82,8 +89,9 @@ def test_output_matrix_odd_widths_short_sequences_and_full_selection(dy):
     s = sel.cpu().numpy()
     assert (s[2, :, :3] >= 0).all()                          # length 3: all three rows selected in every head
     shared = set(s[0, 0][s[0, 0] >= 0]) & set(s[0, 1][s[0, 1] >= 0])
-    _run_all_forms(plan, O, sel, lens, _weights(H, dy, 6, "bf16"), tdt, "bf16", inp["lengths"])
-    assert len(shared) >= 0
+    ran = _run_all_forms(plan, O, sel, lens, _weights(H, dy, 6, "bf16"), tdt, "bf16", inp["lengths"])
+    assert ran["shortcut"] == ("k_project_out_rows" if dy % 64 else "k_project_qkv")
+    assert shared
     plan.close()
 
 
@@ -98,6 +106,8 @@ def test_output_matrix_with_odd_head_counts(H, T):
     inp = wl.make_inputs(wk, n_cols, seed=64 + H, lengths=lengths)
     plan, O, sel, lens, tdt = _forward(inp, "bf16", c)
     _run_all_forms(plan, O, sel, lens, _weights(H, 256, 8, "bf16"), tdt, "bf16", inp["lengths"])
+    ran = _run_all_forms(plan, O, sel, lens, _weights(H, 264, 8, "bf16"), tdt, "bf16", inp["lengths"], forms=("shortcut",))
+    assert ran["shortcut"] == "k_project_out_rows"
     plan.close()
 
 
@@ -122,6 +132,8 @@ def test_output_matrix_with_a_given_selection_shared_by_all_heads():
     sel_d = torch.from_numpy(sel).cuda()
     O = plan.psattn_forward_with_selection(dev["Q"], dev["K"], dev["V"], lengths, sel_d)
     _run_all_forms(plan, O, sel_d, lengths, _weights(H, 512, 7, "bf16"), tdt, "bf16", inp["lengths"])
+    ran = _run_all_forms(plan, O, sel_d, lengths, _weights(H, 520, 7, "bf16"), tdt, "bf16", inp["lengths"], forms=("shortcut",))
+    assert ran["shortcut"] == "k_project_out_rows"
     plan.close()
 
 

@@ -22,7 +22,7 @@ def _poison(n_bytes):
     ("bf16", 257, [257, 128, 129, 0, 1]), ("bf16", 130, [130, 127, 0]), ("bf16", 700, [3, 256, 511, 700]), ("fp32", 70, [70, 1, 0]),
 ])
 def test_padded_rows_of_fresh_outputs_are_zero(dtype, T, lengths):
-    H, B, dx, dy = 2, len(lengths), 128, 64
+    H, B, dx = 2, len(lengths), 128
     tdt = torch.bfloat16 if dtype == "bf16" else torch.float32
     w = wl.Workload("zeroed", 0, B, H, T, 64, dtype, 2.0, 0.1, 3.0)
     pin = wl.make_projection_inputs(w, lengths=lengths, pad_value=float("nan"))
@@ -39,11 +39,13 @@ def test_padded_rows_of_fresh_outputs_are_zero(dtype, T, lengths):
         for b, L in enumerate(lengths):
             assert (got[b, :, L:] == 0).all() and np.abs(got[b, :, :L] - want[b, :, :L]).max(initial=0) < 3e-2
     rng = np.random.default_rng(3)
-    Wot = torch.from_numpy((rng.standard_normal((dy, H * 64)) / 11).astype(np.float32)).to("cuda", tdt)
     idx = torch.zeros((B, T, plan.idx_cols), dtype=torch.int32, device="cuda")
     O, sel = plan.psattn_forward(Q, K, V, ln, idx)
-    for s in (sel, None):
-        _poison(B * T * dy * X.element_size())
+    # width 64: the dense product with and without an index set; width 72: the corrections, and one thread per element
+    for dy, s in ((64, sel), (64, None), (72, sel), (72, None)):
+        Wot = torch.from_numpy((rng.standard_normal((dy, H * 64)) / 11).astype(np.float32)).to("cuda", tdt)
+        for _ in range(3):
+            _poison(B * T * dy * X.element_size())
         Y = plan.psattn_project_out(O, s, ln, Wot).float().cpu().numpy()
         want = orc.project_out(O.float().cpu().numpy(), Wot.float().cpu().numpy(), pin["lengths"], nthreads=2)
         for b, L in enumerate(lengths):
