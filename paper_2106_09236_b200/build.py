@@ -1,6 +1,7 @@
 """Builds libpsattn.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a."""
 from __future__ import annotations
 
+import hashlib
 import os
 import subprocess
 import sys
@@ -24,13 +25,22 @@ def _nvcc() -> str:
     return "nvcc"
 
 
+def built_from() -> bytes:
+    """Digest of the flags and of the sources of libpsattn.so; the library holds it as a string."""
+    h = hashlib.sha1(" ".join(NVCC_FLAGS).encode())
+    files = sorted(os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cu", ".cuh", ".h")))
+    for path in files + [os.path.join(os.path.dirname(HERE), "include", "psattn.h")]:
+        with open(path, "rb") as f:
+            h.update(os.path.basename(path).encode() + f.read())
+    return b"built from " + h.hexdigest().encode()
+
+
 def needs_build() -> bool:
+    """Missing, or built from other sources (by content: a file put back to an older state is older than the library)."""
     if not os.path.exists(LIB):
         return True
-    t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cu", ".cuh", ".h"))]
-    deps.append(os.path.join(os.path.dirname(HERE), "include", "psattn.h"))
-    return any(os.path.getmtime(d) > t for d in deps)
+    with open(LIB, "rb") as f:
+        return built_from() + b"\0" not in f.read()
 
 
 def build(force: bool = False, verbose: bool = False, phase_stamps: bool = False, nvtx: bool = False) -> str:
@@ -44,10 +54,10 @@ def build(force: bool = False, verbose: bool = False, phase_stamps: bool = False
         return _build_variant("libpsattn_nvtx.so", ["-DPSATTN_NVTX"], ".nvtx.o", ["-ldl"])
     if not force and not needs_build():
         return LIB
-    objs = []
+    objs, key = [], built_from().decode()
     for src in SOURCES:
         obj = os.path.join(CSRC, src.replace(".cu", ".o"))
-        cmd = [_nvcc(), *NVCC_FLAGS, "-c", os.path.join(CSRC, src), "-o", obj]
+        cmd = [_nvcc(), *NVCC_FLAGS, '-DPSATTN_BUILT_FROM="%s"' % key, "-c", os.path.join(CSRC, src), "-o", obj]
         if verbose:
             cmd.insert(1, "-Xptxas")
             cmd.insert(2, "-v")

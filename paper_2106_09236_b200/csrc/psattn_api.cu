@@ -54,6 +54,11 @@ struct ApiRange {
 #endif
 #define PSATTN_RANGE() ApiRange api_range_(__func__)
 
+#ifdef PSATTN_BUILT_FROM
+// read back from the file by build.py: a library built from other sources is built again, not loaded
+extern "C" __attribute__((used)) const char psattn_built_from[] = PSATTN_BUILT_FROM;
+#endif
+
 extern "C" int psattn_version(void) { return 1000; }
 
 extern "C" const char *psattn_status_string(int s) {

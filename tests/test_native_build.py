@@ -1,5 +1,6 @@
-"""When the native side of the binding counts as up to date.  Nothing is compiled here."""
+"""When the library and the native side of the binding count as up to date.  Nothing is compiled here."""
 import os
+import shutil
 import sysconfig
 
 import torch
@@ -37,3 +38,19 @@ def test_missing_or_older_module_is_built_again(monkeypatch, tmp_path):
     os.utime(copy, (1, 1))
     monkeypatch.setattr(build, "NATIVE_SOURCE", str(source))
     assert build.native_needs_build()
+
+
+def test_library_of_other_sources_or_flags_is_built_again(monkeypatch, tmp_path):
+    ps.load()
+    assert not build.needs_build()
+    with monkeypatch.context() as m:
+        m.setattr(build, "NVCC_FLAGS", build.NVCC_FLAGS + ["-G"])
+        assert build.needs_build()
+    copy = tmp_path / "csrc"
+    shutil.copytree(build.CSRC, copy, ignore=shutil.ignore_patterns("*.o"))
+    monkeypatch.setattr(build, "CSRC", str(copy))
+    assert not build.needs_build()
+    with open(copy / "psattn_select.cuh", "a") as f:
+        f.write("// changed\n")
+    os.utime(copy / "psattn_select.cuh", (1, 1))         # older than the library, as a file put back to an earlier state
+    assert build.needs_build()
