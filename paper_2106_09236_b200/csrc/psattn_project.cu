@@ -62,6 +62,11 @@ __device__ __forceinline__ int proj_len(const ProjArgs &a, int b) {
     return L;
 }
 
+// ZERO: rows at positions >= the length are written as zeros (else not written).  An instance of its own, and one store for either
+// kind of row: with a second store behind a branch on an argument the drain, which paces the short tiles, cost the calls that write no
+// zeros up to 16 % and the others up to 15 % (us with the branch / so, B64 H4 lengths 40..500: outputs given 23.6 / 20.5, fresh
+// 24.6 / 21.4; B32 H4 T512 16.4 / 14.8, 15.4 / 14.0; B16 H8 T1024 with mean(V) 37.9 / 34.9).
+template <bool ZERO>
 __global__ void __launch_bounds__(kPjThreads, 1) k_project_qkv(ProjArgs a, const __grid_constant__ CUtensorMap tmX,
                                                                const __grid_constant__ CUtensorMap tmW) {
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -159,7 +164,7 @@ __global__ void __launch_bounds__(kPjThreads, 1) k_project_qkv(ProjArgs a, const
             const int b = m / a.tiles_per_seq, tt = m % a.tiles_per_seq;
             const int L = proj_len(a, b);
             if (tt * kPjM >= L) {
-                if (a.zero_pad) {                              // a tile of padding: no product, 64 columns = one row of 8 x 16 bytes
+                if (ZERO) {                                    // a tile of padding: no product, 64 columns = one row of 8 x 16 bytes
                     for (int gc = n * (kPjN / 64); gc < min(a.n_blocks, (n + 1) * (kPjN / 64)); ++gc) {
                         const int role = gc / a.H, h = gc - role * a.H;
                         const long long *st = role == 0 ? a.qs : (role == 1 ? a.ks : a.vs);
@@ -189,6 +194,7 @@ __global__ void __launch_bounds__(kPjThreads, 1) k_project_qkv(ProjArgs a, const
             }
             tc_fence_after();
             const int n_cc = min(kPjN / 64, a.n_blocks - n * (kPjN / 64));   // 64-column blocks of this tile
+            const int t_end = ZERO ? a.T : L;                  // rows are written up to here
             const uint32_t tacc = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * kPjAccCols;
             uint32_t ra[64], rb[64];                           // two blocks in flight: the next one loads while
             tmem_ld32_issue(tacc, ra);                         // the current one is converted and stored
@@ -214,9 +220,9 @@ __global__ void __launch_bounds__(kPjThreads, 1) k_project_qkv(ProjArgs a, const
                 for (int i = 0; i < 8; ++i) {
                     const int rr = 4 * i + (lane >> 3), c = lane & 7;
                     const int tr = tt * kPjM + quarter * 32 + rr;
-                    const uint4 val = stage[rr * 8 + (c ^ (rr & 7))];
-                    if (tr < L) reinterpret_cast<uint4 *>(base + (long long)tr * st[2])[c] = val;
-                    else if (a.zero_pad && tr < a.T) reinterpret_cast<uint4 *>(base + (long long)tr * st[2])[c] = make_uint4(0u, 0u, 0u, 0u);
+                    uint4 val = stage[rr * 8 + (c ^ (rr & 7))];
+                    if (ZERO && tr >= L) val = make_uint4(0u, 0u, 0u, 0u);
+                    if (tr < t_end) reinterpret_cast<uint4 *>(base + (long long)tr * st[2])[c] = val;
                 }
                 if (role == 2 && a.vpart != nullptr) {
                     // column sums of this block over the warp's valid rows, from the values as stored (bf16):
@@ -328,6 +334,13 @@ static EncodeTiledFnP proj_encode_fn() {
     return fn;
 }
 
+// The instance of the kernel, and its grant of shared memory.
+static auto project_kernel(int zero_pad) { return zero_pad ? k_project_qkv<true> : k_project_qkv<false>; }
+static cudaError_t grant_project(int zero_pad) {
+    static SmemGrant grants[2];
+    return grant_dynamic_smem(project_kernel(zero_pad), grants[zero_pad != 0], kPjSmem);
+}
+
 size_t project_vpart_floats(int B, int H, int T) { return (size_t)B * ((T + kPjM - 1) / kPjM) * 4 * H * 64; }
 
 // dtype 0 = bf16, 1 = fp32.  X [B][T][dx], Wt [3][H*64][dx], outputs with g.qs / g.ks / g.vs strides.
@@ -363,8 +376,7 @@ cudaError_t launch_project_qkv(int dtype, int force_simt, int zero_pad, const Ge
                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
         if (ok) {
-            static SmemGrant grant;
-            if (cudaError_t e = grant_dynamic_smem(k_project_qkv, grant, kPjSmem)) return e;
+            if (cudaError_t e = grant_project(zero_pad)) return e;
             // both kernels carry a programmatic dependency on their predecessor in the stream
             cudaLaunchAttribute attr[1];
             attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -376,7 +388,7 @@ cudaError_t launch_project_qkv(int dtype, int force_simt, int zero_pad, const Ge
             cfg.stream = st;
             cfg.attrs = attr;
             cfg.numAttrs = 1;
-            cudaError_t e = cudaLaunchKernelEx(&cfg, k_project_qkv, a, tmX, tmW);
+            cudaError_t e = cudaLaunchKernelEx(&cfg, project_kernel(zero_pad), a, tmX, tmW);
             note_launch();
             if (e == cudaSuccess) e = cudaGetLastError();
             if (e != cudaSuccess || vbar == nullptr) return e;
@@ -437,10 +449,9 @@ cudaError_t launch_project_out_dense(const Geom &g, int zero_pad, int dy, const 
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return cudaErrorNotSupported;
-    static SmemGrant grant;
-    if (cudaError_t e = grant_dynamic_smem(k_project_qkv, grant, kPjSmem)) return e;
+    if (cudaError_t e = grant_project(zero_pad)) return e;
     const int sms = device_sm_count();
-    cudaError_t e = launch_pdl(k_project_qkv, dim3((unsigned)(a.n_tiles < sms ? a.n_tiles : sms)), dim3(kPjThreads), kPjSmem,
+    cudaError_t e = launch_pdl(project_kernel(zero_pad), dim3((unsigned)(a.n_tiles < sms ? a.n_tiles : sms)), dim3(kPjThreads), kPjSmem,
                                st, a, tmX, tmW);
     note_launch();
     return e != cudaSuccess ? e : cudaGetLastError();

@@ -54,7 +54,7 @@ def test_output_matrix_form_by_size(B, H, T, dy, corrections):
     O, sel = plan.psattn_forward(q, k, v, ln, idx)
     Wot = (torch.randn((dy, H * 64), generator=gen, device="cuda") / 16).bfloat16()
     Y, ran = launched(lambda: plan.psattn_project_out(O, sel, ln, Wot))
-    assert ran == {"k_project_out_rows" if corrections else "k_project_qkv"}
+    assert ran == {"k_project_out_rows" if corrections else "k_project_qkv<1>"}
     want = O.permute(0, 2, 1, 3).reshape(B, T, H * 64).double() @ Wot.double().T       # O is zero at padded positions
     err = (Y.double() - want).abs()
     assert bool((err <= 2.0 ** -8 * want.abs() + 1e-3).all())

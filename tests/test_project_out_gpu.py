@@ -69,7 +69,7 @@ def test_output_matrix_on_workloads(name, nb):
     inp = wl.make_inputs(w, n_cols, B=nb)
     plan, O, sel, lengths, tdt = _forward(inp, w.dtype, w.c)
     ran = _run_all_forms(plan, O, sel, lengths, _weights(w.H, w.H * 64, 5, w.dtype), tdt, w.dtype, inp["lengths"])
-    assert ran["dense"] == "k_project_qkv"
+    assert ran["dense"] == "k_project_qkv<0>"
     # a width that the dense tiles do not take: the corrections
     ran = _run_all_forms(plan, O, sel, lengths, _weights(w.H, w.H * 64 + 8, 5, w.dtype), tdt, w.dtype, inp["lengths"], forms=("shortcut",))
     assert ran["shortcut"] == "k_project_out_rows"
@@ -90,7 +90,7 @@ def test_output_matrix_odd_widths_short_sequences_and_full_selection(dy):
     assert (s[2, :, :3] >= 0).all()                          # length 3: all three rows selected in every head
     shared = set(s[0, 0][s[0, 0] >= 0]) & set(s[0, 1][s[0, 1] >= 0])
     ran = _run_all_forms(plan, O, sel, lens, _weights(H, dy, 6, "bf16"), tdt, "bf16", inp["lengths"])
-    assert ran["shortcut"] == ("k_project_out_rows" if dy % 64 else "k_project_qkv")
+    assert ran["shortcut"] == ("k_project_out_rows" if dy % 64 else "k_project_qkv<0>")
     assert shared
     plan.close()
 
