@@ -674,7 +674,8 @@ def run_variants(cx, w, r, dense_ms):
         Wo = torch.from_numpy((rng.standard_normal((dx, dx)) / np.sqrt(dx)).astype(np.float32)).to("cuda", tdt)
         Ys = [torch.empty((w.B, w.T, dx), dtype=tdt, device="cuda") for _ in range(n_sets)]
         o_flops = 2.0 * dx * dx * sum(int(L) for L in host0["lengths"])
-        for key, use_sel in (("output_projection_shortcut", True), ("output_projection_dense", False)):
+        # with the index set the library takes the faster of its two forms for the shape
+        for key, use_sel in (("output_projection_with_index_set", True), ("output_projection_dense", False)):
             def out_proj(s, use_sel=use_sel):
                 d = sets[s]
                 plan.psattn_project_out(d["O"], d["sel"] if use_sel else None, d["lengths"], Wo, Ys[s])

@@ -192,8 +192,8 @@ int psattn_project_qkv_zeroed(psattn_plan_t *plan, const void *X, const void *Wt
  * With sel_idx, the mean(V) fill and bf16 (u_max <= 64, H <= 32, d_y a multiple of 8) the call uses the structure
  * Eq. 12 gives O - every valid row of a unit that its index set does not list equals one fill row F_h - and
  * computes Y[b][t][:] = sum_h F_h W_o^h for all positions plus (O[b][h][t][:] - F_h) W_o^h for the listed ones:
- * O(B H u 64 d_y) products instead of O(B T H 64 d_y) - except where so few positions are given that the dense
- * product (below) is the faster one.  F_h is read from O at the first valid position the set
+ * O(B H u 64 d_y) products instead of O(B T H 64 d_y) - except where the dense product (below) is the faster one
+ * for the sizes, as it is for most shapes but long sequences.  F_h is read from O at the first valid position the set
  * leaves out, so O must really have that structure (rows changed after psattn_forward are not seen).
  * With sel_idx == NULL (any O), the own-value fill, or shapes outside those limits: one dense product (tcgen05 for
  * bf16 with d_y a multiple of 64; one thread per output element for fp32, other d_y, or PSATTN_PATH_STAGED). */

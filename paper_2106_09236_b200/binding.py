@@ -269,7 +269,8 @@ class Plan:
 
     def psattn_project_out(self, O, sel_idx, lengths, Wot, Y=None):
         """Y[b, t, :] = sum_h O[b, h, t, :] W_o^h; Wot [d_y, H*64] holds W_o transposed.  With sel_idx (the index
-        sets psattn_forward wrote for this O) the broadcast-plus-corrections form runs, with None the dense product.
+        sets psattn_forward wrote for this O) the faster of the broadcast-plus-corrections form and the dense
+        product runs, with None the dense product.
         Rows at padded positions of a freshly allocated Y are zero, those of a given one are not written."""
         return self._call.project_out(O, sel_idx, lengths, Wot, Wot.shape[0], Y)
 

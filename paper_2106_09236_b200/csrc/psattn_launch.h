@@ -125,7 +125,7 @@ cudaError_t launch_project_qkv(int dtype, int force_simt, int zero_pad, const Ge
                                void *Q, void *K, void *V, float *vbar, float *vpart, cudaStream_t st);
 // The output matrix of the attention module: Y [B][T][dy] = sum_h O[b][h][t][:] W_o^h, Wot [dy][H * 64].
 // mode 0: with an index set `sel` ([B][H][g.u_max], as psattn_forward writes it) and the mean(V) fill, the
-// broadcast-plus-corrections form; otherwise (and with mode 1) the dense tcgen05 GEMM; mode 2 or fp32: one
+// faster of the broadcast-plus-corrections form and the dense tcgen05 GEMM; otherwise (and with mode 1) the dense GEMM; mode 2 or fp32: one
 // thread per output element.  Rows at padded positions are written as zeros with zero_pad, else not written.
 cudaError_t launch_project_out(int dtype, int mode, int zero_pad, const Geom &g, int dy, const void *O, const int *sel,
                                const void *Wot, void *Y, cudaStream_t st);
