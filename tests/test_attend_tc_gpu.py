@@ -1,0 +1,48 @@
+"""Attention of more than 64 listed rows (k_attend_tc) at the edges of its tiles: rows around a multiple of 128, keys around a multiple
+of 128 with anything (NaN) behind the sequence's end, and rows whose scores grow from one key tile to the next, so that the
+reference of the exponentials moves and the row of O in tensor memory is scaled while products are in flight."""
+import pytest
+import torch
+
+from kernels import launched
+from paper_2106_09236_b200 import binding as ps
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n_rows,lengths,growing", [
+    (65, (1, 127, 128, 129, 300), False), (128, (300, 256, 255, 257, 383), True), (129, (640, 513, 200, 130, 512), True),
+    (257, (1025, 700, 258, 300, 1024), True),
+])
+def test_rows_and_keys_around_tiles(n_rows, lengths, growing):
+    B, H, T = 40, 2, max(lengths)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(n_rows)
+    ln = torch.tensor([lengths[b % len(lengths)] for b in range(B)], dtype=torch.int32, device="cuda")
+    q, k, v = (torch.randn((B, H, T, 64), generator=gen, device="cuda") for _ in range(3))
+    if growing:                                              # scores of the first queries: 1, 4, 7, .. times those of the first key tile
+        k *= 1 + 3 * torch.div(torch.arange(T, device="cuda"), 128, rounding_mode="floor").view(1, 1, T, 1)
+    q, k, v = q.bfloat16(), k.bfloat16(), v.bfloat16()
+    behind = torch.arange(T, device="cuda").view(1, 1, T, 1) >= ln.view(B, 1, 1, 1)
+    k.masked_fill_(behind, float("nan"))
+    v.masked_fill_(behind, float("nan"))
+    rows = torch.randint(0, T, (B, H, n_rows), generator=gen, device="cuda", dtype=torch.int32)
+    rows[rows >= ln.view(B, 1, 1)] = -1                      # entries outside the sequence are ignored
+    rows[:, :, 0] = 0
+    plan = ps.Plan(B, H, T, u_override=n_rows)
+    out, names = launched(lambda: plan.psattn_attend_rows(q, k, v, ln, rows))
+    assert "k_attend_tc" in names and plan.psattn_read_status() == 0
+    for b in range(B):
+        L = int(ln[b])
+        Q, K, V = (x[b, :, :L].double() for x in (q, k, v))
+        at = rows[b].clamp(min=0).long()
+        s = torch.gather(Q, 1, at.unsqueeze(-1).expand(-1, -1, 64)) @ K.transpose(1, 2) / 8
+        ref = torch.softmax(s, -1) @ V
+        ok = (rows[b] >= 0).unsqueeze(-1)
+        # The weights are rounded to bf16 (half a unit in the eighth bit: 2^-8 of each), their sum is not.  A score is 64 products
+        # added in fp32: off by at most 64 roundings of 2^-24 of what |q| |k| / 8 bounds, which moves a weight, and the sum, by
+        # as much of themselves.
+        size = float(Q.norm(dim=2).max() * K.norm(dim=2).max()) / 8
+        bound = float(V.abs().max()) * (2 ** -8 + 2 * 64 * 2 ** -24 * size)
+        assert float(((out[b] - ref) * ok).abs().max()) <= bound
+    plan.close()
