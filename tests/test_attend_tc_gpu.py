@@ -10,12 +10,15 @@ from paper_2106_09236_b200 import binding as ps
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n_rows,lengths,growing", [
-    (65, (1, 127, 128, 129, 300), False), (128, (300, 256, 255, 257, 383), True), (129, (640, 513, 200, 130, 512), True),
-    (257, (1025, 700, 258, 300, 1024), True),
+@pytest.mark.parametrize("B,n_rows,lengths,growing,split", [
+    (40, 65, (1, 127, 128, 129, 300), False, False), (40, 128, (300, 256, 255, 257, 383), True, False),
+    (40, 129, (640, 513, 200, 130, 512), True, False), (40, 257, (1025, 700, 258, 300, 1024), True, False),
+    # few tiles: the keys in four splits, of which short sequences leave some empty
+    (5, 65, (512, 1, 128, 129, 385), True, True), (24, 128, (1025, 100, 257, 513, 512), True, True), (25, 128, (1025, 100, 257, 513, 512), True, False),
+    (24, 128, (384, 100, 257, 383, 129), True, False),
 ])
-def test_rows_and_keys_around_tiles(n_rows, lengths, growing):
-    B, H, T = 40, 2, max(lengths)
+def test_rows_and_keys_around_tiles(B, n_rows, lengths, growing, split):
+    H, T = 2, max(lengths)
     gen = torch.Generator(device="cuda")
     gen.manual_seed(n_rows)
     ln = torch.tensor([lengths[b % len(lengths)] for b in range(B)], dtype=torch.int32, device="cuda")
@@ -32,6 +35,7 @@ def test_rows_and_keys_around_tiles(n_rows, lengths, growing):
     plan = ps.Plan(B, H, T, u_override=n_rows)
     out, names = launched(lambda: plan.psattn_attend_rows(q, k, v, ln, rows))
     assert "k_attend_tc" in names and plan.psattn_read_status() == 0
+    assert any(x.startswith("k_attend_combine") for x in names) == split
     for b in range(B):
         L = int(ln[b])
         Q, K, V = (x[b, :, :L].double() for x in (q, k, v))
