@@ -425,6 +425,12 @@ extern "C" int psattn_forward(psattn_plan_t *plan, const void *Q, const void *K,
         if (e == cudaSuccess) return PSATTN_OK;
         if (e != cudaErrorNotSupported) return cuda_fail(plan, e);
     }
+    if (d.dtype == PSATTN_BF16 && d.path == PSATTN_PATH_AUTO && !d.idx_shared && d.fill_mode == PSATTN_FILL_OWN_V) {
+        // more selected rows than the fused kernel attends to: all but step (d) in one kernel, the attention behind it
+        cudaError_t e = launch_front_fused(g, plan->U_max, Q, K, V, sample_idx, O, sel_idx, M_out, st);
+        if (e == cudaSuccess) return run_attend(plan, g, Q, K, V, sel_idx, plan->u_max, plan->u_max, O, 0, 0, 1, 0, workspace, st);
+        if (e != cudaErrorNotSupported) return cuda_fail(plan, e);
+    }
     float *M = M_out ? M_out : ws_at<float>(workspace, plan->off_M);
     if (d.dtype == PSATTN_BF16 && d.path == PSATTN_PATH_AUTO && fused_from_measure_supported(g, K, V)) {
         // keys too long for shared memory: the measure by itself, the rest in one kernel

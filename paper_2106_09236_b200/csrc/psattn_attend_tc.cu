@@ -92,6 +92,9 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_attend_tc(Geom g, AttendTcArg
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int split = blockIdx.x, tile = blockIdx.y;
+    // (before the allocation too: an earlier grid may still need tensor memory.  For the same reason the next grid of the stream may
+    // start only behind this one's allocations, see below.)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     int b = blockIdx.z / g.H;
     const int h = blockIdx.z % g.H;
     // longest sequences first: the short ones (and the tiles that list nothing) fill the tail of the last wave
@@ -134,6 +137,7 @@ __global__ void __launch_bounds__(kTcThreads, 2) k_attend_tc(Geom g, AttendTcArg
     // Lists are padded to the longest one of the batch: a tile that lists no position of this sequence has only its zero rows to write.
     if (!__syncthreads_or(row_ok)) n_tiles = 0;
     tc_fence_after();
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const uint32_t tmem_base = *tmem_slot;
     auto give_up = [&]() { *abort_flag = 1u; atomicOr(g.status, kStatusWaitExpired); };
 
@@ -399,9 +403,9 @@ cudaError_t launch_attend_tc(const Geom &g, const void *Q, const void *K, const 
     static SmemGrant grant;
     if (cudaError_t e = grant_dynamic_smem(k_attend_tc, grant, kAttendSmem, true)) return e;
     dim3 grid((unsigned)n_splits, (unsigned)((n_rows + kTileRows - 1) / kTileRows), (unsigned)(g.B * g.H));
-    k_attend_tc<<<grid, kTcThreads, kAttendSmem, st>>>(g, a, (const __nv_bfloat16 *)Q, tmK, tmV);
+    cudaError_t e = launch_pdl(k_attend_tc, grid, dim3(kTcThreads), kAttendSmem, st, g, a, (const __nv_bfloat16 *)Q, tmK, tmV);
     note_launch();
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace psattn

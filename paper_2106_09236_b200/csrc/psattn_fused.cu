@@ -59,7 +59,10 @@ __host__ __device__ inline size_t fused_arrays_bytes(int m_floats, int T) { retu
 
 // SPLIT: the unit is shared by the a.split > 1 CTAs of a thread-block cluster.
 // MODE: all steps, or from step (c) on with M~ in global memory (sequences too long for resident keys), or steps (d)+(e).
-enum FusedMode { kAllSteps = 0, kGivenMeasure = 1, kGivenSet = 2 };
+// kFront: steps (a)-(c) and the fill with the query's own value row, for selections too long for step (d) here (k_attend_tc comes
+// behind).  u = L / 2, us per call with measure and selection as kernels of their own and the fill beside them / this: B12 H8 T960
+// 62 / 59, B32 H4 T256 28 / 19, B16 H8 T512 32 / 28, B1 H4 T200 22 / 16 (and the attention started while this kernel drains).
+enum FusedMode { kAllSteps = 0, kGivenMeasure = 1, kGivenSet = 2, kFront = 3 };
 constexpr int kFusedSelectKeys = kSelectMaxSlots * (kFusedThreads - 32);       // longest sequence of the block-wide selection
 
 // S: the shape of the CTA.  ArWide has the SM to itself.  ArHalf (256 threads, half of the shared memory) leaves room for a
@@ -100,7 +103,7 @@ __global__ void __launch_bounds__(S::kThreads, S::kThreads <= 256 ? 2 : 1) k_for
     const int L = seq_len(g, b);
     const int U = min(g.U_tab[L], g.idx_cols);
     const int u = min(min(g.u_tab[L], g.u_max), L);
-    constexpr bool all_steps = MODE == kAllSteps, given = MODE == kGivenSet;
+    constexpr bool front = MODE == kFront, all_steps = MODE == kAllSteps || front, given = MODE == kGivenSet;
     if (tid == 32) {
         mbar_init(&P.bar, 1);
         fence_barrier_init();
@@ -153,11 +156,13 @@ __global__ void __launch_bounds__(S::kThreads, S::kThreads <= 256 ? 2 : 1) k_for
     static_assert(S::kLoader == kSelectors, "the last warp starts the copies");
     const int ahead = given ? 1 : S::kStages;                    // (nothing to hide the copies behind with a given set)
     if (tid >= kSelectors) {
-        if (ok && L > 0 && tid == S::kLoader) attend_rows_start<S>(smem, g, j, &tmK, &tmV, ahead);
+        if (!front && ok && L > 0 && tid == S::kLoader) attend_rows_start<S>(smem, g, j, &tmK, &tmV, ahead);
     } else if (!given) {
         // ---- step (c) ---------------------------------------------------------------------------
+        int *list = front ? reinterpret_cast<int *>(smem) : P.sel;       // (the keys are not needed any more)
+        const int room = front ? g.u_max : kArMaxRows;
         if (all_steps) {
-            block_select_short<3>([&](int i) { return float_key(M_s[i]); }, L, u, kArMaxRows, P.sel, P.select, kSelectors, 1);
+            block_select_short<3>([&](int i) { return float_key(M_s[i]); }, L, u, room, list, P.select, kSelectors, 1);
         } else {
             const float *Mu = a.M_in + (long long)unit * g.T;
             auto key_of = [&](int i) { return float_key(__ldg(Mu + i)); };
@@ -165,7 +170,7 @@ __global__ void __launch_bounds__(S::kThreads, S::kThreads <= 256 ? 2 : 1) k_for
             else block_select_few<kSelectMaxSlots>(key_of, L, u, kArMaxRows, P.sel, P.select, kSelectors, 1);
         }
         for (int r = tid; r < g.u_max; r += kSelectors) {
-            const int i = r < kArMaxRows ? P.sel[r] : -1;
+            const int i = r < room ? list[r] : -1;
             if (part == 0) sel_out[(long long)unit * g.u_max + r] = i;
             if (i >= 0) chosen[i] = 1;
         }
@@ -181,7 +186,7 @@ __global__ void __launch_bounds__(S::kThreads, S::kThreads <= 256 ? 2 : 1) k_for
 
     // ---- step (d), with the column sums of V riding along ------------------------------------------
     // (a CTA of a cluster whose wait for the keys ran out still takes part in the barriers below)
-    if (L > 0 && (ok || SPLIT)) {
+    if (!front && L > 0 && (ok || SPLIT)) {
         float m_run[S::kRows], l_run[S::kRows], acc[S::kRows][8];
         const int c8 = tid & 7;
         if (ok) {
@@ -256,7 +261,7 @@ __global__ void __launch_bounds__(S::kThreads, S::kThreads <= 256 ? 2 : 1) k_for
     }
     __syncthreads();
     phase_stamp(g, 5);                                         // step (e) done
-    if (SPLIT && L > 0) cluster_wait();                    // nobody reads this CTA's states any more
+    if (SPLIT && !front && L > 0) cluster_wait();          // nobody reads this CTA's states any more
 }
 
 bool make_rows_map(CUtensorMap *map, const void *base, const Geom &g, const long long s[3], int box_rows,
@@ -270,9 +275,10 @@ bool make_rows_map(CUtensorMap *map, const void *base, const Geom &g, const long
 static int fused_split(const Geom &g, int mode) {
     static ClusterRecord clusters;
     const int units = g.B * g.H;
-    if (g.T < (mode == kAllSteps ? 192 : 448)) return 1;
+    const bool measures = mode == kAllSteps || mode == kFront;
+    if (g.T < (measures ? 192 : 448)) return 1;
     for (int split = kMaxSplit; split > 1; --split) {
-        if (mode != kAllSteps && split < 4 && g.T < 704) return 1;
+        if (!measures && split < 4 && g.T < 704) return 1;
         if (units <= max_clusters(k_forward_fused<true, kAllSteps, ArWide>, clusters, split, kFusedThreads, kFusedMaxSmem)) return split;
     }
     return 1;
@@ -296,7 +302,7 @@ static bool fused_half(const Geom &g, int mode) {
     const long long units = (long long)g.B * g.H, sms = device_sm_count();
     constexpr int kSelectors = ArHalf::kThreads - 32;
     if (units <= sms) return false;
-    if (mode == kAllSteps) return g.T <= 3 * kSelectors && (units > 2 * sms || g.T <= 208 || (g.T <= 400 && 5 * units >= 8 * sms));
+    if (mode == kAllSteps || mode == kFront) return g.T <= 3 * kSelectors && (units > 2 * sms || g.T <= 208 || (g.T <= 400 && 5 * units >= 8 * sms));
     if (mode == kGivenMeasure && g.T > kSelectMaxSlots * kSelectors) return false;
     const bool many = mode == kGivenSet ? 3 * units >= 4 * sms : 5 * units >= 8 * sms;
     return units > 3 * sms || g.T <= (many ? 1536 : 1024);
@@ -312,24 +318,21 @@ bool fused_from_measure_supported(const Geom &g, const void *K, const void *V) {
            attend64_supported(g, K, V, g.u_max, 1);
 }
 
-// cudaErrorNotSupported when the shape does not fit this kernel (the caller runs the staged schedule):
-// keys + staging beyond shared memory, more than 63 selected rows or 64 samples, no tensor map.
-cudaError_t launch_forward_fused(const Geom &g, int U_max, int own_v, const void *Q, const void *K, const void *V,
-                                 const int *sidx, void *O, int *sel, float *M_out, const int *sel_in, const float *M_in,
-                                 cudaStream_t st) {
+static cudaError_t launch_fused(int mode, const Geom &g, int U_max, int own_v, const void *Q, const void *K, const void *V,
+                                const int *sidx, void *O, int *sel, float *M_out, const int *sel_in, const float *M_in,
+                                cudaStream_t st) {
     if (g.B * g.H == 0) return cudaSuccess;
-    if (g.u_max > kArMaxRows - 1) return cudaErrorNotSupported;
+    if (mode != kFront && g.u_max > kArMaxRows - 1) return cudaErrorNotSupported;
     if (sel_in == nullptr && M_in == nullptr && (U_max > kMeasureMaxU || U_max < 1)) return cudaErrorNotSupported;
     FusedArgs a;
-    const int mode = sel_in != nullptr ? kGivenSet : (M_in != nullptr ? kGivenMeasure : kAllSteps);
-    const bool given = mode != kAllSteps;
+    const bool given = mode == kGivenMeasure || mode == kGivenSet;
     // The shared memory of a CTA of the given shape
     auto layout = [&](int threads, uint32_t attend_bytes) {
         a.k_bytes = given ? 0u : (uint32_t)measure_k_bytes(g.T);
         a.stage_bytes = given ? 0u : (uint32_t)measure_stage_bytes(threads, g.idx_cols);
         a.m_floats = given ? 0 : g.T;
         size_t phase = (size_t)a.k_bytes + kMeasureStages * (size_t)a.stage_bytes;
-        if (phase < attend_bytes) phase = attend_bytes;
+        if (mode != kFront && phase < attend_bytes) phase = attend_bytes;
         a.off_persist = (uint32_t)((phase + 1023) / 1024 * 1024);
         return a.off_persist + fused_arrays_bytes(a.m_floats, g.T) + sizeof(FusedPersist) + 128;
     };
@@ -342,7 +345,7 @@ cudaError_t launch_forward_fused(const Geom &g, int U_max, int own_v, const void
     }
     if (!half) smem = layout(ArWide::kThreads, ArWide::kBytes);
     if (smem > kFusedMaxSmem) return cudaErrorNotSupported;
-    if (mode == kAllSteps && g.T > 3 * (kFusedThreads - 32)) return cudaErrorNotSupported;     // (block_select_short<3>)
+    if (!given && g.T > 3 * (kFusedThreads - 32)) return cudaErrorNotSupported;     // (block_select_short<3>)
     if (mode == kGivenMeasure && g.T > kFusedSelectKeys) return cudaErrorNotSupported;
     CUtensorMap tmKrows, tmK, tmV;
     int p0[3], p1[3], p2[3];
@@ -358,11 +361,12 @@ cudaError_t launch_forward_fused(const Geom &g, int U_max, int own_v, const void
     // the ranking costs B comparisons per sequence in every CTA: only where a second wave exists and B is small
     a.by_length = g.lengths != nullptr && g.B * g.H > device_sm_count() && g.B <= 256;
     using Kernel = decltype(&k_forward_fused<false, kAllSteps, ArWide>);
-    static const Kernel kernels[3][3] = {
+    static const Kernel kernels[4][3] = {
         {k_forward_fused<false, kAllSteps, ArWide>, k_forward_fused<true, kAllSteps, ArWide>, k_forward_fused<false, kAllSteps, ArHalf>},
         {k_forward_fused<false, kGivenMeasure, ArWide>, k_forward_fused<true, kGivenMeasure, ArWide>, k_forward_fused<false, kGivenMeasure, ArHalf>},
-        {k_forward_fused<false, kGivenSet, ArWide>, k_forward_fused<true, kGivenSet, ArWide>, k_forward_fused<false, kGivenSet, ArHalf>}};
-    static SmemGrant grants[3][3];
+        {k_forward_fused<false, kGivenSet, ArWide>, k_forward_fused<true, kGivenSet, ArWide>, k_forward_fused<false, kGivenSet, ArHalf>},
+        {k_forward_fused<false, kFront, ArWide>, k_forward_fused<true, kFront, ArWide>, k_forward_fused<false, kFront, ArHalf>}};
+    static SmemGrant grants[4][3];
     for (int x = 0; x < 3; ++x)
         if (cudaError_t e = grant_dynamic_smem(kernels[mode][x], grants[mode][x], x == 2 ? kFusedHalfSmem : kFusedMaxSmem, x == 2)) return e;
     if (cudaError_t e = grant_dynamic_smem(kernels[0][1], grants[0][1], kFusedMaxSmem)) return e;        // (asked by fused_split)
@@ -375,6 +379,20 @@ cudaError_t launch_forward_fused(const Geom &g, int U_max, int own_v, const void
                                  tmKrows, tmK, tmV);
     note_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+// cudaErrorNotSupported when the shape does not fit this kernel (the caller runs the staged schedule):
+// keys + staging beyond shared memory, more than 63 selected rows or 64 samples, no tensor map.
+cudaError_t launch_forward_fused(const Geom &g, int U_max, int own_v, const void *Q, const void *K, const void *V,
+                                 const int *sidx, void *O, int *sel, float *M_out, const int *sel_in, const float *M_in,
+                                 cudaStream_t st) {
+    return launch_fused(sel_in != nullptr ? kGivenSet : M_in != nullptr ? kGivenMeasure : kAllSteps, g, U_max, own_v, Q, K, V, sidx, O,
+                        sel, M_out, sel_in, M_in, st);
+}
+
+cudaError_t launch_front_fused(const Geom &g, int U_max, const void *Q, const void *K, const void *V, const int *sidx, void *O,
+                               int *sel, float *M_out, cudaStream_t st) {
+    return launch_fused(kFront, g, U_max, 1, Q, K, V, sidx, O, sel, M_out, nullptr, nullptr, st);
 }
 
 }  // namespace psattn

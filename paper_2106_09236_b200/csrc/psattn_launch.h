@@ -66,6 +66,9 @@ cudaError_t launch_measure_mma(const Geom &g, int U_max, const void *Q, const vo
 cudaError_t launch_forward_fused(const Geom &g, int U_max, int own_v, const void *Q, const void *K, const void *V,
                                  const int *sidx, void *O, int *sel, float *M_out, const int *sel_in, const float *M_in,
                                  cudaStream_t st);
+// Steps (a)-(c) and the fill of every other row with its own value row, for selections of any length (step (d) is left).
+cudaError_t launch_front_fused(const Geom &g, int U_max, const void *Q, const void *K, const void *V, const int *sidx, void *O,
+                               int *sel, float *M_out, cudaStream_t st);
 bool fused_from_measure_supported(const Geom &g, const void *K, const void *V);
 // The same for fp32 inputs (psattn_fused_fp32.cu).
 cudaError_t launch_forward_fused_fp32(const Geom &g, int U_max, int own_v, const void *Q, const void *K, const void *V,

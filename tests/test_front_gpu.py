@@ -1,0 +1,42 @@
+"""Selections of more than 63 queries with the own-value fill: measure, selection and fill in one kernel (clusters, one CTA or two CTAs
+per SM), the attention of the list behind it.  The list has to be that of the measure, every other row its own value row to the bit,
+and the selected rows what the attention of listed rows gives."""
+import pytest
+import torch
+
+from kernels import launched
+from paper_2106_09236_b200 import binding as ps
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,H,T,shortest,form", [
+    (1, 4, 203, 203, "1,3,512"), (2, 3, 515, 1, "1,3,512"), (40, 2, 700, 1, "0,3,512"), (80, 2, 200, 1, "0,3,256"), (150, 2, 129, 64, "0,3,256"),
+    (40, 4, 1079, 2, "0,3,512"),
+])
+def test_front(B, H, T, shortest, form):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(T)
+    ln = torch.randint(shortest, T + 1, (B,), generator=gen, device="cuda", dtype=torch.int32)
+    ln[0] = T
+    q, k, v = (torch.randn((B, H, T, 64), generator=gen, device="cuda").bfloat16() for _ in range(3))
+    idx = (torch.rand((B, T, 7), generator=gen, device="cuda") * ln.view(B, 1, 1)).int()
+    plan = ps.Plan(B, H, T, c=1.0, idx_cols=7, r_sparse=0.5, fill_mode=ps.PSATTN_FILL_OWN_V)
+    O = torch.full((B, H, T, 64), float("nan"), dtype=torch.bfloat16, device="cuda")
+    M = torch.empty((B, H, T), device="cuda")
+    (_, sel), names = launched(lambda: plan.psattn_forward(q, k, v, ln, idx, O=O, M_out=M))
+    assert any(x.startswith("k_forward_fused<" + form) for x in names) and "k_attend_tc" in names and len(names) <= 3
+    assert plan.psattn_read_status() == 0
+    torch.testing.assert_close(M, plan.psattn_measure(q, k, ln, idx), atol=1e-5, rtol=1e-5)
+    assert torch.equal(sel, plan.psattn_select(M, ln))
+    rows = plan.psattn_attend_rows(q, k, v, ln, sel)
+    ref = v.clone().float()
+    ref.masked_fill_(torch.arange(T, device="cuda").view(1, 1, T, 1) >= ln.view(B, 1, 1, 1), 0.0)
+    picked = torch.zeros((B, H, T + 1), dtype=torch.bool, device="cuda").scatter_(2, sel.long().where(sel >= 0, T), True)[:, :, :T]
+    assert torch.equal(O.float()[~picked], ref[~picked])
+    at = sel.long().clamp(min=0).unsqueeze(-1).expand(-1, -1, -1, 64)
+    got = torch.gather(O.float(), 2, at)
+    ok = (sel >= 0).unsqueeze(-1)
+    # the same sums, rounded to bf16 (2^-8 of values of at most |V|)
+    assert float(((got - rows) * ok).abs().max()) <= 2 ** -8 * float(v.float().abs().max())
+    plan.close()
