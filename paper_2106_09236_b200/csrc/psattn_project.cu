@@ -2,10 +2,10 @@
 // (d_x x 64) matrix per head and role, written straight into the [B][H][T][64] layout (any b/h/t strides)
 // that the attention kernels read, so no transpose pass sits between the two.
 //
-// bf16: ONE persistent tcgen05 GEMM over all three roles.  A tile is 128 tokens of one sequence x 192 output
-// columns (three 64-wide head blocks); CTAs walk the tiles round-robin.  Warp 0 streams 64-deep slabs of X and
-// of the transposed weights into a 5-stage shared-memory ring by TMA (128-byte swizzle), warp 1 issues
-// tcgen05.mma (M = 128, N = 192, K = 16) into one of two TMEM accumulators, warps 2-5 drain the other
+// bf16: ONE persistent tcgen05 GEMM over all three roles.  A tile is 128 tokens of one sequence x N output
+// columns (N / 64 head blocks; N = 64, 128, 192 or 256, see project_columns); CTAs walk the tiles round-robin.  Warp 0 streams
+// 64-deep slabs of X and of the transposed weights into a shared-memory ring by TMA (128-byte swizzle), warp 1 issues
+// tcgen05.mma (M = 128, N, K = 16) into one of two TMEM accumulators, warps 2-5 drain the other
 // accumulator: TMEM -> registers -> bf16 -> a swizzled staging tile -> whole 128-byte rows at (b, h, t).  The mainloop of tile i + 1 runs
 // under the drain of tile i.  Tiles that lie wholly beyond a sequence's length are skipped; rows beyond it
 // are not written.  For the V blocks every drain warp also adds up the columns of its 32 rows (as rounded to
@@ -19,13 +19,17 @@ namespace psattn {
 
 using namespace sm100;
 
-constexpr int kPjM = 128, kPjN = 192, kPjK = 64, kPjStages = 5;
+constexpr int kPjM = 128, kPjK = 64, kPjThreads = 192;
 constexpr int kPjAccCols = 256;                                // TMEM columns reserved per accumulator
-constexpr uint32_t kPjBytesA = kPjM * kPjK * 2, kPjBytesB = kPjN * kPjK * 2, kPjStage = kPjBytesA + kPjBytesB;
-constexpr uint32_t kPjOffBar = kPjStages * kPjStage;           // mbarriers, TMEM slot, abort flag
-constexpr uint32_t kPjOffStage = kPjOffBar + 128;              // [4 warps][32 rows][128 B] output staging (swizzled)
-constexpr uint32_t kPjSmem = kPjOffStage + 4 * 4096;
-constexpr int kPjThreads = 192;
+constexpr uint32_t kPjBytesA = kPjM * kPjK * 2;
+// Shared memory for tiles of `columns` columns: the ring of slabs, mbarriers | TMEM slot | abort flag, output staging
+// [4 warps][32 rows][128 B] (swizzled).
+constexpr int kPjMaxStages = 8;
+constexpr uint32_t kPjBars = 256, kPjStaging = 4 * 4096;
+__host__ __device__ constexpr uint32_t pj_stage_bytes(int columns) { return kPjBytesA + (uint32_t)columns * kPjK * 2; }
+__host__ __device__ constexpr int pj_stages(int columns) { return columns == 64 ? kPjMaxStages : (columns == 128 ? 6 : (columns == 192 ? 5 : 4)); }
+__host__ __device__ constexpr uint32_t pj_smem(int columns) { return pj_stages(columns) * pj_stage_bytes(columns) + kPjBars + kPjStaging; }
+constexpr uint32_t kPjSmemMax = pj_smem(64) > pj_smem(192) ? pj_smem(64) : pj_smem(192);
 
 __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *m, uint64_t *bar, int c0, int c1) {
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
@@ -43,7 +47,8 @@ struct ProjArgs {
     int n_blocks;                                 // 64-column blocks of all roles together (3 H for Q, K, V)
     int x_heads;                                  // 0: X is [B][T][dx] (3-D tensor map); 1: X is in the attention layout
     int pos_t, pos_h, pos_b;                      //    [B][H_in][T][64] (4-D map, these coordinate slots), dx = H_in * 64
-    int tiles_per_seq, n_tiles_n, n_tiles;        // 128-token tiles per sequence, 192-column tiles, all tiles
+    int columns;                                  // output columns per tile: 64, 128, 192 or 256
+    int tiles_per_seq, n_tiles_n, n_tiles;        // 128-token tiles per sequence, column tiles, all tiles
     long long qs[3], ks[3], vs[3];                // element strides (b, h, t) of the three outputs
     __nv_bfloat16 *Q, *K, *V;
     const int *lengths;
@@ -70,8 +75,12 @@ template <bool ZERO>
 __global__ void __launch_bounds__(kPjThreads, 1) k_project_qkv(ProjArgs a, const __grid_constant__ CUtensorMap tmX,
                                                                const __grid_constant__ CUtensorMap tmW) {
     extern __shared__ __align__(1024) uint8_t smem[];
-    uint64_t *full = reinterpret_cast<uint64_t *>(smem + kPjOffBar), *empty = full + kPjStages;
-    uint64_t *acc_full = empty + kPjStages, *acc_empty = acc_full + 2;
+    // (one kernel for all widths: a layer runs it twice, at different widths, and instances of their own cost it 5 us a pass in
+    // instruction cache misses: B16 H8 T1024, new inputs each pass, 91 us against 86)
+    const int N = a.columns, n_stages = pj_stages(N), tile_blocks = N >> 6;
+    const uint32_t stage_bytes = pj_stage_bytes(N);
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem + n_stages * stage_bytes), *empty = full + kPjMaxStages;
+    uint64_t *acc_full = empty + kPjMaxStages, *acc_empty = acc_full + 2;
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(acc_empty + 2);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -80,7 +89,7 @@ __global__ void __launch_bounds__(kPjThreads, 1) k_project_qkv(ProjArgs a, const
         return;
     }
     if (tid == 0) {
-        for (int s = 0; s < kPjStages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
+        for (int s = 0; s < n_stages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
         for (int s = 0; s < 2; ++s) { mbar_init(&acc_full[s], 1); mbar_init(&acc_empty[s], 4); }
         *abort_flag = 0;
         fence_barrier_init();
@@ -91,7 +100,7 @@ __global__ void __launch_bounds__(kPjThreads, 1) k_project_qkv(ProjArgs a, const
     // griddepcontrol.wait); nothing in global memory is touched before the previous grid has completed
     // (the trigger comes after this CTA's TMEM allocation: a dependent CTA that allocates TMEM and then waits
     // for this grid must never get the columns a CTA of this grid still needs)
-    if (warp == 1) tmem_alloc(tmem_slot, 512);                 // two accumulators, 192 of 256 columns each
+    if (warp == 1) tmem_alloc(tmem_slot, 512);                 // two accumulators, N of 256 columns each
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -103,16 +112,15 @@ __global__ void __launch_bounds__(kPjThreads, 1) k_project_qkv(ProjArgs a, const
     if (warp == 0) {
         // ---- producer: one lane streams the slabs of every tile of this CTA through the ring ----
         if (lane == 0) {
-            uint32_t it = 0;
+            uint32_t s = 0, ph = 0;                            // stage, parity of its use
             for (int tile = blockIdx.x; tile < a.n_tiles && !*abort_flag; tile += gridDim.x) {
                 const int n = tile % a.n_tiles_n, m = tile / a.n_tiles_n;
                 const int b = m / a.tiles_per_seq, tt = m % a.tiles_per_seq;
                 if (tt * kPjM >= proj_len(a, b)) continue;
-                for (int kb = 0; kb < n_kb; ++kb, ++it) {
-                    const uint32_t s = it % kPjStages, ph = (it / kPjStages) & 1u;
+                for (int kb = 0; kb < n_kb; ++kb) {
                     if (!mbar_wait(&empty[s], ph ^ 1u)) { atomicOr(a.status, kStatusWaitExpired); *abort_flag = 1; break; }
-                    uint8_t *sa = smem + s * kPjStage;
-                    mbar_expect_tx(&full[s], kPjStage);
+                    uint8_t *sa = smem + s * stage_bytes;
+                    mbar_expect_tx(&full[s], stage_bytes);
                     if (a.x_heads) {                           // slab kb = head kb of the attention layout
                         const int t0 = tt * kPjM;
                         tma_load_4d(sa, &tmX, &full[s], 0, a.pos_t == 1 ? t0 : (a.pos_h == 1 ? kb : b),
@@ -120,15 +128,16 @@ __global__ void __launch_bounds__(kPjThreads, 1) k_project_qkv(ProjArgs a, const
                     } else {
                         tma_load_3d(sa, &tmX, &full[s], kb * kPjK, tt * kPjM, b);
                     }
-                    tma_load_2d(sa + kPjBytesA, &tmW, &full[s], kb * kPjK, n * kPjN);
+                    tma_load_2d(sa + kPjBytesA, &tmW, &full[s], kb * kPjK, n * N);
+                    if (++s == (uint32_t)n_stages) { s = 0; ph ^= 1u; }
                 }
             }
         }
     } else if (warp == 1) {
         // ---- MMA issuer: one lane; accumulator (tile count & 1) ----
         if (lane == 0) {
-            constexpr uint32_t kIdesc = umma_idesc_bf16(kPjM, kPjN, 0);
-            uint32_t it = 0, tc = 0;
+            const uint32_t idesc = umma_idesc_bf16(kPjM, N, 0);
+            uint32_t s = 0, ph = 0, tc = 0;
             for (int tile = blockIdx.x; tile < a.n_tiles && !*abort_flag; tile += gridDim.x) {
                 const int m = tile / a.n_tiles_n;
                 const int b = m / a.tiles_per_seq, tt = m % a.tiles_per_seq;
@@ -137,16 +146,16 @@ __global__ void __launch_bounds__(kPjThreads, 1) k_project_qkv(ProjArgs a, const
                 if (!mbar_wait(&acc_empty[acc], aph ^ 1u)) { atomicOr(a.status, kStatusWaitExpired); *abort_flag = 1; break; }
                 tc_fence_after();
                 bool ok = true;
-                for (int kb = 0; kb < n_kb; ++kb, ++it) {
-                    const uint32_t s = it % kPjStages, ph = (it / kPjStages) & 1u;
+                for (int kb = 0; kb < n_kb; ++kb) {
                     if (!mbar_wait(&full[s], ph)) { ok = false; break; }
                     tc_fence_after();
-                    const uint32_t sa = smem_u32(smem + s * kPjStage), sb = sa + kPjBytesA;
+                    const uint32_t sa = smem_u32(smem + s * stage_bytes), sb = sa + kPjBytesA;
 #pragma unroll
                     for (int k = 0; k < kPjK / 16; ++k)
                         umma_bf16(tmem_base + acc * kPjAccCols, umma_desc_sw128(sa + k * 32, 16, 1024),
-                                  umma_desc_sw128(sb + k * 32, 16, 1024), kIdesc, (kb | k) != 0);
+                                  umma_desc_sw128(sb + k * 32, 16, 1024), idesc, (kb | k) != 0);
                     umma_commit(&empty[s]);                    // the stage is free once these products have run
+                    if (++s == (uint32_t)n_stages) { s = 0; ph ^= 1u; }
                 }
                 if (!ok) { atomicOr(a.status, kStatusWaitExpired); *abort_flag = 1; break; }
                 umma_commit(&acc_full[acc]);
@@ -157,7 +166,7 @@ __global__ void __launch_bounds__(kPjThreads, 1) k_project_qkv(ProjArgs a, const
         // ---- drain: warp w reads TMEM lanes 32 (w % 4) .. + 31; thread = one token row ----
         const int quarter = warp & 3;
         const int ew = warp - 2;                               // 0..3: slot in the staging buffers
-        uint4 *stage = reinterpret_cast<uint4 *>(smem + kPjOffStage + ew * 4096);
+        uint4 *stage = reinterpret_cast<uint4 *>(smem + n_stages * stage_bytes + kPjBars + ew * 4096);
         uint32_t tc = 0;
         for (int tile = blockIdx.x; tile < a.n_tiles; tile += gridDim.x) {
             const int n = tile % a.n_tiles_n, m = tile / a.n_tiles_n;
@@ -165,7 +174,7 @@ __global__ void __launch_bounds__(kPjThreads, 1) k_project_qkv(ProjArgs a, const
             const int L = proj_len(a, b);
             if (tt * kPjM >= L) {
                 if (ZERO) {                                    // a tile of padding: no product, 64 columns = one row of 8 x 16 bytes
-                    for (int gc = n * (kPjN / 64); gc < min(a.n_blocks, (n + 1) * (kPjN / 64)); ++gc) {
+                    for (int gc = n * (tile_blocks); gc < min(a.n_blocks, (n + 1) * (tile_blocks)); ++gc) {
                         const int role = gc / a.H, h = gc - role * a.H;
                         const long long *st = role == 0 ? a.qs : (role == 1 ? a.ks : a.vs);
                         __nv_bfloat16 *base = (role == 0 ? a.Q : (role == 1 ? a.K : a.V)) + (long long)b * st[0] + (long long)h * st[1];
@@ -193,14 +202,14 @@ __global__ void __launch_bounds__(kPjThreads, 1) k_project_qkv(ProjArgs a, const
                 break;
             }
             tc_fence_after();
-            const int n_cc = min(kPjN / 64, a.n_blocks - n * (kPjN / 64));   // 64-column blocks of this tile
+            const int n_cc = min(tile_blocks, a.n_blocks - n * (tile_blocks));   // 64-column blocks of this tile
             const int t_end = ZERO ? a.T : L;                  // rows are written up to here
             const uint32_t tacc = tmem_base + ((uint32_t)(quarter * 32) << 16) + acc * kPjAccCols;
             uint32_t ra[64], rb[64];                           // two blocks in flight: the next one loads while
             tmem_ld32_issue(tacc, ra);                         // the current one is converted and stored
             tmem_ld32_issue(tacc + 32, ra + 32);
             auto drain_block = [&](uint32_t (&r)[64], int cc) {
-                const int gc = n * (kPjN / 64) + cc;           // role = gc / H, head = gc % H
+                const int gc = n * (tile_blocks) + cc;           // role = gc / H, head = gc % H
                 const int role = gc / a.H, h = gc - role * a.H;
                 uint32_t pk[32];                               // 64 bf16, two per word
 #pragma unroll
@@ -247,7 +256,7 @@ __global__ void __launch_bounds__(kPjThreads, 1) k_project_qkv(ProjArgs a, const
                 __syncwarp();
             };
 #pragma unroll
-            for (int cc = 0; cc < kPjN / 64; cc += 2) {
+            for (int cc = 0; cc < 4; cc += 2) {
                 if (cc < n_cc) {
                     tmem_ld_wait();
                     tmem_ld_fence32(ra); tmem_ld_fence32(ra + 32);
@@ -334,11 +343,44 @@ static EncodeTiledFnP proj_encode_fn() {
     return fn;
 }
 
-// The instance of the kernel, and its grant of shared memory.
-static auto project_kernel(int zero_pad) { return zero_pad ? k_project_qkv<true> : k_project_qkv<false>; }
-static cudaError_t grant_project(int zero_pad) {
+// Columns per tile for m_tiles token tiles and n_blocks 64-column blocks.  Rounds: tiles of the SM with most of them; a tile's
+// time follows the bytes its slabs bring in (128 rows of X and the columns' rows of Wt), so: the least rounds x (128 + columns),
+// the wider one of equals (fewer reads of X).  Many tiles take 192 or 256, whichever fills the last round better; few take
+// the narrowest that still needs one round, whose drain is short.  us at 64 / 128 / 192 / 256 columns (taken: the least, 192 before):
+// Q, K, V of B16 H8 T1024 61.8 / 36.8 / 26.7 / 26.6, B2 H16 T2048 58.2 / 35.1 / 26.3 / 23.8, B3 H4 T130 4.6 / 5.5 / 5.9 / 6.7,
+// B2 H2 T500 4.0 / 4.9 / 5.3 / 6.2; output matrix of B16 H8 T1024 22.7 / 16.1 / 13.6 / 12.1, B64 H4 T500 14.9 / 12.2 / 13.8 / 10.3,
+// B4 H8 T8192 39.9 / 24.8 / 21.6 / 19.6, B2 H16 T2048 23.3 / 14.7 / 15.1 / 11.0, B4 H8 T512 6.0 / 6.9 / 7.2 / 8.0.
+static int project_columns(long long m_tiles, int n_blocks, long long sms) {
+    int columns = 0;
+    long long rounds = 0;
+    for (int n = 256; n >= 64; n -= 64) {
+        const long long r = (m_tiles * ((n_blocks * 64 + n - 1) / n) + sms - 1) / sms;
+        if (columns == 0 || r * (128 + n) < rounds * (128 + columns)) { columns = n; rounds = r; }
+    }
+    return columns;
+}
+
+// The product of all token tiles with the [n_blocks * 64][dx] weights.  cudaErrorNotSupported: no tensor map for the weights.
+static cudaError_t launch_project(ProjArgs a, const CUtensorMap &tmX, const void *Wt, cudaStream_t st) {
+    const int sms = device_sm_count();
+    a.columns = project_columns((long long)a.B * a.tiles_per_seq, a.n_blocks, sms);
+    a.n_tiles_n = (a.n_blocks * 64 + a.columns - 1) / a.columns;
+    a.n_tiles = a.B * a.tiles_per_seq * a.n_tiles_n;
+    CUtensorMap tmW;
+    const cuuint64_t wdim[2] = {(cuuint64_t)a.dx, (cuuint64_t)a.n_blocks * 64};
+    const cuuint64_t wstr[1] = {(cuuint64_t)a.dx * 2};
+    const cuuint32_t wbox[2] = {kPjK, (cuuint32_t)a.columns}, one2[2] = {1, 1};
+    if (proj_encode_fn()(&tmW, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(Wt), wdim, wstr, wbox, one2,
+                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return cudaErrorNotSupported;
+    auto kernel = a.zero_pad ? k_project_qkv<true> : k_project_qkv<false>;
     static SmemGrant grants[2];
-    return grant_dynamic_smem(project_kernel(zero_pad), grants[zero_pad != 0], kPjSmem);
+    if (cudaError_t e = grant_dynamic_smem(kernel, grants[a.zero_pad != 0], kPjSmemMax)) return e;
+    const cudaError_t e = launch_pdl(kernel, dim3((unsigned)(a.n_tiles < sms ? a.n_tiles : sms)), dim3(kPjThreads), pj_smem(a.columns),
+                                     st, a, tmX, tmW);
+    note_launch();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 size_t project_vpart_floats(int B, int H, int T) { return (size_t)B * ((T + kPjM - 1) / kPjM) * 4 * H * 64; }
@@ -353,49 +395,24 @@ cudaError_t launch_project_qkv(int dtype, int force_simt, int zero_pad, const Ge
     a.B = g.B; a.H = g.H; a.T = g.T; a.dx = dx;
     a.n_blocks = 3 * g.H; a.x_heads = 0; a.pos_t = a.pos_h = a.pos_b = 0;
     a.tiles_per_seq = (g.T + kPjM - 1) / kPjM;
-    a.n_tiles_n = (3 * g.H * 64 + kPjN - 1) / kPjN;
-    a.n_tiles = g.B * a.tiles_per_seq * a.n_tiles_n;
     for (int k = 0; k < 3; ++k) { a.qs[k] = g.qs[k]; a.ks[k] = g.ks[k]; a.vs[k] = g.vs[k]; }
     a.Q = (__nv_bfloat16 *)Q; a.K = (__nv_bfloat16 *)K; a.V = (__nv_bfloat16 *)V;
     a.lengths = g.lengths; a.status = g.status; a.zero_pad = zero_pad;
     a.vpart = vbar ? vpart : nullptr;
     EncodeTiledFnP enc = proj_encode_fn();
     if (dtype == 0 && !force_simt && enc && dx % 8 == 0 && (vbar == nullptr || vpart != nullptr)) {
-        CUtensorMap tmX, tmW;
+        CUtensorMap tmX;
         const cuuint64_t xdim[3] = {(cuuint64_t)dx, (cuuint64_t)g.T, (cuuint64_t)g.B};
         const cuuint64_t xstr[2] = {(cuuint64_t)dx * 2, (cuuint64_t)g.T * dx * 2};
         const cuuint32_t xbox[3] = {kPjK, kPjM, 1}, one3[3] = {1, 1, 1};
-        const cuuint64_t wdim[2] = {(cuuint64_t)dx, (cuuint64_t)3 * g.H * 64};
-        const cuuint64_t wstr[1] = {(cuuint64_t)dx * 2};
-        const cuuint32_t wbox[2] = {kPjK, kPjN}, one2[2] = {1, 1};
-        const bool ok =
-            enc(&tmX, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(X), xdim, xstr, xbox, one3,
+        cudaError_t e = cudaErrorNotSupported;
+        if (enc(&tmX, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(X), xdim, xstr, xbox, one3,
                 CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS &&
-            enc(&tmW, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(Wt), wdim, wstr, wbox, one2,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-        if (ok) {
-            if (cudaError_t e = grant_project(zero_pad)) return e;
-            // both kernels carry a programmatic dependency on their predecessor in the stream
-            cudaLaunchAttribute attr[1];
-            attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-            attr[0].val.programmaticStreamSerializationAllowed = 1;
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3((unsigned)(a.n_tiles < device_sm_count() ? a.n_tiles : device_sm_count()));
-            cfg.blockDim = dim3(kPjThreads);
-            cfg.dynamicSmemBytes = kPjSmem;
-            cfg.stream = st;
-            cfg.attrs = attr;
-            cfg.numAttrs = 1;
-            cudaError_t e = cudaLaunchKernelEx(&cfg, project_kernel(zero_pad), a, tmX, tmW);
-            note_launch();
-            if (e == cudaSuccess) e = cudaGetLastError();
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS)
+            e = launch_project(a, tmX, Wt, st);
+        if (e != cudaErrorNotSupported) {
             if (e != cudaSuccess || vbar == nullptr) return e;
-            cfg.gridDim = dim3((unsigned)(g.B * g.H));
-            cfg.blockDim = dim3(512);
-            cfg.dynamicSmemBytes = 0;
-            e = cudaLaunchKernelEx(&cfg, k_project_vbar, a, vbar);
+            e = launch_pdl(k_project_vbar, dim3((unsigned)(g.B * g.H)), dim3(512), 0, st, a, vbar);
             note_launch();
             return e != cudaSuccess ? e : cudaGetLastError();
         }
@@ -431,30 +448,16 @@ cudaError_t launch_project_out_dense(const Geom &g, int zero_pad, int dy, const 
     a.B = g.B; a.H = dy / 64; a.T = g.T; a.dx = g.H * 64;
     a.n_blocks = dy / 64; a.x_heads = 1;
     a.tiles_per_seq = (g.T + kPjM - 1) / kPjM;
-    a.n_tiles_n = (dy + kPjN - 1) / kPjN;
-    a.n_tiles = g.B * a.tiles_per_seq * a.n_tiles_n;
     // Y [B][T][dy] seen as [B][dy / 64][T][64]: block stride 64, token stride dy
     const long long ys[3] = {(long long)g.T * dy, 64, dy};
     for (int k = 0; k < 3; ++k) { a.qs[k] = ys[k]; a.ks[k] = ys[k]; a.vs[k] = ys[k]; }
     a.Q = (__nv_bfloat16 *)Y; a.K = nullptr; a.V = nullptr;
     a.lengths = g.lengths; a.status = g.status; a.vpart = nullptr; a.zero_pad = zero_pad;
-    CUtensorMap tmX, tmW;
+    CUtensorMap tmX;
     int pos[3];
     if (!make_rows_map(&tmX, O, g, g.os, kPjM, 1, pos)) return cudaErrorNotSupported;
     a.pos_t = pos[0]; a.pos_h = pos[1]; a.pos_b = pos[2];
-    const cuuint64_t wdim[2] = {(cuuint64_t)a.dx, (cuuint64_t)dy};
-    const cuuint64_t wstr[1] = {(cuuint64_t)a.dx * 2};
-    const cuuint32_t wbox[2] = {kPjK, kPjN}, one2[2] = {1, 1};
-    if (enc(&tmW, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(Wot), wdim, wstr, wbox, one2,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-        return cudaErrorNotSupported;
-    if (cudaError_t e = grant_project(zero_pad)) return e;
-    const int sms = device_sm_count();
-    cudaError_t e = launch_pdl(project_kernel(zero_pad), dim3((unsigned)(a.n_tiles < sms ? a.n_tiles : sms)), dim3(kPjThreads), kPjSmem,
-                               st, a, tmX, tmW);
-    note_launch();
-    return e != cudaSuccess ? e : cudaGetLastError();
+    return launch_project(a, tmX, Wot, st);
 }
 
 }  // namespace psattn

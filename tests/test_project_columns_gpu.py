@@ -1,0 +1,39 @@
+"""The projections and the dense output matrix at the sizes where their tiles change width (64, 128, 192 or 256 columns, by how many
+tiles the call has): whole and part-empty column tiles, sequences that end within a tile, at its edge and before it."""
+import math
+
+import pytest
+import torch
+
+from paper_2106_09236_b200 import binding as ps
+
+pytestmark = pytest.mark.gpu
+
+
+# few tiles (64 columns); a first round filled at 64, 128, 192, 256 columns; several rounds; one block, three, nine and 48 per product
+@pytest.mark.parametrize("B,H,T", [(1, 1, 1), (3, 4, 130), (6, 8, 129), (10, 8, 128), (4, 8, 512), (32, 4, 511), (70, 3, 257), (150, 1, 127),
+                                   (2, 16, 2048), (24, 8, 1024)])
+def test_projections_and_output_matrix_by_number_of_tiles(B, H, T):
+    gen = torch.Generator(device="cuda").manual_seed(B * T)
+    d = H * 64
+    lengths = torch.randint(0, T + 1, (B,), generator=gen, device="cuda", dtype=torch.int32)
+    lengths[0] = T
+    X = torch.randn((B, T, d), generator=gen, device="cuda").bfloat16()
+    Wt, Wot = ((torch.randn((n, d), generator=gen, device="cuda") / math.sqrt(d)).bfloat16() for n in (3 * d, d))
+    valid = (torch.arange(T, device="cuda") < lengths.view(B, 1)).unsqueeze(-1)
+    plan = ps.Plan(B, H, T, c=5.0)
+    # products of unit variance: half a bf16 ulp (2^-9 of the value, 2^-8 at worst after the tie), and d fp32 additions of terms
+    # of 1 / sqrt(d), below 1e-5 for d <= 1024
+    near = lambda got, want: bool(((got.double() - want).abs() <= 2.0 ** -8 * want.abs() + 1e-4).all())
+    want = torch.where(valid, X.double() @ Wt.double().T, 0.).view(B, T, 3, H, 64)
+    fresh = plan.psattn_project_qkv(X, Wt.view(3, d, d), lengths)
+    given = [torch.full((B, H, T, 64), -7.0, dtype=torch.bfloat16, device="cuda") for _ in range(3)]
+    plan.psattn_project_qkv(X, Wt.view(3, d, d), lengths, *given)
+    for r in range(3):
+        assert near(fresh[r].permute(0, 2, 1, 3), want[:, :, r])
+        assert bool((given[r] == torch.where(valid.view(B, 1, T, 1), fresh[r], -7.0)).all())
+    O = torch.where(valid.view(B, 1, T, 1), fresh[0], 0.)
+    Y = plan.psattn_project_out(O, None, lengths, Wot)
+    assert near(Y, O.permute(0, 2, 1, 3).reshape(B, T, d).double() @ Wot.double().T)
+    assert plan.psattn_read_status() == 0
+    plan.close()
