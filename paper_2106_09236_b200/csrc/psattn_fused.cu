@@ -60,8 +60,7 @@ __host__ __device__ inline size_t fused_arrays_bytes(int m_floats, int T) { retu
 // SPLIT: the unit is shared by the a.split > 1 CTAs of a thread-block cluster.
 // MODE: all steps, or from step (c) on with M~ in global memory (sequences too long for resident keys), or steps (d)+(e).
 // kFront: steps (a)-(c) and the fill with the query's own value row, for selections too long for step (d) here (k_attend_tc comes
-// behind).  u = L / 2, us per call with measure and selection as kernels of their own and the fill beside them / this: B12 H8 T960
-// 62 / 59, B32 H4 T256 28 / 19, B16 H8 T512 32 / 28, B1 H4 T200 22 / 16 (and the attention started while this kernel drains).
+// behind, started while this kernel drains).
 enum FusedMode { kAllSteps = 0, kGivenMeasure = 1, kGivenSet = 2, kFront = 3 };
 constexpr int kFusedSelectKeys = kSelectMaxSlots * (kFusedThreads - 32);       // longest sequence of the block-wide selection
 
@@ -318,6 +317,12 @@ bool fused_from_measure_supported(const Geom &g, const void *K, const void *V) {
            attend64_supported(g, K, V, g.u_max, 1);
 }
 
+// kFront: the longest units of one CTA each.  u = L / 2, us per call on rotating inputs with measure and selection as kernels of
+// their own and the fill beside them / in this kernel: B1 H4 T200 20.1 / 15.6, B32 H4 T256 27.6 / 19.0, B20 H4 T300 26.1 / 22.1, B16 H8 T512
+// 33.3 / 28.9, B12 H8 T700 37.0 / 35.7, B32 H4 T700 42.3 / 41.9; units shared by a cluster B8 H4 T1200 38.6 / 34.8, B2 H8 T1400 41.7 /
+// 42.3.  Long units of one CTA each go the other way, since the kernels of their own share them out over all SMs: B12 H8 T800 46.8 /
+// 48.6, T960 55.9 / 57.8, B16 H8 T960 61.6 / 62.1, B40 H4 T1079 113.7 / 130.5: these are refused here.
+constexpr int kFrontWholeUnit = 768;
 static cudaError_t launch_fused(int mode, const Geom &g, int U_max, int own_v, const void *Q, const void *K, const void *V,
                                 const int *sidx, void *O, int *sel, float *M_out, const int *sel_in, const float *M_in,
                                 cudaStream_t st) {
@@ -371,6 +376,7 @@ static cudaError_t launch_fused(int mode, const Geom &g, int U_max, int own_v, c
         if (cudaError_t e = grant_dynamic_smem(kernels[mode][x], grants[mode][x], x == 2 ? kFusedHalfSmem : kFusedMaxSmem, x == 2)) return e;
     if (cudaError_t e = grant_dynamic_smem(kernels[0][1], grants[0][1], kFusedMaxSmem)) return e;        // (asked by fused_split)
     a.split = half ? 1 : fused_split(g, mode);
+    if (mode == kFront && a.split == 1 && g.T > kFrontWholeUnit) return cudaErrorNotSupported;
     // launched with programmatic stream serialization: the kernel may be scheduled while the previous
     // kernel of the stream drains; it orders itself with griddepcontrol.wait before its first read
     cudaError_t e = launch_split(kernels[mode][half ? 2 : a.split > 1], (unsigned)(g.B * g.H), a.split,
@@ -390,6 +396,7 @@ cudaError_t launch_forward_fused(const Geom &g, int U_max, int own_v, const void
                         sel, M_out, sel_in, M_in, st);
 }
 
+// Steps (a)-(c) and the own-value fill (kFront).  cudaErrorNotSupported as above, and long units of one CTA each.
 cudaError_t launch_front_fused(const Geom &g, int U_max, const void *Q, const void *K, const void *V, const int *sidx, void *O,
                                int *sel, float *M_out, cudaStream_t st) {
     return launch_fused(kFront, g, U_max, 1, Q, K, V, sidx, O, sel, M_out, nullptr, nullptr, st);

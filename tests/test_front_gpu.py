@@ -12,7 +12,7 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("B,H,T,shortest,form", [
     (1, 4, 203, 203, "1,3,512"), (2, 3, 515, 1, "1,3,512"), (40, 2, 700, 1, "0,3,512"), (80, 2, 200, 1, "0,3,256"), (150, 2, 129, 64, "0,3,256"),
-    (40, 4, 1079, 2, "0,3,512"),
+    (40, 4, 768, 2, "0,3,512"), (1, 4, 1079, 1079, "1,3,512"), (40, 4, 769, 2, None), (40, 4, 1079, 2, None),
 ])
 def test_front(B, H, T, shortest, form):
     gen = torch.Generator(device="cuda")
@@ -25,7 +25,10 @@ def test_front(B, H, T, shortest, form):
     O = torch.full((B, H, T, 64), float("nan"), dtype=torch.bfloat16, device="cuda")
     M = torch.empty((B, H, T), device="cuda")
     (_, sel), names = launched(lambda: plan.psattn_forward(q, k, v, ln, idx, O=O, M_out=M))
-    assert any(x.startswith("k_forward_fused<" + form) for x in names) and "k_attend_tc" in names and len(names) <= 3
+    if form is None:                                         # long units of a CTA each: kernels of their own
+        assert not any(x.startswith("k_forward_fused") for x in names) and "k_attend_tc" in names
+    else:
+        assert any(x.startswith("k_forward_fused<" + form) for x in names) and "k_attend_tc" in names and len(names) <= 3
     assert plan.psattn_read_status() == 0
     torch.testing.assert_close(M, plan.psattn_measure(q, k, ln, idx), atol=1e-5, rtol=1e-5)
     assert torch.equal(sel, plan.psattn_select(M, ln))
